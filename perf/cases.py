@@ -71,7 +71,7 @@ def draw(rng):
     if kind == "batch":
         return {"kind": kind, "n": _log(rng, 64, 20_000), "d": d, "k": _log(rng, 256, 8192)}
     if kind == "pruned":
-        n = _log(rng, 300_000, 5_000_000)
+        n = _log(rng, 300_000, 2_000_000)
         return {"kind": kind, "n": n, "d": rng.choice([256, 320, 384, 512]), "k": int(rng.uniform(2.0, 4.0) * math.sqrt(n))}
     if kind == "project":
         n = _log(rng, 20_000, 1_000_000)
@@ -226,9 +226,10 @@ def _inputs(case, seed):
         x = _embeddings(n, d, case["k"], g, rotated=False).to(torch.bfloat16)
         c, a = _settled(x, case["k"], 4, g)
         return {"x": x, "C": c, "prev": a.int()}
+    if kind == "batch":  # the index was built on other points of the same kind
+        x = _embeddings(n + 16 * case["k"], d, _comps(case), g)
+        return {"x": x[:n].clone(), "C": _settled(x[n:], case["k"], 2, g)[0]}
     x = _embeddings(n, d, _comps(case), g)
-    if kind == "batch":
-        return {"x": x, "C": _embeddings(case["k"], d, case["k"], g) * 0.9}
     if kind == "project":
         p = torch.linalg.qr(torch.randn(d, d, generator=torch.Generator().manual_seed(seed)))[0][:, :case["d_out"]]
         return {"x": x, "mean": x[: 1 << 16].mean(0), "P": p.contiguous().cuda()}
