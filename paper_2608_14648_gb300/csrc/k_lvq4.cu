@@ -392,68 +392,6 @@ __global__ void __launch_bounds__(256) assign_lvq4_simt_kernel(const uint32_t *_
     }
 }
 
-// Fixed-point weights in the cluster-sorted order (position q: member perm[q]).
-__global__ void lvq4_q_kernel(const float4 *__restrict__ fac, const int32_t *__restrict__ perm,
-                              const int64_t *__restrict__ offsets, int k, int e, uint32_t *__restrict__ sq,
-                              int64_t *__restrict__ bq) {
-    const int64_t nval = offsets[k];
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nval; q += (int64_t)gridDim.x * blockDim.x) {
-        const float4 f = fac[perm[q]];
-        sq[q] = (uint32_t)fixed_rint(f.x, e);
-        bq[q] = fixed_rint(f.y, e);
-    }
-}
-
-// Rows that do not suit the streamed sums: one warp per run of 128 sorted
-// positions, lane = nibble word (32 words per pass), 8 int64 accumulators per
-// lane, flushed with atomics when the cluster changes.  T[c][d] += Bq.
-__global__ void chunk_sum_lvq4_kernel(const uint32_t *__restrict__ codes, const uint32_t *__restrict__ sq,
-                                      const int64_t *__restrict__ bq, int d, const int32_t *__restrict__ perm,
-                                      const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k,
-                                      unsigned long long *__restrict__ T) {
-    const int lane = threadIdx.x & 31;
-    const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nval = offsets[k];
-    const int64_t q0 = gw * 128;
-    if (q0 >= nval) return;
-    const int cnt = (int)((nval - q0) < 128 ? (nval - q0) : 128);
-    const int W = lvq4_words(d);
-    for (int w0 = 0; w0 < W; w0 += 32) {
-        const int w = w0 + lane;
-        unsigned long long acc[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[j] = 0ull;
-        int64_t us = 0;
-        int cur = scl[q0];
-        auto flush = [&](int c) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int col = 8 * w + j;
-                if (w < W && col < d && acc[j]) atomicAdd(T + (int64_t)c * (d + 1) + col, acc[j]);
-                acc[j] = 0ull;
-            }
-            if (w0 == 0 && lane == 0 && us) atomicAdd(T + (int64_t)c * (d + 1) + d, (unsigned long long)us);
-            us = 0;
-        };
-        for (int i = 0; i < cnt; ++i) {
-            const int64_t q = q0 + i;
-            const int c = scl[q];
-            if (c != cur) {
-                flush(cur);
-                cur = c;
-            }
-            const uint32_t s = sq[q];
-            if (w0 == 0) us += bq[q];
-            if (w < W) {
-                const uint32_t v = codes[(int64_t)perm[q] * W + w];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[j] += (unsigned long long)s * ((v >> (4 * j)) & 15u);
-            }
-        }
-        flush(cur);
-    }
-}
-
 // c_i = (T_i + U) f, f = 2^-e / count formed once per cluster (one block each).
 __global__ void finalize_lvq4_kernel(const int64_t *__restrict__ partial, const int64_t *__restrict__ counts, int k,
                                      int d, int e, float *__restrict__ C) {
@@ -553,25 +491,6 @@ cudaError_t launch_assign_lvq4_simt(const uint32_t *codes, const float4 *fac, in
     }
     assign_lvq4_simt_kernel<<<(unsigned)((n + 255) / 256), 256, smem, st>>>(codes, fac, n, d, yw, info, k, assign,
                                                                             dist);
-    return launched();
-}
-
-cudaError_t launch_lvq4_q(const float4 *fac, const int32_t *perm, const int64_t *offsets, int k, int64_t n, int e,
-                          uint32_t *sq, int64_t *bq, cudaStream_t st) {
-    int64_t blocks = (n + 255) / 256;
-    if (blocks > 152 * 8) blocks = 152 * 8;
-    lvq4_q_kernel<<<(unsigned)(blocks < 1 ? 1 : blocks), 256, 0, st>>>(fac, perm, offsets, k, e, sq, bq);
-    return launched();
-}
-
-cudaError_t launch_chunk_sum_lvq4(const uint32_t *codes, const uint32_t *sq, const int64_t *bq, int64_t n, int d,
-                                  const int32_t *perm, const int32_t *scl, const int64_t *offsets, int k, int64_t *T,
-                                  cudaStream_t st) {
-    if (n == 0) return cudaSuccess;
-    (void)scl;
-    const int64_t warps = (n + 127) / 128;
-    chunk_sum_lvq4_kernel<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, st>>>(
-        codes, sq, bq, d, perm, scl, offsets, k, reinterpret_cast<unsigned long long *>(T));
     return launched();
 }
 

@@ -105,45 +105,49 @@ cudaError_t launch_objective(const void *X, int x_is_bf16, int64_t n, int d, con
     return launched();
 }
 
-__global__ void sum_double_kernel(const double *__restrict__ in, int64_t count,
-                                  double *__restrict__ out) {
-    __shared__ double sh[256];
-    double s = 0.0;
-    for (int64_t i = threadIdx.x; i < count; i += blockDim.x) s += in[i];
-    sh[threadIdx.x] = s;
+// Block sum in a fixed order: a shuffle tree in each warp, the warps' sums in
+// order by thread 0 (its return value; the others' is not used).
+__device__ __forceinline__ double block_sum(double s) {
+    __shared__ double wsum[32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = s;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int i = 0; i < (int)blockDim.x; ++i) t += sh[i];
-        *out = t;
-    }
+    double t = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += wsum[w];
+    return t;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(1024) sum_to_double_kernel(const T *__restrict__ in, int64_t count,
+                                                             double *__restrict__ out) {
+    double s = 0.0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
+        s += (double)in[i];
+    s = block_sum(s);
+    if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
 cudaError_t launch_sum_double(const double *in, int64_t count, double *out, cudaStream_t st) {
-    sum_double_kernel<<<1, 256, 0, st>>>(in, count, out);
+    sum_to_double_kernel<double><<<1, 512, 0, st>>>(in, count, out);
     return launched();
 }
 
-__global__ void sum_float_partial_kernel(const float *__restrict__ in, int64_t count,
-                                         double *__restrict__ partials) {
-    __shared__ double sh[256];
-    double s = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count;
-         i += (int64_t)gridDim.x * blockDim.x)
-        s += (double)in[i];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int i = 0; i < (int)blockDim.x; ++i) t += sh[i];
-        partials[blockIdx.x] = t;
+// A block's 1024 threads read 64 values each in about the time that a second
+// launch costs, so up to SUM1_MAX values take one block and no partials.  (The
+// serial sums over 256 threads this replaces took 11 us a kernel, two kernels
+// for each iteration's objective whatever n.)
+constexpr int64_t SUM1_MAX = 65536;
+cudaError_t launch_sum_float(const float *in, int64_t count, double *partials, int nblk, double *out,
+                             cudaStream_t st) {
+    if (count <= SUM1_MAX) {
+        sum_to_double_kernel<float><<<1, 1024, 0, st>>>(in, count, out);
+        return launched();
     }
-}
-
-cudaError_t launch_sum_float_to_double(const float *in, int64_t count, double *partials,
-                                       int nblk, cudaStream_t st) {
-    sum_float_partial_kernel<<<nblk, 256, 0, st>>>(in, count, partials);
-    return launched();
+    sum_to_double_kernel<float><<<nblk, 512, 0, st>>>(in, count, partials);
+    const cudaError_t e = launched();
+    return e == cudaSuccess ? launch_sum_double(partials, nblk, out, st) : e;
 }
 
 // --------------------------------------------------------------- projection

@@ -2,7 +2,7 @@
 // codes summed exactly in the code domain and, for 1-bit codes, the fused
 // decode-average of Section 3.1 "RabitQ").
 //
-// The cluster-sorted member order is cut into runs of RS_ROWS positions and
+// The cluster-sorted member order is cut into runs of up to RS_ROWS positions and
 // each of the RS_CW warps of a CTA owns one run.  A warp gathers the member
 // rows of its run with cp.async.bulk (global -> shared, completion counted in
 // bytes on one mbarrier per slot) into its own ring of slots, R rows per slot,
@@ -30,7 +30,7 @@ namespace {
 
 constexpr int RS_CW = 8;                      // warps per CTA, one run each
 constexpr int RS_THREADS = 32 * RS_CW;
-constexpr int RS_ROWS = 128;                  // sorted positions per consumer warp
+constexpr int RS_ROWS = SUM_RUN_MAX;          // sorted positions per consumer warp, at most
 constexpr int RS_MAX_SLOTS = 16;              // ring slots per consumer warp
 constexpr int RS_RING_BYTES = 96 * 1024;      // all rings of a CTA
 constexpr unsigned long long RS_WAIT_NS = 2000000000ull;
@@ -88,15 +88,16 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t
         : "memory");
 }
 
-__device__ __forceinline__ int run_len(int64_t nval, int64_t q0) {
+__device__ __forceinline__ int run_len(int64_t nval, int64_t q0, int run) {
     const int64_t r = nval - q0;
-    return r <= 0 ? 0 : (r >= RS_ROWS ? RS_ROWS : (int)r);
+    return r <= 0 ? 0 : (r >= run ? run : (int)r);
 }
 
 // Shared-memory layout of one CTA: ns slots per warp, each holding up to R
 // rows of rb bytes (R <= 32: one row per lane).
 struct RingLayout {
     int ns, R, rb;
+    int run;  // sorted positions per warp (sum_run)
     int lsu;  // 1: rows gathered by 16-byte cp.async per lane (ns == LSU_STAGES)
     __host__ __device__ size_t slot_bytes() const { return (size_t)R * rb; }
     __host__ __device__ size_t ring_bytes() const { return (size_t)RS_CW * ns * slot_bytes(); }
@@ -120,8 +121,8 @@ __device__ __forceinline__ void ring_run(const uint8_t *__restrict__ rows,
     uint64_t *full = reinterpret_cast<uint64_t *>(rs_smem + L.ring_bytes()) + warp * L.ns;
     int32_t *sperm = reinterpret_cast<int32_t *>(rs_smem + L.ring_bytes() + (size_t)RS_CW * L.ns * 8) +
                      warp * RS_ROWS;
-    const int64_t q0 = ((int64_t)blockIdx.x * RS_CW + warp) * RS_ROWS;
-    const int cnt = run_len(nval, q0);
+    const int64_t q0 = ((int64_t)blockIdx.x * RS_CW + warp) * L.run;
+    const int cnt = run_len(nval, q0, L.run);
     if (cnt == 0) return;  // warp-uniform; no other warp waits on this one
     const uint32_t rb = (uint32_t)L.rb;
     if (lane == 0)
@@ -186,8 +187,8 @@ __device__ __forceinline__ void ring_run_lsu(const uint8_t *__restrict__ rows,
     uint8_t *ring = rs_smem + (size_t)warp * LSU_STAGES * sb;
     int32_t *sperm = reinterpret_cast<int32_t *>(rs_smem + L.ring_bytes() + (size_t)RS_CW * L.ns * 8) +
                      warp * RS_ROWS;
-    const int64_t q0 = ((int64_t)blockIdx.x * RS_CW + warp) * RS_ROWS;
-    const int cnt = run_len(nval, q0);
+    const int64_t q0 = ((int64_t)blockIdx.x * RS_CW + warp) * L.run;
+    const int cnt = run_len(nval, q0, L.run);
     if (cnt == 0) return;
     for (int i = lane; i < cnt; i += 32) sperm[i] = perm[q0 + i];
     __syncwarp();
@@ -247,13 +248,21 @@ struct FloatCons {
     int cnt;
     __device__ __forceinline__ void flush(int c, int lane) {
 #pragma unroll
-        for (int t = 0; t < NF; ++t)
+        for (int t = 0; t < NF; ++t) {
+            const int col = 4 * (lane + 32 * t);  // d % 4 == 0: all four columns or none
+            if (col < d) {
+                ACC *dst = S + (int64_t)c * stride + col;
+                if constexpr (sizeof(ACC) == 4) {
+                    atomicAdd(reinterpret_cast<float4 *>(dst),
+                              make_float4(acc[4 * t], acc[4 * t + 1], acc[4 * t + 2], acc[4 * t + 3]));
+                } else {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int col = 4 * (lane + 32 * t) + u;
-                if (col < d) atomicAdd(S + (int64_t)c * stride + col, (ACC)acc[4 * t + u]);
-                acc[4 * t + u] = 0.0f;
+                    for (int u = 0; u < 4; ++u) atomicAdd(dst + u, (ACC)acc[4 * t + u]);
+                }
             }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc[4 * t + u] = 0.0f;
+        }
     }
     __device__ __forceinline__ void start(int64_t q0_, int cnt_, int lane) {
         q0 = q0_;
@@ -305,7 +314,7 @@ __global__ void __launch_bounds__(RS_THREADS) ring_sum_float_kernel(
     const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k, ACC *__restrict__ S,
     int64_t stride, RingLayout L, int32_t *flag) {
     const int64_t nval = offsets[k];
-    if ((int64_t)blockIdx.x * RS_CW * RS_ROWS >= nval) return;
+    if ((int64_t)blockIdx.x * RS_CW * L.run >= nval) return;
     FloatCons<BF16, ACC, NF> cons;
     cons.scl = scl;
     cons.S = S;
@@ -330,7 +339,7 @@ __global__ void __launch_bounds__(RS_THREADS) ring_sum_float_kernel(
 // bits over a run (at most TR_ROWS = 128 weights of at most 2^24) and flush
 // into the int64 accumulators when the cluster changes and at the run's end.
 constexpr int TR_WARPS = 8;
-constexpr int TR_ROWS = 128;
+constexpr int TR_ROWS = SUM_RUN_MAX;
 
 // Lane r holds row r of a 32 x 32 bit matrix (bit i = column i); afterwards
 // lane i holds column i (bit r = row r).  Stage j exchanges j-bit groups with
@@ -367,12 +376,6 @@ __device__ __forceinline__ uint32_t table_sum(uint32_t tbase, uint32_t t) {
     return s;
 }
 
-template <int W4>
-__device__ __forceinline__ uint32_t word_of(const uint4 (&x)[W4], int w) {
-    const uint4 v = x[w >> 2];
-    return (w & 3) == 0 ? v.x : (w & 3) == 1 ? v.y : (w & 3) == 2 ? v.z : v.w;
-}
-
 // PF: the next chunk's words load into registers while this one is summed
 // (two CTAs per SM); without it three CTAs per SM hide the loads instead.
 // Measured on GB300 (kernel time per 1M points): d = 768 81 us with PF
@@ -380,18 +383,23 @@ __device__ __forceinline__ uint32_t word_of(const uint4 (&x)[W4], int w) {
 template <int W4>
 constexpr bool tr_prefetch() { return W4 <= 6; }
 
-template <int W4, bool PF>
+// Rows of WT words; block row blockIdx.y takes the words w0 = 4 W4 blockIdx.y
+// .. + 4 W4 - 1 of every row.  VEC: words a load brings, 4 when the rows are
+// 16-byte aligned and the block rows share their words evenly, else 2 or 1
+// (words past WT are then zero and add nothing).
+template <int W4, int VEC, bool PF>
 __global__ void __launch_bounds__(TR_WARPS * 32, PF ? 2 : 3) rbq1_sum_table_kernel(
-    const uint32_t *__restrict__ codes, const int64_t *__restrict__ fqs, int d,
+    const uint32_t *__restrict__ codes, int WT, const float *__restrict__ F, int e, int d,
     const int32_t *__restrict__ perm, const int32_t *__restrict__ scl,
-    const int64_t *__restrict__ offsets, int k, unsigned long long *__restrict__ T) {
+    const int64_t *__restrict__ offsets, int k, unsigned long long *__restrict__ T, int run) {
     constexpr int W = 4 * W4;
+    const int w0 = W * blockIdx.y, nw = min(W, WT - w0);
     __shared__ __align__(1024) uint32_t tabs[TR_WARPS][256];  // 7 x 32 entries used per warp
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t nval = offsets[k];
-    const int64_t q0 = ((int64_t)blockIdx.x * TR_WARPS + warp) * TR_ROWS;
+    const int64_t q0 = ((int64_t)blockIdx.x * TR_WARPS + warp) * run;
     if (q0 >= nval) return;  // warp-uniform; no other warp waits on this one
-    const int cnt = (int)min((int64_t)TR_ROWS, nval - q0);
+    const int cnt = (int)min((int64_t)run, nval - q0);
     uint32_t *tab = tabs[warp];
     const uint32_t tbase = (uint32_t)__cvta_generic_to_shared(tab);
     uint32_t acc[W];
@@ -403,40 +411,54 @@ __global__ void __launch_bounds__(TR_WARPS * 32, PF ? 2 : 3) rbq1_sum_table_kern
         unsigned long long *Tc = T + (int64_t)c * (d + 1);
 #pragma unroll
         for (int w = 0; w < W; ++w) {
-            const int col = 32 * w + lane;
+            const int col = 32 * (w0 + w) + lane;
             if (col < d && acc[w]) atomicAdd(Tc + col, (unsigned long long)acc[w]);
             acc[w] = 0;
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) usum += __shfl_xor_sync(0xffffffffu, usum, o);
-        if (lane == 0 && usum) atomicAdd(Tc + d, usum);
+        if (lane == 0 && usum && w0 == 0) atomicAdd(Tc + d, usum);
         usum = 0;
     };
     // chunk ch: this lane's row words, cluster id (-1 past the run) and weight
-    auto load = [&](int ch, uint4 (&x)[W4], int &cl, uint32_t &f) {
+    auto load = [&](int ch, uint32_t (&x)[W], int &cl, uint32_t &f) {
         const int i = ch * 32 + lane;
         if (i < cnt) {
             const int64_t q = q0 + i;
             const int64_t row = __ldg(perm + q);
             cl = __ldg(scl + q);
-            f = (uint32_t)__ldg(fqs + q);  // Fq <= 2^24
-            const uint4 *src = reinterpret_cast<const uint4 *>(codes + row * W);
+            f = (uint32_t)fixed_rint(__ldg(F + row), e);  // Fq <= 2^24
+            const uint32_t *src = codes + row * WT + w0;
 #pragma unroll
-            for (int g = 0; g < W4; ++g) x[g] = __ldg(src + g);
+            for (int w = 0; w < W; w += VEC) {
+                if constexpr (VEC == 4) {
+                    const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src + w));
+                    x[w] = v.x;
+                    x[w + 1] = v.y;
+                    x[w + 2] = v.z;
+                    x[w + 3] = v.w;
+                } else if constexpr (VEC == 2) {
+                    const uint2 v = w < nw ? __ldg(reinterpret_cast<const uint2 *>(src + w)) : make_uint2(0u, 0u);
+                    x[w] = v.x;
+                    x[w + 1] = v.y;
+                } else {
+                    x[w] = w < nw ? __ldg(src + w) : 0u;
+                }
+            }
         } else {
             cl = -1;
             f = 0;
 #pragma unroll
-            for (int g = 0; g < W4; ++g) x[g] = make_uint4(0u, 0u, 0u, 0u);
+            for (int w = 0; w < W; ++w) x[w] = 0u;
         }
     };
     const int nch = (cnt + 31) >> 5;
-    uint4 x[W4];
+    uint32_t x[W];
     int cl;
     uint32_t f;
     if (PF) load(0, x, cl, f);
     for (int ch = 0; ch < nch; ++ch) {
-        uint4 xn[W4];
+        uint32_t xn[W];
         int cln = -1;
         uint32_t fn = 0;
         if (PF) {
@@ -471,7 +493,8 @@ __global__ void __launch_bounds__(TR_WARPS * 32, PF ? 2 : 3) rbq1_sum_table_kern
                 }
                 __syncwarp();
 #pragma unroll
-                for (int w = 0; w < W; ++w) acc[w] += table_sum(tbase, bit_transpose32(word_of(x, w), lane));
+                for (int w = 0; w < W; ++w)
+                    if (VEC == 4 || w < nw) acc[w] += table_sum(tbase, bit_transpose32(x[w], lane));
                 const unsigned rest = __ballot_sync(0xffffffffu, valid && cl > c);
                 if (!rest) break;
                 c = __shfl_sync(0xffffffffu, cl, __ffs(rest) - 1);
@@ -489,12 +512,12 @@ __global__ void __launch_bounds__(TR_WARPS * 32, PF ? 2 : 3) rbq1_sum_table_kern
                 if (lane == r) usum += fr;
                 const uint32_t lm = 1u << lane;
 #pragma unroll
-                for (int w = 0; w < W; ++w) add_if_bit(acc[w], __shfl_sync(0xffffffffu, word_of(x, w), r), lm, fr);
+                for (int w = 0; w < W; ++w) add_if_bit(acc[w], __shfl_sync(0xffffffffu, x[w], r), lm, fr);
             }
         }
         if (PF) {
 #pragma unroll
-            for (int g = 0; g < W4; ++g) x[g] = xn[g];
+            for (int w = 0; w < W; ++w) x[w] = xn[w];
             cl = cln;
             f = fn;
         }
@@ -590,7 +613,7 @@ __global__ void __launch_bounds__(RS_THREADS) ring_sum_sq8_kernel(
     const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k,
     unsigned long long *__restrict__ S, RingLayout L, int32_t *flag) {
     const int64_t nval = offsets[k];
-    if ((int64_t)blockIdx.x * RS_CW * RS_ROWS >= nval) return;
+    if ((int64_t)blockIdx.x * RS_CW * L.run >= nval) return;
     Sq8Cons<NG> cons;
     cons.scl = scl;
     cons.S = S;
@@ -608,12 +631,12 @@ template <int NG>
 __global__ void __launch_bounds__(RS_THREADS) direct_sum_sq8_kernel(
     const uint8_t *__restrict__ codes, int d, const int32_t *__restrict__ perm,
     const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k,
-    unsigned long long *__restrict__ S) {
+    unsigned long long *__restrict__ S, int run) {
     __shared__ int32_t sperm_all[RS_CW][RS_ROWS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t nval = offsets[k];
-    const int64_t q0 = ((int64_t)blockIdx.x * RS_CW + warp) * RS_ROWS;
-    const int cnt = run_len(nval, q0);
+    const int64_t q0 = ((int64_t)blockIdx.x * RS_CW + warp) * run;
+    const int cnt = run_len(nval, q0, run);
     if (cnt == 0) return;
     int32_t *sperm = sperm_all[warp];
     for (int i = lane; i < cnt; i += 32) sperm[i] = perm[q0 + i];
@@ -656,12 +679,12 @@ template <typename ACC, int NG>
 __global__ void __launch_bounds__(RS_THREADS) direct_sum_bf16_kernel(
     const uint16_t *__restrict__ X, int d, const int32_t *__restrict__ perm,
     const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k, ACC *__restrict__ S,
-    int64_t stride) {
+    int64_t stride, int run) {
     __shared__ int32_t sperm_all[RS_CW][RS_ROWS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t nval = offsets[k];
-    const int64_t q0 = ((int64_t)blockIdx.x * RS_CW + warp) * RS_ROWS;
-    const int cnt = run_len(nval, q0);
+    const int64_t q0 = ((int64_t)blockIdx.x * RS_CW + warp) * run;
+    const int cnt = run_len(nval, q0, run);
     if (cnt == 0) return;
     int32_t *sperm = sperm_all[warp];
     for (int i = lane; i < cnt; i += 32) sperm[i] = perm[q0 + i];
@@ -742,10 +765,11 @@ __global__ void __launch_bounds__(RS_THREADS) direct_sum_bf16_kernel(
 template <int NW>
 struct Lvq4Cons {
     const int32_t *scl;
-    const uint32_t *sqs;  // Sq in sorted order
-    const int64_t *bqs;   // Bq in sorted order
+    const float4 *fac;     // the points' (s, b, N, A): Sq = rint(s 2^e), Bq = rint(b 2^e)
+    const int32_t *sperm;  // the run's points
+    int e;
     unsigned long long *T;
-    int d, W;
+    int d, W, w0;  // w0: first word of the lane's range
     uint32_t alo[8 * NW], ahi[8 * NW];
     uint32_t pw[NW];  // the row waiting for a partner
     uint32_t psq;
@@ -762,14 +786,14 @@ struct Lvq4Cons {
         for (int t = 0; t < NW; ++t)
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const int col = 8 * (lane + 32 * t) + j;
+                const int col = 8 * (w0 + lane + 32 * t) + j;
                 const unsigned long long v =
                     (unsigned long long)alo[8 * t + j] + ((unsigned long long)ahi[8 * t + j] << 16);
                 if (col < d && v) atomicAdd(T + (int64_t)c * (d + 1) + col, v);
                 alo[8 * t + j] = 0u;
                 ahi[8 * t + j] = 0u;
             }
-        if (lane == 0 && usum) atomicAdd(T + (int64_t)c * (d + 1) + d, (unsigned long long)usum);
+        if (lane == 0 && usum && w0 == 0) atomicAdd(T + (int64_t)c * (d + 1) + d, (unsigned long long)usum);
         usum = 0;
     }
     // rows a (words xa, weight sa) and b (xb, sb) of the current cluster
@@ -801,6 +825,18 @@ struct Lvq4Cons {
             hi[7] = __dp2a_hi(whi, m57, hi[7]);
         }
     }
+    // cluster and weights of position i of the run
+    __device__ __forceinline__ void window(int i, int &cl, uint32_t &sq, int64_t &bq) {
+        cl = -1;
+        sq = 0u;
+        bq = 0;
+        if (i < cnt) {
+            cl = __ldg(scl + q0 + i);
+            const float2 f = __ldg(reinterpret_cast<const float2 *>(fac + sperm[i]));
+            sq = (uint32_t)fixed_rint(f.x, e);
+            bq = fixed_rint(f.y, e);
+        }
+    }
     __device__ __forceinline__ void single() {  // the waiting row with a zero-weight partner
         const uint32_t zero[NW] = {};
         pair(pw, psq, zero, 0u);
@@ -814,23 +850,17 @@ struct Lvq4Cons {
         pend = false;
         psq = 0u;
         usum = 0;
-        clw = lane < cnt ? __ldg(scl + q0 + lane) : -1;
-        cln = 32 + lane < cnt ? __ldg(scl + q0 + 32 + lane) : -1;
-        sqw = lane < cnt ? __ldg(sqs + q0 + lane) : 0u;
-        sqn = 32 + lane < cnt ? __ldg(sqs + q0 + 32 + lane) : 0u;
-        bqw = lane < cnt ? __ldg(bqs + q0 + lane) : 0;
-        bqn = 32 + lane < cnt ? __ldg(bqs + q0 + 32 + lane) : 0;
+        window(lane, clw, sqw, bqw);
+        window(32 + lane, cln, sqn, bqn);
         cur = __shfl_sync(0xffffffffu, clw, 0);
     }
-    __device__ __forceinline__ void row(int i, const uint8_t *slot, int lane) {
+    // row i of the run, the lane's words of it in registers
+    __device__ __forceinline__ void row_regs(int i, const uint32_t (&x)[NW], int lane) {
         if ((i & 31) == 0 && i > 0) {
             clw = cln;
             sqw = sqn;
             bqw = bqn;
-            const int nx = i + 32 + lane;
-            cln = nx < cnt ? __ldg(scl + q0 + nx) : -1;
-            sqn = nx < cnt ? __ldg(sqs + q0 + nx) : 0u;
-            bqn = nx < cnt ? __ldg(bqs + q0 + nx) : 0;
+            window(i + 32 + lane, cln, sqn, bqn);
         }
         const int c = __shfl_sync(0xffffffffu, clw, i & 31);
         const uint32_t sq = __shfl_sync(0xffffffffu, sqw, i & 31);
@@ -841,13 +871,6 @@ struct Lvq4Cons {
             cur = c;
         }
         usum += bq;
-        const uint32_t *words = reinterpret_cast<const uint32_t *>(slot);
-        uint32_t x[NW];
-#pragma unroll
-        for (int t = 0; t < NW; ++t) {
-            const int w = lane + 32 * t;
-            x[t] = w < W ? words[w] : 0u;
-        }
         if (pend) {
             pair(pw, psq, x, sq);
             pend = false;
@@ -864,21 +887,59 @@ struct Lvq4Cons {
     }
 };
 
+// LVQ4 rows straight into registers: lane l loads the words w0 + l + 32 t of a
+// row (coalesced 4-byte loads, whatever the row's alignment), the next
+// LVQ_PF rows of the warp's run in flight while one is summed.  Rows of more
+// than 128 words are taken in ranges of 128 by blockIdx.y (w0).
+constexpr int LVQ_PF = 4;
 template <int NW>
-__global__ void __launch_bounds__(RS_THREADS) ring_sum_lvq4_kernel(
-    const uint32_t *__restrict__ codes, const uint32_t *__restrict__ sqs, const int64_t *__restrict__ bqs, int d,
+__global__ void __launch_bounds__(RS_THREADS) direct_sum_lvq4_kernel(
+    const uint32_t *__restrict__ codes, const float4 *__restrict__ fac, int e, int d,
     const int32_t *__restrict__ perm, const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k,
-    unsigned long long *__restrict__ T, RingLayout L, int32_t *flag) {
+    unsigned long long *__restrict__ T, int run) {
+    __shared__ int32_t sperm_all[RS_CW][RS_ROWS];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t nval = offsets[k];
-    if ((int64_t)blockIdx.x * RS_CW * RS_ROWS >= nval) return;
+    const int64_t q0 = ((int64_t)blockIdx.x * RS_CW + warp) * run;
+    const int cnt = run_len(nval, q0, run);
+    if (cnt == 0) return;
+    int32_t *sperm = sperm_all[warp];
+    for (int i = lane; i < cnt; i += 32) sperm[i] = perm[q0 + i];
+    __syncwarp();
+    const int WT = lvq4_words(d), w0 = 128 * blockIdx.y;
     Lvq4Cons<NW> cons;
     cons.scl = scl;
-    cons.sqs = sqs;
-    cons.bqs = bqs;
+    cons.fac = fac;
+    cons.sperm = sperm;
+    cons.e = e;
     cons.T = T;
     cons.d = d;
-    cons.W = lvq4_words(d);
-    ring_gather(reinterpret_cast<const uint8_t *>(codes), perm, nval, L, flag, cons);
+    cons.W = WT;
+    cons.w0 = w0;
+    auto load = [&](int r, uint32_t(&x)[NW]) {
+        const uint32_t *src = codes + (size_t)sperm[r] * WT + w0;
+#pragma unroll
+        for (int t = 0; t < NW; ++t) {
+            const int w = lane + 32 * t;
+            x[t] = w0 + w < WT ? __ldg(src + w) : 0u;
+        }
+    };
+    uint32_t buf[LVQ_PF][NW];
+#pragma unroll
+    for (int p = 0; p < LVQ_PF; ++p)
+        if (p < cnt) load(p, buf[p]);
+    cons.start(q0, cnt, lane);
+    for (int r0 = 0; r0 < cnt; r0 += LVQ_PF) {
+#pragma unroll
+        for (int p = 0; p < LVQ_PF; ++p) {
+            const int r = r0 + p;
+            if (r < cnt) {  // warp-uniform
+                cons.row_regs(r, buf[p], lane);
+                if (r + LVQ_PF < cnt) load(r + LVQ_PF, buf[p]);
+            }
+        }
+    }
+    cons.finish(lane);
 }
 
 // Rows of [RS_LSU_MIN_ROW, RS_LSU_MAX_ROW) bytes take the LSU path (per-lane
@@ -903,8 +964,8 @@ bool ring_layout(uint32_t rb, RingLayout &L) {
     return L.ns >= 2;
 }
 
-unsigned ring_blocks(int64_t n) {
-    const int64_t per = (int64_t)RS_CW * RS_ROWS;
+unsigned ring_blocks(int64_t n, int run) {
+    const int64_t per = (int64_t)RS_CW * run;
     const int64_t b = (n + per - 1) / per;
     return (unsigned)(b < 1 ? 1 : b);
 }
@@ -913,8 +974,9 @@ template <bool BF16, typename ACC>
 cudaError_t launch_float_nf(int nf, const void *X, int64_t n, int d, const int32_t *perm,
                             const int32_t *scl, const int64_t *offsets, int k, ACC *S, RingLayout L,
                             int32_t *flag, cudaStream_t st) {
+    L.run = sum_run(n, 16, sizeof(ACC) == 4 ? SUM_WARPS_F32 : SUM_WARPS);
     const size_t smem = L.bytes();
-    const unsigned g = ring_blocks(n);
+    const unsigned g = ring_blocks(n, L.run);
 #define RS_CASE(NFV)                                                                                \
     case NFV: {                                                                                     \
         auto kern = ring_sum_float_kernel<BF16, ACC, NFV>;                                          \
@@ -944,25 +1006,21 @@ bool ring_sum_float_ok(const void *X, int x_is_bf16, int d) {
            ring_layout(rb, L);
 }
 
-bool ring_sum_rbq1_ok(const void *codes, int d) {
-    const int W = (d + 31) >> 5;
-    return W % 4 == 0 && W <= 32 && (reinterpret_cast<uintptr_t>(codes) & 15u) == 0;
-}
-
 cudaError_t launch_ring_sum_float(const void *X, int x_is_bf16, int64_t n, int d, const int32_t *perm,
                                   const int32_t *scl, const int64_t *offsets, int k, float *S_f,
                                   double *S_d, int32_t *flag, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     if (x_is_bf16 && d % 8 == 0 && d <= 512 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0) {
         // rows of at most 1 KB: straight into registers
-        const unsigned g = ring_blocks(n);
+        const int run = sum_run(n, 16, SUM_WARPS);
+        const unsigned g = ring_blocks(n, run);
         const uint16_t *Xb = static_cast<const uint16_t *>(X);
         if (d <= 256) {
-            if (S_d) direct_sum_bf16_kernel<double, 1><<<g, RS_THREADS, 0, st>>>(Xb, d, perm, scl, offsets, k, S_d, d);
-            else direct_sum_bf16_kernel<float, 1><<<g, RS_THREADS, 0, st>>>(Xb, d, perm, scl, offsets, k, S_f, d);
+            if (S_d) direct_sum_bf16_kernel<double, 1><<<g, RS_THREADS, 0, st>>>(Xb, d, perm, scl, offsets, k, S_d, d, run);
+            else direct_sum_bf16_kernel<float, 1><<<g, RS_THREADS, 0, st>>>(Xb, d, perm, scl, offsets, k, S_f, d, run);
         } else {
-            if (S_d) direct_sum_bf16_kernel<double, 2><<<g, RS_THREADS, 0, st>>>(Xb, d, perm, scl, offsets, k, S_d, d);
-            else direct_sum_bf16_kernel<float, 2><<<g, RS_THREADS, 0, st>>>(Xb, d, perm, scl, offsets, k, S_f, d);
+            if (S_d) direct_sum_bf16_kernel<double, 2><<<g, RS_THREADS, 0, st>>>(Xb, d, perm, scl, offsets, k, S_d, d, run);
+            else direct_sum_bf16_kernel<float, 2><<<g, RS_THREADS, 0, st>>>(Xb, d, perm, scl, offsets, k, S_f, d, run);
         }
         return launched();
     }
@@ -989,15 +1047,16 @@ cudaError_t launch_ring_sum_sq8(const uint8_t *codes, int64_t n, int d, const in
     if (n == 0) return cudaSuccess;
     RingLayout L;
     if (!ring_layout((uint32_t)d, L)) return cudaErrorInvalidValue;
+    L.run = sum_run(n, 16, SUM_WARPS);
     const size_t smem = L.bytes();
-    const unsigned g = ring_blocks(n);
+    const unsigned g = ring_blocks(n, L.run);
     auto S64 = reinterpret_cast<unsigned long long *>(S);
     const int q = (d / 16 + 31) / 32;  // 16-byte groups per lane
     if (d <= 1024) {  // rows of at most 1 KB: straight into registers
         if (q <= 1)
-            direct_sum_sq8_kernel<1><<<g, RS_THREADS, 0, st>>>(codes, d, perm, scl, offsets, k, S64);
+            direct_sum_sq8_kernel<1><<<g, RS_THREADS, 0, st>>>(codes, d, perm, scl, offsets, k, S64, L.run);
         else
-            direct_sum_sq8_kernel<2><<<g, RS_THREADS, 0, st>>>(codes, d, perm, scl, offsets, k, S64);
+            direct_sum_sq8_kernel<2><<<g, RS_THREADS, 0, st>>>(codes, d, perm, scl, offsets, k, S64, L.run);
         return launched();
     }
 #define RS_CASE(NGV)                                                                                \
@@ -1016,22 +1075,21 @@ cudaError_t launch_ring_sum_sq8(const uint8_t *codes, int64_t n, int d, const in
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_ring_sum_rbq1(const uint32_t *codes, const int64_t *fqs, int64_t n, int d,
-                                 const int32_t *perm, const int32_t *scl, const int64_t *offsets,
-                                 int k, int64_t *T, int32_t *flag, cudaStream_t st) {
-    (void)flag;  // no waits in this kernel
-    if (n == 0) return cudaSuccess;
-    if (!ring_sum_rbq1_ok(codes, d)) return cudaErrorInvalidValue;
-    const int W = (d + 31) >> 5;
-    auto T64 = reinterpret_cast<unsigned long long *>(T);
-    const int64_t per = (int64_t)TR_WARPS * TR_ROWS;
-    const unsigned g = (unsigned)std::max<int64_t>(1, (n + per - 1) / per);
-#define TR_CASE(W4V)                                                                                          \
-    case W4V:                                                                                                 \
-        rbq1_sum_table_kernel<W4V, tr_prefetch<W4V>()><<<g, TR_WARPS * 32, 0, st>>>(codes, fqs, d, perm, scl, \
-                                                                                   offsets, k, T64);           \
+template <int VEC>
+static cudaError_t launch_sum_rbq1_vec(const uint32_t *codes, int WT, const float *F, int e, int64_t n, int d,
+                                       const int32_t *perm, const int32_t *scl, const int64_t *offsets, int k,
+                                       unsigned long long *T, cudaStream_t st) {
+    const int run = sum_run(n, 32, SUM_WARPS);  // whole 32-row chunks
+    const int64_t per = (int64_t)TR_WARPS * run;
+    const int gy = (WT + 31) / 32;                 // at most 32 words of a row in a thread's registers
+    const int w4 = ((WT + gy - 1) / gy + 3) / 4;   // and the blocks' word ranges about equal
+    const dim3 g((unsigned)std::max<int64_t>(1, (n + per - 1) / per), (unsigned)gy);
+#define TR_CASE(W4V)                                                                                       \
+    case W4V:                                                                                              \
+        rbq1_sum_table_kernel<W4V, VEC, tr_prefetch<W4V>()>                                                \
+            <<<g, TR_WARPS * 32, 0, st>>>(codes, WT, F, e, d, perm, scl, offsets, k, T, run);               \
         return launched();
-    switch (W / 4) {
+    switch (w4) {
         TR_CASE(1)
         TR_CASE(2)
         TR_CASE(3)
@@ -1041,47 +1099,43 @@ cudaError_t launch_ring_sum_rbq1(const uint32_t *codes, const int64_t *fqs, int6
         TR_CASE(7)
         TR_CASE(8)
     default:
-        break;
+        return cudaErrorInvalidValue;
     }
 #undef TR_CASE
-    return cudaErrorInvalidValue;
 }
 
-bool ring_sum_lvq4_ok(const void *codes, int d) {
-    RingLayout L;
-    const int W = lvq4_words(d);
-    return W % 4 == 0 && W <= 128 && (reinterpret_cast<uintptr_t>(codes) & 15u) == 0 &&
-           ring_layout((uint32_t)W * 4u, L);
+cudaError_t launch_sum_rbq1(const uint32_t *codes, const float *F, int e, int64_t n, int d, const int32_t *perm,
+                            const int32_t *scl, const int64_t *offsets, int k, int64_t *T, cudaStream_t st) {
+    if (n == 0) return cudaSuccess;
+    const int W = (d + 31) >> 5;
+    auto T64 = reinterpret_cast<unsigned long long *>(T);
+    const uintptr_t a = reinterpret_cast<uintptr_t>(codes);
+    const int gy = (W + 31) / 32;
+    if (W % (4 * gy) == 0 && (a & 15u) == 0) return launch_sum_rbq1_vec<4>(codes, W, F, e, n, d, perm, scl, offsets, k, T64, st);
+    if (W % 2 == 0 && (a & 7u) == 0) return launch_sum_rbq1_vec<2>(codes, W, F, e, n, d, perm, scl, offsets, k, T64, st);
+    return launch_sum_rbq1_vec<1>(codes, W, F, e, n, d, perm, scl, offsets, k, T64, st);
 }
 
-cudaError_t launch_ring_sum_lvq4(const uint32_t *codes, const uint32_t *sq, const int64_t *bq, int64_t n, int d,
-                                 const int32_t *perm, const int32_t *scl, const int64_t *offsets, int k, int64_t *T,
-                                 int32_t *flag, cudaStream_t st) {
+cudaError_t launch_sum_lvq4(const uint32_t *codes, const float4 *fac, int e, int64_t n, int d, const int32_t *perm,
+                            const int32_t *scl, const int64_t *offsets, int k, int64_t *T, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     const int W = lvq4_words(d);
-    RingLayout L;
-    if (!ring_layout((uint32_t)W * 4u, L)) return cudaErrorInvalidValue;
-    const size_t smem = L.bytes();
-    const unsigned g = ring_blocks(n);
     auto T64 = reinterpret_cast<unsigned long long *>(T);
-#define RS_CASE(NWV)                                                                                \
-    case NWV: {                                                                                     \
-        auto kern = ring_sum_lvq4_kernel<NWV>;                                                      \
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-        if (e != cudaSuccess) return e;                                                             \
-        kern<<<g, RS_THREADS, smem, st>>>(codes, sq, bq, d, perm, scl, offsets, k, T64, L, flag);    \
-        return launched();                                                                          \
-    }
-    switch ((W + 31) / 32) {
+    const int run = sum_run(n, 16, SUM_WARPS);
+    const dim3 g(ring_blocks(n, run), (unsigned)((W + 127) / 128));
+#define RS_CASE(NWV)                                                                                           \
+    case NWV:                                                                                                  \
+        direct_sum_lvq4_kernel<NWV><<<g, RS_THREADS, 0, st>>>(codes, fac, e, d, perm, scl, offsets, k, T64, run); \
+        return launched();
+    switch ((std::min(W, 128) + 31) / 32) {
         RS_CASE(1)
         RS_CASE(2)
         RS_CASE(3)
         RS_CASE(4)
     default:
-        break;
+        return cudaErrorInvalidValue;
     }
 #undef RS_CASE
-    return cudaErrorInvalidValue;
 }
 
 }  // namespace skm

@@ -148,6 +148,7 @@ struct TcParams {
     int32_t *resc_rows;
     int32_t *fall_rows;
     int32_t *counters;  // [0] rescore rows, [1] fallback rows, [2] abort flag
+    int64_t *stats;     // code modes: [2] gets the abort flag (may be NULL)
     int32_t *assign;
     const int32_t *nx;  // SQ8: centred ||x||^2
     const int32_t *nc;  // SQ8: centred ||c||^2, padded to 256 with a large value
@@ -1526,6 +1527,9 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
     }
     tc_fence_before();
     __syncthreads();
+    // the screen's counters are added up by the rescoring kernel
+    if ((f8_mode<MODE>() || MODE == MODE_SQ8) && threadIdx.x == 0 && p.stats && *abort_flag)
+        atomicOr(reinterpret_cast<unsigned long long *>(p.stats + 2), 1ull);
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
@@ -1962,17 +1966,23 @@ __device__ __forceinline__ float warp_sqdist(const TX *x, const float *c, int d,
 
 // One warp per listed row: exact fp32 distances to its screen candidates.
 template <typename TX>
-// (count: the call's counters, [0] rows listed, [2] the screen's abort flag.)
+// (count: the call's counters, [0] rows listed, [1] rows of the fallback, [2]
+// the screen's abort flag; thread 0 adds them to the cumulative stats.)
 // SKM_FLAG_WARM: thread 0 stamps the workspace's bounds as complete for this
 // n, d and k unless the screen gave up.
 __global__ void rescore_kernel(const TX *__restrict__ X, int d, const float *__restrict__ C,
                                const int32_t *__restrict__ rows, const int32_t *__restrict__ count,
                                const int32_t *__restrict__ cand, int32_t *__restrict__ assign,
-                               int64_t *__restrict__ warm_hdr, int64_t n, int k) {
+                               int64_t *__restrict__ warm_hdr, int64_t n, int k, int64_t *__restrict__ stats) {
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int64_t cnt = *count;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        stats[0] += count[0];
+        stats[1] += count[1];
+        stats[2] |= count[2];
+    }
     if (warm_hdr && blockIdx.x == 0 && threadIdx.x == 0 && count[2] == 0) {
         warm_hdr[1] = n;
         warm_hdr[2] = d;
@@ -2010,12 +2020,6 @@ __global__ void assigned_dist_kernel(const TX *__restrict__ X, int64_t n, int d,
         const float dd = warp_sqdist<TX>(X + r * d, C + (int64_t)assign[r] * d, d, lane);
         if (lane == 0) dist[r] = dd;
     }
-}
-
-__global__ void add_stats_kernel(const int32_t *__restrict__ counters, int64_t *__restrict__ stats) {
-    stats[0] += counters[0];
-    stats[1] += counters[1];
-    stats[2] |= counters[2];
 }
 
 // ---------------------------------------------------------- segmented mode
@@ -2445,12 +2449,16 @@ void tc_plan_pfront(int64_t n, int d, int k, bool warm, Carver &cv, TcAssignBufs
 //      rows whose lists overflowed pruned over all k.
 // The result is the same as the CUDA-core pruning kernels' bit for bit.
 // End of a front call: the call's list counts into the pruning statistics
-// ([4] finished rows, [5] rows pruned over all k; cumulative in skm_fit) and,
+// ([4] finished rows, [5] rows pruned over all k; cumulative in skm_fit), all
+// counters into the cumulative stats and,
 // with kept bounds (hdr), the stamp when no wait gave up (every row's bound
 // was then written).
 __global__ void pf_done_kernel(int64_t *__restrict__ hdr, const int32_t *__restrict__ counters,
                                unsigned long long *__restrict__ ctr, int64_t n, int d, int k,
-                               const int64_t *__restrict__ cgen) {
+                               const int64_t *__restrict__ cgen, int64_t *__restrict__ stats) {
+    stats[0] += counters[0];
+    stats[1] += counters[1];
+    stats[2] |= counters[2];
     ctr[4] += (unsigned long long)counters[0];
     ctr[5] += (unsigned long long)counters[1];
     if (hdr && counters[2] == 0) {
@@ -2540,9 +2548,7 @@ int tc_assign_pfront(const skm_data *x, const float *C, int k, const int32_t *pr
     SKM_CUDA_TRY(launch_prune_finish(X, d, C, b.pf_thr, b.pf_cand, b.pf_cnt, PF_CAP, nsub, cb.pf_perm, b.resc_rows,
                                      b.counters, assign, dist, rows.wrow, ctr, st));
     SKM_CUDA_TRY(launch_prune_rows_cta(X, d, C, k, rows, b.fall_rows, b.counters + 1, assign, dist, ctr + 6, st));
-    add_stats_kernel<<<1, 1, 0, st>>>(b.counters, b.stats);
-    SKM_CUDA_TRY(launched());
-    pf_done_kernel<<<1, 1, 0, st>>>(warm ? b.pf_whdr : nullptr, b.counters, ctr, n, d, k, cb.pf_cgen);
+    pf_done_kernel<<<1, 1, 0, st>>>(warm ? b.pf_whdr : nullptr, b.counters, ctr, n, d, k, cb.pf_cgen, b.stats);
     SKM_CUDA_TRY(launched());
     return SKM_OK;
 }
@@ -2615,7 +2621,8 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
     const int gw = grid_warps(n);
     if (bf16) {
         const uint16_t *X = static_cast<const uint16_t *>(x->x);
-        rescore_kernel<uint16_t><<<gw, 256, 0, st>>>(X, d, C, b.resc_rows, b.counters, b.cand, assign, hdr, n, k);
+        rescore_kernel<uint16_t><<<gw, 256, 0, st>>>(X, d, C, b.resc_rows, b.counters, b.cand, assign, hdr, n, k,
+                                                   b.stats);
         SKM_CUDA_TRY(launched());
         if (seg) {
             seg_rows_exact_kernel<uint16_t><<<gw, 256, 0, st>>>(X, d, C, b.fall_rows, b.counters + 1, seg->group,
@@ -2631,7 +2638,8 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
         }
     } else {
         const float *X = static_cast<const float *>(x->x);
-        rescore_kernel<float><<<gw, 256, 0, st>>>(X, d, C, b.resc_rows, b.counters, b.cand, assign, hdr, n, k);
+        rescore_kernel<float><<<gw, 256, 0, st>>>(X, d, C, b.resc_rows, b.counters, b.cand, assign, hdr, n, k,
+                                                   b.stats);
         SKM_CUDA_TRY(launched());
         if (seg) {
             seg_rows_exact_kernel<float><<<gw, 256, 0, st>>>(X, d, C, b.fall_rows, b.counters + 1, seg->group,
@@ -2646,8 +2654,6 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
             SKM_CUDA_TRY(launched());
         }
     }
-    add_stats_kernel<<<1, 1, 0, st>>>(b.counters, b.stats);
-    SKM_CUDA_TRY(launched());
     return SKM_OK;
 }
 
@@ -2677,14 +2683,13 @@ int tc_assign_sq8(const skm_data *x, const uint8_t *C, int k, int32_t *nx_plain,
     SKM_CUDA_TRY(cudaMemsetAsync(b.counters, 0, sizeof(int32_t) * 4, st));
     TcParams p{};
     p.counters = b.counters;
+    p.stats = b.stats;
     p.assign = assign;
     p.nx = v.nx;
     p.nc = b.nc;
     p.dist = dist;
     SKM_TRY(seg_setup(seg, n, p, st));
     SKM_TRY(launch_tc<MODE_SQ8>(v.xs, n, dp, d, b.cs, k, p, st));
-    add_stats_kernel<<<1, 1, 0, st>>>(b.counters, b.stats);
-    SKM_CUDA_TRY(launched());
     return SKM_OK;
 }
 
@@ -2713,6 +2718,7 @@ int tc_assign_rbq1(const skm_data *x, const float *C, int k, int32_t *assign, fl
     SKM_CUDA_TRY(cudaMemsetAsync(b.counters, 0, sizeof(int32_t) * 4, st));
     TcParams p{};
     p.counters = b.counters;
+    p.stats = b.stats;
     p.assign = assign;
     p.dist = dist;
     p.rinfo = b.rpair_bs;
@@ -2729,8 +2735,6 @@ int tc_assign_rbq1(const skm_data *x, const float *C, int k, int32_t *assign, fl
     }
     SKM_TRY(seg_setup(seg, n, p, st));
     SKM_TRY(launch_tc<MODE_RBQ1>(v.xs, n, dp, d, b.cs, k, p, st, v.packed));
-    add_stats_kernel<<<1, 1, 0, st>>>(b.counters, b.stats);
-    SKM_CUDA_TRY(launched());
     return SKM_OK;
 }
 
@@ -2751,6 +2755,7 @@ int tc_assign_lvq4(const skm_data *x, const float *C, int k, int32_t *assign, fl
     SKM_CUDA_TRY(cudaMemsetAsync(b.counters, 0, sizeof(int32_t) * 4, st));
     TcParams p{};
     p.counters = b.counters;
+    p.stats = b.stats;
     p.assign = assign;
     p.dist = dist;
     p.rinfo = b.rpair_bs;
@@ -2765,8 +2770,6 @@ int tc_assign_lvq4(const skm_data *x, const float *C, int k, int32_t *assign, fl
     }
     SKM_TRY(seg_setup(seg, n, p, st));
     SKM_TRY(launch_tc<MODE_LVQ4>(v.xs, n, dp, d, b.cs, k, p, st, v.packed));
-    add_stats_kernel<<<1, 1, 0, st>>>(b.counters, b.stats);
-    SKM_CUDA_TRY(launched());
     return SKM_OK;
 }
 

@@ -9,6 +9,8 @@
 //   5. finalise: divide by the counts (or add into caller partial sums).
 // Integer representations accumulate in int64 and are exact, so their result
 // does not depend on the member order produced by the scatter.
+#include <algorithm>
+
 #include "skm_internal.cuh"
 
 namespace skm {
@@ -37,28 +39,6 @@ __global__ void histogram_kernel(const int32_t *__restrict__ assign, int64_t n, 
     }
 }
 
-// One block: the number of zero entries of counts[0..k) into *out.
-__global__ void count_zeros_kernel(const int64_t *__restrict__ counts, int k, int64_t *__restrict__ out) {
-    __shared__ int part[32];
-    int z = 0;
-    for (int j = threadIdx.x; j < k; j += blockDim.x) z += counts[j] == 0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = z;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        z = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-        if (threadIdx.x == 0) *out = z;
-    }
-}
-
-cudaError_t launch_count_zeros(const int64_t *counts, int k, int64_t *out, cudaStream_t st) {
-    count_zeros_kernel<<<1, 1024, 0, st>>>(counts, k, out);
-    return launched();
-}
-
 cudaError_t launch_histogram(const int32_t *assign, int64_t n, int k, int32_t *counts32,
                              cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(counts32, 0, sizeof(int32_t) * (size_t)k, st);
@@ -75,16 +55,25 @@ cudaError_t launch_histogram(const int32_t *assign, int64_t n, int k, int32_t *c
 }
 
 // --------------------------------------------------------------------- scan
-// Single block of 1024 threads; each thread scans a contiguous run of counts.
-__global__ void scan_offsets_kernel(const int32_t *__restrict__ counts, int k,
-                                    int64_t *__restrict__ offsets, int64_t *__restrict__ counts64,
-                                    int accumulate) {
+// Exclusive scan of the counts by one block of 1024 threads, count(j) giving
+// cluster j's members and put(j, offset) taking its offset; each thread has a
+// contiguous run of clusters.  Also the int64 counts, and the number of empty
+// clusters (zeros, may be NULL).
+template <typename Count, typename Put>
+__device__ __forceinline__ void scan_block(int k, Count count, Put put, int64_t *__restrict__ offsets,
+                                           int64_t *__restrict__ counts64, int accumulate,
+                                           int64_t *__restrict__ zeros) {
     __shared__ int64_t wsum[32];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int per = (k + blockDim.x - 1) / blockDim.x;
     const int lo = min(k, t * per), hi = min(k, lo + per);
     int64_t s = 0;
-    for (int j = lo; j < hi; ++j) s += counts[j];
+    int z = 0;
+    for (int j = lo; j < hi; ++j) {
+        const int c = count(j);
+        s += c;
+        z += c == 0;
+    }
     // exclusive scan of the threads' run sums: shuffles inside each warp, then
     // the warp totals (exact integer sums, so any order gives the same offsets)
     int64_t v = s;
@@ -108,22 +97,103 @@ __global__ void scan_offsets_kernel(const int32_t *__restrict__ counts, int k,
     int64_t run = v - s + (w > 0 ? wsum[w - 1] : 0);
     if (t == (int)blockDim.x - 1) offsets[k] = run + s;
     for (int j = lo; j < hi; ++j) {
+        const int c = count(j);
         offsets[j] = run;
-        run += counts[j];
+        put(j, run);
+        run += c;
         if (counts64) {
             if (accumulate)
-                counts64[j] += counts[j];
+                counts64[j] += c;
             else
-                counts64[j] = counts[j];
+                counts64[j] = c;
+        }
+    }
+    if (zeros) {
+        __syncthreads();  // wsum has been read
+        const int64_t zw = __reduce_add_sync(0xffffffffu, z);
+        if (lane == 0) wsum[w] = zw;
+        __syncthreads();
+        if (t == 0) {
+            int64_t tot = 0;
+            for (int i = 0; i < (int)(blockDim.x >> 5); ++i) tot += wsum[i];
+            *zeros = tot;
         }
     }
 }
 
-cudaError_t launch_scan_offsets(const int32_t *counts32, int k, int64_t *offsets,
-                                int64_t *counts64_out, int accumulate_counts, cudaStream_t st) {
-    scan_offsets_kernel<<<1, 1024, 0, st>>>(counts32, k, offsets, counts64_out,
-                                            accumulate_counts);
-    return launched();
+// The blocks after the first clear the cluster sums (bytes a multiple of 4,
+// 16-byte aligned) while the first one sorts or scans, so that the sums need
+// no memset of their own.
+__device__ __forceinline__ void clear_sums(void *__restrict__ sums, size_t bytes) {
+    const size_t nt = (size_t)(gridDim.x - 1) * blockDim.x;
+    const size_t t0 = (size_t)(blockIdx.x - 1) * blockDim.x + threadIdx.x;
+    for (size_t i = t0; i < bytes / 16; i += nt) static_cast<uint4 *>(sums)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (size_t i = bytes / 16 * 4 + t0; i < bytes / 4; i += nt) static_cast<uint32_t *>(sums)[i] = 0u;
+}
+
+__global__ void __launch_bounds__(1024) scan_offsets_kernel(const int32_t *__restrict__ counts, int k,
+                                                            int64_t *__restrict__ offsets,
+                                                            int64_t *__restrict__ counts64, int accumulate,
+                                                            int32_t *__restrict__ cursor, int64_t *__restrict__ zeros,
+                                                            int32_t *__restrict__ flag, void *__restrict__ sums,
+                                                            size_t sum_bytes) {
+    if (flag && blockIdx.x == 0 && threadIdx.x == 0) *flag = 0;
+    if (blockIdx.x > 0) {
+        clear_sums(sums, sum_bytes);
+        return;
+    }
+    scan_block(k, [&](int j) { return counts[j]; }, [&](int j, int64_t) { cursor[j] = 0; }, offsets, counts64,
+               accumulate, zeros);
+}
+
+// Histogram, scan and placement of up to SORT1_MAX points in one block: a
+// thread keeps its points' clusters and their ranks inside them (the values
+// the shared-memory counters returned) in registers between the passes.  Three
+// launches and three memsets became one launch: 20,000 points 16 -> 7 us on
+// the GPU, and the host's launches bound an update of this size.
+constexpr int SORT1_PER = 32;
+constexpr int SORT1_MAX = 1024 * SORT1_PER;
+constexpr int SORT1_MAX_K = 12288;  // 48 KiB of counters; a cluster fits 14 bits, a rank 15
+
+__global__ void __launch_bounds__(1024) sort_one_block_kernel(const int32_t *__restrict__ assign, int n, int k,
+                                                              int64_t *__restrict__ offsets,
+                                                              int64_t *__restrict__ counts64, int accumulate,
+                                                              int32_t *__restrict__ perm, int32_t *__restrict__ scl,
+                                                              int64_t *__restrict__ zeros, int32_t *__restrict__ flag,
+                                                              void *__restrict__ sums, size_t sum_bytes) {
+    if (flag && blockIdx.x == 0 && threadIdx.x == 0) *flag = 0;
+    if (blockIdx.x > 0) {
+        clear_sums(sums, sum_bytes);
+        return;
+    }
+    extern __shared__ int32_t cnt_sh[];
+    for (int j = threadIdx.x; j < k; j += 1024) cnt_sh[j] = 0;
+    uint32_t place[SORT1_PER];
+#pragma unroll
+    for (int i = 0; i < SORT1_PER; ++i) {
+        const int t = threadIdx.x + 1024 * i;
+        place[i] = t < n ? (uint32_t)assign[t] : 0xffffffffu;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < SORT1_PER; ++i) {
+        if (place[i] >= (uint32_t)k)  // out-of-range assignments are skipped
+            place[i] = 0xffffffffu;
+        else
+            place[i] |= (uint32_t)atomicAdd(&cnt_sh[place[i]], 1) << 16;
+    }
+    __syncthreads();
+    scan_block(k, [&](int j) { return cnt_sh[j]; }, [&](int j, int64_t off) { cnt_sh[j] = (int32_t)off; }, offsets,
+               counts64, accumulate, zeros);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < SORT1_PER; ++i) {
+        if (place[i] == 0xffffffffu) continue;
+        const int a = (int)(place[i] & 0xffffu);
+        const int pos = cnt_sh[a] + (int)(place[i] >> 16);
+        perm[pos] = (int32_t)threadIdx.x + 1024 * i;
+        scl[pos] = a;
+    }
 }
 
 // ------------------------------------------------------------------ scatter
@@ -175,9 +245,22 @@ __global__ void __launch_bounds__(SC_THREADS) scatter_blocked_kernel(
     }
 }
 
-cudaError_t launch_scatter(const int32_t *assign, int64_t n, int k, const int64_t *offsets,
-                           int32_t *cursor, int32_t *perm, int32_t *scl, cudaStream_t st) {
-    if (n == 0) return cudaSuccess;
+cudaError_t launch_sort_by_cluster(const int32_t *assign, int64_t n, int k, int32_t *counts32, int32_t *cursor,
+                                   int64_t *offsets, int64_t *counts64, int accumulate, int32_t *perm, int32_t *scl,
+                                   int64_t *zeros, int32_t *flag, void *sums, size_t sum_bytes, cudaStream_t st) {
+    // a block clears 32 KiB or more
+    const unsigned clear = (unsigned)std::min<size_t>(152, (sum_bytes + 32767) / 32768);
+    if (n <= SORT1_MAX && k <= SORT1_MAX_K) {
+        sort_one_block_kernel<<<1 + clear, 1024, sizeof(int32_t) * (size_t)k, st>>>(
+            assign, (int)n, k, offsets, counts64, accumulate, perm, scl, zeros, flag, sums, sum_bytes);
+        return launched();
+    }
+    cudaError_t e = launch_histogram(assign, n, k, counts32, st);
+    if (e != cudaSuccess) return e;
+    scan_offsets_kernel<<<1 + clear, 1024, 0, st>>>(counts32, k, offsets, counts64, accumulate, cursor, zeros, flag,
+                                                    sums, sum_bytes);
+    e = launched();
+    if (e != cudaSuccess) return e;
     if (k <= SC_MAX_K) {
         const int64_t blocks = (n + SC_POINTS - 1) / SC_POINTS;
         scatter_blocked_kernel<<<(unsigned)blocks, SC_THREADS, sizeof(int32_t) * (size_t)k, st>>>(
@@ -317,46 +400,26 @@ __device__ __forceinline__ float rbq1_finish(int64_t T, int64_t U, float m, doub
     return __double2float_rn(__dadd_rn((double)m, __dmul_rn(__ll2double_rn(2 * T - U), f)));
 }
 
-// Fixed-point weights Fq = rint(F 2^e), once per update call, written in the
-// cluster-sorted order (position q holds the weight of member perm[q]).
-__global__ void rbq1_fq_kernel(const float *__restrict__ F, const int32_t *__restrict__ perm,
-                               const int64_t *__restrict__ offsets, int k, int e,
-                               int64_t *__restrict__ fq) {
-    const int64_t nval = offsets[k];
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nval;
-         q += (int64_t)gridDim.x * blockDim.x)
-        fq[q] = fixed_rint(F[perm[q]], e);
-}
-
-cudaError_t launch_rbq1_fq(const float *F, const int32_t *perm, const int64_t *offsets, int k,
-                           int64_t n, int e, int64_t *fq, cudaStream_t st) {
-    int64_t blocks = (n + 255) / 256;
-    if (blocks > 152 * 8) blocks = 152 * 8;
-    if (blocks < 1) blocks = 1;
-    rbq1_fq_kernel<<<(int)blocks, 256, 0, st>>>(F, perm, offsets, k, e, fq);
-    return launched();
-}
-
 // -------------------------------------------- chunked segmented sums (load balanced)
-// Warps take CH_ROWS consecutive members of the cluster-sorted order, so
+// Warps take `run` (at most CH_ROWS) consecutive members of the cluster-sorted order, so
 // every warp has the same work whatever the cluster sizes.  A warp adds its
 // rows into register accumulators and flushes them with global atomics into
 // the cluster's accumulator whenever the cluster changes (and at the end).
 // The member count of the sorted order is offsets[k].
 constexpr int CH_WARPS = 8;
-constexpr int CH_ROWS = 128;
+constexpr int CH_ROWS = SUM_RUN_MAX;
 
 // fp32 / bf16 points -> float or double accumulators S[k][d].
 template <bool BF16, typename ACC>
 __global__ void __launch_bounds__(CH_WARPS * 32) chunk_sum_float_kernel(
     const void *__restrict__ Xv, int d, const int32_t *__restrict__ perm,
     const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k,
-    ACC *__restrict__ S, int64_t stride) {
+    ACC *__restrict__ S, int64_t stride, int run) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t nval = offsets[k];
-    const int64_t q0 = ((int64_t)blockIdx.x * CH_WARPS + warp) * CH_ROWS;
+    const int64_t q0 = ((int64_t)blockIdx.x * CH_WARPS + warp) * run;
     if (q0 >= nval) return;
-    const int64_t q1 = min(nval, q0 + CH_ROWS);
+    const int64_t q1 = min(nval, q0 + run);
     for (int c0 = 0; c0 < d; c0 += SEG_CHUNK) {
         float acc[SEG_CHUNK / 32];
 #pragma unroll
@@ -406,105 +469,8 @@ __global__ void __launch_bounds__(CH_WARPS * 32) chunk_sum_float_kernel(
     }
 }
 
-// 1-bit codes -> int64 accumulators T[k][d+1] (column d holds U = sum Fq);
-// fqs in the sorted order.  Lane l holds dimension l of each code word.  A
-// warp's member ids, cluster ids and weights are read lane-parallel up
-// front; the member rows (W words, lane w loads word w) are read RB_DEPTH
-// rows ahead into a register ring, and each row's words reach every lane by
-// shuffles, so the loads of later rows overlap the sums of earlier ones.
-constexpr int RB_DEPTH = 8;
-
-__device__ __forceinline__ int pick4(const int (&a)[4], int i) {
-    const int t = i >> 5;
-    const int v = t == 0 ? a[0] : t == 1 ? a[1] : t == 2 ? a[2] : a[3];
-    return __shfl_sync(0xffffffffu, v, i & 31);
-}
-__device__ __forceinline__ int64_t pick4(const int64_t (&a)[4], int i) {
-    const int t = i >> 5;
-    const int64_t v = t == 0 ? a[0] : t == 1 ? a[1] : t == 2 ? a[2] : a[3];
-    return __shfl_sync(0xffffffffu, v, i & 31);
-}
-
-template <int WM>
-__global__ void __launch_bounds__(CH_WARPS * 32) chunk_sum_rbq1_kernel(
-    const uint32_t *__restrict__ codes, const int64_t *__restrict__ fqs, int d,
-    const int32_t *__restrict__ perm, const int32_t *__restrict__ scl,
-    const int64_t *__restrict__ offsets, int k, unsigned long long *__restrict__ T) {
-    static_assert(CH_ROWS == 128, "pick4 covers 4 x 32 positions");
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t nval = offsets[k];
-    const int64_t q0 = ((int64_t)blockIdx.x * CH_WARPS + warp) * CH_ROWS;
-    if (q0 >= nval) return;
-    const int cnt = (int)(nval - q0 < CH_ROWS ? nval - q0 : CH_ROWS);
-    const int W = (d + 31) >> 5;
-    const uint32_t lm = 1u << lane;
-    int pp[4], cc[4];
-    int64_t ff[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-        const int i = lane + 32 * t;
-        pp[t] = i < cnt ? perm[q0 + i] : 0;
-        cc[t] = i < cnt ? scl[q0 + i] : -1;
-        ff[t] = i < cnt ? fqs[q0 + i] : 0;
-    }
-    for (int w0 = 0; w0 < W; w0 += WM) {
-        const int nw = min(WM, W - w0);
-        // Fq = hi 2^20 + lo as two 32-bit sums (at most CH_ROWS rows between
-        // flushes: sum lo < 2^27, sum hi <= 2^24)
-        uint32_t alo[WM], ahi[WM];
-#pragma unroll
-        for (int t = 0; t < WM; ++t) alo[t] = ahi[t] = 0u;
-        int64_t usum = 0;
-        int cur = pick4(cc, 0);
-        auto flush = [&](int c) {
-#pragma unroll
-            for (int t = 0; t < WM; ++t) {
-                const int col = 32 * (w0 + t) + lane;
-                const unsigned long long v = ((unsigned long long)ahi[t] << 20) + alo[t];
-                if (t < nw && col < d && v) atomicAdd(T + (int64_t)c * (d + 1) + col, v);
-                alo[t] = ahi[t] = 0u;
-            }
-            if (w0 == 0 && lane == 0 && usum) atomicAdd(T + (int64_t)c * (d + 1) + d, (unsigned long long)usum);
-            usum = 0;
-        };
-        uint32_t buf[RB_DEPTH];
-#pragma unroll
-        for (int r = 0; r < RB_DEPTH; ++r) {
-            const int p = pick4(pp, r);
-            buf[r] = (r < cnt && lane < nw) ? __ldg(codes + (int64_t)p * W + w0 + lane) : 0u;
-        }
-        for (int i0 = 0; i0 < cnt; i0 += RB_DEPTH) {
-#pragma unroll
-            for (int r = 0; r < RB_DEPTH; ++r) {
-                const int i = i0 + r;
-                const uint32_t mine = buf[r];
-                const int in = i + RB_DEPTH;
-                const int pn = pick4(pp, in < CH_ROWS ? in : 0);
-                buf[r] = (in < cnt && lane < nw) ? __ldg(codes + (int64_t)pn * W + w0 + lane) : 0u;
-                if (i < cnt) {  // warp-uniform
-                    const int c = pick4(cc, i);
-                    const int64_t fq = pick4(ff, i);
-                    if (c != cur) {
-                        flush(cur);
-                        cur = c;
-                    }
-                    usum += fq;
-                    const uint32_t flo = (uint32_t)fq & 0xfffffu, fhi = (uint32_t)(fq >> 20);
-#pragma unroll
-                    for (int t = 0; t < WM; ++t) {
-                        if (t < nw) {
-                            add_if_bit2(alo[t], ahi[t], __shfl_sync(0xffffffffu, mine, t), lm, flo, fhi);
-                        }
-                    }
-                }
-            }
-        }
-        flush(cur);
-    }
-}
-
-static unsigned chunk_blocks(int64_t n) {
-    const int64_t per = (int64_t)CH_WARPS * CH_ROWS;
+static unsigned chunk_blocks(int64_t n, int run) {
+    const int64_t per = (int64_t)CH_WARPS * run;
     int64_t b = (n + per - 1) / per;
     return (unsigned)(b < 1 ? 1 : b);
 }
@@ -514,36 +480,19 @@ cudaError_t launch_chunk_sum_float(const void *X, int x_is_bf16, int64_t n, int 
                                    const int64_t *offsets, int k, float *S_f, double *S_d,
                                    cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    const unsigned g = chunk_blocks(n);
+    const int run = sum_run(n, 16, SUM_WARPS);
+    const unsigned g = chunk_blocks(n, run);
     if (S_d) {
         if (x_is_bf16)
-            chunk_sum_float_kernel<true, double><<<g, CH_WARPS * 32, 0, st>>>(X, d, perm, scl, offsets, k, S_d, d);
+            chunk_sum_float_kernel<true, double><<<g, CH_WARPS * 32, 0, st>>>(X, d, perm, scl, offsets, k, S_d, d, run);
         else
-            chunk_sum_float_kernel<false, double><<<g, CH_WARPS * 32, 0, st>>>(X, d, perm, scl, offsets, k, S_d, d);
+            chunk_sum_float_kernel<false, double><<<g, CH_WARPS * 32, 0, st>>>(X, d, perm, scl, offsets, k, S_d, d, run);
     } else {
         if (x_is_bf16)
-            chunk_sum_float_kernel<true, float><<<g, CH_WARPS * 32, 0, st>>>(X, d, perm, scl, offsets, k, S_f, d);
+            chunk_sum_float_kernel<true, float><<<g, CH_WARPS * 32, 0, st>>>(X, d, perm, scl, offsets, k, S_f, d, run);
         else
-            chunk_sum_float_kernel<false, float><<<g, CH_WARPS * 32, 0, st>>>(X, d, perm, scl, offsets, k, S_f, d);
+            chunk_sum_float_kernel<false, float><<<g, CH_WARPS * 32, 0, st>>>(X, d, perm, scl, offsets, k, S_f, d, run);
     }
-    return launched();
-}
-
-cudaError_t launch_chunk_sum_rbq1(const uint32_t *codes, const int64_t *fq, int64_t n, int d,
-                                  const int32_t *perm, const int32_t *scl, const int64_t *offsets,
-                                  int k, int64_t *T, cudaStream_t st) {
-    if (n == 0) return cudaSuccess;
-    const int W = (d + 31) >> 5;
-    auto T64 = reinterpret_cast<unsigned long long *>(T);
-    const unsigned g = chunk_blocks(n);
-    if (W <= 8)
-        chunk_sum_rbq1_kernel<8><<<g, CH_WARPS * 32, 0, st>>>(codes, fq, d, perm, scl, offsets, k, T64);
-    else if (W <= 16)
-        chunk_sum_rbq1_kernel<16><<<g, CH_WARPS * 32, 0, st>>>(codes, fq, d, perm, scl, offsets, k, T64);
-    else if (W <= 24)
-        chunk_sum_rbq1_kernel<24><<<g, CH_WARPS * 32, 0, st>>>(codes, fq, d, perm, scl, offsets, k, T64);
-    else
-        chunk_sum_rbq1_kernel<32><<<g, CH_WARPS * 32, 0, st>>>(codes, fq, d, perm, scl, offsets, k, T64);
     return launched();
 }
 

@@ -207,11 +207,8 @@ static void plan_assign(const skm_data *x, int k, Carver &cv, AssignBufs &b) {
 struct UpdateBufs {
     int32_t *counts32 = nullptr, *cursor = nullptr, *perm = nullptr, *scl = nullptr;
     int64_t *offsets = nullptr;
-    int64_t *fq = nullptr;    // RBQ1: fixed-point weights round(F 2^e)
-    uint32_t *sq = nullptr;   // LVQ4: round(s 2^e), sorted order
-    int64_t *bq = nullptr;    // LVQ4: round(b 2^e), sorted order
     float *sumf = nullptr;    // F32/BF16: cluster sums [k][d]
-    int64_t *sumi = nullptr;  // RBQ1: cluster sums [k][d + 1]; SQ8: [k][d]
+    int64_t *sumi = nullptr;  // RBQ1 / LVQ4: cluster sums [k][d + 1]; SQ8: [k][d]
     int32_t *flag = nullptr;  // raised by a streamed-sum wait that gave up
     int64_t *wsplit = nullptr;  // empty-cluster split: working member counts [k]
 };
@@ -222,15 +219,7 @@ static void plan_update(const skm_data *x, int k, Carver &cv, UpdateBufs &b) {
     b.offsets = cv.take<int64_t>((size_t)k + 1);
     b.perm = cv.take<int32_t>(x->n);
     b.scl = cv.take<int32_t>(x->n);
-    if (x->repr == SKM_REPR_RBQ1) {
-        b.fq = cv.take<int64_t>(x->n);
-        b.sumi = cv.take<int64_t>((size_t)k * (x->d + 1));
-    }
-    if (x->repr == SKM_REPR_LVQ4) {
-        b.sq = cv.take<uint32_t>(x->n);
-        b.bq = cv.take<int64_t>(x->n);
-        b.sumi = cv.take<int64_t>((size_t)k * (x->d + 1));
-    }
+    if (x->repr == SKM_REPR_RBQ1 || x->repr == SKM_REPR_LVQ4) b.sumi = cv.take<int64_t>((size_t)k * (x->d + 1));
     if (x->repr == SKM_REPR_SQ8) b.sumi = cv.take<int64_t>((size_t)k * x->d);
     if (x->repr == SKM_REPR_F32 || x->repr == SKM_REPR_BF16) b.sumf = cv.take<float>((size_t)k * x->d);
     b.flag = cv.take<int32_t>(1);
@@ -259,6 +248,8 @@ __global__ void count_moved_kernel(const int32_t *__restrict__ a, const int32_t 
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
 }
+
+constexpr int OBJ_LOG = 1024;  // objective values kept on the device between copies
 
 struct FitBufs {
     uint8_t *screen = nullptr;  // built once per fit when the caller gave none
@@ -300,7 +291,7 @@ static void plan_fit(const skm_data *x, int k, Carver &cv, FitBufs &b) {
     plan_update(x, k, cv, b.u);
     b.dist = cv.take<float>(x->n);
     b.partials = cv.take<double>(RED_BLOCKS);
-    b.sum = cv.take<double>(1);
+    b.sum = cv.take<double>(OBJ_LOG);
     b.maxbits = cv.take<unsigned int>(1);
     b.e_dev = cv.take<int>(1);
     b.status = cv.take<int>(1);
@@ -387,13 +378,18 @@ static int do_assign(const skm_data *x, const void *C, int k, const int32_t *pre
 }
 
 static int do_update(const skm_data *x, const int32_t *assign, int k, void *C, int64_t *counts,
-                     void *partial, int e, UpdateBufs &b, cudaStream_t st) {
+                     void *partial, int e, UpdateBufs &b, cudaStream_t st, int64_t *zeros = nullptr,
+                     bool clear_flag = false) {
     const int64_t n = x->n;
     const int d = x->d;
-    SKM_CUDA_TRY(launch_histogram(assign, n, k, b.counts32, st));
-    SKM_CUDA_TRY(launch_scan_offsets(b.counts32, k, b.offsets, counts, partial ? 1 : 0, st));
-    SKM_CUDA_TRY(cudaMemsetAsync(b.cursor, 0, sizeof(int32_t) * (size_t)k, st));
-    SKM_CUDA_TRY(launch_scatter(assign, n, k, b.offsets, b.cursor, b.perm, b.scl, st));
+    // the workspace sums the kernels add to (none when partial receives them,
+    // or when the SQ8 rows take the kernel that needs none)
+    void *sums = b.sumf ? static_cast<void *>(b.sumf) : b.sumi;
+    size_t sum_bytes = b.sumf ? sizeof(float) * (size_t)k * d
+                              : sizeof(int64_t) * (size_t)k * (x->repr == SKM_REPR_SQ8 ? d : d + 1);
+    if (partial || (x->repr == SKM_REPR_SQ8 && !ring_sum_sq8_ok(x->x, d))) sum_bytes = 0;
+    SKM_CUDA_TRY(launch_sort_by_cluster(assign, n, k, b.counts32, b.cursor, b.offsets, counts, partial ? 1 : 0, b.perm,
+                                        b.scl, zeros, clear_flag ? b.flag : nullptr, sums, sum_bytes, st));
     switch (x->repr) {
     case SKM_REPR_F32:
     case SKM_REPR_BF16: {
@@ -401,7 +397,6 @@ static int do_update(const skm_data *x, const int32_t *assign, int k, void *C, i
         const bool ring = ring_sum_float_ok(x->x, bf, d);
         float *Sf = partial ? nullptr : b.sumf;
         double *Sd = partial ? static_cast<double *>(partial) : nullptr;
-        if (!partial) SKM_CUDA_TRY(cudaMemsetAsync(b.sumf, 0, sizeof(float) * (size_t)k * d, st));
         if (ring)
             SKM_CUDA_TRY(launch_ring_sum_float(x->x, bf, n, d, b.perm, b.scl, b.offsets, k, Sf, Sd,
                                                b.flag, st));
@@ -415,7 +410,6 @@ static int do_update(const skm_data *x, const int32_t *assign, int k, void *C, i
         const uint8_t *codes = static_cast<const uint8_t *>(x->x);
         if (ring_sum_sq8_ok(codes, d)) {
             int64_t *S = partial ? static_cast<int64_t *>(partial) : b.sumi;
-            if (!partial) SKM_CUDA_TRY(cudaMemsetAsync(S, 0, sizeof(int64_t) * (size_t)k * d, st));
             SKM_CUDA_TRY(launch_ring_sum_sq8(codes, n, d, b.perm, b.scl, b.offsets, k, S, b.flag, st));
             if (!partial)
                 SKM_CUDA_TRY(launch_finalize_sq8(S, counts, k, d, static_cast<uint8_t *>(C), st));
@@ -426,29 +420,18 @@ static int do_update(const skm_data *x, const int32_t *assign, int k, void *C, i
         break;
     }
     case SKM_REPR_RBQ1: {
-        SKM_CUDA_TRY(launch_rbq1_fq(x->F, b.perm, b.offsets, k, n, e, b.fq, st));
         int64_t *T = partial ? static_cast<int64_t *>(partial) : b.sumi;
-        if (!partial) SKM_CUDA_TRY(cudaMemsetAsync(T, 0, sizeof(int64_t) * (size_t)k * (d + 1), st));
         const uint32_t *codes = static_cast<const uint32_t *>(x->x);
-        if (ring_sum_rbq1_ok(codes, d))
-            SKM_CUDA_TRY(launch_ring_sum_rbq1(codes, b.fq, n, d, b.perm, b.scl, b.offsets, k, T,
-                                              b.flag, st));
-        else
-            SKM_CUDA_TRY(launch_chunk_sum_rbq1(codes, b.fq, n, d, b.perm, b.scl, b.offsets, k, T, st));
+        SKM_CUDA_TRY(launch_sum_rbq1(codes, x->F, e, n, d, b.perm, b.scl, b.offsets, k, T, st));
         if (!partial)
             SKM_CUDA_TRY(launch_finalize_rbq1(T, counts, k, d, x->m, e, static_cast<float *>(C), st));
         break;
     }
     case SKM_REPR_LVQ4: {
-        SKM_CUDA_TRY(launch_lvq4_q(reinterpret_cast<const float4 *>(x->lvq), b.perm, b.offsets, k, n, e, b.sq, b.bq,
-                                   st));
         int64_t *T = partial ? static_cast<int64_t *>(partial) : b.sumi;
-        if (!partial) SKM_CUDA_TRY(cudaMemsetAsync(T, 0, sizeof(int64_t) * (size_t)k * (d + 1), st));
         const uint32_t *codes = static_cast<const uint32_t *>(x->x);
-        if (ring_sum_lvq4_ok(codes, d))
-            SKM_CUDA_TRY(launch_ring_sum_lvq4(codes, b.sq, b.bq, n, d, b.perm, b.scl, b.offsets, k, T, b.flag, st));
-        else
-            SKM_CUDA_TRY(launch_chunk_sum_lvq4(codes, b.sq, b.bq, n, d, b.perm, b.scl, b.offsets, k, T, st));
+        SKM_CUDA_TRY(launch_sum_lvq4(codes, reinterpret_cast<const float4 *>(x->lvq), e, n, d, b.perm, b.scl, b.offsets,
+                                     k, T, st));
         if (!partial) SKM_CUDA_TRY(launch_finalize_lvq4(T, counts, k, d, e, static_cast<float *>(C), st));
         break;
     }
@@ -1157,8 +1140,7 @@ int skm_update(const skm_data *x, const int32_t *assign, int k, void *C_inout, i
     UpdateBufs b;
     plan_update(x, k, cv, b);
     SKM_TRY(need_ws(cv, ws_bytes, ws));
-    SKM_CUDA_TRY(cudaMemsetAsync(b.flag, 0, sizeof(int32_t), S(stream)));
-    return do_update(x, assign, k, C_inout, counts, partial, x->rbq1_exp, b, S(stream));
+    return do_update(x, assign, k, C_inout, counts, partial, x->rbq1_exp, b, S(stream), nullptr, true);
 }
 
 int skm_merge_partials(void *dst, const void *src, int64_t count, int elem_type, void *stream) {
@@ -1320,15 +1302,17 @@ int skm_fit(const skm_fit_config *cfg, const skm_data *x, const void *C_init,
             }
         }
         if (want_obj) {
-            SKM_CUDA_TRY(launch_sum_float_to_double(dist, n, b.partials, nblk, st));
-            SKM_CUDA_TRY(launch_sum_double(b.partials, nblk, b.sum, st));
-            SKM_CUDA_TRY(cudaMemcpyAsync(&objective_host[it], b.sum, sizeof(double),
-                                         cudaMemcpyDeviceToHost, st));
+            // kept on the device and read back OBJ_LOG at a time: a copy to the
+            // caller's pageable array would wait for every iteration
+            const int slot = it % OBJ_LOG;
+            SKM_CUDA_TRY(launch_sum_float(dist, n, b.partials, nblk, b.sum + slot, st));
+            if (slot == OBJ_LOG - 1 || it == cfg->iters)
+                SKM_CUDA_TRY(cudaMemcpyAsync(objective_host + (it - slot), b.sum, sizeof(double) * (size_t)(slot + 1),
+                                             cudaMemcpyDeviceToHost, st));
         }
         if (it == cfg->iters) break;
-        SKM_TRY(do_update(&xd, assign, k, C_out, b.counts, nullptr, e, b.u, st));
-        if (stats_host && stats_host->empty_per_iter && it < EMPTY_LOG)
-            SKM_CUDA_TRY(launch_count_zeros(b.counts, k, b.empty_iter + it, st));
+        SKM_TRY(do_update(&xd, assign, k, C_out, b.counts, nullptr, e, b.u, st,
+                          it < EMPTY_LOG ? b.empty_iter + it : nullptr));
         if (cfg->empty_policy == SKM_EMPTY_SPLIT)
             SKM_CUDA_TRY(launch_split_empty(C_out, x->repr == SKM_REPR_SQ8 ? 1 : 4, b.counts, k, x->d,
                                             b.u.wsplit, st));

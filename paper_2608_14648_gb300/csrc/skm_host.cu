@@ -217,8 +217,7 @@ extern "C" int skm_lloyd_step_host(const skm_step_host_config *cfg, const skm_da
             SKM_TRY(skm_update(&v, b.assign[s], k, nullptr, counts, partial, b.ws_u, b.ws_u_bytes, st));
             if (objective_host) {
                 const int nblk = (int)std::min<int64_t>(RED, rows);
-                SKM_CUDA_TRY(launch_sum_float_to_double(b.dist[s], rows, b.red, nblk, st));
-                SKM_CUDA_TRY(launch_sum_double(b.red, nblk, b.chunk_sum + i, st));
+                SKM_CUDA_TRY(launch_sum_float(b.dist[s], rows, b.red, nblk, b.chunk_sum + i, st));
             }
             SKM_CUDA_TRY(cudaMemcpyAsync(assign_host + r0, b.assign[s], sizeof(int32_t) * (size_t)rows,
                                          cudaMemcpyDeviceToHost, st));

@@ -102,20 +102,6 @@ __device__ __forceinline__ void add_if_bit(uint32_t &acc, uint32_t word, uint32_
         : "r"(mask), "r"(f));
 }
 
-// (lo, hi) += (flo, fhi) when (word & mask) != 0, as two predicated 32-bit
-// adds (no branch, no carry); used by the 1-bit decode-average sums, which
-// split each fixed-point weight as hi 2^20 + lo.
-__device__ __forceinline__ void add_if_bit2(uint32_t &lo, uint32_t &hi, uint32_t word, uint32_t mask,
-                                            uint32_t flo, uint32_t fhi) {
-    asm("{\n\t.reg .pred p;\n\t"
-        "and.b32 %2, %2, %3;\n\t"
-        "setp.ne.u32 p, %2, 0;\n\t"
-        "@p add.u32 %0, %0, %4;\n\t"
-        "@p add.u32 %1, %1, %5;\n\t}"
-        : "+r"(lo), "+r"(hi), "+r"(word)
-        : "r"(mask), "r"(flo), "r"(fhi));
-}
-
 // e4m3 encodings of the integers 0..15 (sign 0, exponent bias 7, 3 mantissa
 // bits): 0 -> 0x00, 1 -> 0x38, 2 -> 0x40, 3 -> 0x44, 4 -> 0x48, ... 15 -> 0x57.
 __device__ __forceinline__ uint8_t e4m3_of_code(uint32_t y) {
@@ -269,32 +255,44 @@ cudaError_t launch_assign_rbq1(const uint32_t *codes, const float *nx2, const fl
 // update
 cudaError_t launch_histogram(const int32_t *assign, int64_t n, int k, int32_t *counts32,
                              cudaStream_t st);
-// *out = number of j < k with counts[j] == 0
-cudaError_t launch_count_zeros(const int64_t *counts, int k, int64_t *out, cudaStream_t st);
-cudaError_t launch_scan_offsets(const int32_t *counts32, int k, int64_t *offsets,
-                                int64_t *counts64_out, int accumulate_counts, cudaStream_t st);
-cudaError_t launch_scatter(const int32_t *assign, int64_t n, int k, const int64_t *offsets,
-                           int32_t *cursor, int32_t *perm, int32_t *scl, cudaStream_t st);
-// load-balanced segmented sums over the cluster-sorted order (global atomics)
+// perm / scl: the points in cluster order and their clusters (assignments
+// outside [0, k) left out); offsets[k + 1], counts64 (set, or added to),
+// *zeros = empty clusters (may be NULL); clears *flag (may be NULL) and
+// sum_bytes of sums.  counts32 and cursor: k ints of workspace.
+cudaError_t launch_sort_by_cluster(const int32_t *assign, int64_t n, int k, int32_t *counts32, int32_t *cursor,
+                                   int64_t *offsets, int64_t *counts64, int accumulate, int32_t *perm, int32_t *scl,
+                                   int64_t *zeros, int32_t *flag, void *sums, size_t sum_bytes, cudaStream_t st);
+// Load-balanced segmented sums over the cluster-sorted order (global atomics):
+// a warp sums a run of sum_run(n) consecutive positions.  A long run flushes
+// its sums less often; a short one keeps the GPU full when there are few
+// rows, since a run's rows are summed one after another (at n = 20,000 runs of
+// 128 rows are 157 warps, one per SM, for 66 us of an SQ8 update at d = 128).
+// So: the longest power of two that still gives `warps` warps an SM.  16
+// warps for the code sums (64-bit atomics: 200,000 x 384 SQ8 takes 60 us with
+// 16, 65 with 32, 74 with 64); 64 for fp32 rows, whose flush is one 16-byte
+// atomic per four columns (1M x 768: 510 us with 16, 483 with 64; 350,000 x
+// 100: 114 and 99).
+constexpr int SUM_RUN_MAX = 128;
+constexpr int SUM_WARPS = 16, SUM_WARPS_F32 = 64;
+inline int sum_run(int64_t n, int least, int warps) {
+    int run = SUM_RUN_MAX;
+    while (run > least && n < (int64_t)run * 152 * warps) run >>= 1;
+    return run;
+}
 cudaError_t launch_chunk_sum_float(const void *X, int x_is_bf16, int64_t n, int d,
                                    const int32_t *perm, const int32_t *scl,
                                    const int64_t *offsets, int k, float *S_f, double *S_d,
                                    cudaStream_t st);
-cudaError_t launch_chunk_sum_rbq1(const uint32_t *codes, const int64_t *fq_sorted, int64_t n, int d,
-                                  const int32_t *perm, const int32_t *scl, const int64_t *offsets,
-                                  int k, int64_t *T, cudaStream_t st);
+cudaError_t launch_sum_rbq1(const uint32_t *codes, const float *F, int e, int64_t n, int d, const int32_t *perm,
+                            const int32_t *scl, const int64_t *offsets, int k, int64_t *T, cudaStream_t st);
 cudaError_t launch_finalize_float32(const float *S, const int64_t *counts, int k, int d,
                                     float *C_inout, cudaStream_t st);
 cudaError_t launch_segsum_sq8(const uint8_t *X, int d, const int32_t *perm,
                               const int64_t *offsets, int k, uint8_t *C_inout, int64_t *partial,
                               cudaStream_t st);
-// Fq = round(F[perm[q]] 2^e) for the sorted positions q < offsets[k]
-cudaError_t launch_rbq1_fq(const float *F, const int32_t *perm, const int64_t *offsets, int k,
-                           int64_t n, int e, int64_t *fq_sorted, cudaStream_t st);
 // streamed segmented sums (cp.async.bulk row gathers into shared-memory rings);
 // *_ok says whether the row size and alignment suit them
 bool ring_sum_float_ok(const void *X, int x_is_bf16, int d);
-bool ring_sum_rbq1_ok(const void *codes, int d);
 bool ring_sum_sq8_ok(const void *codes, int d);
 // y = H_D diag(sigma) [x - mean; 0] / sqrt(D), D a power of two in [32, 4096]
 cudaError_t launch_hadamard(const float *X, int64_t n, int d, const float *mean, const float *sigma, int D,
@@ -319,9 +317,6 @@ cudaError_t launch_ring_sum_sq8(const uint8_t *codes, int64_t n, int d, const in
 cudaError_t launch_ring_sum_float(const void *X, int x_is_bf16, int64_t n, int d, const int32_t *perm,
                                   const int32_t *scl, const int64_t *offsets, int k, float *S_f,
                                   double *S_d, int32_t *flag, cudaStream_t st);
-cudaError_t launch_ring_sum_rbq1(const uint32_t *codes, const int64_t *fq_sorted, int64_t n, int d,
-                                 const int32_t *perm, const int32_t *scl, const int64_t *offsets,
-                                 int k, int64_t *T, int32_t *flag, cudaStream_t st);
 cudaError_t launch_finalize_float(const double *partial, const int64_t *counts, int k, int d,
                                   float *C_inout, cudaStream_t st);
 cudaError_t launch_finalize_sq8(const int64_t *partial, const int64_t *counts, int k, int d,
@@ -341,8 +336,9 @@ cudaError_t launch_objective(const void *X, int x_is_bf16, int64_t n, int d, con
                              const int32_t *assign, double *partials, int nblk,
                              cudaStream_t st);
 cudaError_t launch_sum_double(const double *in, int64_t count, double *out, cudaStream_t st);
-cudaError_t launch_sum_float_to_double(const float *in, int64_t count, double *partials,
-                                       int nblk, cudaStream_t st);
+// *out = sum of in[0 .. count) in fp64 (partials: nblk doubles of workspace)
+cudaError_t launch_sum_float(const float *in, int64_t count, double *partials, int nblk, double *out,
+                             cudaStream_t st);
 cudaError_t launch_project(const float *X, int64_t n, int d, const float *mean, const float *P,
                            int d_out, int out_bf16, void *Y, cudaStream_t st);
 cudaError_t launch_cov_partial(const float *X, int64_t n, int d, const float *mean,
@@ -372,16 +368,8 @@ cudaError_t launch_lvq4_pack_pairs(const float4 *info, int k, int kp, float4 *bg
 cudaError_t launch_assign_lvq4_simt(const uint32_t *codes, const float4 *fac, int64_t n, int d,
                                     const uint32_t *yw, const float4 *info, int k, int32_t *assign,
                                     float *dist, cudaStream_t st);
-// Sq = round(s 2^e) (uint32) and Bq = round(b 2^e) (int64) in cluster-sorted order
-cudaError_t launch_lvq4_q(const float4 *fac, const int32_t *perm, const int64_t *offsets, int k, int64_t n,
-                          int e, uint32_t *sq, int64_t *bq, cudaStream_t st);
-bool ring_sum_lvq4_ok(const void *codes, int d);
-cudaError_t launch_ring_sum_lvq4(const uint32_t *codes, const uint32_t *sq, const int64_t *bq, int64_t n,
-                                 int d, const int32_t *perm, const int32_t *scl, const int64_t *offsets,
-                                 int k, int64_t *T, int32_t *flag, cudaStream_t st);
-cudaError_t launch_chunk_sum_lvq4(const uint32_t *codes, const uint32_t *sq, const int64_t *bq, int64_t n,
-                                  int d, const int32_t *perm, const int32_t *scl, const int64_t *offsets,
-                                  int k, int64_t *T, cudaStream_t st);
+cudaError_t launch_sum_lvq4(const uint32_t *codes, const float4 *fac, int e, int64_t n, int d, const int32_t *perm,
+                            const int32_t *scl, const int64_t *offsets, int k, int64_t *T, cudaStream_t st);
 cudaError_t launch_finalize_lvq4(const int64_t *partial, const int64_t *counts, int k, int d, int e,
                                  float *C_inout, cudaStream_t st);
 cudaError_t launch_lvq4_decode_rows(const uint32_t *codes, const float4 *fac, int64_t n, int d, int e,
