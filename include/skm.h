@@ -94,7 +94,8 @@ enum {
      * distance (XOR + POPCOUNT) of the sign codes.  fp32 order: fy =
      * fl32((||rho||^2 / ||rho||_1) / sqrt(d)) per centroid (fp64, blocked
      * order), u = fy (d - 2 h), est = fma(-2 F, u, nx2 + ||rho||^2).  Tensor
-     * cores (e4m3 +-1 codes on both sides) for d <= 1024, XOR + POPC beyond.
+     * cores (e4m3 +-1 codes on both sides) where the plain assignment runs there
+     * (see skm_assign), XOR + POPC elsewhere.
      * The update is unchanged (the points' fused decode-average). */
     SKM_FLAG_SYMMETRIC = 2,
     /* F32 / BF16 (tensor-core screen) only: the points and the workspace are
@@ -427,9 +428,9 @@ int skm_lvq4_exponent(const float *lvq, int64_t n, int *e_host, void *ws, size_t
  * its point tiles into a slot of the workspace, at most 160 x 4 x 128 x
  * round16(d) bytes), so the points occupy their code words in HBM instead of
  * round16(d) bytes; the copy saves that per-tile expansion (measured on
- * GB300, 1M x 768, k = 1000: RBQ1 0.61 ms packed, 0.50 ms from the copy;
- * LVQ4 0.76 and 0.52 ms; at k = 3162 and d = 1024 the gap is 7-9%).
- * Otherwise skm_assign builds the copy in its workspace on every call. */
+ * GB300, 1M x 768, k = 1000: LVQ4 0.63 ms packed, 0.52 ms from the copy).
+ * Otherwise skm_assign builds the copy in its workspace on every call (d <=
+ * 1024; longer rows are then assigned on CUDA cores). */
 size_t skm_screen_bytes(const skm_data *x);
 int skm_screen_prep(const skm_data *x, void *screen, size_t screen_bytes, void *stream);
 
@@ -457,7 +458,10 @@ int skm_screen_prep(const skm_data *x, void *screen, size_t screen_bytes, void *
  *          u = fma(sd, 2P - sum ybar, bd (2 popx - d))
  *          dist = fma(-2 F, u, nx2 + ny2)
  *        where P = sum_i xbar_i ybar_i is an exact integer (tensor cores in
- *        e4m3 for d <= 1024, AND + popcount beyond).
+ *        e4m3 for d <= 1024, and for longer rows read packed, as described
+ *        at skm_screen_bytes; AND + popcount otherwise, and when the
+ *        workspace is smaller than skm_workspace_size but holds the centroids'
+ *        bit planes).
  *   LVQ4 float [k][d] decoded centroids; per call each centroid is
  *        re-encoded with LVQ4 exactly as skm_quantize encodes a point
  *        (s_y, b_y, ybar, N_y; G_y = s_y sum ybar rounded once to fp32) and
@@ -466,7 +470,7 @@ int skm_screen_prep(const skm_data *x, void *screen, size_t screen_bytes, void *
  *          key = fma(G_y, -2 b_x, key)
  *          key = fma(-2 s_x, s_y * P, key)
  *        with P = sum_i xbar_i ybar_i an exact integer (tensor cores in
- *        e4m3 for d <= 1024, __dp4a beyond); the argmin is taken over key
+ *        e4m3, __dp4a otherwise, as for RBQ1); the argmin is taken over key
  *        (N_x is the same for every centroid of a row) and dist = N_x + key.
  *  assign int32[n] (required); dist float[n] (may be NULL).
  *  prev_assign int32[n] or NULL: with SKM_FLAG_PRUNE, seeds each row's

@@ -266,12 +266,25 @@ __global__ void lvq4_exponent_kernel(const unsigned int *__restrict__ maxbits, i
     *e = 31 - c;
 }
 
-// One warp per centroid; info[j] = (s, b, N, G = s * sum ybar).
+// One warp per centroid; (s, b, N, G = s * sum ybar) into info and / or the
+// column pairs.
 __global__ void lvq4_cprep_kernel(const float *__restrict__ C, int k, int d, uint8_t *__restrict__ yq, int dq,
-                                  uint32_t *__restrict__ yw, float4 *__restrict__ info) {
+                                  uint32_t *__restrict__ yw, float4 *__restrict__ info, const CodePairs pairs) {
     const int lane = threadIdx.x & 31;
     const int j = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    if (j >= k) return;  // warp-uniform
+    if (pairs.counters && blockIdx.x == 0 && threadIdx.x < 4) pairs.counters[threadIdx.x] = 0;
+    auto put_pair = [&](float s, float b, float nn, float g) {
+        float *bg = reinterpret_cast<float *>(pairs.bs + (j >> 1)) + (j & 1);
+        float *sn = reinterpret_cast<float *>(pairs.qn + (j >> 1)) + (j & 1);
+        bg[0] = b;
+        bg[2] = g;
+        sn[0] = s;
+        sn[2] = nn;
+    };
+    if (j >= k) {  // warp-uniform
+        if (lane == 0 && j < pairs.kp) put_pair(0.0f, 0.0f, INFINITY, 0.0f);
+        return;
+    }
     const int W = lvq4_words(d);
     const Lvq4Vec r = lvq4_encode_warp(C + (int64_t)j * d, d, lane, [&](int base, int ln, uint32_t c) {
         const int i = base + ln;
@@ -282,9 +295,12 @@ __global__ void lvq4_cprep_kernel(const float *__restrict__ C, int k, int d, uin
             if ((ln & 7) == 0 && wi < W) yw[(int64_t)j * W + wi] = v;
         }
     });
-    if (lane == 0)
-        info[j] = make_float4(r.s, r.lo, __double2float_rn(lvq4_norm(r, d)),
-                              __double2float_rn(__dmul_rn((double)r.s, (double)r.S)));
+    if (lane == 0) {
+        const float nn = __double2float_rn(lvq4_norm(r, d));
+        const float g = __double2float_rn(__dmul_rn((double)r.s, (double)r.S));
+        if (info) info[j] = make_float4(r.s, r.lo, nn, g);
+        if (pairs.bs) put_pair(r.s, r.lo, nn, g);
+    }
 }
 
 // nibble words -> e4m3 bytes (8 per word, one 8-byte store)
@@ -304,30 +320,6 @@ __global__ void lvq4_expand_kernel(const uint32_t *__restrict__ codes, int64_t n
         }
         *reinterpret_cast<uint2 *>(xs + r * dq + 8 * w) = make_uint2(lo, hi);
     }
-}
-
-// Column-pair records of the tensor epilogue; columns past k get N = +inf.
-__global__ void lvq4_pack_pairs_kernel(const float4 *__restrict__ info, int k, int kp, float4 *__restrict__ bg,
-                                      float4 *__restrict__ sn) {
-    const int pp = blockIdx.x * blockDim.x + threadIdx.x;
-    if (2 * pp >= kp) return;
-    float b[2], g[2], s[2], nn[2];
-#pragma unroll
-    for (int o = 0; o < 2; ++o) {
-        const int j = 2 * pp + o;
-        if (j < k) {
-            const float4 in = info[j];
-            s[o] = in.x;
-            b[o] = in.y;
-            nn[o] = in.z;
-            g[o] = in.w;
-        } else {
-            s[o] = b[o] = g[o] = 0.0f;
-            nn[o] = INFINITY;
-        }
-    }
-    bg[pp] = make_float4(b[0], b[1], g[0], g[1]);
-    sn[pp] = make_float4(s[0], s[1], nn[0], nn[1]);
 }
 
 // d > 1024: one thread per point, tiles of SA_KT centroids in shared memory as
@@ -464,8 +456,9 @@ cudaError_t launch_lvq4_exponent(const float4 *fac, int64_t n, unsigned int *max
 }
 
 cudaError_t launch_lvq4_cprep(const float *C, int k, int d, uint8_t *yq, int dq, uint32_t *yw, float4 *info,
-                              cudaStream_t st) {
-    lvq4_cprep_kernel<<<(k + 7) / 8, 256, 0, st>>>(C, k, d, yq, dq, yw, info);
+                              const CodePairs &pairs, cudaStream_t st) {
+    const int rows = k > pairs.kp ? k : pairs.kp;
+    lvq4_cprep_kernel<<<(rows + 7) / 8, 256, 0, st>>>(C, k, d, yq, dq, yw, info, pairs);
     return launched();
 }
 
@@ -473,11 +466,6 @@ cudaError_t launch_lvq4_expand(const uint32_t *codes, int64_t n, int d, uint8_t 
     int64_t blocks = (n * lvq4_words(d) + 255) / 256;
     if (blocks > 152 * 8) blocks = 152 * 8;
     lvq4_expand_kernel<<<(unsigned)(blocks < 1 ? 1 : blocks), 256, 0, st>>>(codes, n, d, xs, dq);
-    return launched();
-}
-
-cudaError_t launch_lvq4_pack_pairs(const float4 *info, int k, int kp, float4 *bg, float4 *sn, cudaStream_t st) {
-    lvq4_pack_pairs_kernel<<<(kp / 2 + 255) / 256, 256, 0, st>>>(info, k, kp, bg, sn);
     return launched();
 }
 

@@ -109,6 +109,7 @@ cudaError_t launch_objective(const void *X, int x_is_bf16, int64_t n, int d, con
 // order by thread 0 (its return value; the others' is not used).
 __device__ __forceinline__ double block_sum(double s) {
     __shared__ double wsum[32];
+    __syncthreads();  // a second call's sums after the first's have been read
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = s;
@@ -119,35 +120,53 @@ __device__ __forceinline__ double block_sum(double s) {
     return t;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(1024) sum_to_double_kernel(const T *__restrict__ in, int64_t count,
-                                                             double *__restrict__ out) {
+__global__ void __launch_bounds__(512) sum_double_kernel(const double *__restrict__ in, int64_t count,
+                                                         double *__restrict__ out) {
+    double s = 0.0;
+    for (int64_t i = threadIdx.x; i < count; i += blockDim.x) s += in[i];
+    s = block_sum(s);
+    if (threadIdx.x == 0) *out = s;
+}
+
+cudaError_t launch_sum_double(const double *in, int64_t count, double *out, cudaStream_t st) {
+    sum_double_kernel<<<1, 512, 0, st>>>(in, count, out);
+    return launched();
+}
+
+// One launch: the blocks' sums, and the last block to finish (ticket: zeroed
+// once by the caller, and back at zero after every call) adds them up in
+// order.  fp64 additions and conversions run at two a clock and SM, so the
+// values are spread over the SMs, 1024 a block, whatever their number.  (Two
+// kernels with serial sums over 256 threads took 23 us for each iteration's
+// objective.)
+__global__ void __launch_bounds__(256) sum_float_kernel(const float *__restrict__ in, int64_t count,
+                                                        double *__restrict__ partials, unsigned int *__restrict__ ticket,
+                                                        double *__restrict__ out) {
+    __shared__ bool last;
     double s = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
         s += (double)in[i];
     s = block_sum(s);
-    if (threadIdx.x == 0) out[blockIdx.x] = s;
-}
-
-cudaError_t launch_sum_double(const double *in, int64_t count, double *out, cudaStream_t st) {
-    sum_to_double_kernel<double><<<1, 512, 0, st>>>(in, count, out);
-    return launched();
-}
-
-// A block's 1024 threads read 64 values each in about the time that a second
-// launch costs, so up to SUM1_MAX values take one block and no partials.  (The
-// serial sums over 256 threads this replaces took 11 us a kernel, two kernels
-// for each iteration's objective whatever n.)
-constexpr int64_t SUM1_MAX = 65536;
-cudaError_t launch_sum_float(const float *in, int64_t count, double *partials, int nblk, double *out,
-                             cudaStream_t st) {
-    if (count <= SUM1_MAX) {
-        sum_to_double_kernel<float><<<1, 1024, 0, st>>>(in, count, out);
-        return launched();
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = s;
+        __threadfence();
+        last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
     }
-    sum_to_double_kernel<float><<<nblk, 512, 0, st>>>(in, count, partials);
-    const cudaError_t e = launched();
-    return e == cudaSuccess ? launch_sum_double(partials, nblk, out, st) : e;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    s = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) s += __ldcg(partials + i);
+    s = block_sum(s);
+    if (threadIdx.x == 0) *out = s;
+}
+
+cudaError_t launch_sum_float(const float *in, int64_t count, double *partials, int nblk, unsigned int *ticket,
+                             double *out, cudaStream_t st) {
+    const int64_t want = (count + 1023) / 1024;
+    const int blocks = (int)(want < nblk ? want : nblk);
+    sum_float_kernel<<<blocks, 256, 0, st>>>(in, count, partials, ticket, out);
+    return launched();
 }
 
 // --------------------------------------------------------------- projection

@@ -125,13 +125,9 @@ constexpr int REC_BYTES = 4096;
 // merge buffer (per group, slices 1..NH/NS-1 publish) and the record buffers
 // (two per group).
 template <int MODE, int NH, int NS>
-constexpr size_t tc_lut_offset() {  // LVQ4 read packed: byte -> two e4m3 codes, after the records
-    return (size_t)STAGES * (A_STAGE + B_STAGE) + 512 + (size_t)(NH - NS) * BM * merge_words<MODE>() * 4 +
-           2 * NS * REC_BYTES;
-}
-template <int MODE, int NH, int NS>
 constexpr size_t tc_smem_bytes() {
-    return 1024 + tc_lut_offset<MODE, NH, NS>() + (MODE == 3 /* MODE_LVQ4 */ ? 512 : 0);
+    return 1024 + (size_t)STAGES * (A_STAGE + B_STAGE) + 512 + (size_t)(NH - NS) * BM * merge_words<MODE>() * 4 +
+           2 * NS * REC_BYTES;
 }
 
 struct TcParams {
@@ -377,6 +373,20 @@ __device__ __forceinline__ uint32_t pm1_e4m3(uint32_t v) {
     return (t & 0x80808080u) ^ 0xB8B8B8B8u;
 }
 
+// The eight nibbles of v -> their e4m3 codes, four bytes in lo and four in hi.
+// A byte permute looks three bits of four nibbles up at once, in the codes of
+// 0..7 and of 8..15; another spreads each nibble's top bit over a byte (sign
+// replication) to choose between the two.
+__device__ __forceinline__ void nibbles_e4m3(uint32_t v, uint32_t &lo, uint32_t &hi) {
+    constexpr uint32_t T0 = 0x44403800u, T1 = 0x4E4C4A48u, T2 = 0x53525150u, T3 = 0x57565554u;
+    const uint32_t s = v & 0x77777777u, e = v << 4;
+    uint32_t ml, mh;  // (__byte_perm takes no sign replication)
+    asm("prmt.b32 %0, %1, %2, 0xD9C8;" : "=r"(ml) : "r"(e), "r"(v));
+    asm("prmt.b32 %0, %1, %2, 0xFBEA;" : "=r"(mh) : "r"(e), "r"(v));
+    lo = (__byte_perm(T0, T1, s) & ~ml) | (__byte_perm(T2, T3, s) & ml);
+    hi = (__byte_perm(T0, T1, s >> 16) & ~mh) | (__byte_perm(T2, T3, s >> 16) & mh);
+}
+
 // min(a, b, c) in one instruction (sm_100 family three-input min)
 __device__ __forceinline__ float fmin3(float a, float b, float c) {
     float r;
@@ -545,11 +555,6 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
     // starts further on, 256 bytes after tmem_slot
     static_assert(8 * (2 * STAGES + 15) + 16 <= 8 * (2 * STAGES + 4) + 256, "group flags inside the barrier area");
     static_assert(!PK || MODE == MODE_RBQ1 || MODE == MODE_LVQ4, "packed points: 1-bit or LVQ4 codes");
-    // PK, LVQ4: lut[b] = e4m3 codes of the two nibbles of byte b (low byte: low nibble)
-    uint16_t *lut = reinterpret_cast<uint16_t *>(smem + tc_lut_offset<MODE, NH, NS>());
-    if (PK && MODE == MODE_LVQ4)
-        for (int i = threadIdx.x; i < 256; i += blockDim.x)
-            lut[i] = (uint16_t)(e4m3_of_code(i & 15) | ((uint32_t)e4m3_of_code(i >> 4) << 8));
     // the epilogue's merge buffer starts 256 bytes after tmem_slot (see tc_smem_bytes)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -792,11 +797,25 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
         // tensor-core operand 2 xbar - 1; rows past n as -1; LVQ4 nibbles ->
         // their e4m3 integer codes, rows past n as 0) into round16(d)
         // e4m3 bytes a row, then make the writes visible to the TMA (async
-        // proxy) and mark the slot ready.  Warp w takes rows w, w + CONV_WARPS,
-        // ..., lanes over a row's 32-bit code words; code bits past d meet
-        // zero centroid columns (the B map's width is d).
+        // proxy) and mark the slot ready.  Code bits past d meet zero centroid
+        // columns (the B map's width is d).
+        // A warp takes 32 consecutive rows, which lie one after another in
+        // memory, as 16-byte pieces of the output in order: every store of the
+        // warp is 512 contiguous bytes, every load a full run of words, and
+        // the loads of the next CW_PASS words a lane (at the end of a tile,
+        // of the next tile) are in flight while these are expanded.  With one
+        // or a few jobs a tile this walk is the kernel's critical path: rows
+        // taken four at a time by whole warps, each batch waiting for its
+        // loads, 1M x 768 1-bit codes against 63 centroids took 511 us.
         const int cw = warp - (2 + 4 * NH);
-        const int npair = (p.pk_dp + 31) >> 5;  // 32-dimension groups in a scratch row
+        constexpr int RPW = BM / CONV_WARPS;               // rows a warp
+        static_assert(RPW == 32, "the piece indexing below");
+        constexpr int CW_PASS = MODE == MODE_RBQ1 ? 8 : 4;  // load rounds in flight
+        constexpr int LW = MODE == MODE_RBQ1 ? 1 : 2;       // words a lane loads a round
+        const int rounds = p.pk_words / LW;                 // load rounds (32 LW words each)
+        const uint32_t cpr = MODE == MODE_RBQ1 ? 2u * p.pk_words : p.pk_words / 2u;  // 16-byte pieces a row
+        const bool contig = 16 * (int)cpr == p.pk_dp;
+        const uint32_t magic = (uint32_t)((0x100000000ull + cpr - 1) / cpr);  // piece / cpr (pieces < 2^13)
         JobStream js[NS];
         int64_t ctile[NS];
         uint32_t ccnt[NS];
@@ -806,86 +825,96 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
             ccnt[s] = 0;
             stream_seek(js[s]);
         }
-        for (int turn = 0;;) {
-            const int sj = stream_pick(js, turn);
-            if (sj < 0) break;
-            int64_t gj;
-            int ct;
-            stream_take(js, sj, gj, ct);
-            turn = (sj + 1) % NS;
-            if ((sj == 0 ? ctile[0] : ctile[NS - 1]) == gj) continue;  // not a tile's first job
-            const uint32_t i = sj == 0 ? ccnt[0] : ccnt[NS - 1];
-            if (sj == 0) {
-                ctile[0] = gj;
-                ccnt[0] = i + 1;
-            } else {
-                ctile[NS - 1] = gj;
-                ccnt[NS - 1] = i + 1;
+        int turn = 0;
+        auto next_tile = [&](int64_t &g) {  // the stream whose next tile comes up, -1: none
+            for (;;) {
+                const int sj = stream_pick(js, turn);
+                if (sj < 0) return -1;
+                int ct;
+                stream_take(js, sj, g, ct);
+                turn = (sj + 1) % NS;
+                if ((sj == 0 ? ctile[0] : ctile[NS - 1]) == g) continue;  // not a tile's first job
+                if (sj == 0)
+                    ctile[0] = g;
+                else
+                    ctile[NS - 1] = g;
+                return sj;
             }
+        };
+        uint32_t buf[CW_PASS][LW];
+        auto load_pass = [&](int64_t g, int u0, uint32_t(&w)[CW_PASS][LW]) {
+            const int64_t row = g * BM + RPW * cw;
+            const int64_t left = p.n - row;  // rows of this warp inside the points
+            const int words = left <= 0 ? 0 : (int)(left < RPW ? left : RPW) * p.pk_words;
+            const uint32_t *src = p.pk_codes + row * p.pk_words;
+#pragma unroll
+            for (int u = 0; u < CW_PASS; ++u) {
+                const int i = (32 * (u0 + u) + lane) * LW;
+                const bool in = u0 + u < rounds && i < words;
+                if constexpr (LW == 1) {
+                    w[u][0] = in ? __ldg(src + i) : 0u;
+                } else {
+                    const uint2 v = in ? __ldg(reinterpret_cast<const uint2 *>(src + i)) : make_uint2(0u, 0u);
+                    w[u][0] = v.x;
+                    w[u][1] = v.y;
+                }
+            }
+        };
+        int64_t gj = 0;
+        int sj = next_tile(gj);
+        if (sj >= 0) load_pass(gj, 0, buf);
+        while (sj >= 0) {
+            const uint32_t i = sj == 0 ? ccnt[0]++ : ccnt[NS - 1]++;
             const uint32_t slot = i & 1u;
             if (!mbar_wait(sfree_bar(sj, slot), ((i >> 1) & 1u) ^ 1u, abort_flag)) goto conv_done;
             // the TMA's reads of the slot's previous tile before these writes
             asm volatile("fence.proxy.async.global;" ::: "memory");
-            uint8_t *dst = p.pk_scratch + (((size_t)blockIdx.x * NS + sj) * 2 + slot) * BM * p.pk_dp;
-            const int64_t r0 = gj * BM;
-            constexpr int RB = 4;
-            if constexpr (MODE == MODE_RBQ1) {
-                // lane q takes code word q of the warp's rows (npair <= 32 for
-                // d <= 1024); RB rows' loads in flight before they are expanded
-                const bool act = lane < npair;
-                for (int rb = 0; rb < BM / CONV_WARPS; rb += RB) {
-                    uint32_t w[RB];
-#pragma unroll
-                    for (int u = 0; u < RB; ++u) {
-                        const int64_t row = r0 + cw + CONV_WARPS * (rb + u);
-                        w[u] = act && row < p.n ? __ldg(p.pk_codes + row * p.pk_words + lane) : 0u;
-                    }
-#pragma unroll
-                    for (int u = 0; u < RB; ++u) {
-                        if (!act) continue;
-                        uint8_t *drow = dst + (size_t)(cw + CONV_WARPS * (rb + u)) * p.pk_dp + 32 * lane;
-                        *reinterpret_cast<uint4 *>(drow) =
-                            make_uint4(pm1_e4m3(w[u]), pm1_e4m3(w[u] >> 4), pm1_e4m3(w[u] >> 8), pm1_e4m3(w[u] >> 12));
-                        if (32 * lane + 16 < p.pk_dp)
-                            *reinterpret_cast<uint4 *>(drow + 16) = make_uint4(
-                                pm1_e4m3(w[u] >> 16), pm1_e4m3(w[u] >> 20), pm1_e4m3(w[u] >> 24), pm1_e4m3(w[u] >> 28));
-                    }
+            uint8_t *dst = p.pk_scratch + ((((size_t)blockIdx.x * NS + sj) * 2 + slot) * BM + RPW * cw) * p.pk_dp;
+            int64_t gn = 0;
+            const int sn = next_tile(gn);
+            auto put = [&](uint32_t piece, uint4 v) {
+                if (contig) {
+                    *reinterpret_cast<uint4 *>(dst + 16 * piece) = v;
+                } else {
+                    const uint32_t r = __umulhi(piece, magic), q = piece - r * cpr;
+                    if (16 * (int)q < p.pk_dp) *reinterpret_cast<uint4 *>(dst + (size_t)r * p.pk_dp + 16 * q) = v;
                 }
-            } else {
-                // LVQ4: lane q takes nibble words q + 32 t (8 dimensions each; at
-                // most 128 words for d <= 1024) of the warp's rows, RB rows' loads
-                // in flight, each byte looked up as two e4m3 codes
-                const int nq = p.pk_dp >> 3;  // 8-dimension words in a scratch row (<= pk_words)
-                for (int rb = 0; rb < BM / CONV_WARPS; rb += RB) {
-                    uint32_t w[RB][4];
+            };
+            for (int u0 = 0; u0 < rounds; u0 += CW_PASS) {
+                uint32_t cur[CW_PASS][LW];
 #pragma unroll
-                    for (int u = 0; u < RB; ++u) {
-                        const int64_t row = r0 + cw + CONV_WARPS * (rb + u);
+                for (int u = 0; u < CW_PASS; ++u)
 #pragma unroll
-                        for (int t = 0; t < 4; ++t) {
-                            const int q = lane + 32 * t;
-                            w[u][t] = q < nq && row < p.n ? __ldg(p.pk_codes + row * p.pk_words + q) : 0u;
+                    for (int t = 0; t < LW; ++t) cur[u][t] = buf[u][t];
+                if (u0 + CW_PASS < rounds)
+                    load_pass(gj, u0 + CW_PASS, buf);
+                else if (sn >= 0)
+                    load_pass(gn, 0, buf);
+#pragma unroll
+                for (int u = 0; u < CW_PASS; ++u) {
+                    if (u0 + u >= rounds) break;  // warp-uniform
+                    if constexpr (MODE == MODE_RBQ1) {
+                        // 32 words are 64 pieces: lane l writes those of half a word
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            uint32_t v = __shfl_sync(0xffffffffu, cur[u][0], 16 * h + (lane >> 1));
+                            v >>= 16 * (lane & 1);
+                            put(64u * (u0 + u) + 32u * h + lane,
+                                make_uint4(pm1_e4m3(v), pm1_e4m3(v >> 4), pm1_e4m3(v >> 8), pm1_e4m3(v >> 12)));
                         }
-                    }
-#pragma unroll
-                    for (int u = 0; u < RB; ++u) {
-                        uint8_t *drow = dst + (size_t)(cw + CONV_WARPS * (rb + u)) * p.pk_dp;
-#pragma unroll
-                        for (int t = 0; t < 4; ++t) {
-                            const int q = lane + 32 * t;
-                            if (q < nq) {
-                                const uint32_t v = w[u][t];
-                                *reinterpret_cast<uint2 *>(drow + 8 * q) =
-                                    make_uint2((uint32_t)lut[v & 255u] | ((uint32_t)lut[(v >> 8) & 255u] << 16),
-                                               (uint32_t)lut[(v >> 16) & 255u] | ((uint32_t)lut[v >> 24] << 16));
-                            }
-                        }
+                    } else {
+                        uint32_t o[4];
+                        nibbles_e4m3(cur[u][0], o[0], o[1]);
+                        nibbles_e4m3(cur[u][LW - 1], o[2], o[3]);
+                        put(32u * (u0 + u) + lane, make_uint4(o[0], o[1], o[2], o[3]));
                     }
                 }
             }
             asm volatile("fence.proxy.async.global;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(sready_bar(sj, slot));
+            sj = sn;
+            gj = gn;
         }
     conv_done:;
     } else {  // ------------------------------------------------------- epilogue
@@ -1859,7 +1888,9 @@ __global__ void pf_gather_kernel(const uint16_t *__restrict__ cs0, const float4 
 }
 
 __global__ void cprep_sq8_kernel(const uint8_t *__restrict__ C, int k, int kp, int d, int dp,
-                                 __nv_bfloat16 *__restrict__ cs, int32_t *__restrict__ nc) {
+                                 __nv_bfloat16 *__restrict__ cs, int32_t *__restrict__ nc,
+                                 int32_t *__restrict__ counters) {
+    if (blockIdx.x == 0 && threadIdx.x < 4) counters[threadIdx.x] = 0;
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
@@ -1910,34 +1941,6 @@ __global__ void screen_prep_rbq1_kernel(const uint32_t *__restrict__ codes, int6
             for (int u = 0; u < nb; ++u) dst[u] = ((bits >> u) & 1u) ? 0x38 : 0xB8;
         }
     }
-}
-
-// Per-centroid estimator terms -> column-pair records for the tensor
-// epilogue: bs[p] = (bd x2, sd x2), qn[p] = (-sum ybar x2, ||c - m||^2 x2);
-// columns past k get ||c - m||^2 = +inf (never the nearest).
-__global__ void pack_rbq1_pairs_kernel(const Rbq1CInfo *__restrict__ info, int k, int kp,
-                                       float4 *__restrict__ bs, float4 *__restrict__ qn) {
-    const int pp = blockIdx.x * blockDim.x + threadIdx.x;
-    if (2 * pp >= kp) return;
-    float b[2], sc[2], q[2], n2[2];
-#pragma unroll
-    for (int o = 0; o < 2; ++o) {
-        const int j = 2 * pp + o;
-        if (j < k) {
-            const Rbq1CInfo in = info[j];
-            b[o] = in.bd;
-            sc[o] = in.sd;
-            q[o] = -(float)in.sumy;
-            n2[o] = in.ny2;
-        } else {
-            b[o] = 0.0f;
-            sc[o] = 0.0f;
-            q[o] = 0.0f;
-            n2[o] = INFINITY;
-        }
-    }
-    bs[pp] = make_float4(b[0], b[1], sc[0], sc[1]);
-    qn[pp] = make_float4(q[0], q[1], n2[0], n2[1]);
 }
 
 // ------------------------------------------------------------ fp32 rescoring
@@ -2211,12 +2214,12 @@ inline int round16(int d) { return (d + 15) & ~15; }
 // bytes, 16-byte aligned); it does so unless the caller supplies the e4m3
 // screening copy
 inline bool rbq1_packed(int d, const void *x) {
-    return d <= TC_RBQ1_MAX_D && ((d + 31) / 32) % 4 == 0 && ((uintptr_t)x & 15) == 0;
+    return d <= TC_WIDE_MAX_D && ((d + 31) / 32) % 4 == 0 && ((uintptr_t)x & 15) == 0;
 }
 // the same for LVQ4 nibble words (then round16(d) <= 8 ceil(d/8): every word
 // a converter reads lies inside the row)
 inline bool lvq4_packed(int d, const void *x) {
-    return d <= TC_LVQ4_MAX_D && ((d + 7) / 8) % 4 == 0 && ((uintptr_t)x & 15) == 0;
+    return d <= TC_WIDE_MAX_D && ((d + 7) / 8) % 4 == 0 && ((uintptr_t)x & 15) == 0;
 }
 
 }  // namespace
@@ -2347,6 +2350,34 @@ bool tc_reads_packed(int repr, int d, const void *x) {
     return (repr == SKM_REPR_RBQ1 && rbq1_packed(d, x)) || (repr == SKM_REPR_LVQ4 && lvq4_packed(d, x));
 }
 
+// 1-bit / LVQ4: the expansion slots (pk: read packed, two per job stream), the
+// centroids' e4m3 codes and their column-pair records
+static void plan_codes(int64_t n, int d, int k, bool pk, Carver &cv, TcAssignBufs &b) {
+    static_assert(TC_NS[MODE_RBQ1] == TC_NS[MODE_LVQ4], "the same slots for both");
+    const size_t kp = (size_t)cdiv(k, BN) * BN;
+    if (pk)
+        b.pk_scratch = cv.take<uint8_t>((size_t)std::min<int64_t>(PK_MAX_CTAS, cdiv(n, BM)) * TC_NS[MODE_RBQ1] * 2 *
+                                        BM * round16(d));
+    b.cs = reinterpret_cast<uint16_t *>(cv.take<uint8_t>((size_t)k * round16(d)));
+    b.rpair_bs = cv.take<float4>(kp / 2);
+    b.rpair_qn = cv.take<float4>(kp / 2);
+}
+
+bool tc_wide_ok(int repr, int d) {
+    return d > TC_RBQ1_MAX_D && ((repr == SKM_REPR_RBQ1 && rbq1_packed(d, nullptr)) ||
+                                 (repr == SKM_REPR_LVQ4 && lvq4_packed(d, nullptr)));
+}
+
+void tc_plan_wide(int repr, int64_t n, int d, int k, Carver &cv, TcAssignBufs &b) {
+    if (!tc_wide_ok(repr, d)) return;
+    Carver t = cv;
+    TcAssignBufs tb = b;
+    plan_codes(n, d, k, true, t, tb);
+    if (cv.base && !t.fits()) return;
+    cv = t;
+    b = tb;
+}
+
 void tc_plan(int repr, int64_t n, int d, int k, const void *x, const void *screen, bool warm, Carver &cv,
              TcAssignBufs &b) {
     b.stats = cv.take<int64_t>(4);
@@ -2365,24 +2396,8 @@ void tc_plan(int repr, int64_t n, int d, int k, const void *x, const void *scree
         b.screen = cv.take<uint8_t>(sb);
     }
     const size_t kp = (size_t)cdiv(k, BN) * BN;  // per-centroid records padded to whole tiles
-    if (repr == SKM_REPR_LVQ4) {
-        if (pk)  // read packed: per-CTA expansion slots (two per job stream)
-            b.pk_scratch = cv.take<uint8_t>((size_t)std::min<int64_t>(PK_MAX_CTAS, cdiv(n, BM)) * TC_NS[MODE_LVQ4] *
-                                            2 * BM * round16(d));
-        b.cs = reinterpret_cast<uint16_t *>(cv.take<uint8_t>((size_t)k * round16(d)));
-        b.linfo = cv.take<float4>(k);
-        b.rpair_bs = cv.take<float4>(kp / 2);
-        b.rpair_qn = cv.take<float4>(kp / 2);
-        return;
-    }
-    if (repr == SKM_REPR_RBQ1) {
-        if (pk)  // read packed: per-CTA expansion slots (two per job stream)
-            b.pk_scratch = cv.take<uint8_t>((size_t)std::min<int64_t>(PK_MAX_CTAS, cdiv(n, BM)) * TC_NS[MODE_RBQ1] *
-                                            2 * BM * round16(d));
-        b.cs = reinterpret_cast<uint16_t *>(cv.take<uint8_t>((size_t)k * round16(d)));
-        b.rinfo = cv.take<Rbq1CInfo>(k);
-        b.rpair_bs = cv.take<float4>(kp / 2);
-        b.rpair_qn = cv.take<float4>(kp / 2);
+    if (repr == SKM_REPR_LVQ4 || repr == SKM_REPR_RBQ1) {
+        plan_codes(n, d, k, pk, cv, b);
         return;
     }
     b.cs = cv.take<uint16_t>((size_t)k * dp);
@@ -2678,9 +2693,9 @@ int tc_assign_sq8(const skm_data *x, const uint8_t *C, int k, int32_t *nx_plain,
     }
     ScreenView v = screen_view(x->repr, n, d, x->x, screen);
     const int kp = (int)(cdiv(k, BN) * BN);
-    cprep_sq8_kernel<<<grid_warps(kp), 256, 0, st>>>(C, k, kp, d, dp, (__nv_bfloat16 *)b.cs, b.nc);
+    cprep_sq8_kernel<<<grid_warps(kp), 256, 0, st>>>(C, k, kp, d, dp, (__nv_bfloat16 *)b.cs, b.nc,
+                                                     b.counters);
     SKM_CUDA_TRY(launched());
-    SKM_CUDA_TRY(cudaMemsetAsync(b.counters, 0, sizeof(int32_t) * 4, st));
     TcParams p{};
     p.counters = b.counters;
     p.stats = b.stats;
@@ -2697,7 +2712,7 @@ int tc_assign_rbq1(const skm_data *x, const float *C, int k, int32_t *assign, fl
                    TcAssignBufs &b, cudaStream_t st, const TcSeg *seg) {
     const int64_t n = x->n;
     const int d = x->d, dp = round16(d);
-    const void *screen = x->screen;
+    const void *screen = d <= TC_RBQ1_MAX_D ? x->screen : nullptr;  // wider rows have no copy
     // without a caller copy the codes are read packed where their layout allows
     if (!screen && !rbq1_packed(d, x->x)) {
         skm_data tmp = *x;
@@ -2706,16 +2721,12 @@ int tc_assign_rbq1(const skm_data *x, const float *C, int k, int32_t *assign, fl
     }
     ScreenView v = screen_view(x->repr, n, d, x->x, screen);
     const int kp = (int)(cdiv(k, BN) * BN);
+    CodePairs pairs{b.rpair_bs, b.rpair_qn, kp, b.counters};
     if (x->flags & SKM_FLAG_SYMMETRIC)
-        SKM_CUDA_TRY(launch_rbq1_cprep_sym(C, k, d, x->m, reinterpret_cast<uint8_t *>(b.cs), dp, nullptr, b.rinfo,
-                                           st));
+        SKM_CUDA_TRY(launch_rbq1_cprep_sym(C, k, d, x->m, reinterpret_cast<uint8_t *>(b.cs), dp, nullptr, nullptr,
+                                           pairs, st));
     else
-        SKM_CUDA_TRY(launch_rbq1_cprep_tc(C, k, d, x->m, reinterpret_cast<uint8_t *>(b.cs), dp, b.rinfo,
-                                          st));
-    pack_rbq1_pairs_kernel<<<(kp / 2 + 255) / 256, 256, 0, st>>>(b.rinfo, k, kp, b.rpair_bs,
-                                                                 b.rpair_qn);
-    SKM_CUDA_TRY(launched());
-    SKM_CUDA_TRY(cudaMemsetAsync(b.counters, 0, sizeof(int32_t) * 4, st));
+        SKM_CUDA_TRY(launch_rbq1_cprep_tc(C, k, d, x->m, reinterpret_cast<uint8_t *>(b.cs), dp, pairs, st));
     TcParams p{};
     p.counters = b.counters;
     p.stats = b.stats;
@@ -2742,7 +2753,7 @@ int tc_assign_lvq4(const skm_data *x, const float *C, int k, int32_t *assign, fl
                    TcAssignBufs &b, cudaStream_t st, const TcSeg *seg) {
     const int64_t n = x->n;
     const int d = x->d, dp = round16(d);
-    const void *screen = x->screen;
+    const void *screen = d <= TC_LVQ4_MAX_D ? x->screen : nullptr;  // wider rows have no copy
     // without a caller copy the codes are read packed where their layout allows
     if (!screen && !lvq4_packed(d, x->x)) {
         SKM_TRY(tc_screen_prep(x, b.screen, st));
@@ -2750,9 +2761,8 @@ int tc_assign_lvq4(const skm_data *x, const float *C, int k, int32_t *assign, fl
     }
     ScreenView v = screen_view(x->repr, n, d, x->x, screen);
     const int kp = (int)(cdiv(k, BN) * BN);
-    SKM_CUDA_TRY(launch_lvq4_cprep(C, k, d, reinterpret_cast<uint8_t *>(b.cs), dp, nullptr, b.linfo, st));
-    SKM_CUDA_TRY(launch_lvq4_pack_pairs(b.linfo, k, kp, b.rpair_bs, b.rpair_qn, st));
-    SKM_CUDA_TRY(cudaMemsetAsync(b.counters, 0, sizeof(int32_t) * 4, st));
+    SKM_CUDA_TRY(launch_lvq4_cprep(C, k, d, reinterpret_cast<uint8_t *>(b.cs), dp, nullptr, nullptr,
+                                   CodePairs{b.rpair_bs, b.rpair_qn, kp, b.counters}, st));
     TcParams p{};
     p.counters = b.counters;
     p.stats = b.stats;

@@ -148,9 +148,11 @@ __global__ void __launch_bounds__(1024) scan_offsets_kernel(const int32_t *__res
 
 // Histogram, scan and placement of up to SORT1_MAX points in one block: a
 // thread keeps its points' clusters and their ranks inside them (the values
-// the shared-memory counters returned) in registers between the passes.  Three
-// launches and three memsets became one launch: 20,000 points 16 -> 7 us on
-// the GPU, and the host's launches bound an update of this size.
+// the shared-memory counters returned) in registers between the passes, and
+// the order is put together in shared memory (16 bits a point) and written
+// out in order: one SM takes 15 us for 20,000 points' scattered stores.
+// Three launches and three memsets became one launch, the host's launches
+// being what bounds an update of this size.
 constexpr int SORT1_PER = 32;
 constexpr int SORT1_MAX = 1024 * SORT1_PER;
 constexpr int SORT1_MAX_K = 12288;  // 48 KiB of counters; a cluster fits 14 bits, a rank 15
@@ -167,6 +169,7 @@ __global__ void __launch_bounds__(1024) sort_one_block_kernel(const int32_t *__r
         return;
     }
     extern __shared__ int32_t cnt_sh[];
+    uint16_t *perm_sh = reinterpret_cast<uint16_t *>(cnt_sh + k), *scl_sh = perm_sh + n;
     for (int j = threadIdx.x; j < k; j += 1024) cnt_sh[j] = 0;
     uint32_t place[SORT1_PER];
 #pragma unroll
@@ -191,8 +194,14 @@ __global__ void __launch_bounds__(1024) sort_one_block_kernel(const int32_t *__r
         if (place[i] == 0xffffffffu) continue;
         const int a = (int)(place[i] & 0xffffu);
         const int pos = cnt_sh[a] + (int)(place[i] >> 16);
-        perm[pos] = (int32_t)threadIdx.x + 1024 * i;
-        scl[pos] = a;
+        perm_sh[pos] = (uint16_t)(threadIdx.x + 1024 * i);
+        scl_sh[pos] = (uint16_t)a;
+    }
+    __syncthreads();
+    const int nval = (int)offsets[k];  // scan_block wrote it before the barriers
+    for (int i = threadIdx.x; i < nval; i += 1024) {
+        perm[i] = perm_sh[i];
+        scl[i] = scl_sh[i];
     }
 }
 
@@ -251,7 +260,13 @@ cudaError_t launch_sort_by_cluster(const int32_t *assign, int64_t n, int k, int3
     // a block clears 32 KiB or more
     const unsigned clear = (unsigned)std::min<size_t>(152, (sum_bytes + 32767) / 32768);
     if (n <= SORT1_MAX && k <= SORT1_MAX_K) {
-        sort_one_block_kernel<<<1 + clear, 1024, sizeof(int32_t) * (size_t)k, st>>>(
+        const size_t smem = sizeof(int32_t) * (size_t)k + 4 * (size_t)n;  // at most 176 KiB
+        if (smem > 48 * 1024 - 512) {
+            const cudaError_t e = cudaFuncSetAttribute(sort_one_block_kernel,
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        sort_one_block_kernel<<<1 + clear, 1024, smem, st>>>(
             assign, (int)n, k, offsets, counts64, accumulate, perm, scl, zeros, flag, sums, sum_bytes);
         return launched();
     }
@@ -779,34 +794,42 @@ cudaError_t launch_stable_sort(const int32_t *key, int64_t n, int m, int32_t *hi
     return launched();
 }
 
-// dst row q = src row perm[q] (rowbytes per row); one warp per row
-__global__ void gather_rows_bytes_kernel(const uint8_t *__restrict__ src, int64_t rowbytes,
-                                         const int32_t *__restrict__ perm, int64_t n, uint8_t *__restrict__ dst,
-                                         int vec16) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t q = warp; q < n; q += nw) {
-        const uint8_t *s = src + (int64_t)perm[q] * rowbytes;
-        uint8_t *t = dst + q * rowbytes;
-        if (vec16) {
-            for (int64_t i = lane; i < rowbytes / 16; i += 32)
-                reinterpret_cast<uint4 *>(t)[i] = __ldg(reinterpret_cast<const uint4 *>(s) + i);
-        } else {
-            for (int64_t i = lane; i < rowbytes; i += 32) t[i] = s[i];
-        }
+// dst row q = src row perm[q], a row being `units` units of T; one thread per
+// unit, so that the writes and each row's reads are contiguous whatever the
+// row's size (a warp per row left most lanes idle: 1M rows of 96 bytes 140 us,
+// of one 4-byte factor as much)
+template <typename T, typename I>
+__global__ void gather_units_kernel(const T *__restrict__ src, int units, const int32_t *__restrict__ perm, I total,
+                                    T *__restrict__ dst) {
+    const I u = (I)units;
+    for (I t = blockIdx.x * (I)blockDim.x + threadIdx.x; t < total; t += (I)gridDim.x * blockDim.x) {
+        const I q = t / u;
+        dst[t] = src[(int64_t)perm[q] * units + (int64_t)(t - q * u)];
     }
+}
+
+template <typename T>
+static cudaError_t launch_gather_units(const void *src, int64_t rowbytes, const int32_t *perm, int64_t n, void *dst,
+                                       cudaStream_t st) {
+    const int units = (int)(rowbytes / (int64_t)sizeof(T));
+    const int64_t total = n * units;
+    const int64_t blocks = std::min<int64_t>(152 * 32, (total + 255) / 256);
+    const T *s = static_cast<const T *>(src);
+    T *d = static_cast<T *>(dst);
+    if (total < (int64_t(1) << 31))  // and a last stride past it stays below 2^32
+        gather_units_kernel<T, uint32_t><<<(unsigned)blocks, 256, 0, st>>>(s, units, perm, (uint32_t)total, d);
+    else
+        gather_units_kernel<T, int64_t><<<(unsigned)blocks, 256, 0, st>>>(s, units, perm, total, d);
+    return launched();
 }
 
 cudaError_t launch_gather_rows_bytes(const void *src, int64_t rowbytes, const int32_t *perm, int64_t n,
                                      void *dst, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    const int vec16 = rowbytes % 16 == 0 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0;
-    int64_t blocks = (n * 32 + 255) / 256;
-    if (blocks > 152 * 16) blocks = 152 * 16;
-    gather_rows_bytes_kernel<<<(int)blocks, 256, 0, st>>>(static_cast<const uint8_t *>(src), rowbytes, perm, n,
-                                                         static_cast<uint8_t *>(dst), vec16);
-    return launched();
+    const uintptr_t a = reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) | (uintptr_t)rowbytes;
+    if ((a & 15) == 0) return launch_gather_units<uint4>(src, rowbytes, perm, n, dst, st);
+    if ((a & 3) == 0) return launch_gather_units<uint32_t>(src, rowbytes, perm, n, dst, st);
+    return launch_gather_units<uint8_t>(src, rowbytes, perm, n, dst, st);
 }
 
 // out[perm[q]] = in[q] (4-byte values)

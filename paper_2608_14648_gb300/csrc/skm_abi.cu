@@ -156,9 +156,10 @@ static void prune_stats_from(const unsigned long long (&h)[PRUNE_CTRS], skm_stat
 struct AssignBufs {
     unsigned long long *prune = nullptr;    // PRUNE_CTRS counters
     int32_t *nx = nullptr, *nc = nullptr;  // SQ8 with d > 1024 (__dp4a path)
-    uint4 *planes = nullptr;                // RBQ1 with d > 1024 (AND + popcount path)
+    // d > 1024 on CUDA cores: codes whose rows the tensor-core kernel cannot read
+    uint4 *planes = nullptr;                // RBQ1 (AND + popcount path)
     Rbq1CInfo *info = nullptr;
-    uint32_t *yw = nullptr;                 // LVQ4 with d > 1024 (__dp4a path): centroid nibbles
+    uint32_t *yw = nullptr;                 // LVQ4 (__dp4a path): centroid nibbles
     float4 *linfo = nullptr;
     TcAssignBufs tc;                        // tensor-core paths (F32, BF16, SQ8, RBQ1)
     Rbq1SegInfo *seginfo = nullptr;         // RBQ1 with SKM_FLAG_PRUNE (planes above)
@@ -249,7 +250,7 @@ __global__ void count_moved_kernel(const int32_t *__restrict__ a, const int32_t 
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
 }
 
-constexpr int OBJ_LOG = 1024;  // objective values kept on the device between copies
+constexpr int OBJ_LOG = 32;  // objective values kept on the device between copies
 
 struct FitBufs {
     uint8_t *screen = nullptr;  // built once per fit when the caller gave none
@@ -263,6 +264,7 @@ struct FitBufs {
     unsigned int *maxbits = nullptr;
     int *e_dev = nullptr;
     int *status = nullptr;
+    unsigned int *ticket = nullptr;  // of the objective's sum; after the status word
     int64_t *counts = nullptr;
     int64_t *init_idx = nullptr;
     int64_t *empty_iter = nullptr;  // empty clusters after each update (first EMPTY_LOG iterations)
@@ -294,10 +296,12 @@ static void plan_fit(const skm_data *x, int k, Carver &cv, FitBufs &b) {
     b.sum = cv.take<double>(OBJ_LOG);
     b.maxbits = cv.take<unsigned int>(1);
     b.e_dev = cv.take<int>(1);
-    b.status = cv.take<int>(1);
+    b.status = cv.take<int>(2);
+    b.ticket = reinterpret_cast<unsigned int *>(b.status ? b.status + 1 : nullptr);
     b.counts = cv.take<int64_t>(k);
     b.init_idx = cv.take<int64_t>(k);  // seeded Forgy indices (host-drawn)
     b.empty_iter = cv.take<int64_t>(EMPTY_LOG);
+    if (!use_prune(x)) tc_plan_wide(x->repr, x->n, x->d, k, cv, b.a.tc);
 }
 
 static int need_ws(const Carver &cv, size_t ws_bytes, void *ws) {
@@ -349,11 +353,12 @@ static int do_assign(const skm_data *x, const void *C, int k, const int32_t *pre
                               b.tc, st));
         break;
     case SKM_REPR_RBQ1:
-        if (d <= TC_RBQ1_MAX_D) {
+        if (d <= TC_RBQ1_MAX_D || (b.tc.cs && tc_reads_packed(x->repr, d, x->x))) {
             SKM_TRY(tc_assign_rbq1(x, static_cast<const float *>(C), k, assign, dist, b.tc, st));
         } else if (x->flags & SKM_FLAG_SYMMETRIC) {
             uint32_t *yw = reinterpret_cast<uint32_t *>(b.planes);  // k sign words per centroid row fit
-            SKM_CUDA_TRY(launch_rbq1_cprep_sym(static_cast<const float *>(C), k, d, x->m, nullptr, 0, yw, b.info, st));
+            SKM_CUDA_TRY(launch_rbq1_cprep_sym(static_cast<const float *>(C), k, d, x->m, nullptr, 0, yw, b.info, CodePairs{},
+                                               st));
             SKM_CUDA_TRY(launch_assign_rbq1_sym(static_cast<const uint32_t *>(x->x), x->nx2, x->F, n, d, yw, b.info, k,
                                                 assign, dist, st));
         } else {
@@ -364,10 +369,11 @@ static int do_assign(const skm_data *x, const void *C, int k, const int32_t *pre
         }
         break;
     case SKM_REPR_LVQ4:
-        if (d <= TC_LVQ4_MAX_D) {
+        if (d <= TC_LVQ4_MAX_D || (b.tc.cs && tc_reads_packed(x->repr, d, x->x))) {
             SKM_TRY(tc_assign_lvq4(x, static_cast<const float *>(C), k, assign, dist, b.tc, st));
         } else {
-            SKM_CUDA_TRY(launch_lvq4_cprep(static_cast<const float *>(C), k, d, nullptr, 0, b.yw, b.linfo, st));
+            SKM_CUDA_TRY(launch_lvq4_cprep(static_cast<const float *>(C), k, d, nullptr, 0, b.yw, b.linfo, CodePairs{},
+                                           st));
             SKM_CUDA_TRY(launch_assign_lvq4_simt(static_cast<const uint32_t *>(x->x),
                                                  reinterpret_cast<const float4 *>(x->lvq), n, d, b.yw, b.linfo, k,
                                                  assign, dist, st));
@@ -496,6 +502,7 @@ size_t skm_workspace_size(int op, const skm_data *x, int k) {
         if (check_data(x, false) || check_k(x, k)) return 0;
         AssignBufs b;
         plan_assign(x, k, cv, b);
+        if (!use_prune(x)) tc_plan_wide(x->repr, x->n, x->d, k, cv, b.tc);
         break;
     }
     case 1: {
@@ -824,6 +831,7 @@ int skm_assign(const skm_data *x, const void *C, int k, const int32_t *prev_assi
     Carver cv(ws, ws_bytes);
     AssignBufs b;
     plan_assign(x, k, cv, b);
+    if (!use_prune(x)) tc_plan_wide(x->repr, x->n, x->d, k, cv, b.tc);
     SKM_TRY(need_ws(cv, ws_bytes, ws));
     if (use_prune(x))
         SKM_CUDA_TRY(cudaMemsetAsync(b.prune, 0, PRUNE_CTRS * sizeof(unsigned long long), S(stream)));
@@ -1243,7 +1251,7 @@ int skm_fit(const skm_fit_config *cfg, const skm_data *x, const void *C_init,
                                      st));
         init_idx = b.init_idx;
     }
-    SKM_CUDA_TRY(cudaMemsetAsync(b.status, 0, sizeof(int), st));
+    SKM_CUDA_TRY(cudaMemsetAsync(b.status, 0, 2 * sizeof(int), st));  // and the ticket
     SKM_CUDA_TRY(cudaMemsetAsync(b.u.flag, 0, sizeof(int32_t), st));
     if (C_init) {
         SKM_CUDA_TRY(cudaMemcpyAsync(C_out, C_init, centroid_bytes(x, k), cudaMemcpyDeviceToDevice,
@@ -1305,7 +1313,7 @@ int skm_fit(const skm_fit_config *cfg, const skm_data *x, const void *C_init,
             // kept on the device and read back OBJ_LOG at a time: a copy to the
             // caller's pageable array would wait for every iteration
             const int slot = it % OBJ_LOG;
-            SKM_CUDA_TRY(launch_sum_float(dist, n, b.partials, nblk, b.sum + slot, st));
+            SKM_CUDA_TRY(launch_sum_float(dist, n, b.partials, nblk, b.ticket, b.sum + slot, st));
             if (slot == OBJ_LOG - 1 || it == cfg->iters)
                 SKM_CUDA_TRY(cudaMemcpyAsync(objective_host + (it - slot), b.sum, sizeof(double) * (size_t)(slot + 1),
                                              cudaMemcpyDeviceToHost, st));

@@ -92,7 +92,7 @@ void plan_host(const skm_step_host_config *cfg, const skm_data *x, Carver &cv, H
     if (!cfg->counts) b.counts = cv.take<int64_t>((size_t)k);
     b.red = cv.take<double>(RED);
     b.chunk_sum = cv.take<double>(MAX_CHUNKS);
-    b.total = cv.take<double>(1);
+    b.total = cv.take<double>(2);  // and the sums' ticket
     // the entry points' own workspaces for a range of rc rows (reused by
     // every range: the compute stream runs them one after another)
     skm_data probe = view_of(x, reinterpret_cast<const void *>(256), rc);
@@ -179,6 +179,8 @@ extern "C" int skm_lloyd_step_host(const skm_step_host_config *cfg, const skm_da
         SKM_CUDA_TRY(cudaMemcpyAsync(b.C, C_host, cbytes, cudaMemcpyHostToDevice, st));
         SKM_CUDA_TRY(cudaMemsetAsync(partial, 0, (size_t)k * d * 8, st));
         SKM_CUDA_TRY(cudaMemsetAsync(counts, 0, sizeof(int64_t) * (size_t)k, st));
+        unsigned int *ticket = reinterpret_cast<unsigned int *>(b.total + 1);
+        if (objective_host) SKM_CUDA_TRY(cudaMemsetAsync(ticket, 0, sizeof(*ticket), st));
         if (cp != st) {  // the copy stream starts after the caller's earlier work on `stream`
             SKM_CUDA_TRY(cudaEventRecord(freed[0], st));
             SKM_CUDA_TRY(cudaStreamWaitEvent(cp, freed[0], 0));
@@ -217,7 +219,7 @@ extern "C" int skm_lloyd_step_host(const skm_step_host_config *cfg, const skm_da
             SKM_TRY(skm_update(&v, b.assign[s], k, nullptr, counts, partial, b.ws_u, b.ws_u_bytes, st));
             if (objective_host) {
                 const int nblk = (int)std::min<int64_t>(RED, rows);
-                SKM_CUDA_TRY(launch_sum_float(b.dist[s], rows, b.red, nblk, b.chunk_sum + i, st));
+                SKM_CUDA_TRY(launch_sum_float(b.dist[s], rows, b.red, nblk, ticket, b.chunk_sum + i, st));
             }
             SKM_CUDA_TRY(cudaMemcpyAsync(assign_host + r0, b.assign[s], sizeof(int32_t) * (size_t)rows,
                                          cudaMemcpyDeviceToHost, st));

@@ -178,11 +178,23 @@ cudaError_t launch_rbq1_cprep(const float *C, int k, int d, const float *m, uint
                               Rbq1CInfo *info, cudaStream_t st);
 // fl(1 / sqrt(d)) as both sides of the estimator use it
 inline float rbq1_isd(int d) { return (float)(1.0 / sqrt((double)d)); }
+// What the tensor-core epilogue reads of the centroids of a code
+// representation, one record per column pair, written by the centroid
+// preparation itself: 1-bit bs = (bd x2, sd x2), qn = (-sum ybar x2,
+// ||c - m||^2 x2); LVQ4 bs = (b x2, G x2), qn = (s x2, N x2).  Columns [k, kp)
+// get +inf in the last place, so they are never the nearest.  Also clears the
+// call's four counters.
+struct CodePairs {
+    float4 *bs = nullptr;
+    float4 *qn = nullptr;
+    int kp = 0;
+    int32_t *counters = nullptr;
+};
 cudaError_t launch_rbq1_cprep_tc(const float *C, int k, int d, const float *m, uint8_t *yq, int dq,
-                                 Rbq1CInfo *info, cudaStream_t st);
+                                 const CodePairs &pairs, cudaStream_t st);
 // symmetric 1-bit variant: binarized centroids (e4m3 +-1 codes and/or sign words)
 cudaError_t launch_rbq1_cprep_sym(const float *C, int k, int d, const float *m, uint8_t *yq, int dq, uint32_t *yw,
-                                  Rbq1CInfo *info, cudaStream_t st);
+                                  Rbq1CInfo *info, const CodePairs &pairs, cudaStream_t st);
 cudaError_t launch_assign_rbq1_sym(const uint32_t *codes, const float *nx2, const float *F, int64_t n, int d,
                                    const uint32_t *yw, const Rbq1CInfo *info, int k, int32_t *assign, float *dist,
                                    cudaStream_t st);
@@ -336,9 +348,11 @@ cudaError_t launch_objective(const void *X, int x_is_bf16, int64_t n, int d, con
                              const int32_t *assign, double *partials, int nblk,
                              cudaStream_t st);
 cudaError_t launch_sum_double(const double *in, int64_t count, double *out, cudaStream_t st);
-// *out = sum of in[0 .. count) in fp64 (partials: nblk doubles of workspace)
-cudaError_t launch_sum_float(const float *in, int64_t count, double *partials, int nblk, double *out,
-                             cudaStream_t st);
+// *out = sum of in[0 .. count) in fp64 (partials: nblk doubles of workspace;
+// ticket: a word that is zero before the first call and not shared by calls
+// that overlap)
+cudaError_t launch_sum_float(const float *in, int64_t count, double *partials, int nblk, unsigned int *ticket,
+                             double *out, cudaStream_t st);
 cudaError_t launch_project(const float *X, int64_t n, int d, const float *mean, const float *P,
                            int d_out, int out_bf16, void *Y, cudaStream_t st);
 cudaError_t launch_cov_partial(const float *X, int64_t n, int d, const float *mean,
@@ -356,15 +370,12 @@ cudaError_t launch_lvq4_encode(const float *X, int64_t n, int d, uint32_t *codes
 cudaError_t launch_lvq4_exponent(const float4 *fac, int64_t n, unsigned int *maxbits, int *e_dev,
                                  cudaStream_t st);
 // centroid re-encoding: yq != nullptr -> e4m3 bytes (row stride dq); yw != nullptr
-// -> nibble words; info (s, b, N, G) per centroid
+// -> nibble words; info (s, b, N, G) per centroid and / or the epilogue's pairs
 cudaError_t launch_lvq4_cprep(const float *C, int k, int d, uint8_t *yq, int dq, uint32_t *yw,
-                              float4 *info, cudaStream_t st);
+                              float4 *info, const CodePairs &pairs, cudaStream_t st);
 // nibble codes -> e4m3 bytes, row stride dq
 cudaError_t launch_lvq4_expand(const uint32_t *codes, int64_t n, int d, uint8_t *xs, int dq,
                                cudaStream_t st);
-// column-pair records for the tensor epilogue: bg = (b x2, G x2), sn = (s x2, N x2)
-cudaError_t launch_lvq4_pack_pairs(const float4 *info, int k, int kp, float4 *bg, float4 *sn,
-                                   cudaStream_t st);
 cudaError_t launch_assign_lvq4_simt(const uint32_t *codes, const float4 *fac, int64_t n, int d,
                                     const uint32_t *yw, const float4 *info, int k, int32_t *assign,
                                     float *dist, cudaStream_t st);

@@ -15,6 +15,13 @@ constexpr int TC_RBQ1_MAX_D = 1024;
 // LVQ4 on the same e4m3 path: P <= 225 d stays below 2^18 up to this d; beyond
 // it the __dp4a kernel is used.
 constexpr int TC_LVQ4_MAX_D = 1024;
+// Both read packed up to this d (no copy of the points is ever made beyond the
+// limits above): P <= 225 d < 2^20 and |2P - sum ybar| <= 15 d < 2^16, still
+// exact integers in the fp32 accumulator.  Longer embeddings are common (1536
+// for text encoders), and the CUDA-core kernels pay 4 POPC a word or a dp4a a
+// byte pair for what one MMA does: 200,000 x 1536, k = 1789, 1-bit: 17.7 ms
+// with AND + popcount.
+constexpr int TC_WIDE_MAX_D = 4096;
 
 struct TcAssignBufs {
     int64_t *stats = nullptr;     // [0] rescored rows, [1] fallback rows, [2] timeout (cumulative)
@@ -32,8 +39,6 @@ struct TcAssignBufs {
     float4 *cinfo = nullptr;      // F32/BF16: per-column-pair bound terms
     float2 *cinfoz = nullptr;
     int32_t *nc = nullptr;        // SQ8: centred ||c||^2
-    Rbq1CInfo *rinfo = nullptr;   // RBQ1: per-centroid estimator terms
-    float4 *linfo = nullptr;      // LVQ4: per-centroid (s, b, N, G)
     float4 *rpair_bs = nullptr;   // RBQ1 / LVQ4: column-pair records (padded)
     float4 *rpair_qn = nullptr;
     int32_t *cand = nullptr;      // F32/BF16: [n][5] screen candidates + count
@@ -81,6 +86,12 @@ int tc_screen_prep(const skm_data *x, void *screen, cudaStream_t st);
 bool tc_reads_packed(int repr, int d, const void *x);
 void tc_plan(int repr, int64_t n, int d, int k, const void *x, const void *screen, bool warm, Carver &cv,
              TcAssignBufs &b);
+// 1-bit / LVQ4 codes with d > 1024 (tc_wide_ok: whole 16-byte rows; the address
+// must be 16-byte aligned too): the tensor-core path's buffers, after
+// everything else in a workspace.  They are left out (b.cs stays NULL, and the
+// CUDA-core kernel runs) when a given workspace ends before them.
+bool tc_wide_ok(int repr, int d);
+void tc_plan_wide(int repr, int64_t n, int d, int k, Carver &cv, TcAssignBufs &b);
 int tc_init_stats(TcAssignBufs &b, cudaStream_t st);
 // Exact dimension pruning of bf16 points with the first dimensions on tensor
 // cores (used when a seed assignment is given): whether these points can take
