@@ -4,6 +4,8 @@
 // a code is an explicit IEEE fp32 operation (no contraction).
 #include <string.h>
 
+#include <algorithm>
+
 #include "skm_internal.cuh"
 
 namespace skm {
@@ -474,6 +476,11 @@ __global__ void colmean_finish_kernel(const double *__restrict__ psum, int nblk,
 // with one fp64 division.  Row shards that use the same s and n add up to
 // exactly the single-process sums.
 // ---------------------------------------------------------------------------
+__host__ __device__ inline int ceil_log2(int64_t n) {
+    int lg = 0;
+    while ((int64_t(1) << lg) < n) ++lg;
+    return lg;
+}
 __host__ __device__ inline int mean_scale_of(unsigned amax_bits, int64_t n) {
     if (amax_bits == 0) return 0;
     const unsigned ef = (amax_bits >> 23) & 0xffu;
@@ -486,9 +493,7 @@ __host__ __device__ inline int mean_scale_of(unsigned amax_bits, int64_t n) {
     } else {
         E = (int)ef - 127 + 1;
     }
-    int lg = 0;
-    while ((int64_t(1) << lg) < n) ++lg;
-    return 61 - lg - E;
+    return 61 - ceil_log2(n) - E;
 }
 
 __global__ void absmax_bits_kernel(const float *__restrict__ X, int64_t count, unsigned *__restrict__ bits) {
@@ -511,64 +516,186 @@ __global__ void absmax_bits_kernel(const float *__restrict__ X, int64_t count, u
     if ((threadIdx.x & 31) == 0 && mx) atomicMax(bits, mx);
 }
 
-__global__ void mean_scale_kernel(const unsigned *__restrict__ bits, int64_t n, int *__restrict__ s_out) {
-    *s_out = mean_scale_of(*bits, n);
+// Where the column sums at the scale of max |x| come from (see mean_pass_kernel):
+// its sums A or B, or the fixed-scale pass.
+enum { MEAN_A = 0, MEAN_B = 1, MEAN_REDO = 2 };
+// What the one-pass mean keeps on the device
+struct MeanState {
+    unsigned amax;    // bits of max |x|
+    unsigned sample;  // ... over the sampled rows
+};
+__device__ __forceinline__ int mean_select(const MeanState &st, int64_t n) {
+    if (st.sample == 0 || st.amax >= 0x7f800000u) return MEAN_REDO;
+    const int sa = mean_scale_of(st.sample, n), s = mean_scale_of(st.amax, n);
+    if (sa < -100 || sa > 120) return MEAN_REDO;  // powers of two outside the fp32 range below
+    return s == sa ? MEAN_A : s == sa - 1 ? MEAN_B : MEAN_REDO;
+}
+
+// max |x| over MEAN_SAMPLE rows spread over the points: its exponent E0 is
+// that of all points or one below it unless the rows differ wildly.
+constexpr int MEAN_SAMPLE = 2048;
+__global__ void mean_sample_kernel(const float *__restrict__ X, int64_t n, int d, MeanState *__restrict__ st) {
+    unsigned mx = 0;
+    const int64_t rows = n < MEAN_SAMPLE ? n : MEAN_SAMPLE;
+    for (int64_t i = blockIdx.x; i < rows; i += gridDim.x) {
+        const float *x = X + i * n / rows * d;
+        for (int c = threadIdx.x; c < d; c += blockDim.x) mx = max(mx, __float_as_uint(__ldg(x + c)) & 0x7fffffffu);
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0 && mx) atomicMax(&st->sample, mx);
+}
+
+// One pass over the points for the fixed-point mean: max |x|, and the column
+// sums of rint(x 2^s) for the two scales that max |x| < 2^(E0 + 1) allows (sums
+// A: s = 61 - L - E0; B: one less).  The scale depends on max |x|, so it took a
+// pass of its own before (489 us at 1M x 768, and the sums, with fixed_rint's 20
+// or so integer instructions a value, 782 us; this is one read of the
+// points at the copy bandwidth: 452 us).
+// A value in fp32 operations only: with s1 = 21 - E0, h = rint(x 2^s1) (|h| <=
+// 2^22, by adding and subtracting 1.5 2^23), r = x - h 2^-s1 (exact: a multiple of
+// x's last place below 2^(-s1-1)), and rint(x 2^s) = h 2^(s-s1) + rint(r 2^s):
+// exact, since r 2^s is (|r 2^s| <= 2^22 for L >= 17) and h 2^(s-s1) is even, so
+// ties fall to the same side.  The integers are the low bits of the sums with
+// 1.5 2^23; they are added up in 32 bits, modulo 2^32, for MEAN_ROWS rows (|sum|
+// <= 2^30), then in 64.
+constexpr int MEAN_ROWS = 256;
+constexpr int MEAN_MIN_LOG2 = 17;  // L >= 17: n > 65536
+constexpr int MEAN_THREADS = 512;
+
+__global__ void __launch_bounds__(MEAN_THREADS, 2) mean_pass_kernel(const float4 *__restrict__ X4, int64_t n, int d4,
+                                                                    int lg, MeanState *__restrict__ st,
+                                                                    unsigned long long *__restrict__ SA,
+                                                                    unsigned long long *__restrict__ SB) {
+    extern __shared__ unsigned long long mean_sh[];  // [2][4 d4]
+    const int d = 4 * d4;
+    for (int c = threadIdx.x; c < 2 * d; c += blockDim.x) mean_sh[c] = 0ull;
+    __syncthreads();
+    const int sa = mean_scale_of(st->sample, n);
+    const int s1 = 21 - (61 - lg - sa);  // E0 = 61 - L - sa
+    const bool ok = st->sample != 0 && sa >= -100 && sa <= 120;
+    auto pow2 = [&](int e) { return ok ? __int_as_float((e + 127) << 23) : 0.0f; };  // |e| <= 123 here
+    const float p1 = pow2(s1), m1 = -pow2(-s1), pa = pow2(sa), pb = 0.5f * pa;
+    constexpr float MAGIC = 12582912.0f;  // 1.5 2^23
+    const uint32_t mb = __float_as_uint(MAGIC);
+    // d4 < blockDim: the block's threads are phases x d4, the phases taking
+    // every phases-th row; wider rows: column groups blockDim apart
+    const int phases = d4 < (int)blockDim.x ? blockDim.x / d4 : 1;
+    const int phase = d4 < (int)blockDim.x ? threadIdx.x / d4 : 0;
+    const int64_t per = (n + gridDim.x - 1) / gridDim.x;
+    const int64_t r0 = (int64_t)blockIdx.x * per, r1 = min(n, r0 + per);
+    unsigned mx = 0;
+    if (phase < phases) {
+        for (int g = d4 < (int)blockDim.x ? threadIdx.x - phase * d4 : threadIdx.x; g < d4; g += blockDim.x) {
+            const float4 *col = X4 + g;
+            for (int64_t rc = r0 + phase; rc < r1; rc += (int64_t)MEAN_ROWS * phases) {
+                const int64_t left = (r1 - rc + phases - 1) / phases;
+                const int cnt = left < MEAN_ROWS ? (int)left : MEAN_ROWS;
+                uint32_t h[4] = {}, a[4] = {}, b[4] = {};
+                auto add = [&](const float4 &v) {
+                    const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        mx = max(mx, __float_as_uint(x[u]) & 0x7fffffffu);
+                        const float t = __fmaf_rn(x[u], p1, MAGIC);
+                        const float r = __fmaf_rn(__fsub_rn(t, MAGIC), m1, x[u]);
+                        h[u] += __float_as_uint(t);
+                        a[u] += __float_as_uint(__fmaf_rn(r, pa, MAGIC));
+                        b[u] += __float_as_uint(__fmaf_rn(r, pb, MAGIC));
+                    }
+                };
+                const float4 *src = col + rc * d4;
+                const int64_t step = (int64_t)phases * d4;
+                int i = 0;
+                for (; i + 4 <= cnt; i += 4, src += 4 * step) {
+                    float4 v[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) v[u] = __ldg(src + u * step);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) add(v[u]);
+                }
+                for (; i < cnt; ++i, src += step) add(__ldg(src));
+                const uint32_t base = (uint32_t)cnt * mb;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int64_t hs = (int32_t)(h[u] - base);
+                    const int64_t va = hs * (int64_t(1) << (40 - lg)) + (int32_t)(a[u] - base);
+                    const int64_t vb = hs * (int64_t(1) << (39 - lg)) + (int32_t)(b[u] - base);
+                    atomicAdd(mean_sh + 4 * g + u, (unsigned long long)va);
+                    atomicAdd(mean_sh + d + 4 * g + u, (unsigned long long)vb);
+                }
+            }
+        }
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0 && mx) atomicMax(&st->amax, mx);
+    __syncthreads();
+    for (int c = threadIdx.x; c < d; c += blockDim.x) {
+        atomicAdd(SA + c, mean_sh[c]);
+        atomicAdd(SB + c, mean_sh[d + c]);
+    }
 }
 
 // S[c] += sum over this launch's rows of rint(x_rc 2^s); blocks take row
-// ranges, threads columns (four at a time when rows are 16-byte aligned).
-__global__ void colsum_fixed_kernel(const float *__restrict__ X, int64_t n, int d, const int *__restrict__ s_dev,
-                                    int s_host, unsigned long long *__restrict__ S) {
-    const int s = s_dev ? *s_dev : s_host;
+// ranges, threads columns (four at a time when rows are 16-byte aligned), and
+// every phases-th row when the columns leave threads over.  s: s_host, or, with
+// st, that of max |x|, and nothing to do unless the one-pass sums miss it.
+__global__ void colsum_fixed_kernel(const float *__restrict__ X, int64_t n, int d, const MeanState *__restrict__ st,
+                                    int only_redo, int s_host, unsigned long long *__restrict__ S) {
+    if (only_redo && mean_select(*st, n) != MEAN_REDO) return;
+    const int s = st ? mean_scale_of(st->amax, n) : s_host;
     const int64_t per = (n + gridDim.x - 1) / gridDim.x;
     const int64_t r0 = (int64_t)blockIdx.x * per, r1 = min(n, r0 + per);
     if (r0 >= r1) return;
-    if ((d & 3) == 0 && ((uintptr_t)X & 15) == 0) {
-        const int d4 = d >> 2;
+    const bool vec = (d & 3) == 0 && ((uintptr_t)X & 15) == 0;
+    const int cols = vec ? d >> 2 : d, nt = blockDim.x;
+    const int phases = cols < nt ? nt / cols : 1, phase = cols < nt ? threadIdx.x / cols : 0;
+    if (phase >= phases) return;
+    const int c0 = cols < nt ? threadIdx.x - phase * cols : threadIdx.x;
+    if (vec) {
         const float4 *X4 = reinterpret_cast<const float4 *>(X);
-        for (int g = threadIdx.x; g < d4; g += blockDim.x) {
+        for (int g = c0; g < cols; g += nt) {
             int64_t a0 = 0, a1 = 0, a2 = 0, a3 = 0;
-            int64_t r = r0;
-            for (; r + 4 <= r1; r += 4) {
-                float4 v[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) v[u] = __ldg(X4 + (r + u) * d4 + g);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    a0 += fixed_rint(v[u].x, s);
-                    a1 += fixed_rint(v[u].y, s);
-                    a2 += fixed_rint(v[u].z, s);
-                    a3 += fixed_rint(v[u].w, s);
-                }
-            }
-            for (; r < r1; ++r) {
-                const float4 v = __ldg(X4 + r * d4 + g);
+            auto add = [&](const float4 &v) {
                 a0 += fixed_rint(v.x, s);
                 a1 += fixed_rint(v.y, s);
                 a2 += fixed_rint(v.z, s);
                 a3 += fixed_rint(v.w, s);
+            };
+            int64_t r = r0 + phase;
+            for (; r + 3 * phases < r1; r += 4 * phases) {
+                float4 v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = __ldg(X4 + (r + u * phases) * cols + g);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) add(v[u]);
             }
+            for (; r < r1; r += phases) add(__ldg(X4 + r * cols + g));
             atomicAdd(S + 4 * g, (unsigned long long)a0);
             atomicAdd(S + 4 * g + 1, (unsigned long long)a1);
             atomicAdd(S + 4 * g + 2, (unsigned long long)a2);
             atomicAdd(S + 4 * g + 3, (unsigned long long)a3);
         }
     } else {
-        for (int c = threadIdx.x; c < d; c += blockDim.x) {
+        for (int c = c0; c < cols; c += nt) {
             int64_t a = 0;
-            for (int64_t r = r0; r < r1; ++r) a += fixed_rint(__ldg(X + r * d + c), s);
+            for (int64_t r = r0 + phase; r < r1; r += phases) a += fixed_rint(__ldg(X + r * d + c), s);
             atomicAdd(S + c, (unsigned long long)a);
         }
     }
 }
 
-__global__ void mean_fixed_finish_kernel(const unsigned long long *__restrict__ S, int d, int64_t n,
-                                         const int *__restrict__ s_dev, int s_host, float *__restrict__ m) {
+// m_c = fl32(S_c / (n 2^s)); with st, s and the sums (S, or the one-pass SA /
+// SB when there are any) are those of max |x|.
+__global__ void mean_fixed_finish_kernel(const unsigned long long *__restrict__ S,
+                                         const unsigned long long *__restrict__ SA,
+                                         const unsigned long long *__restrict__ SB, int d, int64_t n,
+                                         const MeanState *__restrict__ st, int s_host, float *__restrict__ m) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= d) return;
-    const int s = s_dev ? *s_dev : s_host;
-    const double q = __ddiv_rn(__ll2double_rn((long long)S[c]), scalbn((double)n, s));
-    m[c] = __double2float_rn(q);
+    const int s = st ? mean_scale_of(st->amax, n) : s_host;
+    const int sel = SA ? mean_select(*st, n) : MEAN_REDO;
+    const long long v = (long long)(sel == MEAN_A ? SA[c] : sel == MEAN_B ? SB[c] : S[c]);
+    m[c] = __double2float_rn(__ddiv_rn(__ll2double_rn(v), scalbn((double)n, s)));
 }
 
 int host_mean_scale(float amax, int64_t n) {
@@ -577,8 +704,8 @@ int host_mean_scale(float amax, int64_t n) {
     return mean_scale_of(b & 0x7fffffffu, n);
 }
 
-cudaError_t launch_absmax_bits(const float *X, int64_t count, unsigned *bits, cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(bits, 0, sizeof(unsigned), st);
+cudaError_t launch_absmax_bits(const float *X, int64_t count, unsigned *bits, cudaStream_t st, bool zero_first) {
+    const cudaError_t e = zero_first ? cudaMemsetAsync(bits, 0, sizeof(unsigned), st) : cudaSuccess;
     if (e != cudaSuccess) return e;
     int64_t blocks = (count / 4 + 255) / 256;
     blocks = blocks < 1 ? 1 : (blocks > 152 * 8 ? 152 * 8 : blocks);
@@ -586,31 +713,57 @@ cudaError_t launch_absmax_bits(const float *X, int64_t count, unsigned *bits, cu
     return launched();
 }
 
-cudaError_t launch_mean_fixed(const float *X, int64_t n, int d, unsigned *bits, int *s_dev, unsigned long long *S,
-                              float *m, cudaStream_t st) {
-    cudaError_t e = launch_absmax_bits(X, n * (int64_t)d, bits, st);
-    if (e != cudaSuccess) return e;
-    mean_scale_kernel<<<1, 1, 0, st>>>(bits, n, s_dev);
-    if ((e = launched()) != cudaSuccess) return e;
-    if ((e = launch_colsum_fixed(X, n, d, s_dev, 0, S, true, st)) != cudaSuccess) return e;
-    return launch_mean_fixed_finish(S, d, n, s_dev, 0, m, st);
-}
-
-cudaError_t launch_colsum_fixed(const float *X, int64_t n, int d, const int *s_dev, int s_host,
-                                unsigned long long *S, bool zero_first, cudaStream_t st) {
-    if (zero_first) {
-        const cudaError_t e = cudaMemsetAsync(S, 0, sizeof(unsigned long long) * (size_t)d, st);
-        if (e != cudaSuccess) return e;
-    }
-    int64_t blocks = (n + 1023) / 1024;
+// Columns sums at s_host (st NULL), or at the scale of st->amax.
+static cudaError_t colsum_fixed(const float *X, int64_t n, int d, const MeanState *st_dev, bool only_redo, int s_host,
+                                unsigned long long *S, cudaStream_t st) {
+    // 64 rows a phase or more, so that the few atomics a block ends with stay few
+    const int cols = (d & 3) == 0 && ((uintptr_t)X & 15) == 0 ? d >> 2 : d;
+    const int phases = cols < 256 ? 256 / cols : 1;
+    int64_t blocks = (n + 64 * phases - 1) / (64 * phases);
     blocks = blocks < 1 ? 1 : (blocks > 152 * 8 ? 152 * 8 : blocks);
-    colsum_fixed_kernel<<<(unsigned)blocks, 256, 0, st>>>(X, n, d, s_dev, s_host, S);
+    colsum_fixed_kernel<<<(unsigned)blocks, 256, 0, st>>>(X, n, d, st_dev, only_redo ? 1 : 0, s_host, S);
     return launched();
 }
 
-cudaError_t launch_mean_fixed_finish(const unsigned long long *S, int d, int64_t n, const int *s_dev, int s_host,
-                                     float *m, cudaStream_t st) {
-    mean_fixed_finish_kernel<<<(d + 127) / 128, 128, 0, st>>>(S, d, n, s_dev, s_host, m);
+// ws: mean_ws_bytes(d), 16-byte aligned.
+size_t mean_ws_bytes(int d) { return 64 + 3 * sizeof(unsigned long long) * (size_t)d; }
+
+cudaError_t launch_mean_fixed(const float *X, int64_t n, int d, void *ws, float *m, cudaStream_t st) {
+    MeanState *ms = static_cast<MeanState *>(ws);
+    unsigned long long *S = reinterpret_cast<unsigned long long *>(static_cast<char *>(ws) + 64);
+    unsigned long long *SA = S + d, *SB = SA + d;
+    cudaError_t e = cudaMemsetAsync(ws, 0, mean_ws_bytes(d), st);
+    if (e != cudaSuccess) return e;
+    const int lg = ceil_log2(n);
+    const bool one_pass = lg >= MEAN_MIN_LOG2 && (d & 3) == 0 && ((uintptr_t)X & 15) == 0;
+    if (one_pass) {
+        mean_sample_kernel<<<(unsigned)std::min<int64_t>(n, MEAN_SAMPLE), 256, 0, st>>>(X, n, d, ms);
+        if ((e = launched()) != cudaSuccess) return e;
+        const int d4 = d >> 2;
+        const int phases = d4 < MEAN_THREADS ? MEAN_THREADS / d4 : 1;
+        const int threads = d4 < MEAN_THREADS ? (phases * d4 + 31) / 32 * 32 : MEAN_THREADS;
+        const size_t smem = 2 * sizeof(unsigned long long) * (size_t)d;
+        if (smem > 48 * 1024) {
+            e = cudaFuncSetAttribute(mean_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        mean_pass_kernel<<<152 * 2, threads, smem, st>>>(reinterpret_cast<const float4 *>(X), n, d4, lg, ms, SA, SB);
+        if ((e = launched()) != cudaSuccess) return e;
+    } else {
+        e = launch_absmax_bits(X, n * (int64_t)d, &ms->amax, st, false);
+        if (e != cudaSuccess) return e;
+    }
+    if ((e = colsum_fixed(X, n, d, ms, one_pass, 0, S, st)) != cudaSuccess) return e;
+    mean_fixed_finish_kernel<<<(d + 127) / 128, 128, 0, st>>>(S, one_pass ? SA : nullptr, SB, d, n, ms, 0, m);
+    return launched();
+}
+
+cudaError_t launch_colsum_fixed(const float *X, int64_t n, int d, int s, unsigned long long *S, cudaStream_t st) {
+    return colsum_fixed(X, n, d, nullptr, false, s, S, st);
+}
+
+cudaError_t launch_mean_fixed_finish(const unsigned long long *S, int d, int64_t n, int s, float *m, cudaStream_t st) {
+    mean_fixed_finish_kernel<<<(d + 127) / 128, 128, 0, st>>>(S, nullptr, nullptr, d, n, nullptr, s, m);
     return launched();
 }
 

@@ -707,11 +707,12 @@ int skm_quantize(int repr, const float *X, int64_t n, int d, skm_quant_params *q
         if (!qp->m || !qp->nx2 || !qp->F || !qp->popx)
             return set_error(SKM_ERR_INVALID_ARG, "RBQ1 needs m, nx2, F and popx");
         if (qp->fit) {
-            unsigned *bits = cv.take<unsigned>(1);
-            int *s_dev = cv.take<int>(1);
+            // (the two words close the workspace as they always have; the mean
+            // fits the reduction buffers, RED_BLOCKS d doubles)
+            cv.take<unsigned>(1);
+            cv.take<int>(1);
             SKM_TRY(need_ws(cv, ws_bytes, ws));
-            SKM_CUDA_TRY(launch_mean_fixed(X, n, d, bits, s_dev, reinterpret_cast<unsigned long long *>(psum), qp->m,
-                                           st));
+            SKM_CUDA_TRY(launch_mean_fixed(X, n, d, psum, qp->m, st));
         }
         SKM_CUDA_TRY(launch_rbq1_encode(X, n, d, qp->m, static_cast<uint32_t *>(codes), qp->nx2,
                                         qp->F, qp->popx, st));
@@ -763,7 +764,7 @@ int skm_column_sums_fixed(const float *X, int64_t n, int d, int s, int64_t *sums
     if (!X || !sums) return set_error(SKM_ERR_INVALID_ARG, "NULL pointer");
     if (n < 1 || d < 1 || d > MAX_D) return set_error(SKM_ERR_INVALID_ARG, "bad shape n=%lld d=%d", (long long)n, d);
     SKM_CUDA_TRY(
-        launch_colsum_fixed(X, n, d, nullptr, s, reinterpret_cast<unsigned long long *>(sums), false, S(stream)));
+        launch_colsum_fixed(X, n, d, s, reinterpret_cast<unsigned long long *>(sums), S(stream)));
     return SKM_OK;
 }
 
@@ -771,7 +772,7 @@ int skm_mean_from_sums(const int64_t *sums, int64_t n_total, int d, int s, float
     if (!sums || !m) return set_error(SKM_ERR_INVALID_ARG, "NULL pointer");
     if (n_total < 1 || d < 1 || d > MAX_D)
         return set_error(SKM_ERR_INVALID_ARG, "bad shape n=%lld d=%d", (long long)n_total, d);
-    SKM_CUDA_TRY(launch_mean_fixed_finish(reinterpret_cast<const unsigned long long *>(sums), d, n_total, nullptr, s,
+    SKM_CUDA_TRY(launch_mean_fixed_finish(reinterpret_cast<const unsigned long long *>(sums), d, n_total, s,
                                           m, S(stream)));
     return SKM_OK;
 }

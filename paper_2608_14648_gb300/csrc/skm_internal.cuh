@@ -158,15 +158,14 @@ cudaError_t launch_colsum_partial(const float *X, int64_t n, int d, double *psum
                                   cudaStream_t st);
 // the RabitQ mean in exact fixed point (see k_quant.cu): the scale s of a
 // maximum |x| and a point count, the max |x| bits, the column sums at scale s
-// (added into S; s from s_dev when non-NULL, else s_host), and m = S / (n 2^s)
+// (added into S), m = S / (n 2^s), and all of it in one call (ws:
+// mean_ws_bytes(d), 16-byte aligned)
 int host_mean_scale(float amax, int64_t n);
-cudaError_t launch_absmax_bits(const float *X, int64_t count, unsigned *bits, cudaStream_t st);
-cudaError_t launch_colsum_fixed(const float *X, int64_t n, int d, const int *s_dev, int s_host,
-                                unsigned long long *S, bool zero_first, cudaStream_t st);
-cudaError_t launch_mean_fixed_finish(const unsigned long long *S, int d, int64_t n, const int *s_dev, int s_host,
-                                     float *m, cudaStream_t st);
-cudaError_t launch_mean_fixed(const float *X, int64_t n, int d, unsigned *bits, int *s_dev, unsigned long long *S,
-                              float *m, cudaStream_t st);
+cudaError_t launch_absmax_bits(const float *X, int64_t count, unsigned *bits, cudaStream_t st, bool zero_first = true);
+cudaError_t launch_colsum_fixed(const float *X, int64_t n, int d, int s, unsigned long long *S, cudaStream_t st);
+cudaError_t launch_mean_fixed_finish(const unsigned long long *S, int d, int64_t n, int s, float *m, cudaStream_t st);
+size_t mean_ws_bytes(int d);
+cudaError_t launch_mean_fixed(const float *X, int64_t n, int d, void *ws, float *m, cudaStream_t st);
 cudaError_t launch_colmean_finish(const double *psum, int nblk, int d, int64_t n, float *m,
                                   double *mean_d, cudaStream_t st);
 cudaError_t launch_rbq1_encode(const float *X, int64_t n, int d, const float *m, uint32_t *codes,
