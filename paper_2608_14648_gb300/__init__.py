@@ -258,7 +258,7 @@ OP_PROJECT, OP_PROJECT_MIN = 6, 7
 
 def skm_project(X, P, mean=None, out_dtype=DTYPE_F32, stream=None, ws=None, max_ws_bytes=None, cuda_cores=False):
     """Y = (X - mean) P.  Tensor cores (fp32 accuracy from bf16 parts) with a
-    workspace of up to max_ws_bytes (default: one pass over all rows);
+    small workspace for P's parts (max_ws_bytes does not go below it);
     cuda_cores=True selects the fp32 CUDA-core kernel (no workspace)."""
     n, d = X.shape
     d_out = P.shape[1]

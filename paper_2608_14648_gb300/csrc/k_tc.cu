@@ -36,13 +36,11 @@
 //    order, so the result equals the AND+popcount kernel's bit for bit.
 //  LVQ4: point and centroid codes 0..15 in e4m3, the accumulator is the exact
 //    integer P = <xbar, ybar> (<= 225 d) of Eq. final:lvq.
-#include <cuda.h>
-#include <cudaTypedefs.h>
-
 #include <cfloat>
 #include <mutex>
 
 #include "skm_tc.cuh"
+#include "tc_ptx.cuh"
 
 namespace skm {
 namespace {
@@ -65,12 +63,11 @@ constexpr int PK_MAX_CTAS = 160;
 // SKM_FLAG_WARM: stamp word 0 of a workspace whose last call completed
 constexpr int64_t WARM_MAGIC = 0x534b4d5741524d31LL;
 constexpr int TCAND = 4;
-constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;  // 2 s per barrier wait
 
-enum { MODE_SCREEN = 0, MODE_SQ8 = 1, MODE_RBQ1 = 2, MODE_LVQ4 = 3, MODE_GEMM = 4, MODE_PFRONT = 5 };
+enum { MODE_SCREEN = 0, MODE_SQ8 = 1, MODE_RBQ1 = 2, MODE_LVQ4 = 3, MODE_PFRONT = 4 };
 // Epilogue warps per TMEM lane quarter, by mode.  Every CTA works alone
 // (no thread-block clusters): it loads its own centroid slices.
-constexpr int TC_NH[6] = {4, 4, 4, 4, 4, 4};
+constexpr int TC_NH[5] = {4, 4, 4, 4, 4};
 // Job streams per CTA, by mode.  NS = 2: the CTA's point tiles form two
 // streams whose jobs the MMA warp issues alternately, each into its own TMEM
 // accumulator, each drained by its own half of the epilogue warps; an
@@ -80,14 +77,7 @@ constexpr int TC_NH[6] = {4, 4, 4, 4, 4, 4};
 // records.)  Measured at 1M x 1000 x 768 against one stream: 1-bit 0.508 vs
 // 0.574 ms, LVQ4 0.532 vs 0.575, fp32 screen 0.99 vs 1.02, SQ8 (with NH = 4)
 // 0.847 vs 0.882.
-constexpr int TC_NS[6] = {2, 2, 2, 2, 2, 2};
-// GEMM mode (the projection Y = (X - mean) P in fp32 accuracy from bf16
-// parts x = x1 + x2 + x3, P = p1 + p2 + p3): K segments of (A part, B part),
-// the smallest products first; parts i + j > 4 (below 2^-24 relative) are left
-// out.  The A parts are stacked as rows [part][n], the B parts as [part][dout].
-constexpr int GEMM_NSEG = 6;
-__device__ constexpr int GEMM_SEG_A[GEMM_NSEG] = {2, 1, 0, 1, 0, 0};
-__device__ constexpr int GEMM_SEG_B[GEMM_NSEG] = {0, 1, 2, 0, 1, 0};
+constexpr int TC_NS[5] = {2, 2, 2, 2, 2};
 // Columns per TMEM load in the e4m3 epilogues (32: one load and wait per 32
 // columns; 16: two buffers, the next load in flight).  Measured on GB300 at
 // 1M x 1000 x 768 with two job streams: 16 for the 1-bit epilogue (0.511 vs
@@ -178,10 +168,6 @@ struct TcParams {
     const int32_t *seg_group;
     const int32_t *seg_base;
     int nseg;
-    // GEMM mode: Y [n][dout] (fp32, or bf16 bits when y_bf16), row stride ydout
-    void *y;
-    int y_bf16;
-    int ydout;
     // PFRONT: per row (threshold on s~ over the front dimensions, the seed's
     // pruned distance), survivor lists [n][PF_CAP] (sorted positions, one
     // sub-list of PF_CAP / NHG per column slice), per listed row the
@@ -205,136 +191,6 @@ struct TcParams {
     // loaded anything and reports through the abort flag.
     unsigned long long inject_wait_ns;
 };
-
-// ------------------------------------------------------------- PTX helpers
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ unsigned long long globaltimer() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait: false when the abort flag is raised or the limit elapses
-// (the flag is then raised so that every role stops).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int32_t *abort_flag,
-                                          unsigned long long limit_ns = WAIT_LIMIT_NS) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = globaltimer();
-    for (uint32_t i = 1;; ++i) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((i & 255) == 0) {
-            if (*abort_flag) return false;
-            if (globaltimer() - t0 > limit_ns) {
-                *abort_flag = 1;
-                return false;
-            }
-        }
-    }
-}
-// Wait with the limit only (the abort flag is already up): used after a
-// role gave up, to let the asynchronous copies or MMAs it had issued finish
-// before the CTA releases its shared memory and TMEM.
-__device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity) {
-    const unsigned long long t0 = globaltimer();
-    for (uint32_t i = 0;; ++i) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((i & 255) == 255 && globaltimer() - t0 > WAIT_LIMIT_NS) return false;
-    }
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y,
-                                            uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-        : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() {
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                     bar)
-                 : "memory");
-}
-__device__ __forceinline__ void tc_mma(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                       uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(dtmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ void tc_mma_f8(uint32_t dtmem, uint64_t adesc, uint64_t bdesc,
-                                          uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(dtmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// 32 lanes x 32 consecutive 32-bit columns: thread i receives lane (base + i).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-          "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-          "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]),
-          "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]),
-          "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-        : "r"(taddr)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// 16 columns, no wait: the registers are valid only after tmem_wait16 on the
-// same array (which names them as operands, so nothing reads them earlier).
-__device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t (&v)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_wait16(uint32_t (&v)[16]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
-                   "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]),
-                   "+r"(v[15])
-                 :
-                 : "memory");
-}
 
 // Packed fp32 pairs (two IEEE round-to-nearest operations per instruction).
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
@@ -432,18 +288,6 @@ __device__ __forceinline__ uint32_t pickn(const uint32_t (&v)[N], int i) {
         return pick16(v, i);
 }
 
-// Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of
-// 128 bytes in 8-row (1024-byte) groups as written by TMA.  The start address
-// advances by 32 bytes per K=16 step inside the swizzle row.
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
-    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);  // start address
-    d |= (uint64_t)1 << 16;                            // leading byte offset (unused here)
-    d |= (uint64_t)(1024 >> 4) << 32;                  // stride byte offset: 8 rows x 128 B
-    d |= (uint64_t)1 << 46;                            // descriptor version (sm_100 family)
-    d |= (uint64_t)2 << 61;                            // 128-byte swizzle
-    return d;
-}
-
 // Instruction descriptors: D fp32, both operands K-major, N = 256, M = 128;
 // kind::f16 with A/B bf16, kind::f8f6f4 with A/B e4m3.
 constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
@@ -524,7 +368,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
     tc_assign_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const TcParams p) {
     static_assert(NS == 1 || (NS == 2 && NH % 2 == 0), "two job streams: two epilogue groups");
-    static_assert(NS == 1 || MODE == MODE_GEMM ||
+    static_assert(NS == 1 ||
                       epi_threads<NH>() / NS >= (MODE == MODE_SCREEN || MODE == MODE_PFRONT ? 128 : 256),
                   "records staged by one epilogue group");
     static_assert(MODE != MODE_PFRONT || !SEG, "the pruning front has no segmented variant");
@@ -559,7 +403,6 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int32_t *abort_flag = p.counters + 2;
-    constexpr int NSEG = MODE == MODE_GEMM ? GEMM_NSEG : 1;  // K segments per job
     constexpr int KC_ELEMS = f8_mode<MODE>() ? 128 : 64;  // elements per 128-byte row
 
     if (threadIdx.x == 0) {
@@ -683,10 +526,8 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                     arow0 = (((int64_t)blockIdx.x * NS + sj) * 2 + ((pc - 1u) & 1u)) * BM;
                 }
                 {
-                    for (int kt = 0; kt < NSEG * p.nkc; ++kt, ++it) {
-                        const int seg = kt / p.nkc, kc = kt - seg * p.nkc;
-                        const int arow = (int)arow0 + (NSEG > 1 ? GEMM_SEG_A[seg] * (int)p.n : 0);
-                        const int brow = ct * BN + (NSEG > 1 ? GEMM_SEG_B[seg] * p.k : 0);
+                    const int arow = (int)arow0, brow = ct * BN;
+                    for (int kc = 0; kc < p.nkc; ++kc, ++it) {
                         const uint32_t s = it % STAGES, ph = (it / STAGES) & 1u;
                         if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) goto producer_done;
                         mbar_expect_tx(full_bar(s), A_STAGE + B_STAGE);
@@ -756,12 +597,12 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                     if (!mbar_wait(tempty_bar(b), bph ^ 1u, abort_flag)) goto mma_done;
                     tc_fence_after();
                     const uint32_t dcol = tmem + b * BN;
-                    for (int kc = 0; kc < NSEG * p.nkc; ++kc, ++it) {
+                    for (int kc = 0; kc < p.nkc; ++kc, ++it) {
                         const uint32_t s = it % STAGES, ph = (it / STAGES) & 1u;
                         if (!mbar_wait(full_bar(s), ph, abort_flag)) goto mma_done;
                         // PK: the tile's last slice has landed, so no TMA load
                         // reads its scratch slot any more
-                        if (PK && tile_last && kc == NSEG * p.nkc - 1) mbar_arrive(sfree_bar(sj, slot));
+                        if (PK && tile_last && kc == p.nkc - 1) mbar_arrive(sfree_bar(sj, slot));
                         tc_fence_after();
                         const uint64_t ad = sw128_desc(sA + s * A_STAGE);
                         const uint64_t bd = sw128_desc(sB + s * B_STAGE);
@@ -1079,47 +920,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                 const uint8_t *rbuf = rec_base + rb * REC_BYTES;
                 const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + b * BN + slice * SW;
                 const int jh = ct * BN + slice * SW;
-                if (MODE == MODE_GEMM) {
-                    // write the accumulator row out: 32 columns per TMEM load
-#pragma unroll 1
-                    for (int c = 0; c < SW / 32; ++c) {
-                        const int col0 = jh + c * 32;
-                        if (col0 >= p.ydout) break;  // warp-uniform
-                        uint32_t v[32];
-                        tmem_ld32(taddr + c * 32, v);
-                        if (valid) {
-                        if (p.y_bf16) {
-                            uint16_t *yr = static_cast<uint16_t *>(p.y) + row * p.ydout;
-                            if (col0 + 32 <= p.ydout && (p.ydout % 8) == 0) {
-                                uint32_t w[16];
-#pragma unroll
-                                for (int i = 0; i < 16; ++i)
-                                    w[i] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(__uint_as_float(v[2 * i]))) |
-                                           ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(__uint_as_float(v[2 * i + 1]))) << 16);
-                                uint4 *dst = reinterpret_cast<uint4 *>(yr + col0);
-#pragma unroll
-                                for (int q4 = 0; q4 < 4; ++q4)
-                                    dst[q4] = make_uint4(w[4 * q4], w[4 * q4 + 1], w[4 * q4 + 2], w[4 * q4 + 3]);
-                            } else {
-                                for (int i = 0; i < 32 && col0 + i < p.ydout; ++i)
-                                    yr[col0 + i] = __bfloat16_as_ushort(__float2bfloat16_rn(__uint_as_float(pick32(v, i))));
-                            }
-                        } else {
-                            float *yr = static_cast<float *>(p.y) + row * p.ydout;
-                            if (col0 + 32 <= p.ydout && (p.ydout % 4) == 0) {
-                                float4 *dst = reinterpret_cast<float4 *>(yr + col0);
-#pragma unroll
-                                for (int q4 = 0; q4 < 8; ++q4)
-                                    dst[q4] = make_float4(__uint_as_float(v[4 * q4]), __uint_as_float(v[4 * q4 + 1]),
-                                                          __uint_as_float(v[4 * q4 + 2]), __uint_as_float(v[4 * q4 + 3]));
-                            } else {
-                                for (int i = 0; i < 32 && col0 + i < p.ydout; ++i)
-                                    yr[col0 + i] = __uint_as_float(pick32(v, i));
-                            }
-                        }
-                        }
-                    }
-                } else if (MODE == MODE_SCREEN) {
+                if (MODE == MODE_SCREEN) {
                     // chunks of SCR_CW columns (16: the next TMEM load in flight)
                     constexpr int NC = SW / SCR_CW;
                     constexpr int G = SCR_CW / 8;
@@ -1398,7 +1199,6 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
             // (single buffer: a publisher rewrites its slot only at the end of
             // the next point tile, after slice 0 has passed that tile's first
             // job barrier, i.e. after it has read this one)
-            if (MODE == MODE_GEMM) continue;  // no per-row reduction across slices
             if (slice > 0) {
                 uint32_t *slot = merge + ((slice - 1) * BM + rin) * MW;
                 if (MODE == MODE_SCREEN) {
@@ -2089,46 +1889,6 @@ __global__ void seg_rows_exact_kernel(const TX *__restrict__ X, int d, const flo
 }
 
 // ------------------------------------------------------------------ host side
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                             &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    });
-    return fn;
-}
-
-// 2D map over [rows][cols] of 2-byte (bf16) or 1-byte (e4m3, as uint8)
-// elements with row stride `stride_elems`; box = box_rows x 128 bytes.
-int make_map(CUtensorMap *m, const void *ptr, int64_t rows, int cols, int stride_elems,
-             int box_rows, int elem_bytes) {
-    auto fn = encode_fn();
-    if (!fn) return set_error(SKM_ERR_CUDA, "cuTensorMapEncodeTiled entry point not found");
-    cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t gstride[1] = {(cuuint64_t)stride_elems * elem_bytes};
-    cuuint32_t box[2] = {(cuuint32_t)(128 / elem_bytes), (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    const CUtensorMapDataType dt =
-        elem_bytes == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8;
-    CUresult r = fn(m, dt, 2, const_cast<void *>(ptr), gdim, gstride, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return set_error(SKM_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
-    return SKM_OK;
-}
-
-int device_sms() {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? sms : 148;
-}
-
 template <int MODE, bool SEG, bool PK>
 int launch_tc_kind(const void *xs, int64_t n, int dp, int d, const void *cs, int k, const TcParams &p0,
                    cudaStream_t st, int dpb);
@@ -2165,7 +1925,7 @@ int launch_tc_kind(const void *xs, int64_t n, int dp, int d, const void *cs, int
     // the dynamic shared memory attribute, set once per device
     constexpr int MAXDEV = 64;
     static std::mutex mu;
-    static bool attr_set[6][2][2][MAXDEV] = {};
+    static bool attr_set[5][2][2][MAXDEV] = {};
     int dev = 0;
     SKM_CUDA_TRY(cudaGetDevice(&dev));
     {
@@ -2177,17 +1937,15 @@ int launch_tc_kind(const void *xs, int64_t n, int dp, int d, const void *cs, int
     }
     CUtensorMap ma, mb;
     const int eb = f8_mode<MODE>() ? 1 : 2;
-    // GEMM mode: the A and B parts are stacked (rows [part][n], [part][k])
-    const int parts = MODE == MODE_GEMM ? 3 : 1;
     // PK: the A slices come from the CTAs' expansion scratch
     int grid = (int)std::min<int64_t>(device_sms(), cdiv(n, BM));
     if (PK) {
         grid = std::min(grid, PK_MAX_CTAS);
         SKM_TRY(make_map(&ma, p0.pk_scratch, (int64_t)grid * NS * 2 * BM, d, dp, BM, eb));
     } else {
-        SKM_TRY(make_map(&ma, xs, parts * n, d, dp, BM, eb));
+        SKM_TRY(make_map(&ma, xs, n, d, dp, BM, eb));
     }
-    SKM_TRY(make_map(&mb, cs, (int64_t)parts * k, d, dpb, BN, eb));
+    SKM_TRY(make_map(&mb, cs, k, d, dpb, BN, eb));
     TcParams p = p0;
     p.n = n;
     p.nrt = cdiv(n, BM);
@@ -2780,112 +2538,6 @@ int tc_assign_lvq4(const skm_data *x, const float *C, int k, int32_t *assign, fl
     }
     SKM_TRY(seg_setup(seg, n, p, st));
     SKM_TRY(launch_tc<MODE_LVQ4>(v.xs, n, dp, d, b.cs, k, p, st, v.packed));
-    return SKM_OK;
-}
-
-// ------------------------------------------------------------- projection
-namespace {
-// fp32 v -> bf16 parts v1 + v2 + v3 (each the round-to-nearest-even bf16 of
-// the remainder; the remainders are exact in fp32)
-__device__ __forceinline__ void split3(float v, uint16_t &a, uint16_t &b, uint16_t &c) {
-    const __nv_bfloat16 h1 = __float2bfloat16_rn(v);
-    const float r1 = __fsub_rn(v, __bfloat162float(h1));
-    const __nv_bfloat16 h2 = __float2bfloat16_rn(r1);
-    const float r2 = __fsub_rn(r1, __bfloat162float(h2));
-    a = __bfloat16_as_ushort(h1);
-    b = __bfloat16_as_ushort(h2);
-    c = __bfloat16_as_ushort(__float2bfloat16_rn(r2));
-}
-
-// rows [0, n) of X - mean -> A parts [3][n][dp] (8 dimensions per thread)
-__global__ void proj_split_x_kernel(const float *__restrict__ X, int64_t n, int d, const float *__restrict__ mu,
-                                    int dp, uint16_t *__restrict__ A) {
-    const int no = dp / 8;
-    const int64_t total = n * no;
-    const size_t part = (size_t)n * dp;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = t / no;
-        const int i0 = (int)(t - r * no) * 8;
-        uint32_t w[3][4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            uint16_t a[2], b[2], c[2];
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int i = i0 + 2 * q + u;
-                float v = 0.0f;
-                if (i < d) v = mu ? __fsub_rn(X[r * d + i], mu[i]) : X[r * d + i];
-                split3(v, a[u], b[u], c[u]);
-            }
-            w[0][q] = (uint32_t)a[0] | ((uint32_t)a[1] << 16);
-            w[1][q] = (uint32_t)b[0] | ((uint32_t)b[1] << 16);
-            w[2][q] = (uint32_t)c[0] | ((uint32_t)c[1] << 16);
-        }
-#pragma unroll
-        for (int s3 = 0; s3 < 3; ++s3)
-            *reinterpret_cast<uint4 *>(A + s3 * part + r * dp + i0) = make_uint4(w[s3][0], w[s3][1], w[s3][2], w[s3][3]);
-    }
-}
-
-// P [d][dout] -> B parts [3][dout][dp] (transposed: K-major rows per output column)
-__global__ void proj_split_p_kernel(const float *__restrict__ P, int d, int dout, int dp, uint16_t *__restrict__ B) {
-    const int64_t total = (int64_t)dout * dp;
-    const size_t part = (size_t)dout * dp;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int j = (int)(t / dp), i = (int)(t - (int64_t)j * dp);
-        uint16_t a = 0, b = 0, c = 0;
-        if (i < d) split3(P[(int64_t)i * dout + j], a, b, c);
-        B[t] = a;
-        B[part + t] = b;
-        B[2 * part + t] = c;
-    }
-}
-}  // namespace
-
-size_t tc_project_ws_min(int d, int dout) {
-    const size_t dp = (size_t)round8(d);
-    return 256 + 3 * (size_t)dout * dp * 2 + 256 + 3 * (size_t)BM * dp * 2 + 256 + 64;
-}
-
-size_t tc_project_ws_full(int64_t n, int d, int dout) {
-    const size_t dp = (size_t)round8(d);
-    return 256 + 3 * (size_t)dout * dp * 2 + 256 + 3 * (size_t)n * dp * 2 + 256 + 64;
-}
-
-int tc_project(const float *X, int64_t n, int d, const float *mean, const float *P, int dout, int out_bf16, void *Y,
-               void *ws, size_t ws_bytes, cudaStream_t st) {
-    const int dp = round8(d);
-    Carver cv(ws, ws_bytes);
-    int32_t *counters = cv.take<int32_t>(16);
-    uint16_t *B = cv.take<uint16_t>((size_t)3 * dout * dp);
-    const size_t used = cv.off + 256;
-    int64_t rows = ws_bytes > used ? (int64_t)((ws_bytes - used) / ((size_t)3 * dp * 2)) : 0;
-    if (rows >= n) rows = n;
-    else rows = (rows / BM) * BM;
-    if (rows < 1) return set_error(SKM_ERR_NO_MEMORY, "projection workspace too small");
-    uint16_t *A = cv.take<uint16_t>((size_t)3 * rows * dp);
-    if (cv.off > ws_bytes) return set_error(SKM_ERR_NO_MEMORY, "projection workspace too small");
-    {
-        int64_t blocks = ((int64_t)dout * dp + 255) / 256;
-        if (blocks > 152 * 8) blocks = 152 * 8;
-        proj_split_p_kernel<<<(unsigned)blocks, 256, 0, st>>>(P, d, dout, dp, B);
-        SKM_CUDA_TRY(launched());
-    }
-    SKM_CUDA_TRY(cudaMemsetAsync(counters, 0, sizeof(int32_t) * 16, st));
-    for (int64_t r0 = 0; r0 < n; r0 += rows) {
-        const int64_t nr = n - r0 < rows ? n - r0 : rows;
-        int64_t blocks = (nr * (dp / 8) + 255) / 256;
-        if (blocks > 152 * 16) blocks = 152 * 16;
-        proj_split_x_kernel<<<(unsigned)blocks, 256, 0, st>>>(X + r0 * d, nr, d, mean, dp, A);
-        SKM_CUDA_TRY(launched());
-        TcParams p{};
-        p.counters = counters;
-        p.y = out_bf16 ? (void *)(static_cast<uint16_t *>(Y) + r0 * dout) : (void *)(static_cast<float *>(Y) + r0 * dout);
-        p.y_bf16 = out_bf16;
-        p.ydout = dout;
-        p.d = d;
-        SKM_TRY(launch_tc<MODE_GEMM>(A, nr, dp, d, B, dout, p, st));
-    }
     return SKM_OK;
 }
 

@@ -537,13 +537,13 @@ size_t skm_workspace_size(int op, const skm_data *x, int k) {
         cv.take<int>(1);
         break;
     }
-    case 6:  // skm_project on tensor cores, one pass
-    case 7: {  // ... the smallest workspace (rows in chunks)
+    case 6:  // skm_project on tensor cores
+    case 7: {  // ... the smallest workspace it takes, the same
         if (!x || x->d < 1 || x->d > MAX_D || x->n < 1 || k < 1 || k > x->d) {
             set_error(SKM_ERR_INVALID_ARG, "bad skm_data / d_out for op %d", op);
             return 0;
         }
-        return op == 6 ? tc_project_ws_full(x->n, x->d, k) : tc_project_ws_min(x->d, k);
+        return tc_project_ws_min(x->d, k);
     }
     case 4: {  // pca
         if (!x || x->d < 1 || x->d > MAX_D) {
