@@ -137,7 +137,7 @@ struct TcParams {
     int64_t *stats;     // code modes: [2] gets the abort flag (may be NULL)
     int32_t *assign;
     const int32_t *nx;  // SQ8: centred ||x||^2
-    const int32_t *nc;  // SQ8: centred ||c||^2, padded to 256 with a large value
+    const int32_t *nc;  // SQ8: centred ||c||^2 (float bits), padded to 256 with a large value
     float *dist;        // SQ8 / RBQ1 (may be null)
     const float4 *rinfo;     // RBQ1: per column pair (bd x2, sd x2), padded
     const float4 *rinfoq;    // RBQ1: per column pair (-sum ybar x2, ||c - m||^2 x2)
@@ -918,6 +918,14 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                 if (dead) continue;
                 tc_fence_after();
                 const uint8_t *rbuf = rec_base + rb * REC_BYTES;
+                // The warp's last TMEM load of the job has completed (each thread
+                // waited on it): one arrival releases its share, so that the MMA
+                // can refill the accumulator while the last chunk is evaluated.
+                auto release = [&] {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(tempty_bar(b));
+                };
                 const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + b * BN + slice * SW;
                 const int jh = ct * BN + slice * SW;
                 if (MODE == MODE_SCREEN) {
@@ -996,30 +1004,15 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                             }
                         }
                     };
-                    if constexpr (SCR_CW == 32) {
+                    {
+                        const int nv = min(NC, (p.k - jh + 31) / 32);  // chunks inside [0, k) (warp-uniform)
+                        if (nv <= 0) release();
 #pragma unroll 1
-                        for (int c = 0; c < NC; ++c) {
-                            if (jh + c * 32 >= p.k) break;  // warp-uniform
+                        for (int c = 0; c < nv; ++c) {
                             uint32_t v[32];
                             tmem_ld32(taddr + c * 32, v);
+                            if (c == nv - 1) release();
                             chunk(v, c);
-                        }
-                    } else if (jh < p.k) {  // warp-uniform conditions throughout
-                        uint32_t va[16], vb[16];
-                        tmem_ld16_async(taddr, va);
-                        tmem_wait16(va);
-#pragma unroll
-                        for (int c = 0; c < NC; c += 2) {
-                            const bool m1 = c + 1 < NC && jh + (c + 1) * 16 < p.k;
-                            if (m1) tmem_ld16_async(taddr + (c + 1) * 16, vb);
-                            chunk(va, c);
-                            if (!m1) break;
-                            tmem_wait16(vb);
-                            const bool m2 = c + 2 < NC && jh + (c + 2) * 16 < p.k;
-                            if (m2) tmem_ld16_async(taddr + (c + 2) * 16, va);
-                            chunk(vb, c + 1);
-                            if (!m2) break;
-                            tmem_wait16(va);
                         }
                     }
                 } else if (MODE == MODE_PFRONT) {
@@ -1038,22 +1031,14 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                     const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + b * BN;
                     int nvc = 0;  // this slice's chunks inside [0, k) (warp-uniform)
                     while (nvc < SW / 32 && ct * BN + (NHG * nvc + slice) * 32 < p.k) ++nvc;
-                    if (nvc == 0) {
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(tempty_bar(b));
-                    }
+                    if (nvc == 0) release();
 #pragma unroll 1
                     for (int c = 0; c < nvc; ++c) {
                         const int cc = (NHG * c + slice) * 32;  // column offset within the tile
                         const int j0 = ct * BN + cc;
                         uint32_t v[32];
                         tmem_ld32(tbase + cc, v);
-                        if (c == nvc - 1) {  // the warp's loads are complete (each thread waited)
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(tempty_bar(b));
-                        }
+                        if (c == nvc - 1) release();
                         auto f = [&](int i) { return __uint_as_float(v[i]); };
                         float m[11];
 #pragma unroll
@@ -1088,15 +1073,13 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                     auto chunk = [&](const uint32_t(&v)[F8_CW], int c) {
                         const int j0 = jh + c * F8_CW;
                         const int cc = slice * SW + c * F8_CW;
-                        float gb[G];
-                        int gi[G];
 #pragma unroll
                         for (int g = 0; g < G; ++g) {
                             asm volatile("" ::: "memory");
-                            gb[g] = INFINITY;
-                            gi[g] = 0x7fffffff;
+                            float e[8];
 #pragma unroll
-                            for (int i = 8 * g; i < 8 * g + 8; i += 2) {
+                            for (int u = 0; u < 8; u += 2) {
+                                const int i = 8 * g + u;
                                 const float4 r0 = reinterpret_cast<const float4 *>(rbuf)[(cc + i) >> 1];
                                 const float4 r1 = reinterpret_cast<const float4 *>(rbuf)[128 + ((cc + i) >> 1)];
                                 // the accumulator is the exact integer dot product (LVQ4:
@@ -1114,38 +1097,38 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                                     // Eq. final:rabitq in Eq. rabitq_l2: u = fma(sd, 2P -
                                     // sum ybar, bd pc), est = fma(-2F, u, nx2 + ny2)
                                     const float2 t = fmul2(make_float2(r0.x, r0.y), make_float2(rpc, rpc));
-                                    const float2 u = ffma2(make_float2(r0.z, r0.w), P2, t);
+                                    const float2 w = ffma2(make_float2(r0.z, r0.w), P2, t);
                                     const float2 nn = fadd2(make_float2(rnx2, rnx2), make_float2(r1.z, r1.w));
-                                    est = ffma2(make_float2(rf2, rf2), u, nn);
+                                    est = ffma2(make_float2(rf2, rf2), w, nn);
                                 }
                                 if (SEG && (j0 < cb || j0 + F8_CW > ce)) {  // columns outside the row's group
                                     if (j0 + i < cb || j0 + i >= ce) est.x = INFINITY;
                                     if (j0 + i + 1 < cb || j0 + i + 1 >= ce) est.y = INFINITY;
                                 }
-                                if (est.x < gb[g]) {
-                                    gb[g] = est.x;
-                                    gi[g] = j0 + i;
-                                }
-                                if (est.y < gb[g]) {
-                                    gb[g] = est.y;
-                                    gi[g] = j0 + i + 1;
-                                }
+                                e[u] = est.x;
+                                e[u + 1] = est.y;
+                            }
+                            // half an instruction a column for the minimum of eight;
+                            // which of them it was (the first, ties to the lower
+                            // index) is asked only when it is a new best
+                            const float m = fmin3(fmin3(e[0], e[1], e[2]), fmin3(e[3], e[4], e[5]), fminf(e[6], e[7]));
+                            if (m < fbest) {
+                                fbest = m;
+                                int at = 7;
+#pragma unroll
+                                for (int u = 6; u >= 0; --u) at = e[u] == m ? u : at;
+                                besti = j0 + 8 * g + at;
                             }
                         }
-                        // the groups hold increasing columns: the earlier wins ties
-#pragma unroll
-                        for (int g = 0; g < G; ++g)
-                            if (gb[g] < fbest) {
-                                fbest = gb[g];
-                                besti = gi[g];
-                            }
                     };
                     if constexpr (F8_CW == 32) {
+                        const int nv = min(NC, (p.k - jh + 31) / 32);  // chunks inside [0, k) (warp-uniform)
+                        if (nv <= 0) release();
 #pragma unroll 1
-                        for (int c = 0; c < NC; ++c) {
-                            if (jh + c * 32 >= p.k) break;  // warp-uniform
+                        for (int c = 0; c < nv; ++c) {
                             uint32_t v[32];
                             tmem_ld32(taddr + c * 32, v);
+                            if (c == nv - 1) release();
                             chunk(v, c);
                         }
                     } else if (jh < p.k) {  // warp-uniform conditions throughout
@@ -1156,43 +1139,65 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                         for (int c = 0; c < NC; c += 2) {
                             const bool m1 = c + 1 < NC && jh + (c + 1) * 16 < p.k;
                             if (m1) tmem_ld16_async(taddr + (c + 1) * 16, vb);
+                            else release();
                             chunk(va, c);
                             if (!m1) break;
                             tmem_wait16(vb);
                             const bool m2 = c + 2 < NC && jh + (c + 2) * 16 < p.k;
                             if (m2) tmem_ld16_async(taddr + (c + 2) * 16, va);
+                            else release();
                             chunk(vb, c + 1);
                             if (!m2) break;
                             tmem_wait16(va);
                         }
+                    } else {
+                        release();
                     }
-                } else
+                } else {  // MODE_SQ8
+                    const int nv = min(SW / 32, (p.k - jh + 31) / 32);  // chunks inside [0, k) (warp-uniform)
+                    if (nv <= 0) release();
 #pragma unroll 1
-                for (int c = 0; c < SW / 32; ++c) {
-                    const int j0 = jh + c * 32;
-                    const int cc = slice * SW + c * 32;  // column offset within the tile
-                    if (j0 >= p.k) break;  // warp-uniform
-                    uint32_t v[32];
-                    tmem_ld32(taddr + c * 32, v);
-                    if (MODE == MODE_SQ8) {
+                    for (int c = 0; c < nv; ++c) {
+                        const int j0 = jh + c * 32;
+                        const int cc = slice * SW + c * 32;  // column offset within the tile
+                        uint32_t v[32];
+                        tmem_ld32(taddr + c * 32, v);
+                        if (c == nv - 1) release();
+                        // s = ||c||^2 - 2 dot, exact integers in both operands, with
+                        // one rounding at most: rounding is monotone, so only a
+                        // group of eight whose smallest rounded s is below (or,
+                        // past 2^24, not above) the rounded best can hold a
+                        // smaller s; such a group is evaluated in integers
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) {
-                            const int32_t dot = __float2int_rn(__uint_as_float(v[i]));
-                            const int32_t dd = nxr + reinterpret_cast<const int32_t *>(rbuf)[cc + i] - 2 * dot;
-                            if (dd < best && (!SEG || (j0 + i >= cb && j0 + i < ce))) {
-                                best = dd;
-                                besti = j0 + i;
+                        for (int g = 0; g < 4; ++g) {
+                            float m = INFINITY;
+#pragma unroll
+                            for (int u = 0; u < 8; u += 4) {
+                                const int i = 8 * g + u;
+                                const float4 c4 = reinterpret_cast<const float4 *>(rbuf)[(cc + i) >> 2];
+                                const float2 a0 = make_float2(__uint_as_float(v[i]), __uint_as_float(v[i + 1]));
+                                const float2 a1 = make_float2(__uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
+                                const float2 s0 = ffma2(make_float2(-2.0f, -2.0f), a0, make_float2(c4.x, c4.y));
+                                const float2 s1 = ffma2(make_float2(-2.0f, -2.0f), a1, make_float2(c4.z, c4.w));
+                                m = fmin3(m, s0.x, s0.y);
+                                m = fmin3(m, s1.x, s1.y);
+                            }
+                            if (m < fbest || (m == fbest && fabsf(m) >= 16777216.0f)) {
+#pragma unroll
+                                for (int u = 0; u < 8; ++u) {
+                                    const int i = 8 * g + u;
+                                    const int32_t dot = __float2int_rn(__uint_as_float(v[i]));
+                                    const int32_t dd =
+                                        __float2int_rn(reinterpret_cast<const float *>(rbuf)[cc + i]) - 2 * dot;
+                                    if (dd < best && (!SEG || (j0 + i >= cb && j0 + i < ce))) {
+                                        best = dd;
+                                        besti = j0 + i;
+                                    }
+                                }
+                                fbest = best == 0x7fffffff ? INFINITY : __int2float_rn(best);
                             }
                         }
                     }
-                }
-                // the warp's TMEM loads are complete (each thread waited on
-                // them); one arrival for the warp releases its share (PFRONT:
-                // released after its last load already)
-                if (MODE != MODE_PFRONT) {
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(tempty_bar(b));
                 }
             }
             // merge the column slices of each row: slices 1.. publish, slice 0 finishes
@@ -1338,7 +1343,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                     }
                 } else if (MODE == MODE_SQ8) {
                     p.assign[row] = besti;
-                    if (p.dist) p.dist[row] = (float)best;
+                    if (p.dist) p.dist[row] = (float)(nxr + best);
                 } else if (MODE == MODE_LVQ4) {
                     p.assign[row] = besti;
                     if (p.dist) p.dist[row] = __fadd_rn(rnx2, fbest);
@@ -1696,7 +1701,7 @@ __global__ void cprep_sq8_kernel(const uint8_t *__restrict__ C, int k, int kp, i
     const int nw = (gridDim.x * blockDim.x) >> 5;
     for (int j = warp; j < kp; j += nw) {
         if (j >= k) {  // padding records: never the nearest
-            if (lane == 0) nc[j] = 0x3fffffff;
+            if (lane == 0) nc[j] = __float_as_int(1073741824.0f);
             continue;
         }
         int32_t s = 0;
@@ -1707,7 +1712,7 @@ __global__ void cprep_sq8_kernel(const uint8_t *__restrict__ C, int k, int kp, i
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) nc[j] = s;
+        if (lane == 0) nc[j] = __float_as_int((float)s);  // exact: s <= 2^14 d <= 2^24
     }
 }
 
