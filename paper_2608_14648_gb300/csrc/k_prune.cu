@@ -661,28 +661,21 @@ __global__ void __launch_bounds__(TP_WARPS * 32) prune_tiled_kernel(
 // dropped: the pruning kernels, seeded alike, never complete it either
 // (slack is theirs).  A non-finite seed distance keeps everything (the row then
 // overflows to the full pruning).
-// One 32-dimension block of (x_i - c_i)^2 for a lane: x from bf16 (16-byte
-// loads), c from fp32 (16-byte loads), every load issued before the chain;
-// the sum runs in increasing i as in block_partial.  q (when wanted) gets the
-// sum of x_i^2 over the block.  m = dimensions in the block (32 unless it is
-// the ragged last one).
+// One 32-dimension block of (x_i - c_i)^2 for a lane: x (bf16) and c (fp32) from
+// shared memory, both 16-byte aligned; the sum runs in increasing i as in
+// block_partial.  q (when wanted) gets the sum of x_i^2 over the block.  m =
+// dimensions in the block (32 unless it is the ragged last one).
 __device__ __forceinline__ float block_bf16(const uint16_t *xr, const float *cr, int m, bool want_q, float &q) {
     float part = 0.0f;
     q = 0.0f;
     if (m == 32) {
-        uint4 xw[4];
-        float4 cv[8];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) xw[u] = __ldg(reinterpret_cast<const uint4 *>(xr) + u);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) cv[u] = __ldg(reinterpret_cast<const float4 *>(cr) + u);
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const uint32_t w0 = (u & 1) ? xw[u >> 1].z : xw[u >> 1].x;
-            const uint32_t w1 = (u & 1) ? xw[u >> 1].w : xw[u >> 1].y;
-            const float xs[4] = {__uint_as_float(w0 << 16), __uint_as_float(w0 & 0xffff0000u),
-                                 __uint_as_float(w1 << 16), __uint_as_float(w1 & 0xffff0000u)};
-            const float cs[4] = {cv[u].x, cv[u].y, cv[u].z, cv[u].w};
+            const uint2 w = reinterpret_cast<const uint2 *>(xr)[u];
+            const float4 cv = reinterpret_cast<const float4 *>(cr)[u];
+            const float xs[4] = {__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u),
+                                 __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u)};
+            const float cs[4] = {cv.x, cv.y, cv.z, cv.w};
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
                 const float t = __fsub_rn(xs[h], cs[h]);
@@ -692,8 +685,8 @@ __device__ __forceinline__ float block_bf16(const uint16_t *xr, const float *cr,
         }
     } else {
         for (int i = 0; i < m; ++i) {
-            const float xv = __uint_as_float(((uint32_t)__ldg(xr + i)) << 16);
-            const float t = __fsub_rn(xv, __ldg(cr + i));
+            const float xv = __uint_as_float(((uint32_t)xr[i]) << 16);
+            const float t = __fsub_rn(xv, cr[i]);
             part = __fmaf_rn(t, t, part);
             if (want_q) q = __fmaf_rn(xv, xv, q);
         }
@@ -710,7 +703,9 @@ __device__ __forceinline__ float block_bf16(const uint16_t *xr, const float *cr,
 // grows by at most delta (triangle inequality), and the new pruned distance
 // is at most U' = (sqrt(U (1 + g)) + delta)^2 (1 + g), every step rounded up;
 // the threshold is then formed from U' as above, with the kept prefix norms.
-__global__ void front_prep_kernel(const uint16_t *__restrict__ X, int64_t n, int d, int F, int G,
+constexpr int FP_WARPS = 6;   // 43 KiB of shared memory a block, five blocks an SM
+constexpr int FP_LDX = 40;    // bf16 elements from a staged pair's points to the next's
+__global__ void __launch_bounds__(32 * FP_WARPS) front_prep_kernel(const uint16_t *__restrict__ X, int64_t n, int d, int F, int G,
                                   const float *__restrict__ C, int k, const int32_t *__restrict__ prev,
                                   const float *__restrict__ hz, PfRows r, int force_cold,
                                   unsigned long long *__restrict__ ctr) {
@@ -750,15 +745,52 @@ __global__ void front_prep_kernel(const uint16_t *__restrict__ X, int64_t n, int
         }
         return;
     }
+    // The warp's 32 (row, block) pairs are copied to shared memory first, a
+    // pair's 64 bytes of points by 4 lanes and 128 of its seed's centroid by 8
+    // (a lane reading its own pair from global memory touches one line per lane
+    // and load: 2.72 ms for 10M x 256 against the 0.75 that the points take at
+    // the copy bandwidth); pairs 80 and 144 bytes apart, so that the eight lanes
+    // of a 16-byte access phase hit distinct banks.
+    __shared__ __align__(16) uint16_t stage_x[FP_WARPS][32 * FP_LDX];
+    __shared__ __align__(16) float stage_c[FP_WARPS][32 * STG_LD];
+    uint16_t *sx = stage_x[threadIdx.x >> 5];
+    float *sc = stage_c[threadIdx.x >> 5];
+    const uint32_t sx0 = (uint32_t)__cvta_generic_to_shared(sx), sc0 = (uint32_t)__cvta_generic_to_shared(sc);
+    const int gsh = 31 - __clz(G);
+    auto seed_of = [&](int64_t row) {
+        const int v = row < n && prev ? __ldg(prev + row) : 0;
+        return v < 0 || v >= k ? 0 : v;
+    };
+    int seed_next = seed_of(warp * rpw + sub);
     for (int64_t r0 = warp * rpw; r0 < n; r0 += nw * rpw) {
         const int64_t row = r0 + sub;
         const bool act = row < n;
-        int seed = act && prev ? __ldg(prev + row) : 0;
-        if (seed < 0 || seed >= k) seed = 0;
+        const int seed = seed_next;
+        seed_next = seed_of(row + nw * rpw);
+        __syncwarp();  // every lane has read the previous pairs
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int pr = 8 * i + (lane >> 2), u = lane & 3, bb = pr & (G - 1);
+            const int64_t r = r0 + (pr >> gsh);
+            if (r < n && 32 * bb + 8 * u < d)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sx0 + 2u * (pr * FP_LDX + 8 * u)),
+                             "l"(X + r * d + 32 * bb + 8 * u)
+                             : "memory");
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int pr = 4 * i + (lane >> 3), u = lane & 7, bb = pr & (G - 1);
+            const int j = __shfl_sync(0xffffffffu, seed, pr);
+            if (r0 + (pr >> gsh) < n && 32 * bb + 4 * u < d)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sc0 + 4u * (pr * STG_LD + 4 * u)),
+                             "l"(C + (int64_t)j * d + 32 * bb + 4 * u)
+                             : "memory");
+        }
+        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+        __syncwarp();
         float part = 0.0f, q = 0.0f;
         if (act && b < nb)
-            part = block_bf16(X + row * d + 32 * b, C + (int64_t)seed * d + 32 * b, min(32, d - 32 * b), 32 * b < F,
-                              q);
+            part = block_bf16(sx + lane * FP_LDX, sc + lane * STG_LD, min(32, d - 32 * b), 32 * b < F, q);
         // the row's blocks in order (every lane of the group forms the same sum)
         float beta0 = __shfl_sync(0xffffffffu, part, 0, G);
         for (int t = 1; t < nb; ++t) beta0 = __fadd_rn(beta0, __shfl_sync(0xffffffffu, part, t, G));
@@ -1007,11 +1039,14 @@ cudaError_t launch_prune_front_prep(const uint16_t *X, int64_t n, int d, int F, 
     int G = 1;
     while (G < nb) G <<= 1;
     if (G > 32 || F % 32 != 0 || F > d || (d % 8) != 0) return cudaErrorInvalidValue;
-    const int64_t per_block = 256 / G;  // rows per block of 256 threads
+    // the kernel's 16-byte copies (both hold wherever the front is taken)
+    if ((reinterpret_cast<uintptr_t>(C) & 15) != 0 || (reinterpret_cast<uintptr_t>(X) & 15) != 0)
+        return cudaErrorInvalidValue;
+    const int64_t per_block = 32 * FP_WARPS / G;  // rows a block takes at a time
     int64_t blocks = (n + per_block - 1) / per_block;
-    if (blocks > 152 * 16) blocks = 152 * 16;
+    if (blocks > 152 * 10) blocks = 152 * 10;
     if (blocks < 1) blocks = 1;
-    front_prep_kernel<<<(int)blocks, 256, 0, st>>>(X, n, d, F, G, C, k, prev, hz, r, force_cold, ctr);
+    front_prep_kernel<<<(int)blocks, 32 * FP_WARPS, 0, st>>>(X, n, d, F, G, C, k, prev, hz, r, force_cold, ctr);
     return launched();
 }
 

@@ -623,15 +623,18 @@ __global__ void __launch_bounds__(RS_THREADS) ring_sum_sq8_kernel(
 
 // SQ8 rows of at most 1 KB, read straight into registers: no ring.  Lane l
 // loads the 16-byte groups l + 32 t of a row with 128-bit loads; the loads of
-// the next SQ8_PF rows of the warp's run are in flight while a row is summed
+// the next three or four rows of the warp's run are in flight while a row is summed
 // (a row's slot in the register buffer is refilled right after it is read),
 // and with little shared memory many warps fit per SM.
+// (1M x 1024, two groups a lane: 243, 236 and 257 us an update with 2, 3 and 4
+// rows in flight; one group a lane: no difference up to 4, slower beyond)
 constexpr int SQ8_PF = 4;
 template <int NG>
 __global__ void __launch_bounds__(RS_THREADS) direct_sum_sq8_kernel(
     const uint8_t *__restrict__ codes, int d, const int32_t *__restrict__ perm,
     const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k,
     unsigned long long *__restrict__ S, int run) {
+    constexpr int PF = NG == 2 ? 3 : SQ8_PF;
     __shared__ int32_t sperm_all[RS_CW][RS_ROWS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t nval = offsets[k];
@@ -652,18 +655,18 @@ __global__ void __launch_bounds__(RS_THREADS) direct_sum_sq8_kernel(
     cons.scl = scl;
     cons.S = S;
     cons.d = d;
-    uint4 buf[SQ8_PF][NG];
+    uint4 buf[PF][NG];
 #pragma unroll
-    for (int p = 0; p < SQ8_PF; ++p)
+    for (int p = 0; p < PF; ++p)
         if (p < cnt) load(p, buf[p]);
     cons.start(q0, cnt, lane);
-    for (int r0 = 0; r0 < cnt; r0 += SQ8_PF) {
+    for (int r0 = 0; r0 < cnt; r0 += PF) {
 #pragma unroll
-        for (int p = 0; p < SQ8_PF; ++p) {
+        for (int p = 0; p < PF; ++p) {
             const int r = r0 + p;
             if (r < cnt) {  // warp-uniform
                 cons.row_regs(r, buf[p], lane);
-                if (r + SQ8_PF < cnt) load(r + SQ8_PF, buf[p]);
+                if (r + PF < cnt) load(r + PF, buf[p]);
             }
         }
     }
