@@ -38,7 +38,9 @@ __device__ __forceinline__ void argmin_merge(float &bd, int &bi, float d, int i)
 // would otherwise run on a few SMs): each work item covers a range of
 // centroid tiles and merges (dist bits << 32 | index) into its rows' keys with
 // atomicMin — non-negative distances order like their bit patterns, so the
-// smallest key is the nearest centroid with ties to the lowest index.
+// smallest key is the nearest centroid with ties to the lowest index.  The
+// last of a row tile's items to finish writes its rows' assignments; they count
+// themselves in tickets[rows[first row] * tstride], preset to 0.
 template <typename TX>
 __global__ void __launch_bounds__(256) assign_exact_kernel(const TX *__restrict__ X,
                                                            const int32_t *__restrict__ rows,
@@ -47,7 +49,9 @@ __global__ void __launch_bounds__(256) assign_exact_kernel(const TX *__restrict_
                                                            const float *__restrict__ C, int k,
                                                            int32_t *__restrict__ assign,
                                                            float *__restrict__ dist,
-                                                           unsigned long long *__restrict__ keys) {
+                                                           unsigned long long *__restrict__ keys,
+                                                           int32_t *__restrict__ tickets, int tstride) {
+    __shared__ bool last_item;
     __shared__ __align__(16) float xs[32][68];
     __shared__ __align__(16) float cs[32][68];
     const int tid = threadIdx.x;
@@ -153,35 +157,32 @@ __global__ void __launch_bounds__(256) assign_exact_kernel(const TX *__restrict_
 #pragma unroll
             for (int i = 0; i < 4; ++i)
                 if (pval[i]) {
-                    if (keys) {
+                    if (nsplit > 1) {
                         if (besti[i] != 0x7fffffff)
                             atomicMin(keys + row0 + ty * 4 + i,
                                       ((unsigned long long)__float_as_uint(best[i]) << 32) | (uint32_t)besti[i]);
-                    } else {
+                    } else if (!keys || besti[i] != 0x7fffffff) {  // (listed rows without a distance keep theirs)
                         assign[prow[i]] = besti[i];
                         if (dist) dist[prow[i]] = best[i];
                     }
                 }
         }
+        if (nsplit > 1) {  // block-uniform
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) last_item = atomicAdd(tickets + (int64_t)rows[row0] * tstride, 1) == nsplit - 1;
+            __syncthreads();
+            if (last_item && tid < 64 && row0 + tid < nrows) {
+                __threadfence();
+                const unsigned long long key = __ldcg(keys + row0 + tid);
+                const int64_t r = rows[row0 + tid];
+                if (key != ~0ull) {  // (no centroid: k == 0 cannot happen here)
+                    assign[r] = (int32_t)(key & 0xffffffffull);
+                    if (dist) dist[r] = __uint_as_float((uint32_t)(key >> 32));
+                }
+            }
+        }
     }  // work items
-}
-
-__global__ void keys_init_kernel(const int32_t *__restrict__ count, unsigned long long *__restrict__ keys) {
-    const int64_t c = *count;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < c; i += (int64_t)gridDim.x * blockDim.x)
-        keys[i] = ~0ull;
-}
-
-__global__ void keys_finish_kernel(const int32_t *__restrict__ rows, const int32_t *__restrict__ count,
-                                   const unsigned long long *__restrict__ keys, int32_t *__restrict__ assign,
-                                   float *__restrict__ dist) {
-    const int64_t c = *count;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < c; i += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned long long key = keys[i];
-        if (key == ~0ull) continue;  // no centroid (k == 0 cannot happen on this path)
-        assign[rows[i]] = (int32_t)(key & 0xffffffffull);
-        if (dist) dist[rows[i]] = __uint_as_float((uint32_t)(key >> 32));
-    }
 }
 
 static unsigned blocks_for_rows(int64_t nrows) {
@@ -194,7 +195,7 @@ cudaError_t launch_assign_exact_f32(const float *X, int64_t n, int d, const floa
                                     int32_t *assign, float *dist, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     assign_exact_kernel<float><<<blocks_for_rows(n), 256, 0, st>>>(X, nullptr, nullptr, n, d, C,
-                                                                   k, assign, dist, nullptr);
+                                                                   k, assign, dist, nullptr, nullptr, 0);
     return launched();
 }
 
@@ -202,31 +203,25 @@ cudaError_t launch_assign_exact_bf16(const uint16_t *X, int64_t n, int d, const 
                                      int32_t *assign, float *dist, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     assign_exact_kernel<uint16_t><<<blocks_for_rows(n), 256, 0, st>>>(X, nullptr, nullptr, n, d,
-                                                                      C, k, assign, dist, nullptr);
+                                                                      C, k, assign, dist, nullptr, nullptr, 0);
     return launched();
 }
 
 cudaError_t launch_assign_exact_rows(const void *X, int x_is_bf16, const int32_t *rows,
                                      const int32_t *count_dev, int64_t max_rows, int d,
                                      const float *C, int k, int32_t *assign, float *dist,
-                                     unsigned long long *keys, cudaStream_t st) {
+                                     unsigned long long *keys, int32_t *tickets, int tstride, cudaStream_t st) {
     if (max_rows == 0) return cudaSuccess;
     // enough blocks to split the centroids when only a few rows are listed
     const unsigned g = keys ? 152u * 4u : blocks_for_rows(max_rows);
-    if (keys) {
-        keys_init_kernel<<<152, 256, 0, st>>>(count_dev, keys);
-        cudaError_t e = launched();
-        if (e != cudaSuccess) return e;
-    }
     if (x_is_bf16)
         assign_exact_kernel<uint16_t><<<g, 256, 0, st>>>(static_cast<const uint16_t *>(X), rows,
-                                                         count_dev, 0, d, C, k, assign, dist, keys);
+                                                         count_dev, 0, d, C, k, assign, dist, keys, tickets,
+                                                         tstride);
     else
         assign_exact_kernel<float><<<g, 256, 0, st>>>(static_cast<const float *>(X), rows,
-                                                      count_dev, 0, d, C, k, assign, dist, keys);
-    cudaError_t e = launched();
-    if (e != cudaSuccess || !keys) return e;
-    keys_finish_kernel<<<152, 256, 0, st>>>(rows, count_dev, keys, assign, dist);
+                                                      count_dev, 0, d, C, k, assign, dist, keys, tickets,
+                                                      tstride);
     return launched();
 }
 

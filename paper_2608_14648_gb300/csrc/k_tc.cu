@@ -125,6 +125,11 @@ struct TcParams {
     int64_t nrt;  // point tiles
     int k;
     int nct;  // centroid tiles
+    // SCREEN: the centroid tiles of a point tile are shared out to ksplit
+    // CTAs (1: one takes them all), whose rows' states go to part
+    // [n][ksplit][SCREEN_WORDS] for screen_merge_kernel
+    int ksplit;
+    uint32_t *part;
     int nkc;  // 64-wide k-slices
     const float4 *cinfo;  // SCREEN: per column pair (||c||^2 x2, h' x2), padded to 256
     const float *hz;      // SCREEN: (max h', max z) over the centroids
@@ -347,10 +352,82 @@ __device__ __forceinline__ void screen_insert(ScreenRow &s, float L, int j) {
     }
 }
 
-// Centroid tiles [lo, hi) of point tile rt (every tile, or the tile's
-// groups' range in segmented mode; none past the last point tile there).
+constexpr int SCREEN_WORDS = 2 * TCAND + 2;  // a row's screen state
+
+// What the whole screen says of a row (a2 = 2 ||x~||, w2 = 2 W_row): decided,
+// its candidates listed for fp32 rescoring, or left to the fp32 scan.
+__device__ __forceinline__ void screen_decide(const TcParams &p, int64_t row, ScreenRow &sr, float a2, float w2) {
+    // The nearest centroid j* has s~_j* <= min s~ + 2 W_row (its own
+    // and the argmin's intervals), so it is a kept candidate unless the
+    // list overflowed (Lev inside the threshold).
+    const float thr = __fadd_ru(sr.umin, w2);
+    int ncert = 0;
+#pragma unroll
+    for (int t = 0; t < TCAND; ++t) ncert += (sr.L[t] <= thr) ? 1 : 0;
+    const bool overflow = !(sr.lev > thr);
+    int nk = ncert;
+    int kj[TCAND];
+#pragma unroll
+    for (int t = 0; t < TCAND; ++t) kj[t] = sr.J[t];
+    if (!overflow && ncert >= 2) {
+        // refine with each candidate's own interval [s~ - w, s~ + w],
+        // w = 2 ||x~|| h'_j + z_j (rounded outwards)
+        float lo[TCAND], umin = INFINITY;
+#pragma unroll
+        for (int t = 0; t < TCAND; ++t) {
+            lo[t] = INFINITY;
+            if (t < ncert) {
+                const int j = sr.J[t];
+                const float4 ci = __ldg(p.cinfo + (j >> 1));
+                const float2 cz = __ldg(p.cinfoz + (j >> 1));
+                const float w = __fmaf_ru(a2, (j & 1) ? ci.w : ci.z, (j & 1) ? cz.y : cz.x);
+                umin = fminf(umin, __fadd_ru(sr.L[t], w));
+                lo[t] = __fsub_rd(sr.L[t], w);
+            }
+        }
+        nk = 0;
+#pragma unroll
+        for (int t = 0; t < TCAND; ++t)
+            if (t < ncert && lo[t] <= umin) kj[nk++] = sr.J[t];
+    }
+    const int first = kj[0] < p.k ? kj[0] : 0;
+    p.assign[row] = first;
+    if (p.warm_row) {
+        // SKM_FLAG_WARM: a decided row keeps U = s~ + W_row >= s for
+        // its centroid; rows left to the fp32 passes keep none
+        int2 wr = make_int2(__float_as_int(INFINITY), -1);
+        if (!overflow && nk == 1) {
+            float Lj = INFINITY;
+#pragma unroll
+            for (int t = 0; t < TCAND; ++t)
+                if (sr.J[t] == kj[0]) Lj = fminf(Lj, sr.L[t]);
+            wr = make_int2(__float_as_int(__fadd_ru(Lj, 0.5f * w2)), kj[0]);
+        }
+        p.warm_row[row] = wr;
+    }
+    if (!overflow && nk == 1) {
+        // decided by the screen
+    } else if (!overflow && nk >= 2) {
+        int32_t *cr = p.cand + row * (TCAND + 1);
+#pragma unroll
+        for (int t = 0; t < TCAND; ++t) cr[t] = kj[t];
+        cr[TCAND] = nk;
+        p.resc_rows[atomicAdd(&p.counters[0], 1)] = (int32_t)row;
+    } else {
+        p.fall_rows[atomicAdd(&p.counters[1], 1)] = (int32_t)row;
+    }
+}
+
+// Centroid tiles [lo, hi) of work item rt: every tile of a point tile, with
+// ksplit > 1 a share of them, or in segmented mode the tile's groups' range
+// (none past the last point tile there).
 __device__ __forceinline__ void ct_range(const TcParams &p, int64_t rt, int &lo, int &hi) {
-    if (p.seg_ct0) {
+    if (p.ksplit > 1) {
+        const int per = (p.nct + p.ksplit - 1) / p.ksplit;
+        lo = (int)(rt % p.ksplit) * per;
+        hi = min(p.nct, lo + per);
+        if (lo >= hi) lo = hi = 0;
+    } else if (p.seg_ct0) {
         if (rt < p.nrt) {
             lo = p.seg_ct0[rt];
             hi = lo + p.seg_nct[rt];
@@ -440,7 +517,8 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
     // CTA b takes the point tiles b, b + grid, b + 2 grid, ...
     const int64_t g0 = (int64_t)blockIdx.x;
     const int64_t gstep = (int64_t)gridDim.x;
-    const int64_t ngroups = p.nrt;
+    const int64_t ngroups = p.nrt * p.ksplit;
+    auto tile_of = [&](int64_t g) { return MODE == MODE_SCREEN && p.ksplit > 1 ? g / p.ksplit : g; };
 
     // Job order (producer and MMA issuer walk it identically): stream s takes
     // the CTA's point-tile groups g0 + (s + NS i) gstep; the streams' jobs
@@ -507,7 +585,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                 int64_t gj;
                 int ct;
                 stream_take(js, sj, gj, ct);
-                const int64_t rt = gj;
+                const int64_t rt = tile_of(gj);
                 turn = (sj + 1) % NS;
                 int64_t arow0 = rt * BM;
                 if (PK) {  // A comes from the stream's scratch slot of this tile
@@ -820,7 +898,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
         uint32_t job = 0;  // jobs of this group so far (NS = 1: of the CTA)
         unsigned long long pf_alive = 0;  // PFRONT: survivors of this thread's rows
         for (int64_t g = g0 + grp * gstep; g < ngroups; g += NS * gstep) {
-            const int64_t rt = g;
+            const int64_t rt = tile_of(g);
             const int64_t row = rt * BM + rin;
             const bool valid = row < p.n;
             ScreenRow sr;
@@ -848,7 +926,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                 ce = p.seg_base[gi + 1];
             }
             int ct_lo, ct_hi;
-            ct_range(p, rt, ct_lo, ct_hi);
+            ct_range(p, g, ct_lo, ct_hi);
             int next_lo = 0;
             {
                 int nhi;
@@ -1282,64 +1360,17 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                     }
                 }
                 if (MODE == MODE_SCREEN) {
-                    // The nearest centroid j* has s~_j* <= min s~ + 2 W_row (its own
-                    // and the argmin's intervals), so it is a kept candidate unless the
-                    // list overflowed (Lev inside the threshold).
-                    const float thr = __fadd_ru(sr.umin, w2);
-                    int ncert = 0;
-#pragma unroll
-                    for (int t = 0; t < TCAND; ++t) ncert += (sr.L[t] <= thr) ? 1 : 0;
-                    const bool overflow = !(sr.lev > thr);
-                    int nk = ncert;
-                    int kj[TCAND];
-#pragma unroll
-                    for (int t = 0; t < TCAND; ++t) kj[t] = sr.J[t];
-                    if (!overflow && ncert >= 2) {
-                        // refine with each candidate's own interval [s~ - w, s~ + w],
-                        // w = 2 ||x~|| h'_j + z_j (rounded outwards)
-                        float lo[TCAND], umin = INFINITY;
+                    if (p.ksplit > 1) {
+                        uint32_t *o = p.part + (row * p.ksplit + g % p.ksplit) * SCREEN_WORDS;
 #pragma unroll
                         for (int t = 0; t < TCAND; ++t) {
-                            lo[t] = INFINITY;
-                            if (t < ncert) {
-                                const int j = sr.J[t];
-                                const float4 ci = __ldg(p.cinfo + (j >> 1));
-                                const float2 cz = __ldg(p.cinfoz + (j >> 1));
-                                const float w = __fmaf_ru(a2, (j & 1) ? ci.w : ci.z, (j & 1) ? cz.y : cz.x);
-                                umin = fminf(umin, __fadd_ru(sr.L[t], w));
-                                lo[t] = __fsub_rd(sr.L[t], w);
-                            }
+                            o[t] = __float_as_uint(sr.L[t]);
+                            o[TCAND + t] = (uint32_t)sr.J[t];
                         }
-                        nk = 0;
-#pragma unroll
-                        for (int t = 0; t < TCAND; ++t)
-                            if (t < ncert && lo[t] <= umin) kj[nk++] = sr.J[t];
-                    }
-                    const int first = kj[0] < p.k ? kj[0] : 0;
-                    p.assign[row] = first;
-                    if (p.warm_row) {
-                        // SKM_FLAG_WARM: a decided row keeps U = s~ + W_row >= s for
-                        // its centroid; rows left to the fp32 passes keep none
-                        int2 wr = make_int2(__float_as_int(INFINITY), -1);
-                        if (!overflow && nk == 1) {
-                            float Lj = INFINITY;
-#pragma unroll
-                            for (int t = 0; t < TCAND; ++t)
-                                if (sr.J[t] == kj[0]) Lj = fminf(Lj, sr.L[t]);
-                            wr = make_int2(__float_as_int(__fadd_ru(Lj, 0.5f * w2)), kj[0]);
-                        }
-                        p.warm_row[row] = wr;
-                    }
-                    if (!overflow && nk == 1) {
-                        // decided by the screen
-                    } else if (!overflow && nk >= 2) {
-                        int32_t *cr = p.cand + row * (TCAND + 1);
-#pragma unroll
-                        for (int t = 0; t < TCAND; ++t) cr[t] = kj[t];
-                        cr[TCAND] = nk;
-                        p.resc_rows[atomicAdd(&p.counters[0], 1)] = (int32_t)row;
+                        o[2 * TCAND] = __float_as_uint(sr.umin);
+                        o[2 * TCAND + 1] = __float_as_uint(sr.lev);
                     } else {
-                        p.fall_rows[atomicAdd(&p.counters[1], 1)] = (int32_t)row;
+                        screen_decide(p, row, sr, a2, w2);
                     }
                 } else if (MODE == MODE_SQ8) {
                     p.assign[row] = besti;
@@ -1476,6 +1507,18 @@ __global__ void screen_prep_sq8_kernel(const uint8_t *__restrict__ X, int64_t n,
     }
 }
 
+// ||c||^2, h' and z (see below) from the fp64 sums of c^2 and (c~ - c)^2
+__device__ __forceinline__ void prep_bounds(double c2, double e2, double rho, float eps_acc, float eps_s, float &c2f,
+                                            float &hf, float &zf) {
+    const double up = 1.0 + 1e-6;
+    const double cn = sqrt(c2) * up, e = sqrt(e2) * up;
+    const double g = (cn + e) * up;
+    const double h = (e + ((double)eps_acc + (double)eps_s) * g + rho * cn) * up;
+    c2f = __double2float_rn(c2);
+    hf = __double2float_ru(h);
+    zf = __double2float_ru((double)eps_s * c2 * up);
+}
+
 // Centroids (fp32) -> bf16 operand + (||c||^2, h', z, 0) with
 // h' = e + (eps_acc + eps_s) (||c|| + e) + rho_max ||c||, e = ||c~ - c||,
 // z = eps_s ||c||^2, where rho_max >= ||x~ - x|| / ||x~|| over all points, so
@@ -1486,7 +1529,7 @@ __global__ void screen_prep_sq8_kernel(const uint8_t *__restrict__ X, int64_t n,
 // column pair p = (2p, 2p+1) -> cinfo[p] = (||c||^2 x2, h' x2), cinfoz[p] = (z x2);
 // hz_bits (zeroed by the caller) receives max h' and max z over j < k.
 //
-// SKM_FLAG_WARM (cprev non-NULL): also shift[j] = (||c_j||^2 - ||cprev_j||^2,
+// For SKM_FLAG_WARM (cprep_cold_kernel is the form without): also shift[j] = (||c_j||^2 - ||cprev_j||^2,
 // ||c_j - cprev_j||), each rounded up (fp64 sums of products of fp32 values,
 // plus a margin far above their rounding), then cprev_j = c_j; thread 0
 // publishes in *warm_ok whether the stamp names this n, d and k (the bounds
@@ -1503,7 +1546,7 @@ __global__ void cprep_f32_kernel(const float *__restrict__ C, int k, int kp, int
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     const double rho = (double)*rho_max;
-    if (cprev && blockIdx.x == 0 && threadIdx.x == 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         // cgen (the pruning front): cprev's generation, which the stamp must
         // name too (bounds taken against exactly these previous centroids)
         const int64_t g = cgen ? *cgen : 0;
@@ -1525,8 +1568,7 @@ __global__ void cprep_f32_kernel(const float *__restrict__ C, int k, int kp, int
             continue;
         }
         double c2 = 0.0, e2 = 0.0, p2 = 0.0, dd = 0.0, dn = 0.0;
-        const int iend = cprev ? d : dr;
-        for (int i = lane; i < iend; i += 32) {
+        for (int i = lane; i < d; i += 32) {
             const float c = C[(int64_t)j * d + i];
             if (i < dr) {
                 const __nv_bfloat16 cb = __float2bfloat16_rn(c);
@@ -1535,36 +1577,120 @@ __global__ void cprep_f32_kernel(const float *__restrict__ C, int k, int kp, int
                 c2 += (double)c * (double)c;
                 e2 += (cf - (double)c) * (cf - (double)c);
             }
-            if (cprev) {
-                const double cq = (double)cprev[(int64_t)j * d + i];
-                p2 += cq * cq;
-                dd += ((double)c - cq) * ((double)c - cq);
-                dn += ((double)c - cq) * ((double)c + cq);
-                cprev[(int64_t)j * d + i] = c;
-            }
+            const double cq = (double)cprev[(int64_t)j * d + i];
+            p2 += cq * cq;
+            dd += ((double)c - cq) * ((double)c - cq);
+            dn += ((double)c - cq) * ((double)c + cq);
+            cprev[(int64_t)j * d + i] = c;
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             c2 += __shfl_xor_sync(0xffffffffu, c2, o);
             e2 += __shfl_xor_sync(0xffffffffu, e2, o);
-            if (cprev) {
-                p2 += __shfl_xor_sync(0xffffffffu, p2, o);
-                dd += __shfl_xor_sync(0xffffffffu, dd, o);
-                dn += __shfl_xor_sync(0xffffffffu, dn, o);
-            }
+            p2 += __shfl_xor_sync(0xffffffffu, p2, o);
+            dd += __shfl_xor_sync(0xffffffffu, dd, o);
+            dn += __shfl_xor_sync(0xffffffffu, dn, o);
         }
-        if (cprev && lane == 0) {
+        if (lane == 0) {
             const double margin = 1e-12 * (c2 + p2);
             shift[j] = make_float2(__double2float_ru(dn + margin), __double2float_ru(sqrt(dd + margin) * (1.0 + 1e-12)));
         }
         if (lane == 0) {
-            const double up = 1.0 + 1e-6;
-            const double cn = sqrt(c2) * up, e = sqrt(e2) * up;
-            const double g = (cn + e) * up;
-            const double h = (e + ((double)eps_acc + (double)eps_s) * g + rho * cn) * up;
-            const double z = (double)eps_s * c2 * up;
-            cf[4 * pp + o] = __double2float_rn(c2);
-            const float hf = __double2float_ru(h), zf1 = __double2float_ru(z);
+            float c2f, hf, zf1;
+            prep_bounds(c2, e2, rho, eps_acc, eps_s, c2f, hf, zf1);
+            cf[4 * pp + o] = c2f;
+            cf[4 * pp + 2 + o] = hf;
+            zf[2 * pp + o] = zf1;
+            // maxima over the centroids (non-negative: bits order like values)
+            atomicMax(hz_bits, __float_as_uint(hf));
+            atomicMax(hz_bits + 1, __float_as_uint(zf1));
+        }
+    }
+}
+
+// The same records for calls that keep no bounds, in fp32: GB300 issues two fp64
+// lanes a clock and SM, and this kernel's few fp64 operations a value were its
+// time (1000 x 768: 16.6 us).  ||c||^2 is a double-float sum (error-free products
+// and TwoSums, about 2^-45 relative) rounded once; e and the bounds are rounded
+// upwards throughout, the fp32 sum of e^2 scaled up by its error bound first.
+// A centroid whose ||c||^2 leaves [2^-40, 2^100], where squares could
+// underflow unseen by the bounds or overflow, is done in fp64 as above.
+__device__ __forceinline__ void two_sum(float &hi, float &lo, float v) {
+    const float s = __fadd_rn(hi, v), bb = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(v, bb)));
+    hi = s;
+}
+__global__ void cprep_cold_kernel(const float *__restrict__ C, int k, int kp, int d, int dp, int dr, float eps_acc,
+                                  float eps_s, const float *__restrict__ rho_max, __nv_bfloat16 *__restrict__ cs,
+                                  float4 *__restrict__ cinfo, float2 *__restrict__ cinfoz,
+                                  unsigned int *__restrict__ hz_bits) {
+    const int lane = threadIdx.x & 31;
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nw = (gridDim.x * blockDim.x) >> 5;
+    const float rho = *rho_max;
+    float *cf = reinterpret_cast<float *>(cinfo);
+    float *zf = reinterpret_cast<float *>(cinfoz);
+    for (int j = warp; j < kp; j += nw) {
+        const int pp = j >> 1, o = j & 1;
+        if (j >= k) {
+            if (lane == 0) {
+                cf[4 * pp + o] = INFINITY;
+                cf[4 * pp + 2 + o] = 0.0f;
+                zf[2 * pp + o] = 0.0f;
+            }
+            continue;
+        }
+        const float *src = C + (int64_t)j * d;
+        float hi = 0.0f, lo = 0.0f, e2 = 0.0f;
+        for (int i0 = lane; i0 - lane < dr; i0 += 32 * PREP_UNROLL) {
+            float v[PREP_UNROLL];
+#pragma unroll
+            for (int u = 0; u < PREP_UNROLL; ++u) v[u] = i0 + 32 * u < dr ? __ldg(src + i0 + 32 * u) : 0.0f;
+#pragma unroll
+            for (int u = 0; u < PREP_UNROLL; ++u) {
+                const int i = i0 + 32 * u;
+                if (i >= dr) continue;
+                const __nv_bfloat16 cb = __float2bfloat16_rn(v[u]);
+                cs[(int64_t)j * dp + i] = cb;
+                const float e = __fsub_rn(__bfloat162float(cb), v[u]);
+                e2 = __fmaf_rn(e, e, e2);
+                const float p = __fmul_rn(v[u], v[u]);
+                lo = __fadd_rn(lo, __fmaf_rn(v[u], v[u], -p));
+                two_sum(hi, lo, p);
+            }
+        }
+#pragma unroll
+        for (int w = 16; w > 0; w >>= 1) {
+            e2 = __fadd_rn(e2, __shfl_xor_sync(0xffffffffu, e2, w));
+            const float h2 = __shfl_xor_sync(0xffffffffu, hi, w), l2 = __shfl_xor_sync(0xffffffffu, lo, w);
+            two_sum(hi, lo, h2);
+            lo = __fadd_rn(lo, l2);
+        }
+        float c2 = __fadd_rn(hi, lo), hf, zf1;
+        c2 = __shfl_sync(0xffffffffu, c2, 0);  // (one value decides the path for the warp)
+        const float up = 1.0f + 1e-6f;
+        if (c2 >= 0x1p-40f && c2 <= 0x1p100f) {
+            const float c2u = __fmul_ru(c2, up);
+            const float cn = __fsqrt_ru(c2u), e = sumsq_upper_norm(e2, (dr + 31) / 32 + 5);
+            const float g = __fadd_ru(cn, e);
+            hf = __fmul_ru(__fmaf_ru(rho, cn, __fmaf_ru(__fadd_ru(eps_acc, eps_s), g, e)), up);
+            zf1 = __fmul_ru(__fmul_ru(eps_s, c2u), up);
+        } else {
+            double c2d = 0.0, e2d = 0.0;
+            for (int i = lane; i < dr; i += 32) {
+                const double c = (double)src[i], t = (double)__bfloat162float(__float2bfloat16_rn(src[i])) - c;
+                c2d += c * c;
+                e2d += t * t;
+            }
+#pragma unroll
+            for (int w = 16; w > 0; w >>= 1) {
+                c2d += __shfl_xor_sync(0xffffffffu, c2d, w);
+                e2d += __shfl_xor_sync(0xffffffffu, e2d, w);
+            }
+            prep_bounds(c2d, e2d, (double)rho, eps_acc, eps_s, c2, hf, zf1);
+        }
+        if (lane == 0) {
+            cf[4 * pp + o] = c2;
             cf[4 * pp + 2 + o] = hf;
             zf[2 * pp + o] = zf1;
             // maxima over the centroids (non-negative: bits order like values)
@@ -1748,6 +1874,25 @@ __global__ void screen_prep_rbq1_kernel(const uint32_t *__restrict__ codes, int6
     }
 }
 
+// ksplit > 1: the shares' states of a row merged in centroid order, then the
+// decision the epilogue takes otherwise.
+__global__ void screen_merge_kernel(const TcParams p) {
+    const int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (row >= p.n || p.counters[2]) return;  // (a share that gave up left no states)
+    ScreenRow sr;
+    screen_init(sr);
+    const float a2 = 2.0f * p.xinfo[row].x;
+    const float w2 = 2.0f * __fmaf_ru(a2, __ldg(p.hz), __ldg(p.hz + 1));
+    for (int h = 0; h < p.ksplit; ++h) {
+        const uint32_t *o = p.part + (row * p.ksplit + h) * SCREEN_WORDS;
+        sr.umin = fminf(sr.umin, __uint_as_float(o[2 * TCAND]));
+        sr.lev = fminf(sr.lev, __uint_as_float(o[2 * TCAND + 1]));
+#pragma unroll
+        for (int t = 0; t < TCAND; ++t) screen_insert(sr, __uint_as_float(o[t]), (int)o[TCAND + t]);
+    }
+    screen_decide(p, row, sr, a2, w2);
+}
+
 // ------------------------------------------------------------ fp32 rescoring
 template <typename TX>
 __device__ __forceinline__ float ldx(const TX *p);
@@ -1760,10 +1905,27 @@ __device__ __forceinline__ float ldx<uint16_t>(const uint16_t *p) {
     return __uint_as_float(((uint32_t)__ldg(p)) << 16);
 }
 
+// Lane l sums the dimensions l, l + 32, ... in order; the loads of eight of
+// them are issued together (one at a time a row's latency was its length:
+// 2,000 rows of 768 20 us for their candidates and 13 for their distances).
 template <typename TX>
 __device__ __forceinline__ float warp_sqdist(const TX *x, const float *c, int d, int lane) {
+    constexpr int U = 8;
     float s = 0.0f;
-    for (int i = lane; i < d; i += 32) {
+    int i = lane;
+    for (; i + 32 * (U - 1) < d; i += 32 * U) {
+        float a[U], b[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) a[u] = ldx<TX>(x + i + 32 * u);
+#pragma unroll
+        for (int u = 0; u < U; ++u) b[u] = __ldg(c + i + 32 * u);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const float t = __fsub_rn(a[u], b[u]);
+            s = __fmaf_rn(t, t, s);
+        }
+    }
+    for (; i < d; i += 32) {
         const float t = __fsub_rn(ldx<TX>(x + i), __ldg(c + i));
         s = __fmaf_rn(t, t, s);
     }
@@ -1781,7 +1943,16 @@ template <typename TX>
 __global__ void rescore_kernel(const TX *__restrict__ X, int d, const float *__restrict__ C,
                                const int32_t *__restrict__ rows, const int32_t *__restrict__ count,
                                const int32_t *__restrict__ cand, int32_t *__restrict__ assign,
-                               int64_t *__restrict__ warm_hdr, int64_t n, int k, int64_t *__restrict__ stats) {
+                               int64_t *__restrict__ warm_hdr, int64_t n, int k, int64_t *__restrict__ stats,
+                               const int32_t *__restrict__ fall_rows, unsigned long long *__restrict__ fall_keys,
+                               int32_t *__restrict__ fall_tickets) {
+    // the fallback scan's keys and tickets (launch_assign_exact_rows)
+    if (fall_keys)
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count[1];
+             i += (int64_t)gridDim.x * blockDim.x) {
+            fall_keys[i] = ~0ull;
+            if ((i & 63) == 0) fall_tickets[(int64_t)fall_rows[i] * (TCAND + 1)] = 0;
+        }
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1943,7 +2114,7 @@ int launch_tc_kind(const void *xs, int64_t n, int dp, int d, const void *cs, int
     CUtensorMap ma, mb;
     const int eb = f8_mode<MODE>() ? 1 : 2;
     // PK: the A slices come from the CTAs' expansion scratch
-    int grid = (int)std::min<int64_t>(device_sms(), cdiv(n, BM));
+    int grid = (int)std::min<int64_t>(device_sms(), cdiv(n, BM) * std::max(1, p0.ksplit));
     if (PK) {
         grid = std::min(grid, PK_MAX_CTAS);
         SKM_TRY(make_map(&ma, p0.pk_scratch, (int64_t)grid * NS * 2 * BM, d, dp, BM, eb));
@@ -1956,6 +2127,7 @@ int launch_tc_kind(const void *xs, int64_t n, int dp, int d, const void *cs, int
     p.nrt = cdiv(n, BM);
     p.k = k;
     p.nct = (int)cdiv(k, BN);
+    p.ksplit = std::max(1, p0.ksplit);
     p.nkc = (int)cdiv(d, 128 / eb);
     p.inject_wait_ns = fault_take(SKM_FAULT_WAIT) ? 1000000ull : 0ull;  // 1 ms
     tc_timer_mark(st, 0);
@@ -2111,6 +2283,24 @@ int tc_screen_prep(const skm_data *x, void *screen, cudaStream_t st) {
 
 bool tc_reads_packed(int repr, int d, const void *x) {
     return (repr == SKM_REPR_RBQ1 && rbq1_packed(d, x)) || (repr == SKM_REPR_LVQ4 && lvq4_packed(d, x));
+}
+
+// Few points against many centroids: a point tile's centroid tiles shared out
+// to as many CTAs as the GPU has room for, at most one tile each.  (2,000 rows x
+// 768 against 1,000: 16 CTAs of 4 tiles each, one after another, take 35 us.)
+constexpr int SPLIT_SMS = 152;
+static int screen_split(int64_t n, int k) {
+    const int64_t nct = cdiv(k, BN), most = std::min<int64_t>(nct, SPLIT_SMS / cdiv(n, BM));
+    return most < 2 ? 1 : (int)cdiv(nct, cdiv(nct, most));  // no share empty
+}
+
+void tc_plan_split(int repr, int64_t n, int k, Carver &cv, TcAssignBufs &b) {
+    if ((repr != SKM_REPR_F32 && repr != SKM_REPR_BF16) || screen_split(n, k) < 2) return;
+    Carver t = cv;
+    uint32_t *part = t.take<uint32_t>((size_t)n * screen_split(n, k) * SCREEN_WORDS);
+    if (cv.base && !t.fits()) return;
+    cv = t;
+    b.scr_part = part;
 }
 
 // 1-bit / LVQ4: the expansion slots (pk: read packed, two per job stream), the
@@ -2276,12 +2466,16 @@ int tc_assign_pfront(const skm_data *x, const float *C, int k, const int32_t *pr
         const float eps_acc = (float)(((F / BK) * (BK / 16) + 4) * 0x1p-18);
         const float eps_s = 0x1p-21f;
         // bf16 points are their own operand: no residual term (counters[7] = 0.0f)
-        cprep_f32_kernel<<<grid_warps(kp), 256, 0, st>>>(C, k, kp, d, F, F, eps_acc, eps_s,
-                                                         reinterpret_cast<const float *>(b.counters + 7),
-                                                         (__nv_bfloat16 *)b.pf_cs0, b.pf_cinfo0, b.cinfoz,
-                                                         reinterpret_cast<unsigned int *>(b.counters + 4),
-                                                         warm ? b.pf_cprev : nullptr, b.pf_shift, b.pf_whdr, n,
-                                                         b.counters + 6, warm ? b.pf_cgen : nullptr);
+        const float *rho = reinterpret_cast<const float *>(b.counters + 7);
+        unsigned int *hz = reinterpret_cast<unsigned int *>(b.counters + 4);
+        if (warm)
+            cprep_f32_kernel<<<grid_warps(kp), 256, 0, st>>>(C, k, kp, d, F, F, eps_acc, eps_s, rho,
+                                                             (__nv_bfloat16 *)b.pf_cs0, b.pf_cinfo0, b.cinfoz, hz,
+                                                             b.pf_cprev, b.pf_shift, b.pf_whdr, n, b.counters + 6,
+                                                             b.pf_cgen);
+        else
+            cprep_cold_kernel<<<grid_warps(kp), 256, 0, st>>>(C, k, kp, d, F, F, eps_acc, eps_s, rho,
+                                                              (__nv_bfloat16 *)b.pf_cs0, b.pf_cinfo0, b.cinfoz, hz);
         SKM_CUDA_TRY(launched());
         // columns sorted by ||c_F||^2 (a chunk's columns then share a tight bound)
         pf_sort_kernel<<<1, 1024, 0, st>>>(b.pf_cinfo0, k, kp, b.pf_perm);
@@ -2372,11 +2566,14 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
     SKM_CUDA_TRY(cudaMemsetAsync(b.counters, 0, sizeof(int32_t) * 8, st));
     // SKM_FLAG_WARM (not in segmented calls): bounds carried between calls
     const bool warm = !seg && (x->flags & SKM_FLAG_WARM) && b.warm_hdr;
-    cprep_f32_kernel<<<grid_warps(kp), 256, 0, st>>>(C, k, kp, d, dp, d, eps_acc, eps_s, v.rho_max,
-                                                     (__nv_bfloat16 *)b.cs, b.cinfo, b.cinfoz,
-                                                     reinterpret_cast<unsigned int *>(b.counters + 4),
-                                                     warm ? b.warm_cprev : nullptr, b.warm_shift, b.warm_hdr, n,
-                                                     b.counters + 6, nullptr);
+    unsigned int *hz = reinterpret_cast<unsigned int *>(b.counters + 4);
+    if (warm)
+        cprep_f32_kernel<<<grid_warps(kp), 256, 0, st>>>(C, k, kp, d, dp, d, eps_acc, eps_s, v.rho_max,
+                                                         (__nv_bfloat16 *)b.cs, b.cinfo, b.cinfoz, hz, b.warm_cprev,
+                                                         b.warm_shift, b.warm_hdr, n, b.counters + 6, nullptr);
+    else
+        cprep_cold_kernel<<<grid_warps(kp), 256, 0, st>>>(C, k, kp, d, dp, d, eps_acc, eps_s, v.rho_max,
+                                                          (__nv_bfloat16 *)b.cs, b.cinfo, b.cinfoz, hz);
     SKM_CUDA_TRY(launched());
     TcParams p{};
     p.cinfo = b.cinfo;
@@ -2394,13 +2591,23 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
         p.warm_ok = b.counters + 6;
     }
     SKM_TRY(seg_setup(seg, n, p, st));
+    if (!seg && b.scr_part) {
+        p.ksplit = screen_split(n, k);
+        p.part = b.scr_part;
+    }
     SKM_TRY(launch_tc<MODE_SCREEN>(v.xs, n, dp, d, b.cs, k, p, st));
+    if (p.ksplit > 1) {
+        p.n = n;
+        p.k = k;
+        screen_merge_kernel<<<(unsigned)cdiv(n, 64), 64, 0, st>>>(p);
+        SKM_CUDA_TRY(launched());
+    }
     int64_t *hdr = warm ? b.warm_hdr : nullptr;
     const int gw = grid_warps(n);
     if (bf16) {
         const uint16_t *X = static_cast<const uint16_t *>(x->x);
         rescore_kernel<uint16_t><<<gw, 256, 0, st>>>(X, d, C, b.resc_rows, b.counters, b.cand, assign, hdr, n, k,
-                                                   b.stats);
+                                                   b.stats, b.fall_rows, seg ? nullptr : b.fall_keys, b.cand);
         SKM_CUDA_TRY(launched());
         if (seg) {
             seg_rows_exact_kernel<uint16_t><<<gw, 256, 0, st>>>(X, d, C, b.fall_rows, b.counters + 1, seg->group,
@@ -2408,7 +2615,7 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
             SKM_CUDA_TRY(launched());
         } else {
             SKM_CUDA_TRY(launch_assign_exact_rows(X, 1, b.fall_rows, b.counters + 1, n, d, C, k, assign,
-                                                  nullptr, b.fall_keys, st));
+                                                  nullptr, b.fall_keys, b.cand, TCAND + 1, st));
         }
         if (dist) {
             assigned_dist_kernel<uint16_t><<<gw, 256, 0, st>>>(X, n, d, C, assign, dist);
@@ -2417,7 +2624,7 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
     } else {
         const float *X = static_cast<const float *>(x->x);
         rescore_kernel<float><<<gw, 256, 0, st>>>(X, d, C, b.resc_rows, b.counters, b.cand, assign, hdr, n, k,
-                                                   b.stats);
+                                                   b.stats, b.fall_rows, seg ? nullptr : b.fall_keys, b.cand);
         SKM_CUDA_TRY(launched());
         if (seg) {
             seg_rows_exact_kernel<float><<<gw, 256, 0, st>>>(X, d, C, b.fall_rows, b.counters + 1, seg->group,
@@ -2425,7 +2632,7 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
             SKM_CUDA_TRY(launched());
         } else {
             SKM_CUDA_TRY(launch_assign_exact_rows(X, 0, b.fall_rows, b.counters + 1, n, d, C, k, assign,
-                                                  nullptr, b.fall_keys, st));
+                                                  nullptr, b.fall_keys, b.cand, TCAND + 1, st));
         }
         if (dist) {
             assigned_dist_kernel<float><<<gw, 256, 0, st>>>(X, n, d, C, assign, dist);

@@ -205,6 +205,14 @@ static void plan_assign(const skm_data *x, int k, Carver &cv, AssignBufs &b) {
     tc_plan(x->repr, n, d, k, x->x, x->screen, (x->flags & SKM_FLAG_WARM) != 0, cv, b.tc);
 }
 
+// Buffers that only make an assignment faster, at the end of its workspace: a
+// workspace that ends before them does without.
+static void plan_assign_extra(const skm_data *x, int k, Carver &cv, TcAssignBufs &b) {
+    if (use_prune(x)) return;
+    tc_plan_wide(x->repr, x->n, x->d, k, cv, b);
+    tc_plan_split(x->repr, x->n, k, cv, b);
+}
+
 struct UpdateBufs {
     int32_t *counts32 = nullptr, *cursor = nullptr, *perm = nullptr, *scl = nullptr;
     int64_t *offsets = nullptr;
@@ -301,7 +309,7 @@ static void plan_fit(const skm_data *x, int k, Carver &cv, FitBufs &b) {
     b.counts = cv.take<int64_t>(k);
     b.init_idx = cv.take<int64_t>(k);  // seeded Forgy indices (host-drawn)
     b.empty_iter = cv.take<int64_t>(EMPTY_LOG);
-    if (!use_prune(x)) tc_plan_wide(x->repr, x->n, x->d, k, cv, b.a.tc);
+    plan_assign_extra(x, k, cv, b.a.tc);
 }
 
 static int need_ws(const Carver &cv, size_t ws_bytes, void *ws) {
@@ -502,7 +510,7 @@ size_t skm_workspace_size(int op, const skm_data *x, int k) {
         if (check_data(x, false) || check_k(x, k)) return 0;
         AssignBufs b;
         plan_assign(x, k, cv, b);
-        if (!use_prune(x)) tc_plan_wide(x->repr, x->n, x->d, k, cv, b.tc);
+        plan_assign_extra(x, k, cv, b.tc);
         break;
     }
     case 1: {
@@ -832,7 +840,7 @@ int skm_assign(const skm_data *x, const void *C, int k, const int32_t *prev_assi
     Carver cv(ws, ws_bytes);
     AssignBufs b;
     plan_assign(x, k, cv, b);
-    if (!use_prune(x)) tc_plan_wide(x->repr, x->n, x->d, k, cv, b.tc);
+    plan_assign_extra(x, k, cv, b.tc);
     SKM_TRY(need_ws(cv, ws_bytes, ws));
     if (use_prune(x))
         SKM_CUDA_TRY(cudaMemsetAsync(b.prune, 0, PRUNE_CTRS * sizeof(unsigned long long), S(stream)));

@@ -42,6 +42,7 @@ struct TcAssignBufs {
     float4 *rpair_bs = nullptr;   // RBQ1 / LVQ4: column-pair records (padded)
     float4 *rpair_qn = nullptr;
     int32_t *cand = nullptr;      // F32/BF16: [n][5] screen candidates + count
+    uint32_t *scr_part = nullptr;  // F32/BF16, few points: the centroid shares' row states
     int32_t *resc_rows = nullptr;
     int32_t *fall_rows = nullptr;
     unsigned long long *fall_keys = nullptr;  // F32/BF16: per fallback row, (dist bits, index)
@@ -92,6 +93,9 @@ void tc_plan(int repr, int64_t n, int d, int k, const void *x, const void *scree
 // CUDA-core kernel runs) when a given workspace ends before them.
 bool tc_wide_ok(int repr, int d);
 void tc_plan_wide(int repr, int64_t n, int d, int k, Carver &cv, TcAssignBufs &b);
+// F32 / BF16 screens of few points: the buffer that lets several CTAs share a
+// point tile's centroids, likewise last and likewise left out when it does not fit.
+void tc_plan_split(int repr, int64_t n, int k, Carver &cv, TcAssignBufs &b);
 int tc_init_stats(TcAssignBufs &b, cudaStream_t st);
 // Exact dimension pruning of bf16 points with the first dimensions on tensor
 // cores (used when a seed assignment is given): whether these points can take
