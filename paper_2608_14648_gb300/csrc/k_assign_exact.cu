@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(256) assign_exact_kernel(const TX *__restrict_
                                                            float *__restrict__ dist,
                                                            unsigned long long *__restrict__ keys,
                                                            int32_t *__restrict__ tickets, int tstride) {
+    dep_sync();
     __shared__ bool last_item;
     __shared__ __align__(16) float xs[32][68];
     __shared__ __align__(16) float cs[32][68];
@@ -194,7 +195,7 @@ static unsigned blocks_for_rows(int64_t nrows) {
 cudaError_t launch_assign_exact_f32(const float *X, int64_t n, int d, const float *C, int k,
                                     int32_t *assign, float *dist, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    assign_exact_kernel<float><<<blocks_for_rows(n), 256, 0, st>>>(X, nullptr, nullptr, n, d, C,
+    launch_dep(assign_exact_kernel<float>, blocks_for_rows(n), 256, 0, st, X, nullptr, nullptr, n, d, C,
                                                                    k, assign, dist, nullptr, nullptr, 0);
     return launched();
 }
@@ -202,7 +203,7 @@ cudaError_t launch_assign_exact_f32(const float *X, int64_t n, int d, const floa
 cudaError_t launch_assign_exact_bf16(const uint16_t *X, int64_t n, int d, const float *C, int k,
                                      int32_t *assign, float *dist, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    assign_exact_kernel<uint16_t><<<blocks_for_rows(n), 256, 0, st>>>(X, nullptr, nullptr, n, d,
+    launch_dep(assign_exact_kernel<uint16_t>, blocks_for_rows(n), 256, 0, st, X, nullptr, nullptr, n, d,
                                                                       C, k, assign, dist, nullptr, nullptr, 0);
     return launched();
 }
@@ -215,11 +216,11 @@ cudaError_t launch_assign_exact_rows(const void *X, int x_is_bf16, const int32_t
     // enough blocks to split the centroids when only a few rows are listed
     const unsigned g = keys ? 152u * 4u : blocks_for_rows(max_rows);
     if (x_is_bf16)
-        assign_exact_kernel<uint16_t><<<g, 256, 0, st>>>(static_cast<const uint16_t *>(X), rows,
+        launch_dep(assign_exact_kernel<uint16_t>, g, 256, 0, st, static_cast<const uint16_t *>(X), rows,
                                                          count_dev, 0, d, C, k, assign, dist, keys, tickets,
                                                          tstride);
     else
-        assign_exact_kernel<float><<<g, 256, 0, st>>>(static_cast<const float *>(X), rows,
+        launch_dep(assign_exact_kernel<float>, g, 256, 0, st, static_cast<const float *>(X), rows,
                                                       count_dev, 0, d, C, k, assign, dist, keys, tickets,
                                                       tstride);
     return launched();

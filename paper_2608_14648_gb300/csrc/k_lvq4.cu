@@ -270,6 +270,7 @@ __global__ void lvq4_exponent_kernel(const unsigned int *__restrict__ maxbits, i
 // column pairs.
 __global__ void lvq4_cprep_kernel(const float *__restrict__ C, int k, int d, uint8_t *__restrict__ yq, int dq,
                                   uint32_t *__restrict__ yw, float4 *__restrict__ info, const CodePairs pairs) {
+    dep_sync();
     const int lane = threadIdx.x & 31;
     const int j = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     if (pairs.counters && blockIdx.x == 0 && threadIdx.x < 4) pairs.counters[threadIdx.x] = 0;
@@ -387,6 +388,7 @@ __global__ void __launch_bounds__(256) assign_lvq4_simt_kernel(const uint32_t *_
 // c_i = (T_i + U) f, f = 2^-e / count formed once per cluster (one block each).
 __global__ void finalize_lvq4_kernel(const int64_t *__restrict__ partial, const int64_t *__restrict__ counts, int k,
                                      int d, int e, float *__restrict__ C) {
+    dep_sync();
     __shared__ double fs;
     const int j = blockIdx.x;
     const int64_t c = counts[j];
@@ -458,7 +460,7 @@ cudaError_t launch_lvq4_exponent(const float4 *fac, int64_t n, unsigned int *max
 cudaError_t launch_lvq4_cprep(const float *C, int k, int d, uint8_t *yq, int dq, uint32_t *yw, float4 *info,
                               const CodePairs &pairs, cudaStream_t st) {
     const int rows = k > pairs.kp ? k : pairs.kp;
-    lvq4_cprep_kernel<<<(rows + 7) / 8, 256, 0, st>>>(C, k, d, yq, dq, yw, info, pairs);
+    launch_dep(lvq4_cprep_kernel, (rows + 7) / 8, 256, 0, st, C, k, d, yq, dq, yw, info, pairs);
     return launched();
 }
 
@@ -484,7 +486,7 @@ cudaError_t launch_assign_lvq4_simt(const uint32_t *codes, const float4 *fac, in
 
 cudaError_t launch_finalize_lvq4(const int64_t *partial, const int64_t *counts, int k, int d, int e, float *C_inout,
                                  cudaStream_t st) {
-    finalize_lvq4_kernel<<<k, 256, 0, st>>>(partial, counts, k, d, e, C_inout);
+    launch_dep(finalize_lvq4_kernel, k, 256, 0, st, partial, counts, k, d, e, C_inout);
     return launched();
 }
 

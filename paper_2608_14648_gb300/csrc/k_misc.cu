@@ -142,6 +142,7 @@ cudaError_t launch_sum_double(const double *in, int64_t count, double *out, cuda
 __global__ void __launch_bounds__(256) sum_float_kernel(const float *__restrict__ in, int64_t count,
                                                         double *__restrict__ partials, unsigned int *__restrict__ ticket,
                                                         double *__restrict__ out) {
+    dep_sync();
     __shared__ bool last;
     double s = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
@@ -165,7 +166,7 @@ cudaError_t launch_sum_float(const float *in, int64_t count, double *partials, i
                              double *out, cudaStream_t st) {
     const int64_t want = (count + 1023) / 1024;
     const int blocks = (int)(want < nblk ? want : nblk);
-    sum_float_kernel<<<blocks, 256, 0, st>>>(in, count, partials, ticket, out);
+    launch_dep(sum_float_kernel, blocks, 256, 0, st, in, count, partials, ticket, out);
     return launched();
 }
 

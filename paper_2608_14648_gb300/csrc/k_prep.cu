@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(CPREP_WARPS * 32) rbq1_cprep_kernel(
     const float *__restrict__ C, int k, int d, const float *__restrict__ m,
     uint4 *__restrict__ planes, Rbq1CInfo *__restrict__ info, uint8_t *__restrict__ yq, int dq,
     float isd, const CodePairs pairs) {
+    dep_sync();
     extern __shared__ __align__(8) uint8_t sh_prep[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int W = (d + 31) >> 5;
@@ -155,7 +156,7 @@ static cudaError_t launch_cprep_common(const float *C, int k, int d, const float
         if (e != cudaSuccess) return e;
     }
     const int rows = k > pairs.kp ? k : pairs.kp;
-    rbq1_cprep_kernel<<<(rows + CPREP_WARPS - 1) / CPREP_WARPS, CPREP_WARPS * 32, smem, st>>>(
+    launch_dep(rbq1_cprep_kernel, (rows + CPREP_WARPS - 1) / CPREP_WARPS, CPREP_WARPS * 32, smem, st, 
         C, k, d, m, planes, info, yq, dq, rbq1_isd(d), pairs);
     return launched();
 }

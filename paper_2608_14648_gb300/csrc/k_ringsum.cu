@@ -26,6 +26,7 @@
 #include "skm_internal.cuh"
 
 namespace skm {
+
 namespace {
 
 constexpr int RS_CW = 8;                      // warps per CTA, one run each
@@ -313,6 +314,7 @@ __global__ void __launch_bounds__(RS_THREADS) ring_sum_float_kernel(
     const void *__restrict__ X, int d, const int32_t *__restrict__ perm,
     const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k, ACC *__restrict__ S,
     int64_t stride, RingLayout L, int32_t *flag) {
+    dep_sync();
     const int64_t nval = offsets[k];
     if ((int64_t)blockIdx.x * RS_CW * L.run >= nval) return;
     FloatCons<BF16, ACC, NF> cons;
@@ -392,6 +394,7 @@ __global__ void __launch_bounds__(TR_WARPS * 32, PF ? 2 : 3) rbq1_sum_table_kern
     const uint32_t *__restrict__ codes, int WT, const float *__restrict__ F, int e, int d,
     const int32_t *__restrict__ perm, const int32_t *__restrict__ scl,
     const int64_t *__restrict__ offsets, int k, unsigned long long *__restrict__ T, int run) {
+    dep_sync();
     constexpr int W = 4 * W4;
     const int w0 = W * blockIdx.y, nw = min(W, WT - w0);
     __shared__ __align__(1024) uint32_t tabs[TR_WARPS][256];  // 7 x 32 entries used per warp
@@ -612,6 +615,7 @@ __global__ void __launch_bounds__(RS_THREADS) ring_sum_sq8_kernel(
     const uint8_t *__restrict__ codes, int d, const int32_t *__restrict__ perm,
     const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k,
     unsigned long long *__restrict__ S, RingLayout L, int32_t *flag) {
+    dep_sync();
     const int64_t nval = offsets[k];
     if ((int64_t)blockIdx.x * RS_CW * L.run >= nval) return;
     Sq8Cons<NG> cons;
@@ -634,6 +638,7 @@ __global__ void __launch_bounds__(RS_THREADS) direct_sum_sq8_kernel(
     const uint8_t *__restrict__ codes, int d, const int32_t *__restrict__ perm,
     const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k,
     unsigned long long *__restrict__ S, int run) {
+    dep_sync();
     constexpr int PF = NG == 2 ? 3 : SQ8_PF;
     __shared__ int32_t sperm_all[RS_CW][RS_ROWS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -683,6 +688,7 @@ __global__ void __launch_bounds__(RS_THREADS) direct_sum_bf16_kernel(
     const uint16_t *__restrict__ X, int d, const int32_t *__restrict__ perm,
     const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k, ACC *__restrict__ S,
     int64_t stride, int run) {
+    dep_sync();
     __shared__ int32_t sperm_all[RS_CW][RS_ROWS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t nval = offsets[k];
@@ -900,6 +906,7 @@ __global__ void __launch_bounds__(RS_THREADS) direct_sum_lvq4_kernel(
     const uint32_t *__restrict__ codes, const float4 *__restrict__ fac, int e, int d,
     const int32_t *__restrict__ perm, const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k,
     unsigned long long *__restrict__ T, int run) {
+    dep_sync();
     __shared__ int32_t sperm_all[RS_CW][RS_ROWS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t nval = offsets[k];
@@ -985,7 +992,7 @@ cudaError_t launch_float_nf(int nf, const void *X, int64_t n, int d, const int32
         auto kern = ring_sum_float_kernel<BF16, ACC, NFV>;                                          \
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
         if (e != cudaSuccess) return e;                                                             \
-        kern<<<g, RS_THREADS, smem, st>>>(X, d, perm, scl, offsets, k, S, d, L, flag);               \
+        launch_dep(kern, g, RS_THREADS, smem, st, X, d, perm, scl, offsets, k, S, d, L, flag);               \
         return launched();                                                                          \
     }
     switch (nf) {
@@ -1019,11 +1026,11 @@ cudaError_t launch_ring_sum_float(const void *X, int x_is_bf16, int64_t n, int d
         const unsigned g = ring_blocks(n, run);
         const uint16_t *Xb = static_cast<const uint16_t *>(X);
         if (d <= 256) {
-            if (S_d) direct_sum_bf16_kernel<double, 1><<<g, RS_THREADS, 0, st>>>(Xb, d, perm, scl, offsets, k, S_d, d, run);
-            else direct_sum_bf16_kernel<float, 1><<<g, RS_THREADS, 0, st>>>(Xb, d, perm, scl, offsets, k, S_f, d, run);
+            if (S_d) launch_dep(direct_sum_bf16_kernel<double, 1>, g, RS_THREADS, 0, st, Xb, d, perm, scl, offsets, k, S_d, d, run);
+            else launch_dep(direct_sum_bf16_kernel<float, 1>, g, RS_THREADS, 0, st, Xb, d, perm, scl, offsets, k, S_f, d, run);
         } else {
-            if (S_d) direct_sum_bf16_kernel<double, 2><<<g, RS_THREADS, 0, st>>>(Xb, d, perm, scl, offsets, k, S_d, d, run);
-            else direct_sum_bf16_kernel<float, 2><<<g, RS_THREADS, 0, st>>>(Xb, d, perm, scl, offsets, k, S_f, d, run);
+            if (S_d) launch_dep(direct_sum_bf16_kernel<double, 2>, g, RS_THREADS, 0, st, Xb, d, perm, scl, offsets, k, S_d, d, run);
+            else launch_dep(direct_sum_bf16_kernel<float, 2>, g, RS_THREADS, 0, st, Xb, d, perm, scl, offsets, k, S_f, d, run);
         }
         return launched();
     }
@@ -1057,9 +1064,9 @@ cudaError_t launch_ring_sum_sq8(const uint8_t *codes, int64_t n, int d, const in
     const int q = (d / 16 + 31) / 32;  // 16-byte groups per lane
     if (d <= 1024) {  // rows of at most 1 KB: straight into registers
         if (q <= 1)
-            direct_sum_sq8_kernel<1><<<g, RS_THREADS, 0, st>>>(codes, d, perm, scl, offsets, k, S64, L.run);
+            launch_dep(direct_sum_sq8_kernel<1>, g, RS_THREADS, 0, st, codes, d, perm, scl, offsets, k, S64, L.run);
         else
-            direct_sum_sq8_kernel<2><<<g, RS_THREADS, 0, st>>>(codes, d, perm, scl, offsets, k, S64, L.run);
+            launch_dep(direct_sum_sq8_kernel<2>, g, RS_THREADS, 0, st, codes, d, perm, scl, offsets, k, S64, L.run);
         return launched();
     }
 #define RS_CASE(NGV)                                                                                \
@@ -1067,7 +1074,7 @@ cudaError_t launch_ring_sum_sq8(const uint8_t *codes, int64_t n, int d, const in
         auto kern = ring_sum_sq8_kernel<NGV>;                                                       \
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
         if (e != cudaSuccess) return e;                                                             \
-        kern<<<g, RS_THREADS, smem, st>>>(codes, d, perm, scl, offsets, k, S64, L, flag);            \
+        launch_dep(kern, g, RS_THREADS, smem, st, codes, d, perm, scl, offsets, k, S64, L, flag);            \
         return launched();                                                                          \
     }
     RS_CASE(1)
@@ -1128,7 +1135,7 @@ cudaError_t launch_sum_lvq4(const uint32_t *codes, const float4 *fac, int e, int
     const dim3 g(ring_blocks(n, run), (unsigned)((W + 127) / 128));
 #define RS_CASE(NWV)                                                                                           \
     case NWV:                                                                                                  \
-        direct_sum_lvq4_kernel<NWV><<<g, RS_THREADS, 0, st>>>(codes, fac, e, d, perm, scl, offsets, k, T64, run); \
+        launch_dep(direct_sum_lvq4_kernel<NWV>, g, RS_THREADS, 0, st, codes, fac, e, d, perm, scl, offsets, k, T64, run); \
         return launched();
     switch ((std::min(W, 128) + 31) / 32) {
         RS_CASE(1)

@@ -421,8 +421,9 @@ __device__ __forceinline__ void screen_decide(const TcParams &p, int64_t row, Sc
 // Centroid tiles [lo, hi) of work item rt: every tile of a point tile, with
 // ksplit > 1 a share of them, or in segmented mode the tile's groups' range
 // (none past the last point tile there).
+template <int MODE>
 __device__ __forceinline__ void ct_range(const TcParams &p, int64_t rt, int &lo, int &hi) {
-    if (p.ksplit > 1) {
+    if (MODE == MODE_SCREEN && p.ksplit > 1) {
         const int per = (p.nct + p.ksplit - 1) / p.ksplit;
         lo = (int)(rt % p.ksplit) * per;
         hi = min(p.nct, lo + per);
@@ -510,14 +511,16 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    dep_wait();  // the setup above reads nothing that an earlier kernel writes
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    dep_launch();  // after the allocation: the next such kernel cannot take the TMEM first
     const uint32_t tmem = *tmem_slot;
     // CTA b takes the point tiles b, b + grid, b + 2 grid, ...
     const int64_t g0 = (int64_t)blockIdx.x;
     const int64_t gstep = (int64_t)gridDim.x;
-    const int64_t ngroups = p.nrt * p.ksplit;
+    const int64_t ngroups = MODE == MODE_SCREEN ? p.nrt * p.ksplit : p.nrt;
     auto tile_of = [&](int64_t g) { return MODE == MODE_SCREEN && p.ksplit > 1 ? g / p.ksplit : g; };
 
     // Job order (producer and MMA issuer walk it identically): stream s takes
@@ -530,7 +533,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
     auto stream_seek = [&](JobStream &js) {  // the first job at or after group js.g
         while (js.g < ngroups) {
             int lo, hi;
-            ct_range(p, js.g, lo, hi);
+            ct_range<MODE>(p, js.g, lo, hi);
             if (lo < hi) {
                 js.ct = lo;
                 js.hi = hi;
@@ -889,7 +892,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
         };
         {
             int lo0, hi0;
-            ct_range(p, g0 + grp * gstep, lo0, hi0);
+            ct_range<MODE>(p, g0 + grp * gstep, lo0, hi0);
             rec_load(lo0);
         }
         // A warp whose barrier wait gave up stops computing but keeps taking part
@@ -926,11 +929,11 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                 ce = p.seg_base[gi + 1];
             }
             int ct_lo, ct_hi;
-            ct_range(p, g, ct_lo, ct_hi);
+            ct_range<MODE>(p, g, ct_lo, ct_hi);
             int next_lo = 0;
             {
                 int nhi;
-                ct_range(p, g + NS * gstep, next_lo, nhi);
+                ct_range<MODE>(p, g + NS * gstep, next_lo, nhi);
             }
             if (MODE == MODE_SCREEN) {
                 a2 = valid ? 2.0f * p.xinfo[row].x : 0.0f;
@@ -1542,6 +1545,7 @@ __global__ void cprep_f32_kernel(const float *__restrict__ C, int k, int kp, int
                                  float *__restrict__ cprev, float2 *__restrict__ shift,
                                  int64_t *__restrict__ warm_hdr, int64_t n, int32_t *__restrict__ warm_ok,
                                  int64_t *__restrict__ cgen) {
+    dep_sync();
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
@@ -1624,6 +1628,7 @@ __global__ void cprep_cold_kernel(const float *__restrict__ C, int k, int kp, in
                                   float eps_s, const float *__restrict__ rho_max, __nv_bfloat16 *__restrict__ cs,
                                   float4 *__restrict__ cinfo, float2 *__restrict__ cinfoz,
                                   unsigned int *__restrict__ hz_bits) {
+    dep_sync();
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
@@ -1709,6 +1714,7 @@ __global__ void cprep_cold_kernel(const float *__restrict__ C, int k, int kp, in
 constexpr int PF_NB = 4096;
 __global__ void __launch_bounds__(1024) pf_sort_kernel(const float4 *__restrict__ cinfo, int k, int kp,
                                                        int32_t *__restrict__ perm) {
+    dep_sync();
     __shared__ unsigned int cnt[PF_NB];
     __shared__ float red[2][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1791,6 +1797,7 @@ __global__ void __launch_bounds__(1024) pf_sort_kernel(const float4 *__restrict_
 __global__ void pf_gather_kernel(const uint16_t *__restrict__ cs0, const float4 *__restrict__ cinfo0, int k, int kp,
                                  int F, const int32_t *__restrict__ perm, uint16_t *__restrict__ cs,
                                  float4 *__restrict__ cinfo, float *__restrict__ cmin) {
+    dep_sync();
     const int lane = threadIdx.x & 31;
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1821,6 +1828,7 @@ __global__ void pf_gather_kernel(const uint16_t *__restrict__ cs0, const float4 
 __global__ void cprep_sq8_kernel(const uint8_t *__restrict__ C, int k, int kp, int d, int dp,
                                  __nv_bfloat16 *__restrict__ cs, int32_t *__restrict__ nc,
                                  int32_t *__restrict__ counters) {
+    dep_sync();
     if (blockIdx.x == 0 && threadIdx.x < 4) counters[threadIdx.x] = 0;
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1877,6 +1885,7 @@ __global__ void screen_prep_rbq1_kernel(const uint32_t *__restrict__ codes, int6
 // ksplit > 1: the shares' states of a row merged in centroid order, then the
 // decision the epilogue takes otherwise.
 __global__ void screen_merge_kernel(const TcParams p) {
+    dep_sync();
     const int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (row >= p.n || p.counters[2]) return;  // (a share that gave up left no states)
     ScreenRow sr;
@@ -1946,6 +1955,7 @@ __global__ void rescore_kernel(const TX *__restrict__ X, int d, const float *__r
                                int64_t *__restrict__ warm_hdr, int64_t n, int k, int64_t *__restrict__ stats,
                                const int32_t *__restrict__ fall_rows, unsigned long long *__restrict__ fall_keys,
                                int32_t *__restrict__ fall_tickets) {
+    dep_sync();
     // the fallback scan's keys and tickets (launch_assign_exact_rows)
     if (fall_keys)
         for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count[1];
@@ -1992,6 +2002,7 @@ template <typename TX>
 __global__ void assigned_dist_kernel(const TX *__restrict__ X, int64_t n, int d,
                                      const float *__restrict__ C, const int32_t *__restrict__ assign,
                                      float *__restrict__ dist) {
+    dep_sync();
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -2006,6 +2017,7 @@ __global__ void assigned_dist_kernel(const TX *__restrict__ X, int64_t n, int d,
 // (min and max group over the tile's rows, ids clamped into [0, nseg)).
 __global__ void seg_tiles_kernel(const int32_t *__restrict__ group, const int32_t *__restrict__ base, int nseg,
                                  int64_t n, int64_t nrt, int32_t *__restrict__ ct0, int32_t *__restrict__ nct) {
+    dep_sync();
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -2131,7 +2143,7 @@ int launch_tc_kind(const void *xs, int64_t n, int dp, int d, const void *cs, int
     p.nkc = (int)cdiv(d, 128 / eb);
     p.inject_wait_ns = fault_take(SKM_FAULT_WAIT) ? 1000000ull : 0ull;  // 1 ms
     tc_timer_mark(st, 0);
-    kern<<<grid, tc_threads<NH, PK>(), SMEM, st>>>(ma, mb, p);
+    launch_dep(kern, grid, tc_threads<NH, PK>(), SMEM, st, ma, mb, p);
     tc_timer_mark(st, 1);
     SKM_CUDA_TRY(launched());
     return SKM_OK;
@@ -2424,6 +2436,7 @@ void tc_plan_pfront(int64_t n, int d, int k, bool warm, Carver &cv, TcAssignBufs
 __global__ void pf_done_kernel(int64_t *__restrict__ hdr, const int32_t *__restrict__ counters,
                                unsigned long long *__restrict__ ctr, int64_t n, int d, int k,
                                const int64_t *__restrict__ cgen, int64_t *__restrict__ stats) {
+    dep_sync();
     stats[0] += counters[0];
     stats[1] += counters[1];
     stats[2] |= counters[2];
@@ -2469,18 +2482,18 @@ int tc_assign_pfront(const skm_data *x, const float *C, int k, const int32_t *pr
         const float *rho = reinterpret_cast<const float *>(b.counters + 7);
         unsigned int *hz = reinterpret_cast<unsigned int *>(b.counters + 4);
         if (warm)
-            cprep_f32_kernel<<<grid_warps(kp), 256, 0, st>>>(C, k, kp, d, F, F, eps_acc, eps_s, rho,
+            launch_dep(cprep_f32_kernel, grid_warps(kp), 256, 0, st, C, k, kp, d, F, F, eps_acc, eps_s, rho,
                                                              (__nv_bfloat16 *)b.pf_cs0, b.pf_cinfo0, b.cinfoz, hz,
                                                              b.pf_cprev, b.pf_shift, b.pf_whdr, n, b.counters + 6,
                                                              b.pf_cgen);
         else
-            cprep_cold_kernel<<<grid_warps(kp), 256, 0, st>>>(C, k, kp, d, F, F, eps_acc, eps_s, rho,
+            launch_dep(cprep_cold_kernel, grid_warps(kp), 256, 0, st, C, k, kp, d, F, F, eps_acc, eps_s, rho,
                                                               (__nv_bfloat16 *)b.pf_cs0, b.pf_cinfo0, b.cinfoz, hz);
         SKM_CUDA_TRY(launched());
         // columns sorted by ||c_F||^2 (a chunk's columns then share a tight bound)
-        pf_sort_kernel<<<1, 1024, 0, st>>>(b.pf_cinfo0, k, kp, b.pf_perm);
+        launch_dep(pf_sort_kernel, 1, 1024, 0, st, b.pf_cinfo0, k, kp, b.pf_perm);
         SKM_CUDA_TRY(launched());
-        pf_gather_kernel<<<std::max(1, std::min(kp / 32 / 8, 152 * 8)), 256, 0, st>>>(b.pf_cs0, b.pf_cinfo0, k, kp, F,
+        launch_dep(pf_gather_kernel, std::max(1, std::min(kp / 32 / 8, 152 * 8)), 256, 0, st, b.pf_cs0, b.pf_cinfo0, k, kp, F,
                                                                                       b.pf_perm, b.cs, b.cinfo,
                                                                                       b.pf_cmin);
         SKM_CUDA_TRY(launched());
@@ -2520,7 +2533,7 @@ int tc_assign_pfront(const skm_data *x, const float *C, int k, const int32_t *pr
     SKM_CUDA_TRY(launch_prune_finish(X, d, C, b.pf_thr, b.pf_cand, b.pf_cnt, PF_CAP, nsub, cb.pf_perm, b.resc_rows,
                                      b.counters, assign, dist, rows.wrow, ctr, st));
     SKM_CUDA_TRY(launch_prune_rows_cta(X, d, C, k, rows, b.fall_rows, b.counters + 1, assign, dist, ctr + 6, st));
-    pf_done_kernel<<<1, 1, 0, st>>>(warm ? b.pf_whdr : nullptr, b.counters, ctr, n, d, k, cb.pf_cgen, b.stats);
+    launch_dep(pf_done_kernel, 1, 1, 0, st, warm ? b.pf_whdr : nullptr, b.counters, ctr, n, d, k, cb.pf_cgen, b.stats);
     SKM_CUDA_TRY(launched());
     return SKM_OK;
 }
@@ -2536,7 +2549,7 @@ static int seg_setup(const TcSeg *seg, int64_t n, TcParams &p, cudaStream_t st) 
     const int64_t nrt = cdiv(n, BM);
     int64_t blocks = (nrt * 32 + 255) / 256;
     if (blocks > 152 * 8) blocks = 152 * 8;
-    seg_tiles_kernel<<<(int)(blocks < 1 ? 1 : blocks), 256, 0, st>>>(seg->group, seg->base, seg->nseg, n, nrt,
+    launch_dep(seg_tiles_kernel, (int)(blocks < 1 ? 1 : blocks), 256, 0, st, seg->group, seg->base, seg->nseg, n, nrt,
                                                                     seg->ct0, seg->nct);
     SKM_CUDA_TRY(launched());
     p.seg_ct0 = seg->ct0;
@@ -2568,11 +2581,11 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
     const bool warm = !seg && (x->flags & SKM_FLAG_WARM) && b.warm_hdr;
     unsigned int *hz = reinterpret_cast<unsigned int *>(b.counters + 4);
     if (warm)
-        cprep_f32_kernel<<<grid_warps(kp), 256, 0, st>>>(C, k, kp, d, dp, d, eps_acc, eps_s, v.rho_max,
+        launch_dep(cprep_f32_kernel, grid_warps(kp), 256, 0, st, C, k, kp, d, dp, d, eps_acc, eps_s, v.rho_max,
                                                          (__nv_bfloat16 *)b.cs, b.cinfo, b.cinfoz, hz, b.warm_cprev,
                                                          b.warm_shift, b.warm_hdr, n, b.counters + 6, nullptr);
     else
-        cprep_cold_kernel<<<grid_warps(kp), 256, 0, st>>>(C, k, kp, d, dp, d, eps_acc, eps_s, v.rho_max,
+        launch_dep(cprep_cold_kernel, grid_warps(kp), 256, 0, st, C, k, kp, d, dp, d, eps_acc, eps_s, v.rho_max,
                                                           (__nv_bfloat16 *)b.cs, b.cinfo, b.cinfoz, hz);
     SKM_CUDA_TRY(launched());
     TcParams p{};
@@ -2599,14 +2612,14 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
     if (p.ksplit > 1) {
         p.n = n;
         p.k = k;
-        screen_merge_kernel<<<(unsigned)cdiv(n, 64), 64, 0, st>>>(p);
+        launch_dep(screen_merge_kernel, (unsigned)cdiv(n, 64), 64, 0, st, p);
         SKM_CUDA_TRY(launched());
     }
     int64_t *hdr = warm ? b.warm_hdr : nullptr;
     const int gw = grid_warps(n);
     if (bf16) {
         const uint16_t *X = static_cast<const uint16_t *>(x->x);
-        rescore_kernel<uint16_t><<<gw, 256, 0, st>>>(X, d, C, b.resc_rows, b.counters, b.cand, assign, hdr, n, k,
+        launch_dep(rescore_kernel<uint16_t>, gw, 256, 0, st, X, d, C, b.resc_rows, b.counters, b.cand, assign, hdr, n, k,
                                                    b.stats, b.fall_rows, seg ? nullptr : b.fall_keys, b.cand);
         SKM_CUDA_TRY(launched());
         if (seg) {
@@ -2618,12 +2631,12 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
                                                   nullptr, b.fall_keys, b.cand, TCAND + 1, st));
         }
         if (dist) {
-            assigned_dist_kernel<uint16_t><<<gw, 256, 0, st>>>(X, n, d, C, assign, dist);
+            launch_dep(assigned_dist_kernel<uint16_t>, gw, 256, 0, st, X, n, d, C, assign, dist);
             SKM_CUDA_TRY(launched());
         }
     } else {
         const float *X = static_cast<const float *>(x->x);
-        rescore_kernel<float><<<gw, 256, 0, st>>>(X, d, C, b.resc_rows, b.counters, b.cand, assign, hdr, n, k,
+        launch_dep(rescore_kernel<float>, gw, 256, 0, st, X, d, C, b.resc_rows, b.counters, b.cand, assign, hdr, n, k,
                                                    b.stats, b.fall_rows, seg ? nullptr : b.fall_keys, b.cand);
         SKM_CUDA_TRY(launched());
         if (seg) {
@@ -2635,7 +2648,7 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
                                                   nullptr, b.fall_keys, b.cand, TCAND + 1, st));
         }
         if (dist) {
-            assigned_dist_kernel<float><<<gw, 256, 0, st>>>(X, n, d, C, assign, dist);
+            launch_dep(assigned_dist_kernel<float>, gw, 256, 0, st, X, n, d, C, assign, dist);
             SKM_CUDA_TRY(launched());
         }
     }
@@ -2663,7 +2676,7 @@ int tc_assign_sq8(const skm_data *x, const uint8_t *C, int k, int32_t *nx_plain,
     }
     ScreenView v = screen_view(x->repr, n, d, x->x, screen);
     const int kp = (int)(cdiv(k, BN) * BN);
-    cprep_sq8_kernel<<<grid_warps(kp), 256, 0, st>>>(C, k, kp, d, dp, (__nv_bfloat16 *)b.cs, b.nc,
+    launch_dep(cprep_sq8_kernel, grid_warps(kp), 256, 0, st, C, k, kp, d, dp, (__nv_bfloat16 *)b.cs, b.nc,
                                                      b.counters);
     SKM_CUDA_TRY(launched());
     TcParams p{};

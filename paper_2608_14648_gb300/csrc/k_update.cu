@@ -137,6 +137,7 @@ __global__ void __launch_bounds__(1024) scan_offsets_kernel(const int32_t *__res
                                                             int32_t *__restrict__ cursor, int64_t *__restrict__ zeros,
                                                             int32_t *__restrict__ flag, void *__restrict__ sums,
                                                             size_t sum_bytes) {
+    dep_sync();
     if (flag && blockIdx.x == 0 && threadIdx.x == 0) *flag = 0;
     if (blockIdx.x > 0) {
         clear_sums(sums, sum_bytes);
@@ -163,6 +164,7 @@ __global__ void __launch_bounds__(1024) sort_one_block_kernel(const int32_t *__r
                                                               int32_t *__restrict__ perm, int32_t *__restrict__ scl,
                                                               int64_t *__restrict__ zeros, int32_t *__restrict__ flag,
                                                               void *__restrict__ sums, size_t sum_bytes) {
+    dep_sync();
     if (flag && blockIdx.x == 0 && threadIdx.x == 0) *flag = 0;
     if (blockIdx.x > 0) {
         clear_sums(sums, sum_bytes);
@@ -230,6 +232,7 @@ constexpr int SC_MAX_K = 12288;  // 48 KiB of counters
 __global__ void __launch_bounds__(SC_THREADS) scatter_blocked_kernel(
     const int32_t *__restrict__ assign, int64_t n, int k, const int64_t *__restrict__ offsets,
     int32_t *__restrict__ cursor, int32_t *__restrict__ perm, int32_t *__restrict__ scl) {
+    dep_sync();
     extern __shared__ int32_t cnt_sh[];
     const int64_t p0 = (int64_t)blockIdx.x * SC_POINTS;
     const int64_t p1 = min(n, p0 + SC_POINTS);
@@ -266,19 +269,19 @@ cudaError_t launch_sort_by_cluster(const int32_t *assign, int64_t n, int k, int3
                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        sort_one_block_kernel<<<1 + clear, 1024, smem, st>>>(
+        launch_dep(sort_one_block_kernel, 1 + clear, 1024, smem, st, 
             assign, (int)n, k, offsets, counts64, accumulate, perm, scl, zeros, flag, sums, sum_bytes);
         return launched();
     }
     cudaError_t e = launch_histogram(assign, n, k, counts32, st);
     if (e != cudaSuccess) return e;
-    scan_offsets_kernel<<<1 + clear, 1024, 0, st>>>(counts32, k, offsets, counts64, accumulate, cursor, zeros, flag,
+    launch_dep(scan_offsets_kernel, 1 + clear, 1024, 0, st, counts32, k, offsets, counts64, accumulate, cursor, zeros, flag,
                                                     sums, sum_bytes);
     e = launched();
     if (e != cudaSuccess) return e;
     if (k <= SC_MAX_K) {
         const int64_t blocks = (n + SC_POINTS - 1) / SC_POINTS;
-        scatter_blocked_kernel<<<(unsigned)blocks, SC_THREADS, sizeof(int32_t) * (size_t)k, st>>>(
+        launch_dep(scatter_blocked_kernel, (unsigned)blocks, SC_THREADS, sizeof(int32_t) * (size_t)k, st, 
             assign, n, k, offsets, cursor, perm, scl);
         return launched();
     }
@@ -430,6 +433,7 @@ __global__ void __launch_bounds__(CH_WARPS * 32) chunk_sum_float_kernel(
     const void *__restrict__ Xv, int d, const int32_t *__restrict__ perm,
     const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k,
     ACC *__restrict__ S, int64_t stride, int run) {
+    dep_sync();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t nval = offsets[k];
     const int64_t q0 = ((int64_t)blockIdx.x * CH_WARPS + warp) * run;
@@ -499,14 +503,14 @@ cudaError_t launch_chunk_sum_float(const void *X, int x_is_bf16, int64_t n, int 
     const unsigned g = chunk_blocks(n, run);
     if (S_d) {
         if (x_is_bf16)
-            chunk_sum_float_kernel<true, double><<<g, CH_WARPS * 32, 0, st>>>(X, d, perm, scl, offsets, k, S_d, d, run);
+            launch_dep(chunk_sum_float_kernel<true, double>, g, CH_WARPS * 32, 0, st, X, d, perm, scl, offsets, k, S_d, d, run);
         else
-            chunk_sum_float_kernel<false, double><<<g, CH_WARPS * 32, 0, st>>>(X, d, perm, scl, offsets, k, S_d, d, run);
+            launch_dep(chunk_sum_float_kernel<false, double>, g, CH_WARPS * 32, 0, st, X, d, perm, scl, offsets, k, S_d, d, run);
     } else {
         if (x_is_bf16)
-            chunk_sum_float_kernel<true, float><<<g, CH_WARPS * 32, 0, st>>>(X, d, perm, scl, offsets, k, S_f, d, run);
+            launch_dep(chunk_sum_float_kernel<true, float>, g, CH_WARPS * 32, 0, st, X, d, perm, scl, offsets, k, S_f, d, run);
         else
-            chunk_sum_float_kernel<false, float><<<g, CH_WARPS * 32, 0, st>>>(X, d, perm, scl, offsets, k, S_f, d, run);
+            launch_dep(chunk_sum_float_kernel<false, float>, g, CH_WARPS * 32, 0, st, X, d, perm, scl, offsets, k, S_f, d, run);
     }
     return launched();
 }
@@ -515,6 +519,7 @@ cudaError_t launch_chunk_sum_float(const void *X, int x_is_bf16, int64_t n, int 
 __global__ void finalize_float32_kernel(const float *__restrict__ S,
                                         const int64_t *__restrict__ counts, int k, int d,
                                         float *__restrict__ C) {
+    dep_sync();
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= (int64_t)k * d) return;
     const int64_t c = counts[t / d];
@@ -524,7 +529,7 @@ __global__ void finalize_float32_kernel(const float *__restrict__ S,
 cudaError_t launch_finalize_float32(const float *S, const int64_t *counts, int k, int d,
                                     float *C_inout, cudaStream_t st) {
     const int64_t tot = (int64_t)k * d;
-    finalize_float32_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(S, counts, k, d, C_inout);
+    launch_dep(finalize_float32_kernel, (unsigned)((tot + 255) / 256), 256, 0, st, S, counts, k, d, C_inout);
     return launched();
 }
 
@@ -550,6 +555,7 @@ cudaError_t launch_finalize_float(const double *partial, const int64_t *counts, 
 __global__ void finalize_sq8_kernel(const int64_t *__restrict__ partial,
                                     const int64_t *__restrict__ counts, int k, int d,
                                     uint8_t *__restrict__ C) {
+    dep_sync();
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= (int64_t)k * d) return;
     const int j = (int)(t / d);
@@ -560,7 +566,7 @@ __global__ void finalize_sq8_kernel(const int64_t *__restrict__ partial,
 cudaError_t launch_finalize_sq8(const int64_t *partial, const int64_t *counts, int k, int d,
                                 uint8_t *C_inout, cudaStream_t st) {
     const int64_t tot = (int64_t)k * d;
-    finalize_sq8_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(partial, counts, k, d,
+    launch_dep(finalize_sq8_kernel, (unsigned)((tot + 255) / 256), 256, 0, st, partial, counts, k, d,
                                                                        C_inout);
     return launched();
 }
@@ -571,6 +577,7 @@ cudaError_t launch_finalize_sq8(const int64_t *partial, const int64_t *counts, i
 __global__ void finalize_rbq1_kernel(const int64_t *__restrict__ partial,
                                      const int64_t *__restrict__ counts, int k, int d,
                                      const float *__restrict__ m, int e, float *__restrict__ C) {
+    dep_sync();
     __shared__ double fs;
     const int j = blockIdx.x;
     const int64_t c = counts[j];
@@ -588,7 +595,7 @@ __global__ void finalize_rbq1_kernel(const int64_t *__restrict__ partial,
 
 cudaError_t launch_finalize_rbq1(const int64_t *partial, const int64_t *counts, int k, int d,
                                  const float *m, int e, float *C_inout, cudaStream_t st) {
-    finalize_rbq1_kernel<<<k, 256, 0, st>>>(partial, counts, k, d, m, e, C_inout);
+    launch_dep(finalize_rbq1_kernel, k, 256, 0, st, partial, counts, k, d, m, e, C_inout);
     return launched();
 }
 
