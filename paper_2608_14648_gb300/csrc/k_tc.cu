@@ -131,6 +131,9 @@ struct TcParams {
     int ksplit;
     uint32_t *part;
     int nkc;  // 64-wide k-slices
+    // ONE: the centroids rounded up to 32 (the MMAs' N and the B loads' rows)
+    int bn;
+    int sw;  // ONE: columns of an epilogue slice
     const float4 *cinfo;  // SCREEN: per column pair (||c||^2 x2, h' x2), padded to 256
     const float *hz;      // SCREEN: (max h', max z) over the centroids
     const float2 *cinfoz; // SCREEN: per column pair (z x2)
@@ -421,9 +424,12 @@ __device__ __forceinline__ void screen_decide(const TcParams &p, int64_t row, Sc
 // Centroid tiles [lo, hi) of work item rt: every tile of a point tile, with
 // ksplit > 1 a share of them, or in segmented mode the tile's groups' range
 // (none past the last point tile there).
-template <int MODE>
+template <int MODE, bool ONE>
 __device__ __forceinline__ void ct_range(const TcParams &p, int64_t rt, int &lo, int &hi) {
-    if (MODE == MODE_SCREEN && p.ksplit > 1) {
+    if (ONE) {
+        lo = 0;
+        hi = 1;
+    } else if (MODE == MODE_SCREEN && p.ksplit > 1) {
         const int per = (p.nct + p.ksplit - 1) / p.ksplit;
         lo = (int)(rt % p.ksplit) * per;
         hi = min(p.nct, lo + per);
@@ -441,7 +447,8 @@ __device__ __forceinline__ void ct_range(const TcParams &p, int64_t rt, int &lo,
     }
 }
 
-template <int MODE, int NH, bool SEG, int NS, bool PK>
+// ONE: all centroids in one tile (k <= BN), which is only as wide as they are.
+template <int MODE, int NH, bool SEG, int NS, bool PK, bool ONE>
 __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
     tc_assign_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const TcParams p) {
@@ -533,7 +540,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
     auto stream_seek = [&](JobStream &js) {  // the first job at or after group js.g
         while (js.g < ngroups) {
             int lo, hi;
-            ct_range<MODE>(p, js.g, lo, hi);
+            ct_range<MODE, ONE>(p, js.g, lo, hi);
             if (lo < hi) {
                 js.ct = lo;
                 js.hi = hi;
@@ -611,7 +618,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                     for (int kc = 0; kc < p.nkc; ++kc, ++it) {
                         const uint32_t s = it % STAGES, ph = (it / STAGES) & 1u;
                         if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) goto producer_done;
-                        mbar_expect_tx(full_bar(s), A_STAGE + B_STAGE);
+                        mbar_expect_tx(full_bar(s), A_STAGE + (ONE ? (uint32_t)p.bn * (B_STAGE / BN) : B_STAGE));
                         tma_load_2d(sA + s * A_STAGE, &tmA, kc * KC_ELEMS, arow, full_bar(s));
                         tma_load_2d(sB + s * B_STAGE, &tmB, kc * KC_ELEMS, brow, full_bar(s));
                     }
@@ -630,6 +637,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
     } else if (warp == 1) {
         if (lane == 0) {  // ---------------------------------------- MMA issuer
             uint32_t it = 0, job = 0;
+            const uint32_t idesc = (f8_mode<MODE>() ? IDESC_F8 : IDESC) - (ONE ? (uint32_t)((BN - p.bn) >> 3) << 17 : 0u);
             bool issued = false, gave_up = true;
             uint32_t jc[NS];
             JobStream js[NS];
@@ -690,9 +698,9 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {  // 4 x 32-byte K steps per 128-byte row
                             if (f8_mode<MODE>())
-                                tc_mma_f8(dcol, ad + 2u * kk, bd + 2u * kk, IDESC_F8, (kc | kk) != 0);
+                                tc_mma_f8(dcol, ad + 2u * kk, bd + 2u * kk, idesc, (kc | kk) != 0);
                             else
-                                tc_mma(dcol, ad + 2u * kk, bd + 2u * kk, IDESC, (kc | kk) != 0);
+                                tc_mma(dcol, ad + 2u * kk, bd + 2u * kk, idesc, (kc | kk) != 0);
                         }
                         issued = true;
                         tc_commit(empty_bar(s));
@@ -842,7 +850,8 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
     } else {  // ------------------------------------------------------- epilogue
         constexpr int NHG = NH / NS;     // warps per TMEM lane quarter in a group
         constexpr int GT = epi_threads<NH>() / NS;  // threads per group
-        constexpr int SW = BN / NHG;     // columns per slice
+        constexpr int SW = BN / NHG;     // columns per slice, at most
+        const int sw = ONE ? p.sw : SW;
         constexpr int MW = merge_words<MODE>();
         const int e = warp - 2;          // 0 .. 4 NH - 1
         const int q = warp & 3;          // TMEM lane quarter this warp may access
@@ -892,7 +901,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
         };
         {
             int lo0, hi0;
-            ct_range<MODE>(p, g0 + grp * gstep, lo0, hi0);
+            ct_range<MODE, ONE>(p, g0 + grp * gstep, lo0, hi0);
             rec_load(lo0);
         }
         // A warp whose barrier wait gave up stops computing but keeps taking part
@@ -929,11 +938,11 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                 ce = p.seg_base[gi + 1];
             }
             int ct_lo, ct_hi;
-            ct_range<MODE>(p, g, ct_lo, ct_hi);
+            ct_range<MODE, ONE>(p, g, ct_lo, ct_hi);
             int next_lo = 0;
             {
                 int nhi;
-                ct_range<MODE>(p, g + NS * gstep, next_lo, nhi);
+                ct_range<MODE, ONE>(p, g + NS * gstep, next_lo, nhi);
             }
             if (MODE == MODE_SCREEN) {
                 a2 = valid ? 2.0f * p.xinfo[row].x : 0.0f;
@@ -1007,15 +1016,16 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tempty_bar(b));
                 };
-                const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + b * BN + slice * SW;
-                const int jh = ct * BN + slice * SW;
+                const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + b * BN + slice * sw;
+                const int jh = ct * BN + slice * sw;
+                const int jend = ONE ? min(p.k, jh + sw) : p.k;
                 if (MODE == MODE_SCREEN) {
                     // chunks of SCR_CW columns (16: the next TMEM load in flight)
                     constexpr int NC = SW / SCR_CW;
                     constexpr int G = SCR_CW / 8;
                     auto chunk = [&](uint32_t(&v)[SCR_CW], int c) {
                         const int j0 = jh + c * SCR_CW;
-                        const int cc = slice * SW + c * SCR_CW;  // column offset within the tile
+                        const int cc = slice * sw + c * SCR_CW;  // column offset within the tile
                         // pass 1, two columns per packed op: s~ = ||c||^2 - 2 acc (kept in
                         // v) and the chunk's smallest s~.  Records past k have ||c||^2 =
                         // +inf, so s~ = +inf.
@@ -1086,7 +1096,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                         }
                     };
                     {
-                        const int nv = min(NC, (p.k - jh + 31) / 32);  // chunks inside [0, k) (warp-uniform)
+                        const int nv = min(NC, (jend - jh + 31) / 32);  // chunks inside [0, k) (warp-uniform)
                         if (nv <= 0) release();
 #pragma unroll 1
                         for (int c = 0; c < nv; ++c) {
@@ -1153,7 +1163,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                     constexpr int G = F8_CW / 8;
                     auto chunk = [&](const uint32_t(&v)[F8_CW], int c) {
                         const int j0 = jh + c * F8_CW;
-                        const int cc = slice * SW + c * F8_CW;
+                        const int cc = slice * sw + c * F8_CW;
 #pragma unroll
                         for (int g = 0; g < G; ++g) {
                             asm volatile("" ::: "memory");
@@ -1203,7 +1213,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                         }
                     };
                     if constexpr (F8_CW == 32) {
-                        const int nv = min(NC, (p.k - jh + 31) / 32);  // chunks inside [0, k) (warp-uniform)
+                        const int nv = min(NC, (jend - jh + 31) / 32);  // chunks inside [0, k) (warp-uniform)
                         if (nv <= 0) release();
 #pragma unroll 1
                         for (int c = 0; c < nv; ++c) {
@@ -1212,19 +1222,19 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                             if (c == nv - 1) release();
                             chunk(v, c);
                         }
-                    } else if (jh < p.k) {  // warp-uniform conditions throughout
+                    } else if (jh < jend) {  // warp-uniform conditions throughout
                         uint32_t va[16], vb[16];
                         tmem_ld16_async(taddr, va);
                         tmem_wait16(va);
 #pragma unroll
                         for (int c = 0; c < NC; c += 2) {
-                            const bool m1 = c + 1 < NC && jh + (c + 1) * 16 < p.k;
+                            const bool m1 = c + 1 < NC && jh + (c + 1) * 16 < jend;
                             if (m1) tmem_ld16_async(taddr + (c + 1) * 16, vb);
                             else release();
                             chunk(va, c);
                             if (!m1) break;
                             tmem_wait16(vb);
-                            const bool m2 = c + 2 < NC && jh + (c + 2) * 16 < p.k;
+                            const bool m2 = c + 2 < NC && jh + (c + 2) * 16 < jend;
                             if (m2) tmem_ld16_async(taddr + (c + 2) * 16, va);
                             else release();
                             chunk(vb, c + 1);
@@ -1235,12 +1245,12 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                         release();
                     }
                 } else {  // MODE_SQ8
-                    const int nv = min(SW / 32, (p.k - jh + 31) / 32);  // chunks inside [0, k) (warp-uniform)
+                    const int nv = min(SW / 32, (jend - jh + 31) / 32);  // chunks inside [0, k) (warp-uniform)
                     if (nv <= 0) release();
 #pragma unroll 1
                     for (int c = 0; c < nv; ++c) {
                         const int j0 = jh + c * 32;
-                        const int cc = slice * SW + c * 32;  // column offset within the tile
+                        const int cc = slice * sw + c * 32;  // column offset within the tile
                         uint32_t v[32];
                         tmem_ld32(taddr + c * 32, v);
                         if (c == nv - 1) release();
@@ -2077,7 +2087,7 @@ __global__ void seg_rows_exact_kernel(const TX *__restrict__ X, int d, const flo
 }
 
 // ------------------------------------------------------------------ host side
-template <int MODE, bool SEG, bool PK>
+template <int MODE, bool SEG, bool PK, bool ONE>
 int launch_tc_kind(const void *xs, int64_t n, int dp, int d, const void *cs, int k, const TcParams &p0,
                    cudaStream_t st, int dpb);
 
@@ -2090,37 +2100,39 @@ int launch_tc(const void *xs, int64_t n, int dp, int d, const void *cs, int k, c
     if (dpb < 0) dpb = dp;
     if constexpr (MODE == MODE_RBQ1 || MODE == MODE_LVQ4) {
         if (packed) {
-            if (p0.seg_group) return launch_tc_kind<MODE, true, true>(xs, n, dp, d, cs, k, p0, st, dpb);
-            return launch_tc_kind<MODE, false, true>(xs, n, dp, d, cs, k, p0, st, dpb);
+            if (p0.seg_group) return launch_tc_kind<MODE, true, true, false>(xs, n, dp, d, cs, k, p0, st, dpb);
+            if (k <= BN) return launch_tc_kind<MODE, false, true, true>(xs, n, dp, d, cs, k, p0, st, dpb);
+            return launch_tc_kind<MODE, false, true, false>(xs, n, dp, d, cs, k, p0, st, dpb);
         }
     }
-    if constexpr (MODE != MODE_PFRONT)
-        if (p0.seg_group) return launch_tc_kind<MODE, true, false>(xs, n, dp, d, cs, k, p0, st, dpb);
-    return launch_tc_kind<MODE, false, false>(xs, n, dp, d, cs, k, p0, st, dpb);
+    if constexpr (MODE != MODE_PFRONT) {
+        if (p0.seg_group) return launch_tc_kind<MODE, true, false, false>(xs, n, dp, d, cs, k, p0, st, dpb);
+        if (k <= BN) return launch_tc_kind<MODE, false, false, true>(xs, n, dp, d, cs, k, p0, st, dpb);
+    }
+    return launch_tc_kind<MODE, false, false, false>(xs, n, dp, d, cs, k, p0, st, dpb);
 }
 
 // One persistent CTA per SM (at most one point tile per CTA when there are
 // fewer tiles than SMs).
-template <int MODE, bool SEG, bool PK>
+template <int MODE, bool SEG, bool PK, bool ONE>
 int launch_tc_kind(const void *xs, int64_t n, int dp, int d, const void *cs, int k, const TcParams &p0,
                    cudaStream_t st, int dpb) {
     constexpr int NH = TC_NH[MODE];
     constexpr int NS = TC_NS[MODE];
     constexpr size_t SMEM = tc_smem_bytes<MODE, NH, NS>();
     static_assert(SMEM <= 227 * 1024, "shared memory per CTA");
-    auto kern = tc_assign_kernel<MODE, NH, SEG, NS, PK>;
-    const int segi = SEG ? 1 : 0, pki = PK ? 1 : 0;
-    // the dynamic shared memory attribute, set once per device
+    auto kern = tc_assign_kernel<MODE, NH, SEG, NS, PK, ONE>;
+    // the dynamic shared memory attribute, set once per device and instantiation
     constexpr int MAXDEV = 64;
     static std::mutex mu;
-    static bool attr_set[5][2][2][MAXDEV] = {};
+    static bool attr_set[MAXDEV] = {};
     int dev = 0;
     SKM_CUDA_TRY(cudaGetDevice(&dev));
     {
         std::lock_guard<std::mutex> lock(mu);
-        if (dev >= MAXDEV || !attr_set[MODE][segi][pki][dev]) {
+        if (dev >= MAXDEV || !attr_set[dev]) {
             SKM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM));
-            if (dev < MAXDEV) attr_set[MODE][segi][pki][dev] = true;
+            if (dev < MAXDEV) attr_set[dev] = true;
         }
     }
     CUtensorMap ma, mb;
@@ -2133,12 +2145,23 @@ int launch_tc_kind(const void *xs, int64_t n, int dp, int d, const void *cs, int
     } else {
         SKM_TRY(make_map(&ma, xs, n, d, dp, BM, eb));
     }
-    SKM_TRY(make_map(&mb, cs, k, d, dpb, BN, eb));
     TcParams p = p0;
+    const int nct = (int)cdiv(k, BN);
+    // Few centroids (the meso pass of a hierarchical fit): a full tile's B loads
+    // and MMAs would be mostly padding, repeated for each point tile, and its
+    // second epilogue slice would idle.  1M x 768 against about 60 centroids:
+    // 1-bit codes packed 390 -> 225 us, from the copy 282 -> 131 us; LVQ4 packed
+    // 532 -> 406; fp32 643 -> 264; SQ8 d = 128, k = 100: 117 -> 88.  With more
+    // tiles a narrow last one gives nothing (4M x 1024 against 3162, 90 columns
+    // left: 7.35 -> 7.36 ms), and slices of a width known at run time cost 2 to
+    // 15%, so all are BN wide there.
+    p.bn = ONE ? (k + 31) / 32 * 32 : BN;
+    p.sw = (p.bn / (NH / NS) + 31) / 32 * 32;
+    SKM_TRY(make_map(&mb, cs, k, d, dpb, p.bn, eb));
     p.n = n;
     p.nrt = cdiv(n, BM);
     p.k = k;
-    p.nct = (int)cdiv(k, BN);
+    p.nct = nct;
     p.ksplit = std::max(1, p0.ksplit);
     p.nkc = (int)cdiv(d, 128 / eb);
     p.inject_wait_ns = fault_take(SKM_FAULT_WAIT) ? 1000000ull : 0ull;  // 1 ms
