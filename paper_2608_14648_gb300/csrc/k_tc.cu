@@ -131,7 +131,8 @@ struct TcParams {
     int ksplit;
     uint32_t *part;
     int nkc;  // 64-wide k-slices
-    // ONE: the centroids rounded up to 32 (the MMAs' N and the B loads' rows)
+    // a job's columns (the MMAs' N and the B loads' rows): BN; ONE: the centroids
+    // rounded up to 32; segmented: see seg_setup
     int bn;
     int sw;  // ONE: columns of an epilogue slice
     const float4 *cinfo;  // SCREEN: per column pair (||c||^2 x2, h' x2), padded to 256
@@ -169,8 +170,8 @@ struct TcParams {
     const int32_t *warm_ok;
     // Segmented mode (all NULL otherwise): the point rows are sorted by
     // group and row r may only take centroids [seg_base[g], seg_base[g + 1])
-    // of its group g = seg_group[r]; point tile rt covers the centroid tiles
-    // seg_ct0[rt] .. seg_ct0[rt] + seg_nct[rt] - 1.
+    // of its group g = seg_group[r]; point tile rt covers seg_nct[rt] x 32
+    // columns from 32 seg_ct0[rt] on, in jobs of bn columns (128 or 256).
     const int32_t *seg_ct0;
     const int32_t *seg_nct;
     const int32_t *seg_group;
@@ -528,6 +529,10 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
     const int64_t g0 = (int64_t)blockIdx.x;
     const int64_t gstep = (int64_t)gridDim.x;
     const int64_t ngroups = MODE == MODE_SCREEN ? p.nrt * p.ksplit : p.nrt;
+    // job columns: segmented tiles start at any multiple of 32 and are counted
+    // in those, the others in whole tiles
+    constexpr int CTW = SEG ? 32 : BN;
+    const int cts = SEG ? p.bn / 32 : 1;
     auto tile_of = [&](int64_t g) { return MODE == MODE_SCREEN && p.ksplit > 1 ? g / p.ksplit : g; };
 
     // Job order (producer and MMA issuer walk it identically): stream s takes
@@ -550,7 +555,8 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
         }
     };
     auto stream_advance = [&](JobStream &js) {
-        if (++js.ct >= js.hi) {
+        js.ct += cts;
+        if (js.ct >= js.hi) {
             js.g += NS * gstep;
             stream_seek(js);
         }
@@ -614,11 +620,11 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                     arow0 = (((int64_t)blockIdx.x * NS + sj) * 2 + ((pc - 1u) & 1u)) * BM;
                 }
                 {
-                    const int arow = (int)arow0, brow = ct * BN;
+                    const int arow = (int)arow0, brow = ct * CTW;
                     for (int kc = 0; kc < p.nkc; ++kc, ++it) {
                         const uint32_t s = it % STAGES, ph = (it / STAGES) & 1u;
                         if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) goto producer_done;
-                        mbar_expect_tx(full_bar(s), A_STAGE + (ONE ? (uint32_t)p.bn * (B_STAGE / BN) : B_STAGE));
+                        mbar_expect_tx(full_bar(s), A_STAGE + (ONE || SEG ? (uint32_t)p.bn * (B_STAGE / BN) : B_STAGE));
                         tma_load_2d(sA + s * A_STAGE, &tmA, kc * KC_ELEMS, arow, full_bar(s));
                         tma_load_2d(sB + s * B_STAGE, &tmB, kc * KC_ELEMS, brow, full_bar(s));
                     }
@@ -637,7 +643,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
     } else if (warp == 1) {
         if (lane == 0) {  // ---------------------------------------- MMA issuer
             uint32_t it = 0, job = 0;
-            const uint32_t idesc = (f8_mode<MODE>() ? IDESC_F8 : IDESC) - (ONE ? (uint32_t)((BN - p.bn) >> 3) << 17 : 0u);
+            const uint32_t idesc = (f8_mode<MODE>() ? IDESC_F8 : IDESC) - (ONE || SEG ? (uint32_t)((BN - p.bn) >> 3) << 17 : 0u);
             bool issued = false, gave_up = true;
             uint32_t jc[NS];
             JobStream js[NS];
@@ -674,7 +680,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                             }
                         }
                         slot = (mc - 1u) & 1u;
-                        tile_last = ctj == hij - 1;
+                        tile_last = ctj + cts >= hij;
                     }
                 }
                 turn = (sj + 1) % NS;
@@ -873,19 +879,21 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
         float4 pre4 = make_float4(0.f, 0.f, 0.f, 0.f);
         float2 pre2 = make_float2(0.f, 0.f);
         int32_t pre1 = 0;
+        // column pairs of a job (segmented: those past a narrow job may lie past the records)
+        const int rec_pairs = SEG ? p.bn / 2 : 128;
         auto rec_load = [&](int ctn) {
             if (MODE == MODE_SCREEN || MODE == MODE_PFRONT) {
-                if (te < 128) {
-                    const float4 ci = __ldg(p.cinfo + ctn * 128 + te);
+                if (te < rec_pairs) {
+                    const float4 ci = __ldg(p.cinfo + ctn * (CTW / 2) + te);
                     pre2 = make_float2(ci.x, ci.y);
                 } else if (MODE == MODE_PFRONT && te < 130) {  // the tile's 8 chunk minima
                     pre4 = __ldg(reinterpret_cast<const float4 *>(p.pf_cmin + ctn * 8) + (te - 128));
                 }
             } else if (f8_mode<MODE>()) {
-                if (te < 128) pre4 = __ldg(p.rinfo + ctn * 128 + te);
-                else if (te < 256) pre4 = __ldg(p.rinfoq + ctn * 128 + (te - 128));
+                if (te < rec_pairs) pre4 = __ldg(p.rinfo + ctn * (CTW / 2) + te);
+                else if (te >= 128 && te < 128 + rec_pairs) pre4 = __ldg(p.rinfoq + ctn * (CTW / 2) + (te - 128));
             } else if (MODE == MODE_SQ8) {
-                if (te < 256) pre1 = __ldg(p.nc + ctn * 256 + te);
+                if (te < 2 * rec_pairs) pre1 = __ldg(p.nc + ctn * CTW + te);
             }
         };
         auto rec_store = [&](uint32_t buf) {
@@ -937,6 +945,12 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                 cb = p.seg_base[gi];
                 ce = p.seg_base[gi + 1];
             }
+            int wlo = 0, whi = 0;  // the warp's rows' columns
+            if (SEG) {
+                wlo = __reduce_min_sync(0xffffffffu, valid ? cb : 0x7fffffff);
+                whi = min(p.k, __reduce_max_sync(0xffffffffu, valid ? ce : 0));
+                if (whi <= wlo) wlo = whi = 0;
+            }
             int ct_lo, ct_hi;
             ct_range<MODE, ONE>(p, g, ct_lo, ct_hi);
             int next_lo = 0;
@@ -978,7 +992,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                 rf2 = valid ? __fmul_rn(-2.0f, p.F[row]) : 0.0f;  // exact
                 rpc = valid ? (float)(2 * p.popx[row] - p.d) : 0.0f;
             }
-            for (int ct = ct_lo; ct < ct_hi; ++ct, ++job) {
+            for (int ct = ct_lo; ct < ct_hi; ct += cts, ++job) {
                 // accumulator b (NS = 2: the group's own; NS = 1: alternating), its
                 // use parity, and the record buffer (two per group, alternating)
                 const uint32_t b = NS == 2 ? (uint32_t)grp : (job & 1u);
@@ -1004,7 +1018,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                     rec_store(rb);
                     asm volatile("bar.sync %0, %1;" ::"r"(2 + grp), "n"(GT) : "memory");
                 }
-                rec_load(ct + 1 < ct_hi ? ct + 1 : next_lo);
+                rec_load(ct + cts < ct_hi ? ct + cts : next_lo);
                 if (dead) continue;
                 tc_fence_after();
                 const uint8_t *rbuf = rec_base + rb * REC_BYTES;
@@ -1016,16 +1030,23 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tempty_bar(b));
                 };
-                const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + b * BN + slice * sw;
-                const int jh = ct * BN + slice * sw;
+                const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + b * BN + (SEG ? 0 : slice * sw);
+                const int jh = ct * CTW + (SEG ? 0 : slice * sw);
                 const int jend = ONE ? min(p.k, jh + sw) : p.k;
+                // Segmented: the slices take alternate chunks of CW columns, and
+                // only those that meet the range of some row of the warp.
+                auto seg_chunks = [&](int CW, int &c0, int &c1) {
+                    const int st = NHG * CW, at = jh + slice * CW;
+                    c0 = wlo < at + CW ? 0 : (wlo - at - CW) / st + 1;
+                    c1 = min(p.bn / st, whi > at ? (whi - at + st - 1) / st : 0);
+                };
                 if (MODE == MODE_SCREEN) {
                     // chunks of SCR_CW columns (16: the next TMEM load in flight)
                     constexpr int NC = SW / SCR_CW;
                     constexpr int G = SCR_CW / 8;
                     auto chunk = [&](uint32_t(&v)[SCR_CW], int c) {
-                        const int j0 = jh + c * SCR_CW;
-                        const int cc = slice * sw + c * SCR_CW;  // column offset within the tile
+                        const int cc = SEG ? (NHG * c + slice) * SCR_CW : slice * sw + c * SCR_CW;
+                        const int j0 = SEG ? jh + cc : jh + c * SCR_CW;  // column offset within the tile
                         // pass 1, two columns per packed op: s~ = ||c||^2 - 2 acc (kept in
                         // v) and the chunk's smallest s~.  Records past k have ||c||^2 =
                         // +inf, so s~ = +inf.
@@ -1096,12 +1117,13 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                         }
                     };
                     {
-                        const int nv = min(NC, (jend - jh + 31) / 32);  // chunks inside [0, k) (warp-uniform)
-                        if (nv <= 0) release();
+                        int c0 = 0, nv = min(NC, (jend - jh + 31) / 32);  // chunks inside [0, k) (warp-uniform)
+                        if (SEG) seg_chunks(SCR_CW, c0, nv);
+                        if (nv <= c0) release();
 #pragma unroll 1
-                        for (int c = 0; c < nv; ++c) {
+                        for (int c = c0; c < nv; ++c) {
                             uint32_t v[32];
-                            tmem_ld32(taddr + c * 32, v);
+                            tmem_ld32(taddr + (SEG ? (NHG * c + slice) * 32 : c * 32), v);
                             if (c == nv - 1) release();
                             chunk(v, c);
                         }
@@ -1162,8 +1184,8 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                     constexpr int NC = SW / F8_CW;
                     constexpr int G = F8_CW / 8;
                     auto chunk = [&](const uint32_t(&v)[F8_CW], int c) {
-                        const int j0 = jh + c * F8_CW;
-                        const int cc = slice * sw + c * F8_CW;
+                        const int cc = SEG ? (NHG * c + slice) * F8_CW : slice * sw + c * F8_CW;
+                        const int j0 = SEG ? jh + cc : jh + c * F8_CW;
 #pragma unroll
                         for (int g = 0; g < G; ++g) {
                             asm volatile("" ::: "memory");
@@ -1212,7 +1234,23 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                             }
                         }
                     };
-                    if constexpr (F8_CW == 32) {
+                    if constexpr (SEG) {
+                        int c0, c1;
+                        seg_chunks(F8_CW, c0, c1);
+                        if (c1 <= c0) release();
+#pragma unroll 1
+                        for (int c = c0; c < c1; ++c) {
+                            uint32_t v[F8_CW];
+                            if constexpr (F8_CW == 32) {
+                                tmem_ld32(taddr + (NHG * c + slice) * 32, v);
+                            } else {
+                                tmem_ld16_async(taddr + (NHG * c + slice) * 16, v);
+                                tmem_wait16(v);
+                            }
+                            if (c == c1 - 1) release();
+                            chunk(v, c);
+                        }
+                    } else if constexpr (F8_CW == 32) {
                         const int nv = min(NC, (jend - jh + 31) / 32);  // chunks inside [0, k) (warp-uniform)
                         if (nv <= 0) release();
 #pragma unroll 1
@@ -1245,14 +1283,15 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                         release();
                     }
                 } else {  // MODE_SQ8
-                    const int nv = min(SW / 32, (jend - jh + 31) / 32);  // chunks inside [0, k) (warp-uniform)
-                    if (nv <= 0) release();
+                    int c0 = 0, nv = min(SW / 32, (jend - jh + 31) / 32);  // chunks inside [0, k) (warp-uniform)
+                    if (SEG) seg_chunks(32, c0, nv);
+                    if (nv <= c0) release();
 #pragma unroll 1
-                    for (int c = 0; c < nv; ++c) {
-                        const int j0 = jh + c * 32;
-                        const int cc = slice * sw + c * 32;  // column offset within the tile
+                    for (int c = c0; c < nv; ++c) {
+                        const int cc = SEG ? (NHG * c + slice) * 32 : slice * sw + c * 32;  // column offset within the tile
+                        const int j0 = SEG ? jh + cc : jh + c * 32;
                         uint32_t v[32];
-                        tmem_ld32(taddr + c * 32, v);
+                        tmem_ld32(taddr + (SEG ? cc : c * 32), v);
                         if (c == nv - 1) release();
                         // s = ||c||^2 - 2 dot, exact integers in both operands, with
                         // one rounding at most: rounding is monotone, so only a
@@ -2026,7 +2065,8 @@ __global__ void assigned_dist_kernel(const TX *__restrict__ X, int64_t n, int d,
 // Centroid tiles of each point tile: the union of its rows' group ranges
 // (min and max group over the tile's rows, ids clamped into [0, nseg)).
 __global__ void seg_tiles_kernel(const int32_t *__restrict__ group, const int32_t *__restrict__ base, int nseg,
-                                 int64_t n, int64_t nrt, int32_t *__restrict__ ct0, int32_t *__restrict__ nct) {
+                                 int64_t n, int64_t nrt, int k, int bn, int32_t *__restrict__ ct0,
+                                 int32_t *__restrict__ nct) {
     dep_sync();
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -2048,11 +2088,14 @@ __global__ void seg_tiles_kernel(const int32_t *__restrict__ group, const int32_
             gmax = max(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
         }
         if (lane == 0) {
-            const int lo = base[gmin], hi = base[gmax + 1];
-            const int t0 = lo / BN;
-            const int t1 = hi > lo ? (hi + BN - 1) / BN : t0 + 1;
-            ct0[rt] = t0;
-            nct[rt] = t1 - t0;
+            // from the groups' first column (rounded down to 32), as many jobs of
+            // bn columns as reach their last; none past the padded records
+            const int hi = min(base[gmax + 1], k);
+            int c = max(0, min(base[gmin], k - 1)) & ~31;
+            const int jobs = hi > c ? (hi - c + bn - 1) / bn : 1;
+            c = min(c, (k + BN - 1) / BN * BN - jobs * bn);
+            ct0[rt] = c / 32;
+            nct[rt] = jobs * (bn / 32);
         }
     }
 }
@@ -2155,7 +2198,7 @@ int launch_tc_kind(const void *xs, int64_t n, int dp, int d, const void *cs, int
     // tiles a narrow last one gives nothing (4M x 1024 against 3162, 90 columns
     // left: 7.35 -> 7.36 ms), and slices of a width known at run time cost 2 to
     // 15%, so all are BN wide there.
-    p.bn = ONE ? (k + 31) / 32 * 32 : BN;
+    p.bn = ONE ? (k + 31) / 32 * 32 : SEG ? p0.bn : BN;
     p.sw = (p.bn / (NH / NS) + 31) / 32 * 32;
     SKM_TRY(make_map(&mb, cs, k, d, dpb, p.bn, eb));
     p.n = n;
@@ -2567,13 +2610,18 @@ int tc_init_stats(TcAssignBufs &b, cudaStream_t st) {
 }
 
 // point tiles' centroid-tile ranges for a segmented call (none otherwise)
-static int seg_setup(const TcSeg *seg, int64_t n, TcParams &p, cudaStream_t st) {
+static int seg_setup(const TcSeg *seg, int64_t n, int k, TcParams &p, cudaStream_t st) {
     if (!seg) return SKM_OK;
+    // A tile's jobs start at its groups' first column and are 128 columns wide
+    // when groups have at most 96 on average (rounded out to 32 one mostly
+    // fits; a larger one takes several jobs).  From 256-column tiles at fixed
+    // places, 1M x 768 1-bit codes in 63 groups of about 63: 215 -> 142 us (read at 5.5 TB/s).
+    p.bn = k <= 96LL * seg->nseg ? 128 : BN;
     const int64_t nrt = cdiv(n, BM);
     int64_t blocks = (nrt * 32 + 255) / 256;
     if (blocks > 152 * 8) blocks = 152 * 8;
     launch_dep(seg_tiles_kernel, (int)(blocks < 1 ? 1 : blocks), 256, 0, st, seg->group, seg->base, seg->nseg, n, nrt,
-                                                                    seg->ct0, seg->nct);
+               k, p.bn, seg->ct0, seg->nct);
     SKM_CUDA_TRY(launched());
     p.seg_ct0 = seg->ct0;
     p.seg_nct = seg->nct;
@@ -2626,7 +2674,7 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
         p.warm_shift = b.warm_shift;
         p.warm_ok = b.counters + 6;
     }
-    SKM_TRY(seg_setup(seg, n, p, st));
+    SKM_TRY(seg_setup(seg, n, k, p, st));
     if (!seg && b.scr_part) {
         p.ksplit = screen_split(n, k);
         p.part = b.scr_part;
@@ -2709,7 +2757,7 @@ int tc_assign_sq8(const skm_data *x, const uint8_t *C, int k, int32_t *nx_plain,
     p.nx = v.nx;
     p.nc = b.nc;
     p.dist = dist;
-    SKM_TRY(seg_setup(seg, n, p, st));
+    SKM_TRY(seg_setup(seg, n, k, p, st));
     SKM_TRY(launch_tc<MODE_SQ8>(v.xs, n, dp, d, b.cs, k, p, st));
     return SKM_OK;
 }
@@ -2750,7 +2798,7 @@ int tc_assign_rbq1(const skm_data *x, const float *C, int k, int32_t *assign, fl
         p.pk_words = words_of(d);
         p.pk_dp = dp;
     }
-    SKM_TRY(seg_setup(seg, n, p, st));
+    SKM_TRY(seg_setup(seg, n, k, p, st));
     SKM_TRY(launch_tc<MODE_RBQ1>(v.xs, n, dp, d, b.cs, k, p, st, v.packed));
     return SKM_OK;
 }
@@ -2784,7 +2832,7 @@ int tc_assign_lvq4(const skm_data *x, const float *C, int k, int32_t *assign, fl
         p.pk_words = lvq4_words(d);
         p.pk_dp = dp;
     }
-    SKM_TRY(seg_setup(seg, n, p, st));
+    SKM_TRY(seg_setup(seg, n, k, p, st));
     SKM_TRY(launch_tc<MODE_LVQ4>(v.xs, n, dp, d, b.cs, k, p, st, v.packed));
     return SKM_OK;
 }
