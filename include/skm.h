@@ -428,7 +428,7 @@ int skm_lvq4_exponent(const float *lvq, int64_t n, int *e_host, void *ws, size_t
  * its point tiles into a slot of the workspace, at most 160 x 4 x 128 x
  * round16(d) bytes), so the points occupy their code words in HBM instead of
  * round16(d) bytes; the copy saves that per-tile expansion (measured on
- * GB300, 1M x 768, k = 1000: LVQ4 0.63 ms packed, 0.52 ms from the copy).
+ * GB300, 1M x 768, k = 1000: LVQ4 0.57 ms packed, 0.48 ms from the copy).
  * Otherwise skm_assign builds the copy in its workspace on every call (d <=
  * 1024; longer rows are then assigned on CUDA cores). */
 size_t skm_screen_bytes(const skm_data *x);
