@@ -21,6 +21,7 @@
 //
 // 1-bit codes take a separate kernel (rows read straight into registers, bit
 // transposes and subset-sum tables; see "1-bit rows" below).
+#include <type_traits>
 #include <algorithm>
 
 #include "skm_internal.cuh"
@@ -678,17 +679,20 @@ __global__ void __launch_bounds__(RS_THREADS) direct_sum_sq8_kernel(
     cons.finish(lane);
 }
 
-// bf16 rows of at most 1 KB (d <= 512, d % 8 == 0) straight into registers
-// like the SQ8 rows: lane l loads the 16-byte groups l + 32 t (columns
-// 8 (l + 32 t) .. + 7) of a row, a whole row per load instruction of the warp,
-// with the next SQ8_PF rows' loads in flight while one is summed (one bulk
-// copy per 512-byte row left the copy engine, not HBM, as the limit).
-template <typename ACC, int NG>
+// bf16 rows of at most 1 KB (d <= 512) straight into registers like the SQ8
+// rows: lane l loads the groups l + 32 t of VEC columns of a row (VEC 8, one
+// 16-byte load, where d % 8 == 0; else 4, 8-byte loads, where d % 4 == 0), a
+// whole row per load instruction of the warp, with the next SQ8_PF rows' loads in
+// flight while one is summed (one bulk copy per 512-byte row left the copy
+// engine, not HBM, as the limit; rows of 100 or 300 columns, two bytes a lane
+// and two rows in flight: 338k x 100 343 us).
+template <typename ACC, int NG, int VEC>
 __global__ void __launch_bounds__(RS_THREADS) direct_sum_bf16_kernel(
     const uint16_t *__restrict__ X, int d, const int32_t *__restrict__ perm,
     const int32_t *__restrict__ scl, const int64_t *__restrict__ offsets, int k, ACC *__restrict__ S,
     int64_t stride, int run) {
     dep_sync();
+    using V = std::conditional_t<VEC == 8, uint4, uint2>;
     __shared__ int32_t sperm_all[RS_CW][RS_ROWS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t nval = offsets[k];
@@ -698,31 +702,31 @@ __global__ void __launch_bounds__(RS_THREADS) direct_sum_bf16_kernel(
     int32_t *sperm = sperm_all[warp];
     for (int i = lane; i < cnt; i += 32) sperm[i] = perm[q0 + i];
     __syncwarp();
-    const int ng = d >> 3;
-    auto load = [&](int r, uint4(&w)[NG]) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(X + (size_t)sperm[r] * d);
+    const int ng = d / VEC;
+    auto load = [&](int r, V(&w)[NG]) {
+        const V *src = reinterpret_cast<const V *>(X + (size_t)sperm[r] * d);
 #pragma unroll
         for (int t = 0; t < NG; ++t)
             if (lane + 32 * t < ng) w[t] = __ldg(src + lane + 32 * t);
     };
-    float acc[8 * NG];
+    float acc[VEC * NG];
 #pragma unroll
-    for (int t = 0; t < 8 * NG; ++t) acc[t] = 0.0f;
+    for (int t = 0; t < VEC * NG; ++t) acc[t] = 0.0f;
     auto flush = [&](int c) {
 #pragma unroll
         for (int t = 0; t < NG; ++t)
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int col = 8 * (lane + 32 * t) + u;
-                if (col < d) atomicAdd(S + (int64_t)c * stride + col, (ACC)acc[8 * t + u]);
-                acc[8 * t + u] = 0.0f;
+            for (int u = 0; u < VEC; ++u) {
+                const int col = VEC * (lane + 32 * t) + u;
+                if (col < d) atomicAdd(S + (int64_t)c * stride + col, (ACC)acc[VEC * t + u]);
+                acc[VEC * t + u] = 0.0f;
             }
     };
     // cluster ids of positions 32 b .. 32 b + 31 (lane-held), this and the next window
     int clw = lane < cnt ? __ldg(scl + q0 + lane) : -1;
     int cln = 32 + lane < cnt ? __ldg(scl + q0 + 32 + lane) : -1;
     int cur = __shfl_sync(0xffffffffu, clw, 0);
-    uint4 buf[SQ8_PF][NG];
+    V buf[SQ8_PF][NG];
 #pragma unroll
     for (int p = 0; p < SQ8_PF; ++p)
         if (p < cnt) load(p, buf[p]);
@@ -744,12 +748,11 @@ __global__ void __launch_bounds__(RS_THREADS) direct_sum_bf16_kernel(
 #pragma unroll
                 for (int t = 0; t < NG; ++t) {
                     if (lane + 32 * t < ng) {
-                        const uint4 w = buf[p][t];
-                        const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+                        const uint32_t *ww = reinterpret_cast<const uint32_t *>(&buf[p][t]);
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            acc[8 * t + 2 * u] += __uint_as_float(ww[u] << 16);
-                            acc[8 * t + 2 * u + 1] += __uint_as_float(ww[u] & 0xffff0000u);
+                        for (int u = 0; u < VEC / 2; ++u) {
+                            acc[VEC * t + 2 * u] += __uint_as_float(ww[u] << 16);
+                            acc[VEC * t + 2 * u + 1] += __uint_as_float(ww[u] & 0xffff0000u);
                         }
                     }
                 }
@@ -1009,7 +1012,15 @@ cudaError_t launch_float_nf(int nf, const void *X, int64_t n, int d, const int32
 
 }  // namespace
 
+// columns a load of the direct bf16 sums takes, 0: not such rows
+static int direct_bf16_vec(const void *X, int d) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(X);
+    if (d > 512) return 0;
+    return d % 8 == 0 && (a & 15u) == 0 ? 8 : d % 4 == 0 && (a & 7u) == 0 ? 4 : 0;
+}
+
 bool ring_sum_float_ok(const void *X, int x_is_bf16, int d) {
+    if (x_is_bf16 && direct_bf16_vec(X, d)) return true;
     RingLayout L;
     const uint32_t rb = (uint32_t)d * (x_is_bf16 ? 2u : 4u);
     return d % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0 && d <= 12 * 128 &&
@@ -1020,17 +1031,21 @@ cudaError_t launch_ring_sum_float(const void *X, int x_is_bf16, int64_t n, int d
                                   const int32_t *scl, const int64_t *offsets, int k, float *S_f,
                                   double *S_d, int32_t *flag, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    if (x_is_bf16 && d % 8 == 0 && d <= 512 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0) {
-        // rows of at most 1 KB: straight into registers
+    if (x_is_bf16 && direct_bf16_vec(X, d)) {
         const int run = sum_run(n, 16, SUM_WARPS);
         const unsigned g = ring_blocks(n, run);
         const uint16_t *Xb = static_cast<const uint16_t *>(X);
-        if (d <= 256) {
-            if (S_d) launch_dep(direct_sum_bf16_kernel<double, 1>, g, RS_THREADS, 0, st, Xb, d, perm, scl, offsets, k, S_d, d, run);
-            else launch_dep(direct_sum_bf16_kernel<float, 1>, g, RS_THREADS, 0, st, Xb, d, perm, scl, offsets, k, S_f, d, run);
+        auto go = [&](auto fd, auto ff) {
+            if (S_d) launch_dep(fd, g, RS_THREADS, 0, st, Xb, d, perm, scl, offsets, k, S_d, (int64_t)d, run);
+            else launch_dep(ff, g, RS_THREADS, 0, st, Xb, d, perm, scl, offsets, k, S_f, (int64_t)d, run);
+        };
+        if (direct_bf16_vec(X, d) == 8) {
+            if (d <= 256) go(direct_sum_bf16_kernel<double, 1, 8>, direct_sum_bf16_kernel<float, 1, 8>);
+            else go(direct_sum_bf16_kernel<double, 2, 8>, direct_sum_bf16_kernel<float, 2, 8>);
         } else {
-            if (S_d) launch_dep(direct_sum_bf16_kernel<double, 2>, g, RS_THREADS, 0, st, Xb, d, perm, scl, offsets, k, S_d, d, run);
-            else launch_dep(direct_sum_bf16_kernel<float, 2>, g, RS_THREADS, 0, st, Xb, d, perm, scl, offsets, k, S_f, d, run);
+            if (d <= 128) go(direct_sum_bf16_kernel<double, 1, 4>, direct_sum_bf16_kernel<float, 1, 4>);
+            else if (d <= 256) go(direct_sum_bf16_kernel<double, 2, 4>, direct_sum_bf16_kernel<float, 2, 4>);
+            else go(direct_sum_bf16_kernel<double, 4, 4>, direct_sum_bf16_kernel<float, 4, 4>);
         }
         return launched();
     }

@@ -94,3 +94,23 @@ def test_fit_objective_sum(skm, n):
                                      init_idx=torch.zeros(1, dtype=torch.int64, device=DEV))
     want = float(dist.double().sum())
     assert abs(obj[0] - want) <= max(n, 2) * 2.0 ** -52 * want
+
+
+@pytest.mark.parametrize("d", [64, 100, 101, 300, 512, 516, 515])
+@pytest.mark.parametrize("offset", [0, 4, 1])
+def test_bf16_sums_by_alignment(skm, d, offset):
+    """Rows that start on 16, 8 and 2 bytes; integer points, so that the sums are exact."""
+    n, k = 5003, 37
+    g = torch.Generator().manual_seed(d + offset)
+    X = torch.randint(-100, 101, (n, d), generator=g).float()
+    a = _assign(n, k, d)
+    ok = (a >= 0) & (a < k)
+    buf = torch.zeros(n * d + 8, dtype=torch.int16, device=DEV)
+    x = buf[offset : offset + n * d].view(n, d)
+    x.copy_(X.to(torch.bfloat16).view(torch.int16))
+    C0 = torch.randn(k, d, generator=g)
+    C, counts = skm.skm_update(skm.Points(skm.REPR_BF16, x, d), a.to(DEV), C0.to(DEV))
+    S = torch.zeros(k, d).index_add_(0, a[ok].long(), X[ok])
+    co = torch.bincount(a[ok].long(), minlength=k)
+    want = torch.where(co[:, None] > 0, S / co.clamp_min(1)[:, None].float(), C0)
+    assert torch.equal(counts.cpu(), co) and torch.equal(C.cpu(), want)
