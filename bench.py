@@ -326,7 +326,7 @@ def setup_head(dev, rank, world, dist, peaks):
     proj = {"ms": t_proj, "bound": "tensor", "achieved": flops / (t_proj / 1e3) / 1e12, "peak": peaks["bf16_tflops"],
             "unit": "TFLOP/s", "in_step": False,
             "algorithmic": f"6 bf16 part products x 2*N*D*d' = {flops:.3e} flop (fp32-accurate projection, "
-                           "one-time preparation; includes the split pass)"}
+                           "one-time preparation)"}
     proj["frac"] = proj["achieved"] / proj["peak"]
     return Yb, C, idx, proj
 
