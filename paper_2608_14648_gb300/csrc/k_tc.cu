@@ -1297,10 +1297,14 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                         // one rounding at most: rounding is monotone, so only a
                         // group of eight whose smallest rounded s is below (or,
                         // past 2^24, not above) the rounded best can hold a
-                        // smaller s; such a group is evaluated in integers
+                        // smaller s; below 2^24 the floats are exact and say
+                        // which column it is, else the group is evaluated in
+                        // integers (such a group always in integers: a step on
+                        // 969k x 96 against 1353 centroids 677 us, now 583)
 #pragma unroll
                         for (int g = 0; g < 4; ++g) {
                             float m = INFINITY;
+                            float e[8];
 #pragma unroll
                             for (int u = 0; u < 8; u += 4) {
                                 const int i = 8 * g + u;
@@ -1311,8 +1315,19 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                                 const float2 s1 = ffma2(make_float2(-2.0f, -2.0f), a1, make_float2(c4.z, c4.w));
                                 m = fmin3(m, s0.x, s0.y);
                                 m = fmin3(m, s1.x, s1.y);
+                                e[u] = s0.x;
+                                e[u + 1] = s0.y;
+                                e[u + 2] = s1.x;
+                                e[u + 3] = s1.y;
                             }
-                            if (m < fbest || (m == fbest && fabsf(m) >= 16777216.0f)) {
+                            if (!SEG && m < fbest && fabsf(m) < 16777216.0f) {
+                                int at = 7;
+#pragma unroll
+                                for (int u = 6; u >= 0; --u) at = e[u] == m ? u : at;
+                                fbest = m;
+                                best = __float2int_rn(m);
+                                besti = j0 + 8 * g + at;
+                            } else if (m < fbest || (m == fbest && fabsf(m) >= 16777216.0f)) {
 #pragma unroll
                                 for (int u = 0; u < 8; ++u) {
                                     const int i = 8 * g + u;
