@@ -1958,11 +1958,16 @@ __global__ void screen_prep_rbq1_kernel(const uint32_t *__restrict__ codes, int6
 }
 
 // ksplit > 1: the shares' states of a row merged in centroid order, then the
-// decision the epilogue takes otherwise.
+// decision the epilogue takes otherwise.  A share that gave up left no states:
+// no row is assigned then.
 __global__ void screen_merge_kernel(const TcParams p) {
     dep_sync();
     const int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (row >= p.n || p.counters[2]) return;  // (a share that gave up left no states)
+    if (row >= p.n) return;
+    if (p.counters[2]) {
+        p.assign[row] = -1;
+        return;
+    }
     ScreenRow sr;
     screen_init(sr);
     const float a2 = 2.0f * p.xinfo[row].x;
@@ -2072,17 +2077,21 @@ __global__ void rescore_kernel(const TX *__restrict__ X, int d, const float *__r
     }
 }
 
-// dist[r] = fp32 sum of squared differences to the assigned centroid.
+// dist[r] = fp32 sum of squared differences to the assigned centroid.  When the
+// screen gave up (counters[2]) rows may be left with whatever their assignment
+// held before: no centroid is read then, and every distance is +inf.
 template <typename TX>
 __global__ void assigned_dist_kernel(const TX *__restrict__ X, int64_t n, int d,
-                                     const float *__restrict__ C, const int32_t *__restrict__ assign,
-                                     float *__restrict__ dist) {
+                                     const float *__restrict__ C, int k, const int32_t *__restrict__ assign,
+                                     const int32_t *__restrict__ counters, float *__restrict__ dist) {
     dep_sync();
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const uint32_t valid = counters[2] ? 0u : (uint32_t)k;
     for (int64_t r = warp; r < n; r += nw) {
-        const float dd = warp_sqdist<TX>(X + r * d, C + (int64_t)assign[r] * d, d, lane);
+        const uint32_t j = (uint32_t)assign[r];
+        const float dd = j < valid ? warp_sqdist<TX>(X + r * d, C + (int64_t)j * d, d, lane) : INFINITY;
         if (lane == 0) dist[r] = dd;
     }
 }
@@ -2728,7 +2737,7 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
                                                   nullptr, b.fall_keys, b.cand, TCAND + 1, st));
         }
         if (dist) {
-            launch_dep(assigned_dist_kernel<uint16_t>, gw, 256, 0, st, X, n, d, C, assign, dist);
+            launch_dep(assigned_dist_kernel<uint16_t>, gw, 256, 0, st, X, n, d, C, k, assign, b.counters, dist);
             SKM_CUDA_TRY(launched());
         }
     } else {
@@ -2745,7 +2754,7 @@ int tc_assign_float(const skm_data *x, const float *C, int k, int32_t *assign, f
                                                   nullptr, b.fall_keys, b.cand, TCAND + 1, st));
         }
         if (dist) {
-            launch_dep(assigned_dist_kernel<float>, gw, 256, 0, st, X, n, d, C, assign, dist);
+            launch_dep(assigned_dist_kernel<float>, gw, 256, 0, st, X, n, d, C, k, assign, b.counters, dist);
             SKM_CUDA_TRY(launched());
         }
     }

@@ -1,0 +1,49 @@
+"""What a call leaves behind when a device wait runs out (the injected short wait,
+before anything is loaded): nothing is read through an assignment that was never
+written, and the next call is as before."""
+import pytest
+import torch
+
+import synth
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+WAIT = 4
+
+
+@pytest.fixture(scope="module")
+def skm(cuda_ok):
+    import paper_2608_14648_gb300 as skm
+
+    skm.lib()
+    yield skm
+    skm.skm_inject_fault(WAIT, 0)
+
+
+# centroid tiles shared out to several blocks; one tile; several tiles, one block a point tile
+@pytest.mark.parametrize("n,k,shared", [(2000, 1000, True), (2000, 200, False), (40000, 300, False)])
+@pytest.mark.parametrize("kind", ["f32", "bf16"])
+def test_distances_without_assignments(skm, kind, n, k, shared):
+    d = 64
+    X = synth.gmm_points(n, d, 30, seed=n + k).to(DEV)
+    if kind == "bf16":
+        p = skm.Points(skm.REPR_BF16, X.to(torch.bfloat16).view(torch.int16), d)
+    else:
+        p = skm.Points(skm.REPR_F32, X, d)
+    C = X[:k].clone()
+    ws = skm.workspace(skm.OP_ASSIGN, p, k)
+    a0, d0 = skm.skm_assign(p, C, ws=ws)
+    out = torch.full((n,), -1, dtype=torch.int32, device=DEV)
+    dist = torch.zeros(n, device=DEV)
+    skm.skm_inject_fault(WAIT, 1)
+    skm.skm_assign(p, C, ws=ws, out=out, dist_out=dist)
+    torch.cuda.synchronize()
+    assert skm.skm_fault_armed(WAIT) == 0
+    assert (out == -1).all() and torch.isinf(dist).all()
+    if shared:  # rows of shared tiles are set, whatever the array held
+        out.fill_(k - 1)
+        skm.skm_inject_fault(WAIT, 1)
+        skm.skm_assign(p, C, ws=ws, out=out, dist_out=dist)
+        assert (out == -1).all() and torch.isinf(dist).all()
+    a1, d1 = skm.skm_assign(p, C, ws=ws)
+    assert torch.equal(a1, a0) and torch.equal(d1, d0)
