@@ -802,7 +802,9 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
         while (sj >= 0) {
             const uint32_t i = sj == 0 ? ccnt[0]++ : ccnt[NS - 1]++;
             const uint32_t slot = i & 1u;
-            if (!mbar_wait(sfree_bar(sj, slot), ((i >> 1) & 1u) ^ 1u, abort_flag)) goto conv_done;
+            // (a vote: the shuffles below take the whole warp)
+            if (!__all_sync(0xffffffffu, mbar_wait(sfree_bar(sj, slot), ((i >> 1) & 1u) ^ 1u, abort_flag)))
+                goto conv_done;
             // the TMA's reads of the slot's previous tile before these writes
             asm volatile("fence.proxy.async.global;" ::: "memory");
             uint8_t *dst = p.pk_scratch + ((((size_t)blockIdx.x * NS + sj) * 2 + slot) * BM + RPW * cw) * p.pk_dp;

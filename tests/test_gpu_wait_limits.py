@@ -47,3 +47,28 @@ def test_distances_without_assignments(skm, kind, n, k, shared):
         assert (out == -1).all() and torch.isinf(dist).all()
     a1, d1 = skm.skm_assign(p, C, ws=ws)
     assert torch.equal(a1, a0) and torch.equal(d1, d0)
+
+
+# packed codes with three point tiles or more a job stream, so that the converter
+# warps come to wait for an expansion slot that is never freed
+@pytest.mark.parametrize("k", [30, 300])
+@pytest.mark.parametrize("kind", ["rbq1", "lvq4"])
+def test_packed_codes(skm, kind, k):
+    n, d = 152 * 128 * 7, 128
+    X = synth.gmm_points(n, d, 30, seed=k).to(DEV)
+    if kind == "rbq1":
+        p = skm.rbq1_points(skm.skm_quantize(skm.REPR_RBQ1, X), d)
+    else:
+        p = skm.lvq4_points(skm.skm_quantize(skm.REPR_LVQ4, X), d)
+    idx = synth.forgy_indices(n, k, seed=1).to(DEV)
+
+    def fit():
+        return skm.skm_fit(p, k, 1, init_idx=idx, want_objective=False, want_dist=False)[:2]
+
+    C0, a0 = fit()
+    skm.skm_inject_fault(WAIT, 1)
+    with pytest.raises(skm.SkmError) as ei:
+        fit()
+    assert ei.value.code == 5 and skm.skm_fault_armed(WAIT) == 0
+    C1, a1 = fit()
+    assert torch.equal(C1, C0) and torch.equal(a1, a0)
