@@ -213,10 +213,11 @@ int skm_version(void); /* major*10000 + minor*100 + patch */
  *  SKM_FAULT_STATUS     skm_fit's final read of its device status word finds
  *                       it set (the fault writes it on the device), so the
  *                       call returns SKM_ERR_DEVICE_CHECK;
- *  SKM_FAULT_WAIT       a tensor-core assignment launch starts with a 1 ms
- *                       bounded wait on a barrier that nothing arrives on: it
- *                       gives up before loading anything, raises its abort
- *                       flag, and skm_fit reports SKM_ERR_TIMEOUT.
+ *  SKM_FAULT_WAIT       a tensor-core assignment or projection launch starts
+ *                       with a 1 ms bounded wait on a barrier that nothing
+ *                       arrives on: it gives up before loading anything and
+ *                       raises its abort flag; skm_fit reports
+ *                       SKM_ERR_TIMEOUT, skm_project leaves NaN in Y.
  * The environment variable SKM_FAULT=workspace|launch|status|wait arms one
  * occurrence when the library first checks.  Nothing faults the GPU: every
  * injected failure is a status the host reads.  Returns SKM_OK, or
@@ -253,7 +254,8 @@ size_t skm_workspace_size(int op, const skm_data *x, int k);
  * the six products with i + j <= 4 are accumulated in fp32, the five small ones
  * apart from x1 p1 (the three left out are below 2^-24 relative).  The
  * workspace holds P's parts; X's are formed on the fly.  ws == NULL (or smaller): an
- * fp32 CUDA-core tile GEMM.  Asynchronous. */
+ * fp32 CUDA-core tile GEMM.  Asynchronous; device waits are bounded (2 s), and
+ * the part of Y that a wait which ran out kept from being formed is NaN. */
 int skm_project(const float *X, int64_t n, int d, const float *mean, const float *P,
                 int d_out, int out_dtype, void *Y, void *ws, size_t ws_bytes, void *stream);
 

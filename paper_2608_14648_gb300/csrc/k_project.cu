@@ -62,6 +62,7 @@ struct ProjParams {
     int vec;            // X rows and the mean can be read 16 bytes at a time
     int yvec;           // Y is 16-byte aligned
     int32_t *abort_flag;
+    unsigned long long inject_wait_ns;  // fault injection: see mbar_wait below
 };
 
 // fp32 v -> bf16 parts v1 + v2 + v3 (each the round-to-nearest-even bf16 of
@@ -103,8 +104,9 @@ __global__ void __launch_bounds__(THREADS, 1) project_tc_kernel(const __grid_con
     auto bempty = [&](uint32_t s) { return bar0 + 8u * (B_SLOTS + s); };
     auto afull = [&](uint32_t s) { return bar0 + 8u * (2 * B_SLOTS + s); };
     auto aempty = [&](uint32_t s) { return bar0 + 8u * (2 * B_SLOTS + A_BUFS + s); };
-    const uint32_t tfull = bar0 + 8u * (2 * B_SLOTS + 2 * A_BUFS), tempty = tfull + 8u, drain_bar = tfull + 16u;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * B_SLOTS + 2 * A_BUFS + 3);
+    const uint32_t tfull = bar0 + 8u * (2 * B_SLOTS + 2 * A_BUFS), tempty = tfull + 8u, drain_bar = tfull + 16u,
+                   inject_bar = tfull + 24u;  // (nothing arrives on the last)
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * B_SLOTS + 2 * A_BUFS + 4);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int32_t *abort_flag = p.abort_flag;
 
@@ -120,6 +122,7 @@ __global__ void __launch_bounds__(THREADS, 1) project_tc_kernel(const __grid_con
         mbar_init(tfull, 1);
         mbar_init(tempty, EPI_WARPS);
         mbar_init(drain_bar, 1);
+        mbar_init(inject_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
     }
@@ -139,6 +142,7 @@ __global__ void __launch_bounds__(THREADS, 1) project_tc_kernel(const __grid_con
     if (warp == 0) {
         if (lane == 0) {  // ---------------------------------------- TMA producer
             uint32_t it = 0;
+            if (p.inject_wait_ns && !mbar_wait(inject_bar, 0u, abort_flag, p.inject_wait_ns)) goto producer_done;
             for (int64_t t = t0; t < p.ntiles; t += tstep) {
                 const int col0 = (int)(t % p.nct) * p.ncols;
                 for (int kc = 0; kc < p.nslices; ++kc)
@@ -205,11 +209,14 @@ __global__ void __launch_bounds__(THREADS, 1) project_tc_kernel(const __grid_con
         const int half = (warp - 2) >> 2;          // which half of the 32-column groups
         const int groups = (p.ncols + 31) / 32;
         uint32_t tiles = 0;
+        // a wait ran out: this tile and those after it are written as NaN, so that
+        // whoever reads Y sees it (the call has long returned)
+        bool gave_up = false;
         for (int64_t t = t0; t < p.ntiles; t += tstep, ++tiles) {
             const int64_t row = (t / p.nct) * PM + q * 32 + lane;
             const int col0 = (int)(t % p.nct) * p.ncols;
             const int colw = min(p.ncols, p.dout - col0);
-            if (!__all_sync(0xffffffffu, mbar_wait(tfull, tiles & 1u, abort_flag))) break;
+            if (!gave_up) gave_up = !__all_sync(0xffffffffu, mbar_wait(tfull, tiles & 1u, abort_flag));
             tc_fence_after();
             const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16);
 #pragma unroll 1
@@ -219,7 +226,8 @@ __global__ void __launch_bounds__(THREADS, 1) project_tc_kernel(const __grid_con
                 tmem_ld32(taddr + PN + 32 * g, w);
 #pragma unroll
                 for (int i = 0; i < 32; ++i)
-                    v[i] = __float_as_uint(__fadd_rn(__uint_as_float(v[i]), __uint_as_float(w[i])));
+                    v[i] = gave_up ? 0x7fffffffu
+                                   : __float_as_uint(__fadd_rn(__uint_as_float(v[i]), __uint_as_float(w[i])));
                 const int c0 = 32 * g, cn = row < p.n ? min(32, colw - c0) : 0;
                 if (cn <= 0) {
                     // nothing of this group inside Y
@@ -257,7 +265,7 @@ __global__ void __launch_bounds__(THREADS, 1) project_tc_kernel(const __grid_con
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(tempty);
+            if (lane == 0 && !gave_up) mbar_arrive(tempty);  // (no accumulator is handed on unread)
         }
     } else {  // ------------------------------------------------------- converters
         // thread ct: dimensions 8 c .. 8 c + 7 (c = ct mod 8) of the slice, rows
@@ -407,6 +415,7 @@ int tc_project(const float *X, int64_t n, int d, const float *mean, const float 
     p.vec = d % 4 == 0 && ((uintptr_t)X & 15) == 0 && ((uintptr_t)mean & 15) == 0;
     p.yvec = ((uintptr_t)Y & 15) == 0;
     p.abort_flag = flag;
+    p.inject_wait_ns = fault_take(SKM_FAULT_WAIT) ? 1000000ull : 0ull;  // 1 ms
     CUtensorMap mb;
     SKM_TRY(make_map(&mb, B, (int64_t)PARTS * dout, d, dp, p.ncols, 2));
     SKM_CUDA_TRY(cudaFuncSetAttribute(project_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM));

@@ -72,3 +72,23 @@ def test_packed_codes(skm, kind, k):
     assert ei.value.code == 5 and skm.skm_fault_armed(WAIT) == 0
     C1, a1 = fit()
     assert torch.equal(C1, C0) and torch.equal(a1, a0)
+
+
+# one tile; several row and column tiles a block; more tiles than blocks
+@pytest.mark.parametrize("n,d,dout", [(100, 64, 16), (3000, 600, 300), (152 * 128 * 2 + 5, 128, 48)])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_projection(skm, bf16, n, d, dout):
+    g = torch.Generator().manual_seed(d)
+    X, P = torch.randn(n, d, generator=g).to(DEV), torch.randn(d, dout, generator=g).to(DEV)
+    dt = skm.DTYPE_BF16 if bf16 else skm.DTYPE_F32
+
+    def project():
+        Y = skm.skm_project(X, P, out_dtype=dt)
+        return Y.view(torch.bfloat16) if bf16 else Y
+
+    want = project()
+    assert torch.isfinite(want).all()
+    skm.skm_inject_fault(WAIT, 1)
+    assert torch.isnan(project()).all()
+    assert skm.skm_fault_armed(WAIT) == 0
+    assert torch.equal(project(), want)
