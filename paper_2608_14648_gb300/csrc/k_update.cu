@@ -798,6 +798,11 @@ cudaError_t launch_stable_sort(const int32_t *key, int64_t n, int m, int32_t *hi
     ss_hist_kernel<<<nblk, 256, sm, st>>>(key, n, m, hist);
     cudaError_t e = launched();
     if (e != cudaSuccess) return e;
+    // with the most groups the counters are 48 KiB, and the kernel's own words come
+    // on top (the limit belongs to the process: always the largest any call needs)
+    constexpr int SS_MAX_M = 12288;
+    e = cudaFuncSetAttribute(ss_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(int32_t) * SS_MAX_M);
+    if (e != cudaSuccess) return e;
     ss_scan_kernel<<<1, 1024, sm, st>>>(hist, nblk, m, sizes);
     e = launched();
     if (e != cudaSuccess) return e;
