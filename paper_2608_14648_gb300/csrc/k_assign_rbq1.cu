@@ -155,12 +155,7 @@ cudaError_t launch_assign_rbq1_sym(const uint32_t *codes, const float *nx2, cons
                                    const uint32_t *yw, const Rbq1CInfo *info, int k, int32_t *assign, float *dist,
                                    cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    const size_t smem = (size_t)SYM_KT * ((d + 31) >> 5) * sizeof(uint32_t);
-    if (smem > 48 * 1024) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(assign_rbq1_sym_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const size_t smem = (size_t)SYM_KT * ((d + 31) >> 5) * sizeof(uint32_t);  // at most 16 KiB
     assign_rbq1_sym_kernel<<<(unsigned)((n + RBQ1_THREADS - 1) / RBQ1_THREADS), RBQ1_THREADS, smem, st>>>(
         codes, nx2, F, n, d, yw, info, k, assign, dist);
     return launched();
@@ -174,13 +169,13 @@ cudaError_t launch_assign_rbq1(const uint32_t *codes, const float *nx2, const fl
     const int W = (d + 31) >> 5;
     const size_t xs_bytes = (size_t)W * RBQ1_THREADS * 4;
     const size_t per_c = (size_t)W * 16 + sizeof(Rbq1CInfo);
-    const size_t budget = 96 * 1024;
+    constexpr size_t budget = 96 * 1024;  // more than 4 centroids and the points' words take at any d
+    static_assert(4 * (MAX_D / 32 * 16 + sizeof(Rbq1CInfo)) + MAX_D / 32 * RBQ1_THREADS * 4 <= budget, "");
     int kc = (int)((budget > xs_bytes ? budget - xs_bytes : per_c) / per_c);
     kc = max(4, min(kc, 256));
     kc = min(kc, max(4, k));
     const size_t smem = (size_t)kc * per_c + xs_bytes + 16;
-    cudaError_t e = cudaFuncSetAttribute(assign_rbq1_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = smem_limit(assign_rbq1_kernel, budget + 16);
     if (e != cudaSuccess) return e;
     assign_rbq1_kernel<<<(unsigned)((n + RBQ1_THREADS - 1) / RBQ1_THREADS), RBQ1_THREADS, smem,
                          st>>>(codes, nx2, F, popx, n, d, planes, info, k, kc, assign, dist);

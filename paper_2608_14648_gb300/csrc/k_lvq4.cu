@@ -476,7 +476,7 @@ cudaError_t launch_assign_lvq4_simt(const uint32_t *codes, const float4 *fac, in
     const size_t smem = (size_t)SA_KT * 2 * lvq4_words(d) * sizeof(uint32_t);
     if (smem > 48 * 1024) {
         const cudaError_t e =
-            cudaFuncSetAttribute(assign_lvq4_simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            smem_limit(assign_lvq4_simt_kernel, (size_t)SA_KT * 2 * lvq4_words(MAX_D) * sizeof(uint32_t));
         if (e != cudaSuccess) return e;
     }
     assign_lvq4_simt_kernel<<<(unsigned)((n + 255) / 256), 256, smem, st>>>(codes, fac, n, d, yw, info, k, assign,

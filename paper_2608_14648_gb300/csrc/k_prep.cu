@@ -151,8 +151,8 @@ static cudaError_t launch_cprep_common(const float *C, int k, int d, const float
                                        Rbq1CInfo *info, uint8_t *yq, int dq, const CodePairs &pairs, cudaStream_t st) {
     const size_t smem = (size_t)CPREP_WARPS * (words_of(d) * sizeof(double) + d * sizeof(float));
     if (smem > 48 * 1024 - 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(
-            rbq1_cprep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = smem_limit(
+            rbq1_cprep_kernel, (size_t)CPREP_WARPS * (words_of(MAX_D) * sizeof(double) + MAX_D * sizeof(float)));
         if (e != cudaSuccess) return e;
     }
     const int rows = k > pairs.kp ? k : pairs.kp;

@@ -418,7 +418,7 @@ int tc_project(const float *X, int64_t n, int d, const float *mean, const float 
     p.inject_wait_ns = fault_take(SKM_FAULT_WAIT) ? 1000000ull : 0ull;  // 1 ms
     CUtensorMap mb;
     SKM_TRY(make_map(&mb, B, (int64_t)PARTS * dout, d, dp, p.ncols, 2));
-    SKM_CUDA_TRY(cudaFuncSetAttribute(project_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM));
+    SKM_CUDA_TRY(smem_limit(project_tc_kernel, SMEM));
     const int grid = (int)std::min<int64_t>(device_sms(), p.ntiles);
     tc_timer_mark(st, 0);
     project_tc_kernel<<<grid, THREADS, SMEM, st>>>(mb, p);

@@ -945,24 +945,27 @@ cudaError_t launch_prune_assign_sq8(const uint8_t *X, int64_t n, int d, const ui
     return launched();
 }
 
+// shared memory of prune_tiled_kernel
+static size_t tiled_bytes(int d) {
+    const int dx = (d + 31) & ~31, dp = dx + 4;
+    return ((size_t)TP_KC * dp + (size_t)TP_PTS * dx + 2 * TP_PTS) * sizeof(float);
+}
+
 cudaError_t launch_prune_assign(const void *X, int x_is_bf16, int64_t n, int d, const float *C,
                                 int k, const int32_t *prev, int32_t *assign, float *dist,
                                 unsigned long long *counters, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     if (d <= TP_MAX_D_F32 && (reinterpret_cast<uintptr_t>(C) & 15) == 0) {
-        const int dx = (d + 31) & ~31, dp = dx + 4;
-        const size_t smem = ((size_t)TP_KC * dp + (size_t)TP_PTS * dx + 2 * TP_PTS) * sizeof(float);
+        const size_t smem = tiled_bytes(d);
         const int64_t blocks = (n + TP_PTS - 1) / TP_PTS;
         if (x_is_bf16) {
-            cudaError_t e = cudaFuncSetAttribute(prune_tiled_kernel<uint16_t, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem);
+            cudaError_t e = smem_limit(prune_tiled_kernel<uint16_t, false>, tiled_bytes(TP_MAX_D_F32));
             if (e != cudaSuccess) return e;
             prune_tiled_kernel<uint16_t, false><<<(unsigned)blocks, TP_WARPS * 32, smem, st>>>(
                 static_cast<const uint16_t *>(X), n, d, C, k, prev, assign, dist, counters, nullptr, nullptr, 0,
                 nullptr, nullptr, nullptr);
         } else {
-            cudaError_t e = cudaFuncSetAttribute(prune_tiled_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem);
+            cudaError_t e = smem_limit(prune_tiled_kernel<float, false>, tiled_bytes(TP_MAX_D_F32));
             if (e != cudaSuccess) return e;
             prune_tiled_kernel<float, false><<<(unsigned)blocks, TP_WARPS * 32, smem, st>>>(
                 static_cast<const float *>(X), n, d, C, k, prev, assign, dist, counters, nullptr, nullptr, 0,
@@ -978,8 +981,7 @@ cudaError_t launch_prune_assign(const void *X, int x_is_bf16, int64_t n, int d, 
     cudaError_t e = cudaSuccess;
     if (x_is_bf16) {
         if (stg) {
-            e = cudaFuncSetAttribute(prune_assign_kernel<uint16_t, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     stg_bytes);
+            e = smem_limit(prune_assign_kernel<uint16_t, true>, stg_bytes);
             if (e != cudaSuccess) return e;
             prune_assign_kernel<uint16_t, true><<<(int)blocks, PR_WARPS * 32, stg_bytes, st>>>(
                 static_cast<const uint16_t *>(X), n, d, C, k, prev, assign, dist, counters);
@@ -989,8 +991,7 @@ cudaError_t launch_prune_assign(const void *X, int x_is_bf16, int64_t n, int d, 
         }
     } else {
         if (stg) {
-            e = cudaFuncSetAttribute(prune_assign_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     stg_bytes);
+            e = smem_limit(prune_assign_kernel<float, true>, stg_bytes);
             if (e != cudaSuccess) return e;
             prune_assign_kernel<float, true><<<(int)blocks, PR_WARPS * 32, stg_bytes, st>>>(
                 static_cast<const float *>(X), n, d, C, k, prev, assign, dist, counters);
@@ -1015,17 +1016,15 @@ cudaError_t launch_prune_rows_cta(const uint16_t *X, int d, const float *C, int 
     if ((d % 4) != 0 || (reinterpret_cast<uintptr_t>(C) & 15) != 0 || (int64_t)k * d > (1LL << 26))
         return cudaErrorInvalidValue;
     const int stg_bytes = PRC_WARPS * 32 * STG_LD * (int)sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(prune_rows_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, stg_bytes);
+    cudaError_t e = smem_limit(prune_rows_cta_kernel, stg_bytes);
     if (e != cudaSuccess) return e;
     prune_rows_cta_kernel<<<152 * 3, PRC_WARPS * 32, stg_bytes, st>>>(X, d, C, k, r.seed, r.thr, r.wrow, rows, nrows,
                                                                       assign, dist, counters,
                                                                       tiled ? LONG_LIST : INT_MAX);
     e = launched();
     if (e != cudaSuccess || !tiled) return e;
-    const int dx = (d + 31) & ~31, dp = dx + 4;
-    const size_t smem = ((size_t)TP_KC * dp + (size_t)TP_PTS * dx + 2 * TP_PTS) * sizeof(float);
-    e = cudaFuncSetAttribute(prune_tiled_kernel<uint16_t, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+    const size_t smem = tiled_bytes(d);
+    e = smem_limit(prune_tiled_kernel<uint16_t, true>, tiled_bytes(TP_MAX_D_F32));
     if (e != cudaSuccess) return e;
     prune_tiled_kernel<uint16_t, true><<<152, TP_WARPS * 32, smem, st>>>(X, 0, d, C, k, nullptr, assign, dist, counters,
                                                                     rows, nrows, LONG_LIST, r.seed, r.thr, r.wrow);

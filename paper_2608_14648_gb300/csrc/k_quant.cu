@@ -744,7 +744,7 @@ cudaError_t launch_mean_fixed(const float *X, int64_t n, int d, void *ws, float 
         const int threads = d4 < MEAN_THREADS ? (phases * d4 + 31) / 32 * 32 : MEAN_THREADS;
         const size_t smem = 2 * sizeof(unsigned long long) * (size_t)d;
         if (smem > 48 * 1024) {
-            e = cudaFuncSetAttribute(mean_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            e = smem_limit(mean_pass_kernel, 2 * sizeof(unsigned long long) * MAX_D);
             if (e != cudaSuccess) return e;
         }
         mean_pass_kernel<<<152 * 2, threads, smem, st>>>(reinterpret_cast<const float4 *>(X), n, d4, lg, ms, SA, SB);

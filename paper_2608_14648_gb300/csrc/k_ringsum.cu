@@ -108,6 +108,9 @@ struct RingLayout {
     }
 };
 
+// of any row size (the rings of a CTA take at most RS_RING_BYTES, see ring_layout)
+constexpr size_t RS_SMEM_MAX = RS_RING_BYTES + (size_t)RS_CW * RS_MAX_SLOTS * 8 + (size_t)RS_CW * RS_ROWS * 4;
+
 // Gather loop shared by every row type.  A warp calls cons.start(q0, cnt,
 // lane) before the first row of its run (positions q0 .. q0 + cnt - 1),
 // cons.row(i, row, lane) for its i-th row (in shared memory), and
@@ -993,7 +996,7 @@ cudaError_t launch_float_nf(int nf, const void *X, int64_t n, int d, const int32
 #define RS_CASE(NFV)                                                                                \
     case NFV: {                                                                                     \
         auto kern = ring_sum_float_kernel<BF16, ACC, NFV>;                                          \
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+        cudaError_t e = smem_limit(kern, RS_SMEM_MAX);                                              \
         if (e != cudaSuccess) return e;                                                             \
         launch_dep(kern, g, RS_THREADS, smem, st, X, d, perm, scl, offsets, k, S, d, L, flag);               \
         return launched();                                                                          \
@@ -1087,7 +1090,7 @@ cudaError_t launch_ring_sum_sq8(const uint8_t *codes, int64_t n, int d, const in
 #define RS_CASE(NGV)                                                                                \
     if (q <= NGV) {                                                                                 \
         auto kern = ring_sum_sq8_kernel<NGV>;                                                       \
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+        cudaError_t e = smem_limit(kern, RS_SMEM_MAX);                                              \
         if (e != cudaSuccess) return e;                                                             \
         launch_dep(kern, g, RS_THREADS, smem, st, codes, d, perm, scl, offsets, k, S64, L, flag);            \
         return launched();                                                                          \

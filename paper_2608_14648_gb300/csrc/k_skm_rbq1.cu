@@ -386,12 +386,7 @@ cudaError_t launch_rbq1_seg_cprep(const float *C, int k, int d, const float *m, 
     rbq1_seg_bounds(d, &d1, &d2);
     const float i0 = (float)(1.0 / sqrt((double)d1)), i1 = (float)(1.0 / sqrt((double)(d2 - d1))),
                 i2 = (float)(1.0 / sqrt((double)(d - d2)));
-    const size_t smem = (size_t)SEG_CPREP_WARPS * d * sizeof(float);
-    if (smem > 48 * 1024) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(rbq1_seg_cprep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const size_t smem = (size_t)SEG_CPREP_WARPS * d * sizeof(float);  // at most 16 KiB (d <= 1024)
     rbq1_seg_cprep_kernel<<<(k + SEG_CPREP_WARPS - 1) / SEG_CPREP_WARPS, SEG_CPREP_WARPS * 32, smem, st>>>(
         C, k, d, m, d1, d2, i0, i1, i2, planes, info);
     return launched();
@@ -407,10 +402,12 @@ cudaError_t launch_assign_rbq1_seg(const uint32_t *codes, const float *nx2s, con
     float g[2];
     rbq1_seg_factors(d, d1, d2, g);
     const int W = (d + 31) >> 5;
-    const size_t smem = (size_t)SEG_KC * (W + 1) * sizeof(uint4) + (size_t)SEG_KC * sizeof(Rbq1SegInfo) +
-                        (size_t)SEG_PTS * W * sizeof(uint32_t) + (size_t)SEG_PTS * 16;
-    const cudaError_t e =
-        cudaFuncSetAttribute(assign_rbq1_seg_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto bytes = [](int words) {
+        return (size_t)SEG_KC * (words + 1) * sizeof(uint4) + (size_t)SEG_KC * sizeof(Rbq1SegInfo) +
+               (size_t)SEG_PTS * words * sizeof(uint32_t) + (size_t)SEG_PTS * 16;
+    };
+    const size_t smem = bytes(W);
+    const cudaError_t e = smem_limit(assign_rbq1_seg_kernel, bytes(SEG_MAXW));
     if (e != cudaSuccess) return e;
     const int64_t blocks = (n + SEG_PTS - 1) / SEG_PTS;
     assign_rbq1_seg_kernel<<<(unsigned)blocks, SEG_WARPS * 32, smem, st>>>(

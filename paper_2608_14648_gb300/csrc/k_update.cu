@@ -265,8 +265,7 @@ cudaError_t launch_sort_by_cluster(const int32_t *assign, int64_t n, int k, int3
     if (n <= SORT1_MAX && k <= SORT1_MAX_K) {
         const size_t smem = sizeof(int32_t) * (size_t)k + 4 * (size_t)n;  // at most 176 KiB
         if (smem > 48 * 1024 - 512) {
-            const cudaError_t e = cudaFuncSetAttribute(sort_one_block_kernel,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            const cudaError_t e = smem_limit(sort_one_block_kernel, sizeof(int32_t) * SORT1_MAX_K + 4 * SORT1_MAX);
             if (e != cudaSuccess) return e;
         }
         launch_dep(sort_one_block_kernel, 1 + clear, 1024, smem, st, 
@@ -799,9 +798,9 @@ cudaError_t launch_stable_sort(const int32_t *key, int64_t n, int m, int32_t *hi
     cudaError_t e = launched();
     if (e != cudaSuccess) return e;
     // with the most groups the counters are 48 KiB, and the kernel's own words come
-    // on top (the limit belongs to the process: always the largest any call needs)
+    // on top
     constexpr int SS_MAX_M = 12288;
-    e = cudaFuncSetAttribute(ss_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(int32_t) * SS_MAX_M);
+    e = smem_limit(ss_scan_kernel, sizeof(int32_t) * SS_MAX_M);
     if (e != cudaSuccess) return e;
     ss_scan_kernel<<<1, 1024, sm, st>>>(hist, nblk, m, sizes);
     e = launched();

@@ -69,7 +69,6 @@ int set_error(int code, const char *fmt, ...) {
 
 static inline cudaStream_t S(void *s) { return static_cast<cudaStream_t>(s); }
 
-constexpr int MAX_D = 4096;
 constexpr int MAX_K = 65536;
 constexpr int64_t MAX_N = (int64_t(1) << 31) - 1;
 constexpr int64_t MAX_N_RBQ1 = int64_t(1) << 24;

@@ -44,6 +44,8 @@ void tc_timer_mark(cudaStream_t st, int which);
 // ---- workspace carving ------------------------------------------------------
 // Sub-buffers are carved from the caller's workspace at 256-byte boundaries.
 // With base == nullptr the carver only measures (used by skm_workspace_size).
+constexpr int MAX_D = 4096;  // dimensions of a point, at most
+
 struct Carver {
     char *base;
     size_t off = 0;
@@ -89,6 +91,15 @@ inline void launch_dep(void (*kern)(K...), dim3 grid, dim3 block, size_t smem, c
     cfg.attrs = &at;
     cfg.numAttrs = (uint64_t)grid.x * grid.y <= 2 * 152 ? 1 : 0;
     (void)cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);  // the caller checks launched()
+}
+
+// Lets `kern` take up to `most` bytes of dynamic shared memory.  The limit belongs
+// to the process, not to a call: `most` is the largest that any call of the
+// kernel asks for, so that calls of several threads all write the same value
+// (each call's own size could be lowered again between this and its launch).
+template <typename... K>
+inline cudaError_t smem_limit(void (*kern)(K...), size_t most) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
 inline int words_of(int d) { return (d + 31) / 32; }
