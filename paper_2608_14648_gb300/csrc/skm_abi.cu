@@ -1289,7 +1289,18 @@ int skm_fit(const skm_fit_config *cfg, const skm_data *x, const void *C_init,
     int32_t *assign = assign_out;
     bool pruning = false;                 // adaptive: the pruned assignment is in use
     unsigned long long surv_seen = 0;     // adaptive: front survivors counted so far
-    for (int it = 0; it <= cfg->iters; ++it) {
+    // Objective values are kept on the device and read back OBJ_LOG at a time (a
+    // copy to the caller's pageable array would wait for every iteration), and
+    // before a return with an error, so that every finished iteration's is written.
+    int obj_formed = 0, obj_read = 0;
+    auto read_objective = [&]() -> cudaError_t {
+        const int from = obj_read, count = obj_formed - obj_read;
+        obj_read = obj_formed;
+        return count == 0 ? cudaSuccess
+                          : cudaMemcpyAsync(objective_host + from, b.sum + from % OBJ_LOG, sizeof(double) * (size_t)count,
+                                            cudaMemcpyDeviceToHost, st);
+    };
+    auto iterate = [&](int it) -> int {
         const bool want_obj = objective_host != nullptr;
         float *dist_it = (want_obj || it == cfg->iters) ? dist : nullptr;
         if (adaptive && !pruning) {
@@ -1318,20 +1329,24 @@ int skm_fit(const skm_fit_config *cfg, const skm_data *x, const void *C_init,
             }
         }
         if (want_obj) {
-            // kept on the device and read back OBJ_LOG at a time: a copy to the
-            // caller's pageable array would wait for every iteration
-            const int slot = it % OBJ_LOG;
-            SKM_CUDA_TRY(launch_sum_float(dist, n, b.partials, nblk, b.ticket, b.sum + slot, st));
-            if (slot == OBJ_LOG - 1 || it == cfg->iters)
-                SKM_CUDA_TRY(cudaMemcpyAsync(objective_host + (it - slot), b.sum, sizeof(double) * (size_t)(slot + 1),
-                                             cudaMemcpyDeviceToHost, st));
+            SKM_CUDA_TRY(launch_sum_float(dist, n, b.partials, nblk, b.ticket, b.sum + it % OBJ_LOG, st));
+            obj_formed = it + 1;
+            if (obj_formed % OBJ_LOG == 0 || it == cfg->iters) SKM_CUDA_TRY(read_objective());
         }
-        if (it == cfg->iters) break;
+        if (it == cfg->iters) return SKM_OK;
         SKM_TRY(do_update(&xd, assign, k, C_out, b.counts, nullptr, e, b.u, st,
                           it < EMPTY_LOG ? b.empty_iter + it : nullptr));
         if (cfg->empty_policy == SKM_EMPTY_SPLIT)
             SKM_CUDA_TRY(launch_split_empty(C_out, x->repr == SKM_REPR_SQ8 ? 1 : 4, b.counts, k, x->d,
                                             b.u.wsplit, st));
+        return SKM_OK;
+    };
+    for (int it = 0; it <= cfg->iters; ++it) {
+        const int rc = iterate(it);
+        if (rc != SKM_OK) {
+            if (read_objective() != cudaSuccess) (void)cudaGetLastError();  // the first error is the one reported
+            return rc;
+        }
     }
     if (fault_take(SKM_FAULT_STATUS)) SKM_CUDA_TRY(cudaMemsetAsync(b.status, 0xff, sizeof(int), st));
     {
