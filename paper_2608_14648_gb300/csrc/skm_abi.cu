@@ -277,7 +277,7 @@ struct FitBufs {
     int64_t *empty_iter = nullptr;  // empty clusters after each update (first EMPTY_LOG iterations)
 };
 
-static void plan_fit(const skm_data *x, int k, Carver &cv, FitBufs &b) {
+static void plan_fit(const skm_data *x, int k, Carver &cv, FitBufs &b, bool extra = true) {
     skm_data xs = *x;
     if (x->repr == SKM_REPR_F32 || x->repr == SKM_REPR_BF16) xs.flags |= SKM_FLAG_WARM;  // as skm_fit
     // 1-bit codes the tensor-core kernel reads packed: no copy of the points
@@ -308,7 +308,7 @@ static void plan_fit(const skm_data *x, int k, Carver &cv, FitBufs &b) {
     b.counts = cv.take<int64_t>(k);
     b.init_idx = cv.take<int64_t>(k);  // seeded Forgy indices (host-drawn)
     b.empty_iter = cv.take<int64_t>(EMPTY_LOG);
-    plan_assign_extra(x, k, cv, b.a.tc);
+    if (extra) plan_assign_extra(x, k, cv, b.a.tc);
 }
 
 static int need_ws(const Carver &cv, size_t ws_bytes, void *ws) {
@@ -506,11 +506,7 @@ size_t skm_workspace_size(int op, const skm_data *x, int k) {
     Carver cv(nullptr, 0);
     switch (op) {
     case 0: {
-        if (check_data(x, false) || check_k(x, k)) return 0;
-        AssignBufs b;
-        plan_assign(x, k, cv, b);
-        plan_assign_extra(x, k, cv, b.tc);
-        break;
+        return assign_ws_bytes(x, k, true);
     }
     case 1: {
         if (check_data(x, false) || check_k(x, k)) return 0;
@@ -942,12 +938,14 @@ struct HierBufs {
     int *e_dev = nullptr;
 };
 
-static void plan_hier(const skm_data *x, int k, int m, Carver &cv, HierBufs &b) {
+// extra: with the meso fit's buffers that only make it faster (see
+// plan_assign_extra); a workspace too small for them does without
+static void plan_hier(const skm_data *x, int k, int m, Carver &cv, HierBufs &b, bool extra = true) {
     const int64_t n = x->n;
     {
         Carver mc(nullptr, 0);
         FitBufs fb;
-        plan_fit(x, m, mc, fb);
+        plan_fit(x, m, mc, fb, extra);
         b.meso_ws_bytes = mc.off;
     }
     b.meso_ws = cv.take<uint8_t>(b.meso_ws_bytes);
@@ -1040,6 +1038,10 @@ int skm_fit_hierarchical(const skm_hier_config *cfg, const skm_data *x, const in
     Carver cv(ws, ws_bytes);
     HierBufs b;
     plan_hier(x, k, m, cv, b);
+    if (!cv.fits()) {
+        cv = Carver(ws, ws_bytes);
+        plan_hier(x, k, m, cv, b, false);
+    }
     SKM_TRY(need_ws(cv, ws_bytes, ws));
 
     // MESO-CLUSTERING: Lloyd with m clusters from the given Forgy indices
@@ -1439,6 +1441,15 @@ int skm_sq8_decode(const uint8_t *codes, int64_t n, int d, const float *b, const
 }  // extern "C"
 
 namespace skm {
+
+size_t assign_ws_bytes(const skm_data *x, int k, bool extra) {
+    if (check_data(x, false) || check_k(x, k)) return 0;
+    Carver cv(nullptr, 0);
+    AssignBufs b;
+    plan_assign(x, k, cv, b);
+    if (extra) plan_assign_extra(x, k, cv, b.tc);
+    return cv.off < 256 ? 256 : cv.off;
+}
 
 // skm_lloyd_step_host's pruned ranges after the first: the tensor-core
 // front's centroid side (operand, records, sort, the centroids' moves) was

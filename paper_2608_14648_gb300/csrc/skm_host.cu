@@ -77,7 +77,9 @@ bool host_warm(const skm_step_host_config *cfg, const skm_data *x) {
     return cfg->warm && (x->repr == SKM_REPR_F32 || x->repr == SKM_REPR_BF16);
 }
 
-void plan_host(const skm_step_host_config *cfg, const skm_data *x, Carver &cv, HostBufs &b) {
+// extra: with the part of the assignments' workspaces that only makes small
+// ones faster; a workspace too small for it does without
+void plan_host(const skm_step_host_config *cfg, const skm_data *x, Carver &cv, HostBufs &b, bool extra = true) {
     const int64_t rc = cdiv(x->n, cfg->chunks);
     const int64_t rb = host_row_bytes(x);
     const int k = cfg->k, d = x->d;
@@ -98,7 +100,7 @@ void plan_host(const skm_step_host_config *cfg, const skm_data *x, Carver &cv, H
     skm_data probe = view_of(x, reinterpret_cast<const void *>(256), rc);
     if (host_warm(cfg, x)) probe.flags |= SKM_FLAG_WARM;
     if (cfg->prune) probe.flags |= SKM_FLAG_PRUNE;
-    b.ws_a_bytes = skm_workspace_size(0, &probe, k);
+    b.ws_a_bytes = assign_ws_bytes(&probe, k, extra);
     probe.flags = 0;
     b.ws_u_bytes = skm_workspace_size(1, &probe, k);
     // warm: one assignment workspace per range (each keeps its rows' bounds)
@@ -132,6 +134,10 @@ extern "C" int skm_lloyd_step_host(const skm_step_host_config *cfg, const skm_da
     Carver cv(ws, ws_bytes);
     HostBufs b;
     plan_host(cfg, x, cv, b);
+    if (!cv.fits()) {
+        cv = Carver(ws, ws_bytes);
+        plan_host(cfg, x, cv, b, false);
+    }
     if (b.ws_a_bytes == 0 || b.ws_u_bytes == 0) return SKM_ERR_INVALID_ARG;  // message set by skm_workspace_size
     if (fault_take(SKM_FAULT_WORKSPACE))
         return set_error(SKM_ERR_NO_MEMORY, "injected fault: workspace reported too small");

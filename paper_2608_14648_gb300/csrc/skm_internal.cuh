@@ -41,11 +41,11 @@ bool fault_take(int kind);
 // before, 1 after; nothing unless skm_kernel_timer enabled it)
 void tc_timer_mark(cudaStream_t st, int which);
 
+constexpr int MAX_D = 4096;  // dimensions of a point, at most
+
 // ---- workspace carving ------------------------------------------------------
 // Sub-buffers are carved from the caller's workspace at 256-byte boundaries.
 // With base == nullptr the carver only measures (used by skm_workspace_size).
-constexpr int MAX_D = 4096;  // dimensions of a point, at most
-
 struct Carver {
     char *base;
     size_t off = 0;
@@ -285,6 +285,9 @@ cudaError_t launch_prune_rows_cta(const uint16_t *X, int d, const float *C, int 
 // (hz = (max h', max z) of the front's centroid records); with kept bounds
 // that apply and force_cold == 0, the seed and a bound from the kept state
 // instead, without reading the points.
+// bytes of skm_assign's workspace, with or without the buffers at its end that
+// only make it faster (skm_abi.cu); 0: invalid arguments
+size_t assign_ws_bytes(const skm_data *x, int k, bool extra);
 // skm_lloyd_step_host's pruned ranges after the first (skm_abi.cu): the
 // tensor-core front on centroids prepared by the first range's call this step
 // (its workspace ws0, planned for x0); otherwise a plain skm_assign.
