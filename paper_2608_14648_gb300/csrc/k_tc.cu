@@ -1678,96 +1678,101 @@ __global__ void cprep_f32_kernel(const float *__restrict__ C, int k, int kp, int
     }
 }
 
-// The same records for calls that keep no bounds, in fp32: GB300 issues two fp64
-// lanes a clock and SM, and this kernel's few fp64 operations a value were its
-// time (1000 x 768: 16.6 us).  ||c||^2 is a double-float sum (error-free products
-// and TwoSums, about 2^-45 relative) rounded once; e and the bounds are rounded
-// upwards throughout, the fp32 sum of e^2 scaled up by its error bound first.
-// A centroid whose ||c||^2 leaves [2^-40, 2^100], where squares could
-// underflow unseen by the bounds or overflow, is done in fp64 as above.
-__device__ __forceinline__ void two_sum(float &hi, float &lo, float v) {
-    const float s = __fadd_rn(hi, v), bb = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(v, bb)));
-    hi = s;
+// The same records for calls that keep no bounds, the sums in fp32 operations:
+// GB300 issues two fp64 lanes a clock and SM, and this kernel's few fp64 operations
+// a value were its time (1000 x 768: 16.6 us).  Both sums are held as three floats
+// (error-free products and TwoSums; 2^-70 of the sum, against the 2^-53 of a
+// double), and only a lane's totals are fp64.  Products below 2^-100 are not
+// error-free: a centroid with ||c||^2 outside [2^-40, 2^100], or with so small a
+// sum of (c~ - c)^2 that those could count, is summed in fp64 as above.  The
+// bounds are formed from the fp64 sums by one warp for the block's centroids
+// side by side.
+struct Sum3 {
+    float a = 0.0f, b = 0.0f, c = 0.0f;
+    static __device__ __forceinline__ float two_sum(float &s, float v) {  // s += v; returns the rounding error
+        const float t = __fadd_rn(s, v), bb = __fsub_rn(t, s);
+        const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(v, bb));
+        s = t;
+        return err;
+    }
+    __device__ __forceinline__ void add_square(float v) {
+        const float p = __fmul_rn(v, v), q = __fmaf_rn(v, v, -p);
+        const float r = two_sum(b, two_sum(a, p));
+        c = __fadd_rn(c, __fadd_rn(r, two_sum(b, q)));
+    }
+    __device__ __forceinline__ double total() const { return __dadd_rn((double)a, __dadd_rn((double)b, (double)c)); }
+};
+// Sums over the warp of x (in the lower 16 lanes) and y (in the upper 16)
+__device__ __forceinline__ double warp_sum_pair(double x, double y, int lane) {
+    const bool up = (lane & 16) != 0;
+    double s = __dadd_rn(up ? y : x, __shfl_xor_sync(0xffffffffu, up ? x : y, 16));
+#pragma unroll
+    for (int w = 8; w > 0; w >>= 1) s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, w));
+    return s;
 }
-__global__ void cprep_cold_kernel(const float *__restrict__ C, int k, int kp, int d, int dp, int dr, float eps_acc,
-                                  float eps_s, const float *__restrict__ rho_max, __nv_bfloat16 *__restrict__ cs,
-                                  float4 *__restrict__ cinfo, float2 *__restrict__ cinfoz,
-                                  unsigned int *__restrict__ hz_bits) {
+constexpr int CC_WARPS = 8;
+__global__ void __launch_bounds__(32 * CC_WARPS) cprep_cold_kernel(
+    const float *__restrict__ C, int k, int kp, int d, int dp, int dr, float eps_acc, float eps_s,
+    const float *__restrict__ rho_max, __nv_bfloat16 *__restrict__ cs, float4 *__restrict__ cinfo,
+    float2 *__restrict__ cinfoz, unsigned int *__restrict__ hz_bits) {
     dep_sync();
-    const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
+    __shared__ double sums[2][CC_WARPS];  // ||c||^2 and ||c~ - c||^2 of the block's centroids
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float rho = *rho_max;
     float *cf = reinterpret_cast<float *>(cinfo);
     float *zf = reinterpret_cast<float *>(cinfoz);
-    for (int j = warp; j < kp; j += nw) {
-        const int pp = j >> 1, o = j & 1;
-        if (j >= k) {
-            if (lane == 0) {
-                cf[4 * pp + o] = INFINITY;
-                cf[4 * pp + 2 + o] = 0.0f;
-                zf[2 * pp + o] = 0.0f;
-            }
-            continue;
-        }
-        const float *src = C + (int64_t)j * d;
-        float hi = 0.0f, lo = 0.0f, e2 = 0.0f;
-        for (int i0 = lane; i0 - lane < dr; i0 += 32 * PREP_UNROLL) {
-            float v[PREP_UNROLL];
+    for (int j0 = blockIdx.x * CC_WARPS; j0 < kp; j0 += gridDim.x * CC_WARPS) {
+        if (j0 + warp < k) {  // warp-uniform
+            const int j = j0 + warp;
+            const float *src = C + (int64_t)j * d;
+            Sum3 c2, e2;
+            bool inexact = false;  // some c~ differs from c
+            for (int i0 = lane; i0 - lane < dr; i0 += 32 * PREP_UNROLL) {
+                float v[PREP_UNROLL];
 #pragma unroll
-            for (int u = 0; u < PREP_UNROLL; ++u) v[u] = i0 + 32 * u < dr ? __ldg(src + i0 + 32 * u) : 0.0f;
+                for (int u = 0; u < PREP_UNROLL; ++u) v[u] = i0 + 32 * u < dr ? __ldg(src + i0 + 32 * u) : 0.0f;
 #pragma unroll
-            for (int u = 0; u < PREP_UNROLL; ++u) {
-                const int i = i0 + 32 * u;
-                if (i >= dr) continue;
-                const __nv_bfloat16 cb = __float2bfloat16_rn(v[u]);
-                cs[(int64_t)j * dp + i] = cb;
-                const float e = __fsub_rn(__bfloat162float(cb), v[u]);
-                e2 = __fmaf_rn(e, e, e2);
-                const float p = __fmul_rn(v[u], v[u]);
-                lo = __fadd_rn(lo, __fmaf_rn(v[u], v[u], -p));
-                two_sum(hi, lo, p);
+                for (int u = 0; u < PREP_UNROLL; ++u) {
+                    const int i = i0 + 32 * u;
+                    if (i >= dr) continue;
+                    const __nv_bfloat16 cb = __float2bfloat16_rn(v[u]);
+                    cs[(int64_t)j * dp + i] = cb;
+                    const float e = __fsub_rn(__bfloat162float(cb), v[u]);  // exact
+                    inexact = inexact || e != 0.0f;
+                    e2.add_square(e);
+                    c2.add_square(v[u]);
+                }
             }
-        }
-#pragma unroll
-        for (int w = 16; w > 0; w >>= 1) {
-            e2 = __fadd_rn(e2, __shfl_xor_sync(0xffffffffu, e2, w));
-            const float h2 = __shfl_xor_sync(0xffffffffu, hi, w), l2 = __shfl_xor_sync(0xffffffffu, lo, w);
-            two_sum(hi, lo, h2);
-            lo = __fadd_rn(lo, l2);
-        }
-        float c2 = __fadd_rn(hi, lo), hf, zf1;
-        c2 = __shfl_sync(0xffffffffu, c2, 0);  // (one value decides the path for the warp)
-        const float up = 1.0f + 1e-6f;
-        if (c2 >= 0x1p-40f && c2 <= 0x1p100f) {
-            const float c2u = __fmul_ru(c2, up);
-            const float cn = __fsqrt_ru(c2u), e = sumsq_upper_norm(e2, (dr + 31) / 32 + 5);
-            const float g = __fadd_ru(cn, e);
-            hf = __fmul_ru(__fmaf_ru(rho, cn, __fmaf_ru(__fadd_ru(eps_acc, eps_s), g, e)), up);
-            zf1 = __fmul_ru(__fmul_ru(eps_s, c2u), up);
-        } else {
-            double c2d = 0.0, e2d = 0.0;
-            for (int i = lane; i < dr; i += 32) {
-                const double c = (double)src[i], t = (double)__bfloat162float(__float2bfloat16_rn(src[i])) - c;
-                c2d += c * c;
-                e2d += t * t;
+            inexact = __any_sync(0xffffffffu, inexact);
+            double s = warp_sum_pair(c2.total(), e2.total(), lane);
+            const bool ok = lane < 16 ? s >= 0x1p-40 && s <= 0x1p100 : s >= 0x1p-80 || (s == 0.0 && !inexact);
+            if (!__all_sync(0xffffffffu, ok)) {
+                double c2d = 0.0, e2d = 0.0;
+                for (int i = lane; i < dr; i += 32) {
+                    const double c = (double)src[i], t = (double)__bfloat162float(__float2bfloat16_rn(src[i])) - c;
+                    c2d += c * c;
+                    e2d += t * t;
+                }
+                s = warp_sum_pair(c2d, e2d, lane);
             }
-#pragma unroll
-            for (int w = 16; w > 0; w >>= 1) {
-                c2d += __shfl_xor_sync(0xffffffffu, c2d, w);
-                e2d += __shfl_xor_sync(0xffffffffu, e2d, w);
-            }
-            prep_bounds(c2d, e2d, (double)rho, eps_acc, eps_s, c2, hf, zf1);
+            if ((lane & 15) == 0) sums[lane >> 4][warp] = s;
         }
-        if (lane == 0) {
-            cf[4 * pp + o] = c2;
+        __syncthreads();
+        const int j = j0 + lane;
+        if (warp == 0 && lane < CC_WARPS && j < kp) {
+            float c2f = INFINITY, hf = 0.0f, zf1 = 0.0f;  // records past k: never the nearest
+            if (j < k) {
+                prep_bounds(sums[0][lane], sums[1][lane], (double)rho, eps_acc, eps_s, c2f, hf, zf1);
+                // maxima over the centroids (non-negative: bits order like values)
+                atomicMax(hz_bits, __float_as_uint(hf));
+                atomicMax(hz_bits + 1, __float_as_uint(zf1));
+            }
+            const int pp = j >> 1, o = j & 1;
+            cf[4 * pp + o] = c2f;
             cf[4 * pp + 2 + o] = hf;
             zf[2 * pp + o] = zf1;
-            // maxima over the centroids (non-negative: bits order like values)
-            atomicMax(hz_bits, __float_as_uint(hf));
-            atomicMax(hz_bits + 1, __float_as_uint(zf1));
         }
+        __syncthreads();  // sums is free again
     }
 }
 
