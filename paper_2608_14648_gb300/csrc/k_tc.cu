@@ -2436,13 +2436,9 @@ static void plan_codes(int64_t n, int d, int k, bool pk, Carver &cv, TcAssignBuf
     b.rpair_qn = cv.take<float4>(kp / 2);
 }
 
-bool tc_wide_ok(int repr, int d) {
-    return d > TC_RBQ1_MAX_D && ((repr == SKM_REPR_RBQ1 && rbq1_packed(d, nullptr)) ||
-                                 (repr == SKM_REPR_LVQ4 && lvq4_packed(d, nullptr)));
-}
-
-void tc_plan_wide(int repr, int64_t n, int d, int k, Carver &cv, TcAssignBufs &b) {
-    if (!tc_wide_ok(repr, d)) return;
+void tc_plan_wide(int repr, int64_t n, int d, int k, const void *x, Carver &cv, TcAssignBufs &b) {
+    static_assert(TC_RBQ1_MAX_D == TC_LVQ4_MAX_D, "the same line for both");
+    if (d <= TC_RBQ1_MAX_D || !tc_reads_packed(repr, d, x)) return;
     Carver t = cv;
     TcAssignBufs tb = b;
     plan_codes(n, d, k, true, t, tb);

@@ -208,7 +208,7 @@ static void plan_assign(const skm_data *x, int k, Carver &cv, AssignBufs &b) {
 // workspace that ends before them does without.
 static void plan_assign_extra(const skm_data *x, int k, Carver &cv, TcAssignBufs &b) {
     if (use_prune(x)) return;
-    tc_plan_wide(x->repr, x->n, x->d, k, cv, b);
+    tc_plan_wide(x->repr, x->n, x->d, k, x->x, cv, b);
     tc_plan_split(x->repr, x->n, k, cv, b);
 }
 

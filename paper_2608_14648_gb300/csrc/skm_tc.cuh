@@ -87,12 +87,12 @@ int tc_screen_prep(const skm_data *x, void *screen, cudaStream_t st);
 bool tc_reads_packed(int repr, int d, const void *x);
 void tc_plan(int repr, int64_t n, int d, int k, const void *x, const void *screen, bool warm, Carver &cv,
              TcAssignBufs &b);
-// 1-bit / LVQ4 codes with d > 1024 (tc_wide_ok: whole 16-byte rows; the address
-// must be 16-byte aligned too): the tensor-core path's buffers, after
-// everything else in a workspace.  They are left out (b.cs stays NULL, and the
-// CUDA-core kernel runs) when a given workspace ends before them.
-bool tc_wide_ok(int repr, int d);
-void tc_plan_wide(int repr, int64_t n, int d, int k, Carver &cv, TcAssignBufs &b);
+// 1-bit / LVQ4 codes with d > 1024 that can be read packed (whole 16-byte rows at
+// a 16-byte aligned address; none yet, NULL, counts as aligned): the tensor-core
+// path's buffers, after everything else in a workspace.  They are left out (b.cs
+// stays NULL, and the CUDA-core kernel runs) when a given workspace ends before
+// them.
+void tc_plan_wide(int repr, int64_t n, int d, int k, const void *x, Carver &cv, TcAssignBufs &b);
 // F32 / BF16 screens of few points: the buffer that lets several CTAs share a
 // point tile's centroids, likewise last and likewise left out when it does not fit.
 void tc_plan_split(int repr, int64_t n, int k, Carver &cv, TcAssignBufs &b);
