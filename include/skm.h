@@ -248,7 +248,7 @@ size_t skm_workspace_size(int op, const skm_data *x, int k);
  *   Y      out_dtype [n][d_out]: SKM_DTYPE_F32 (float) or SKM_DTYPE_BF16
  *          (bf16 bit patterns, rounded half to even from the fp32 result)
  * fp32 accuracy.  d_out <= d.  With a workspace of at least
- * skm_workspace_size(6, x = {n, d}, k = d_out) bytes the product runs on the
+ * skm_workspace_size(6, x = {n, d}, k = d_out) bytes, and n < 2^29, the product runs on the
  * tensor cores: x - mean and P are split into three bf16 parts each (x = x1 +
  * x2 + x3 exactly, each part the round-to-nearest bf16 of the remainder) and
  * the six products with i + j <= 4 are accumulated in fp32, the five small ones

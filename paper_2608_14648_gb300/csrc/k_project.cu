@@ -382,12 +382,12 @@ inline int round8(int d) { return (d + 7) & ~7; }
 
 }  // namespace
 
-// P's parts and the flag; the rest is what a 128-row slab of X's parts took
-// when they went through the workspace, kept so that the sizes callers have
-// still select the same path.
+// the flag and P's parts, as tc_project carves them
 size_t tc_project_ws_min(int d, int dout) {
-    const size_t dp = (size_t)round8(d);
-    return 256 + 3 * (size_t)dout * dp * 2 + 256 + 3 * (size_t)PM * dp * 2 + 256 + 64;
+    Carver cv(nullptr, 0);
+    cv.take<int32_t>(16);
+    cv.take<uint16_t>((size_t)PARTS * dout * round8(d));
+    return cv.off;
 }
 
 int tc_project(const float *X, int64_t n, int d, const float *mean, const float *P, int dout, int out_bf16, void *Y,
