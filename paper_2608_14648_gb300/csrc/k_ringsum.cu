@@ -784,7 +784,7 @@ struct Lvq4Cons {
     const int32_t *sperm;  // the run's points
     int e;
     unsigned long long *T;
-    int d, W, w0;  // w0: first word of the lane's range
+    int d, w0;  // w0: first word of the lane's range
     uint32_t alo[8 * NW], ahi[8 * NW];
     uint32_t pw[NW];  // the row waiting for a partner
     uint32_t psq;
@@ -930,7 +930,6 @@ __global__ void __launch_bounds__(RS_THREADS) direct_sum_lvq4_kernel(
     cons.e = e;
     cons.T = T;
     cons.d = d;
-    cons.W = WT;
     cons.w0 = w0;
     auto load = [&](int r, uint32_t(&x)[NW]) {
         const uint32_t *src = codes + (size_t)sperm[r] * WT + w0;
@@ -994,7 +993,10 @@ cudaError_t launch_float_nf(int nf, const void *X, int64_t n, int d, const int32
     const size_t smem = L.bytes();
     const unsigned g = ring_blocks(n, L.run);
 #define RS_CASE(NFV)                                                                                \
-    case NFV: {                                                                                     \
+    case NFV:                                                                                       \
+        if constexpr (BF16 && NFV <= 4) { /* those rows are summed by direct_sum_bf16_kernel */     \
+            return cudaErrorInvalidValue;                                                           \
+        } else {                                                                                    \
         auto kern = ring_sum_float_kernel<BF16, ACC, NFV>;                                          \
         cudaError_t e = smem_limit(kern, RS_SMEM_MAX);                                              \
         if (e != cudaSuccess) return e;                                                             \
@@ -1079,7 +1081,7 @@ cudaError_t launch_ring_sum_sq8(const uint8_t *codes, int64_t n, int d, const in
     const size_t smem = L.bytes();
     const unsigned g = ring_blocks(n, L.run);
     auto S64 = reinterpret_cast<unsigned long long *>(S);
-    const int q = (d / 16 + 31) / 32;  // 16-byte groups per lane
+    const int q = (d / 16 + 31) / 32;  // 16-byte groups per lane (3 or more past 1024)
     if (d <= 1024) {  // rows of at most 1 KB: straight into registers
         if (q <= 1)
             launch_dep(direct_sum_sq8_kernel<1>, g, RS_THREADS, 0, st, codes, d, perm, scl, offsets, k, S64, L.run);
@@ -1095,8 +1097,6 @@ cudaError_t launch_ring_sum_sq8(const uint8_t *codes, int64_t n, int d, const in
         launch_dep(kern, g, RS_THREADS, smem, st, codes, d, perm, scl, offsets, k, S64, L, flag);            \
         return launched();                                                                          \
     }
-    RS_CASE(1)
-    RS_CASE(2)
     RS_CASE(4)
     RS_CASE(8)
 #undef RS_CASE

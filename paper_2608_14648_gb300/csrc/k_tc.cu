@@ -279,23 +279,6 @@ __device__ __forceinline__ uint32_t pick32(const uint32_t (&v)[32], int i) {
     return (i & 1) ? w2[1] : w2[0];
 }
 
-__device__ __forceinline__ __attribute__((unused)) uint32_t pick16(const uint32_t (&v)[16], int i) {
-    uint32_t w8[8], w4[4], w2[2];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) w8[t] = (i & 8) ? v[t + 8] : v[t];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) w4[t] = (i & 4) ? w8[t + 4] : w8[t];
-#pragma unroll
-    for (int t = 0; t < 2; ++t) w2[t] = (i & 2) ? w4[t + 2] : w4[t];
-    return (i & 1) ? w2[1] : w2[0];
-}
-template <int N>
-__device__ __forceinline__ uint32_t pickn(const uint32_t (&v)[N], int i) {
-    if constexpr (N == 32)
-        return pick32(v, i);
-    else
-        return pick16(v, i);
-}
 
 // Instruction descriptors: D fp32, both operands K-major, N = 256, M = 128;
 // kind::f16 with A/B bf16, kind::f8f6f4 with A/B e4m3.
@@ -1043,7 +1026,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                     c1 = min(p.bn / st, whi > at ? (whi - at + st - 1) / st : 0);
                 };
                 if (MODE == MODE_SCREEN) {
-                    // chunks of SCR_CW columns (16: the next TMEM load in flight)
+                    // chunks of SCR_CW columns, one TMEM load each
                     constexpr int NC = SW / SCR_CW;
                     constexpr int G = SCR_CW / 8;
                     auto chunk = [&](uint32_t(&v)[SCR_CW], int c) {
@@ -1113,7 +1096,7 @@ __global__ void __launch_bounds__(tc_threads<NH, PK>(), 1)
                                 while (mask) {
                                     const int i = __ffs(mask) - 1;
                                     mask &= mask - 1;
-                                    screen_insert(sr, __uint_as_float(pickn<SCR_CW>(v, i)), j0 + i);
+                                    screen_insert(sr, __uint_as_float(pick32(v, i)), j0 + i);
                                 }
                             }
                         }
