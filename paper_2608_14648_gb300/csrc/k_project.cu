@@ -14,8 +14,8 @@
 //                accumulator, the five small ones into another, so that the
 //                small terms are not rounded at the size of the large one's sum
 //   warps 2 ..   epilogue: the two accumulators added once and written out
-// So X is read once and its parts never leave the SM.  1M x 1024 -> 256: 1.88
-// ms, bound by the six products (1.62 ms at the measured bf16 rate; X and Y
+// So X is read once and its parts never leave the SM.  1M x 1024 -> 256: 1.9 to
+// 2.0 ms, bound by the six products (1.62 ms at the measured bf16 rate; X and Y
 // take 0.68 ms at the copy bandwidth).  Split by a kernel of its own into 6
 // bytes a value that a GEMM kernel then read it took 2.02 + 1.92 ms.  The error
 // against 64 bits (relative 2-norm, embeddings, d = 256 .. 1536) is 2.3e-7 ..

@@ -2218,8 +2218,8 @@ int launch_tc_kind(const void *xs, int64_t n, int dp, int d, const void *cs, int
     // Few centroids (the meso pass of a hierarchical fit): a full tile's B loads
     // and MMAs would be mostly padding, repeated for each point tile, and its
     // second epilogue slice would idle.  1M x 768 against about 60 centroids:
-    // 1-bit codes packed 390 -> 225 us, from the copy 282 -> 131 us; LVQ4 packed
-    // 532 -> 406; fp32 643 -> 264; SQ8 d = 128, k = 100: 117 -> 88.  With more
+    // 1-bit codes packed 390 -> 217 us, from the copy 282 -> 131 us; LVQ4 packed
+    // 532 -> 404; fp32 643 -> 262; SQ8 d = 128, k = 100: 117 -> 74.  With more
     // tiles a narrow last one gives nothing (4M x 1024 against 3162, 90 columns
     // left: 7.35 -> 7.36 ms), and slices of a width known at run time cost 2 to
     // 15%, so all are BN wide there.
@@ -2637,6 +2637,14 @@ static int seg_setup(const TcSeg *seg, int64_t n, int k, TcParams &p, cudaStream
     // when groups have at most 96 on average (rounded out to 32 one mostly
     // fits; a larger one takes several jobs).  From 256-column tiles at fixed
     // places, 1M x 768 1-bit codes in 63 groups of about 63: 215 -> 142 us (read at 5.5 TB/s).
+    // The line: 500,000 x 768 from the copy in 63 groups of 0.6 to 1.4 times the average,
+    // us with 128 / 256 columns,
+    //   average       24        64        80        96       112       160
+    //   fp32     501/508   679/708   770/789   827/860   948/915 1354/1263
+    //   1-bit      93/96   114/116   123/120   139/132   151/134   188/153
+    //   SQ8      141/147   151/150   155/149   169/152   186/161   220/164
+    // (the screen crosses at about 100, where most of the time is at stake, the
+    // codes at about 70).
     p.bn = k <= 96LL * seg->nseg ? 128 : BN;
     const int64_t nrt = cdiv(n, BM);
     int64_t blocks = (nrt * 32 + 255) / 256;

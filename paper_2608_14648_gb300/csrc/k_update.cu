@@ -3,9 +3,10 @@
 //   1. histogram of assignments (shared-memory privatised counters),
 //   2. exclusive scan -> per-cluster offsets,
 //   3. scatter point ids (and their cluster) into cluster-contiguous order,
-//   4. fp32/bf16 and 1-bit: warps take equal runs of the sorted order and
-//      flush per-cluster register sums with global atomics (load balanced
-//      whatever the cluster sizes); SQ8: one CTA per cluster;
+//   4. warps take equal runs of the sorted order and flush per-cluster register
+//      sums with global atomics (load balanced whatever the cluster sizes);
+//      SQ8 rows of no multiple of 16 bytes, or not 16-byte aligned: one CTA
+//      per cluster;
 //   5. finalise: divide by the counts (or add into caller partial sums).
 // Integer representations accumulate in int64 and are exact, so their result
 // does not depend on the member order produced by the scatter.

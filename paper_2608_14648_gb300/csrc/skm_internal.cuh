@@ -64,10 +64,14 @@ struct Carver {
 // Kernels of a few microseconds that follow one another on a stream: with
 // programmatic stream serialization a kernel's blocks are placed while the
 // previous kernel still runs and wait at dep_sync for its end (and its writes),
-// so the launch gaps between them (2 to 3 us each) disappear.  Every kernel
-// launched this way calls dep_sync before anything else, in every thread, so
-// that each waits for its predecessor, that one for its own, and so on; kernels
-// launched normally wait for the end of everything before them, as ever.
+// so the launch gaps between them (2 to 3 us each) disappear.  In every kernel
+// launched this way every thread waits (dep_wait) before it reads or writes
+// anything that other kernels touch, so that each waits for its predecessor, that
+// one for its own, and so on; kernels launched normally wait for the end of
+// everything before them, as ever.  All but one wait first of all and let their
+// successor's blocks in at once (dep_sync); the tensor-core kernel sets up its
+// barriers and TMEM before the wait and lets successors in only after its TMEM is
+// allocated, so that the next such kernel cannot take it first.
 // Only grids of at most two blocks for each SM are placed early: a larger one
 // that fits the chip at once would be spread over whatever the previous kernel
 // leaves free instead of evenly (measured on the SQ8 sums of 1M x 1024 points:
