@@ -989,7 +989,7 @@ template <bool BF16, typename ACC>
 cudaError_t launch_float_nf(int nf, const void *X, int64_t n, int d, const int32_t *perm,
                             const int32_t *scl, const int64_t *offsets, int k, ACC *S, RingLayout L,
                             int32_t *flag, cudaStream_t st) {
-    L.run = sum_run(n, 16, sizeof(ACC) == 4 ? SUM_WARPS_F32 : SUM_WARPS);
+    L.run = sizeof(ACC) == 4 ? sum_run(n, k, 16, SUM_WARPS_F32, SUM_FLUSH_F32) : sum_run(n, k, 16, SUM_WARPS, SUM_FLUSH_F64);
     const size_t smem = L.bytes();
     const unsigned g = ring_blocks(n, L.run);
 #define RS_CASE(NFV)                                                                                \
@@ -1037,7 +1037,7 @@ cudaError_t launch_ring_sum_float(const void *X, int x_is_bf16, int64_t n, int d
                                   double *S_d, int32_t *flag, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     if (x_is_bf16 && direct_bf16_vec(X, d)) {
-        const int run = sum_run(n, 16, SUM_WARPS);
+        const int run = sum_run(n, k, 16, SUM_WARPS, SUM_FLUSH);
         const unsigned g = ring_blocks(n, run);
         const uint16_t *Xb = static_cast<const uint16_t *>(X);
         auto go = [&](auto fd, auto ff) {
@@ -1077,7 +1077,9 @@ cudaError_t launch_ring_sum_sq8(const uint8_t *codes, int64_t n, int d, const in
     if (n == 0) return cudaSuccess;
     RingLayout L;
     if (!ring_layout((uint32_t)d, L)) return cudaErrorInvalidValue;
-    L.run = sum_run(n, 16, SUM_WARPS);
+    // rows past 1 KB keep a warp busy for longer, and cost more atomics (100,000 x
+    // 4096, k = 100: 198 us with 16 warps, 182 with 4)
+    L.run = sum_run(n, k, 16, std::max(1, SUM_WARPS * std::min(1024, d) / d), SUM_FLUSH);
     const size_t smem = L.bytes();
     const unsigned g = ring_blocks(n, L.run);
     auto S64 = reinterpret_cast<unsigned long long *>(S);
@@ -1107,7 +1109,7 @@ template <int VEC>
 static cudaError_t launch_sum_rbq1_vec(const uint32_t *codes, int WT, const float *F, int e, int64_t n, int d,
                                        const int32_t *perm, const int32_t *scl, const int64_t *offsets, int k,
                                        unsigned long long *T, cudaStream_t st) {
-    const int run = sum_run(n, 32, SUM_WARPS);  // whole 32-row chunks
+    const int run = sum_run(n, k, 32, SUM_WARPS, SUM_FLUSH_RBQ1);  // whole 32-row chunks
     const int64_t per = (int64_t)TR_WARPS * run;
     const int gy = (WT + 31) / 32;                 // at most 32 words of a row in a thread's registers
     const int w4 = ((WT + gy - 1) / gy + 3) / 4;   // and the blocks' word ranges about equal
@@ -1149,7 +1151,8 @@ cudaError_t launch_sum_lvq4(const uint32_t *codes, const float4 *fac, int e, int
     if (n == 0) return cudaSuccess;
     const int W = lvq4_words(d);
     auto T64 = reinterpret_cast<unsigned long long *>(T);
-    const int run = sum_run(n, 16, SUM_WARPS);
+    // (as for SQ8, from 256 dimensions, a word a lane, on)
+    const int run = sum_run(n, k, 16, std::max(1, SUM_WARPS * std::min(256, d) / d), SUM_FLUSH);
     const dim3 g(ring_blocks(n, run), (unsigned)((W + 127) / 128));
 #define RS_CASE(NWV)                                                                                           \
     case NWV:                                                                                                  \

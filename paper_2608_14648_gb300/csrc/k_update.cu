@@ -461,7 +461,7 @@ cudaError_t launch_chunk_sum_float(const void *X, int x_is_bf16, int64_t n, int 
                                    const int64_t *offsets, int k, float *S_f, double *S_d,
                                    cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    const int run = sum_run(n, 16, SUM_WARPS);
+    const int run = sum_run(n, k, 16, SUM_WARPS, SUM_FLUSH_F32);
     const unsigned g = chunk_blocks(n, run);
     if (S_d) {
         if (x_is_bf16)

@@ -327,20 +327,31 @@ cudaError_t launch_sort_by_cluster(const int32_t *assign, int64_t n, int k, int3
                                    int64_t *offsets, int64_t *counts64, int accumulate, int32_t *perm, int32_t *scl,
                                    int64_t *zeros, int32_t *flag, void *sums, size_t sum_bytes, cudaStream_t st);
 // Load-balanced segmented sums over the cluster-sorted order (global atomics):
-// a warp sums a run of sum_run(n) consecutive positions.  A long run flushes
-// its sums less often; a short one keeps the GPU full when there are few
-// rows, since a run's rows are summed one after another (at n = 20,000 runs of
-// 128 rows are 157 warps, one per SM, for 66 us of an SQ8 update at d = 128).
-// So: the longest power of two that still gives `warps` warps an SM.  16
-// warps for the code sums (64-bit atomics: 200,000 x 384 SQ8 takes 60 us with
-// 16, 65 with 32, 74 with 64); 64 for fp32 rows, whose flush is one 16-byte
-// atomic per four columns (1M x 768: 510 us with 16, 483 with 64; 350,000 x
-// 100: 114 and 99).
+// a warp sums a run of sum_run consecutive positions.  A long run flushes its sums
+// less often; a short one keeps the GPU full when there are few rows, since a
+// run's rows are summed one after another (at n = 20,000 runs of 128 rows are 157
+// warps, one per SM, for 66 us of an SQ8 update at d = 128).  So: the longest
+// power of two that still gives `warps` warps an SM.  16 warps for the code sums
+// (64-bit atomics: 200,000 x 384 SQ8 takes 60 us with 16, 65 with 32, 74 with 64);
+// 64 for fp32 rows, whose flush is one 16-byte atomic per four columns (1M x 768:
+// 510 us with 16, 483 with 64; 350,000 x 100: 114 and 99).
+// With few clusters the flushes meet at the same addresses, n / (run k) at each,
+// one after another: run rows in a row cost as much as they do where run^2 k is
+// about n / flush, flush being the rows summed in the time of some flushes.  A run
+// is no shorter than that (us of an update with runs of 16, 32, 64, 128; rule *):
+//   SQ8  60,000 x 1024, k = 2        168   94   65*  62      flush 5
+//   LVQ4 60,000 x 4096, k = 2        451  207  127   92*     5
+//   bf16 60,000 x 128,  k = 8         74   46   40*  49      5
+//   bf16 60,000 x 128,  k = 1000      36*  33   40   53      5
+//   fp64 partial sums, 1-bit tables                          10, 20
+//   fp32 200,000 x 768, k = 2        169  133* 139  120      100 (16-byte atomics)
 constexpr int SUM_RUN_MAX = 128;
 constexpr int SUM_WARPS = 16, SUM_WARPS_F32 = 64;
-inline int sum_run(int64_t n, int least, int warps) {
+constexpr int SUM_FLUSH = 5, SUM_FLUSH_F64 = 10, SUM_FLUSH_RBQ1 = 20, SUM_FLUSH_F32 = 100;
+inline int sum_run(int64_t n, int k, int least, int warps, int flush) {
     int run = SUM_RUN_MAX;
     while (run > least && n < (int64_t)run * 152 * warps) run >>= 1;
+    while (run < SUM_RUN_MAX && (int64_t)run * run * k * flush < n) run <<= 1;
     return run;
 }
 cudaError_t launch_chunk_sum_float(const void *X, int x_is_bf16, int64_t n, int d,
