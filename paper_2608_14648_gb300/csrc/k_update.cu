@@ -57,67 +57,78 @@ cudaError_t launch_histogram(const int32_t *assign, int64_t n, int k, int32_t *c
 
 // --------------------------------------------------------------------- scan
 // Exclusive scan of the counts by one block of 1024 threads, count(j) giving
-// cluster j's members and put(j, offset) taking its offset; each thread has a
-// contiguous run of clusters.  Also the int64 counts, and the number of empty
-// clusters (zeros, may be NULL).
+// cluster j's members and put(j, offset) taking its offset.  Also the int64
+// counts, and the number of empty clusters (zeros, may be NULL).  Each warp has a
+// contiguous range of clusters and goes through it twice, for its sum and for the
+// offsets, 32 neighbours a step, so that reads and writes are contiguous (a range a
+// thread: 60,000 clusters 83 us when only offsets and counts were written, 113
+// with the cursors and the empty clusters too; now 31).
 template <typename Count, typename Put>
 __device__ __forceinline__ void scan_block(int k, Count count, Put put, int64_t *__restrict__ offsets,
                                            int64_t *__restrict__ counts64, int accumulate,
                                            int64_t *__restrict__ zeros) {
-    __shared__ int64_t wsum[32];
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int per = (k + blockDim.x - 1) / blockDim.x;
-    const int lo = min(k, t * per), hi = min(k, lo + per);
-    int64_t s = 0;
-    int z = 0;
-    for (int j = lo; j < hi; ++j) {
-        const int c = count(j);
-        s += c;
-        z += c == 0;
-    }
-    // exclusive scan of the threads' run sums: shuffles inside each warp, then
-    // the warp totals (exact integer sums, so any order gives the same offsets)
-    int64_t v = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int64_t u = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += u;
-    }
-    if (lane == 31) wsum[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        int64_t x = lane < (int)(blockDim.x >> 5) ? wsum[lane] : 0;
+    __shared__ int wsum[32], wzero[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int seg = (k + 1023) / 1024 * 32;
+    const int lo = min(k, w * seg), hi = min(k, lo + seg);
+    auto warp_incl = [&](int v) {
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int64_t u = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += u;
+            const int u = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += u;
         }
-        wsum[lane] = x;  // inclusive over warps
+        return v;
+    };
+    constexpr int U = 4;  // steps whose counts are read together
+    auto read = [&](int j0, int(&c)[U]) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int j = j0 + 32 * u + lane;
+            c[u] = j < hi ? count(j) : 0;
+        }
+    };
+    int s = 0, z = 0;  // (counts add up to fewer than 2^31)
+    for (int j0 = lo; j0 < hi; j0 += 32 * U) {
+        int c[U];
+        read(j0, c);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            s += c[u];
+            z += j0 + 32 * u + lane < hi && c[u] == 0;
+        }
+    }
+    s = __reduce_add_sync(0xffffffffu, s);
+    z = __reduce_add_sync(0xffffffffu, z);
+    if (lane == 0) {
+        wsum[w] = s;
+        wzero[w] = z;
     }
     __syncthreads();
-    int64_t run = v - s + (w > 0 ? wsum[w - 1] : 0);
-    if (t == (int)blockDim.x - 1) offsets[k] = run + s;
-    for (int j = lo; j < hi; ++j) {
-        const int c = count(j);
-        offsets[j] = run;
-        put(j, run);
-        run += c;
-        if (counts64) {
-            if (accumulate)
-                counts64[j] += c;
-            else
-                counts64[j] = c;
-        }
+    const int x = wsum[lane], xi = warp_incl(x);  // over the 32 warps, in each of them
+    int run = __shfl_sync(0xffffffffu, xi - x, w);
+    if (w == 0) {
+        z = __reduce_add_sync(0xffffffffu, wzero[lane]);
+        if (lane == 31) offsets[k] = xi;
+        if (zeros && lane == 0) *zeros = z;
     }
-    if (zeros) {
-        __syncthreads();  // wsum has been read
-        const int64_t zw = __reduce_add_sync(0xffffffffu, z);
-        if (lane == 0) wsum[w] = zw;
-        __syncthreads();
-        if (t == 0) {
-            int64_t tot = 0;
-            for (int i = 0; i < (int)(blockDim.x >> 5); ++i) tot += wsum[i];
-            *zeros = tot;
+    for (int j0 = lo; j0 < hi; j0 += 32 * U) {
+        int c[U];
+        read(j0, c);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int j = j0 + 32 * u + lane;
+            const int v = warp_incl(c[u]);
+            if (j < hi) {
+                offsets[j] = run + v - c[u];
+                put(j, run + v - c[u]);
+                if (counts64) {
+                    if (accumulate)
+                        counts64[j] += c[u];
+                    else
+                        counts64[j] = c[u];
+                }
+            }
+            run += __shfl_sync(0xffffffffu, v, 31);
         }
     }
 }
