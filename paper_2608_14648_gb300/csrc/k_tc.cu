@@ -1663,29 +1663,57 @@ __global__ void cprep_f32_kernel(const float *__restrict__ C, int k, int kp, int
 
 // The same records for calls that keep no bounds, the sums in fp32 operations:
 // GB300 issues two fp64 lanes a clock and SM, and this kernel's few fp64 operations
-// a value were its time (1000 x 768: 16.6 us).  Both sums are held as three floats
-// (error-free products and TwoSums; 2^-70 of the sum, against the 2^-53 of a
-// double), and only a lane's totals are fp64.  Products below 2^-100 are not
-// error-free: a centroid with ||c||^2 outside [2^-40, 2^100], or with so small a
-// sum of (c~ - c)^2 that those could count, is summed in fp64 as above.  The
-// bounds are formed from the fp64 sums by one warp for the block's centroids
-// side by side.
+// a value were its time (1000 x 768: 16.6 us, now 8).  Both sums are held as
+// three floats (error-free products and TwoSums; over up to 128 squares the error
+// was at most 2^-67 of the sum, that of an fp64 sum 2^-50).  Products below 2^-100
+// are not error-free: a centroid with ||c||^2 outside [2^-40, 2^100], or with so
+// small a sum of (c~ - c)^2 that those could count, is summed in fp64 as above.
+// The bounds are formed in fp64 by one warp for the block's centroids side by
+// side.
+// s += v; returns the rounding error (both sums at once: two IEEE operations an
+// instruction)
+__device__ __forceinline__ float2 two_sum2(float2 &s, float2 v) {
+    const float2 m1 = make_float2(-1.0f, -1.0f);
+    const float2 t = fadd2(s, v), bb = ffma2(s, m1, t);
+    const float2 err = fadd2(ffma2(ffma2(bb, m1, t), m1, s), ffma2(bb, m1, v));
+    s = t;
+    return err;
+}
+__device__ __forceinline__ float two_sum(float &s, float v) {
+    const float t = __fadd_rn(s, v), bb = __fsub_rn(t, s);
+    const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(v, bb));
+    s = t;
+    return err;
+}
 struct Sum3 {
-    float a = 0.0f, b = 0.0f, c = 0.0f;
-    static __device__ __forceinline__ float two_sum(float &s, float v) {  // s += v; returns the rounding error
-        const float t = __fadd_rn(s, v), bb = __fsub_rn(t, s);
-        const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(v, bb));
-        s = t;
-        return err;
-    }
-    __device__ __forceinline__ void add_square(float v) {
-        const float p = __fmul_rn(v, v), q = __fmaf_rn(v, v, -p);
-        const float r = two_sum(b, two_sum(a, p));
-        c = __fadd_rn(c, __fadd_rn(r, two_sum(b, q)));
+    float a, b, c;
+    __device__ __forceinline__ void merge(float a2, float b2, float c2) {
+        const float r = two_sum(b, two_sum(a, a2));
+        c = __fadd_rn(__fadd_rn(c, c2), __fadd_rn(r, two_sum(b, b2)));
     }
     __device__ __forceinline__ double total() const { return __dadd_rn((double)a, __dadd_rn((double)b, (double)c)); }
 };
-// Sums over the warp of x (in the lower 16 lanes) and y (in the upper 16)
+struct Sum3x2 {
+    float2 a = make_float2(0.0f, 0.0f), b = a, c = a;
+    __device__ __forceinline__ void add_squares(float2 v) {
+        const float2 p = fmul2(v, v), q = ffma2(v, v, fmul2(p, make_float2(-1.0f, -1.0f)));
+        const float2 r = two_sum2(b, two_sum2(a, p));
+        c = fadd2(c, fadd2(r, two_sum2(b, q)));
+    }
+};
+// Sums over the warp: the first in the lower 16 lanes, the second in the upper 16
+__device__ __forceinline__ Sum3 warp_sum_pair(const Sum3x2 &x, int lane) {
+    const bool up = (lane & 16) != 0;
+    Sum3 s = up ? Sum3{x.a.y, x.b.y, x.c.y} : Sum3{x.a.x, x.b.x, x.c.x};
+    const Sum3 o = up ? Sum3{x.a.x, x.b.x, x.c.x} : Sum3{x.a.y, x.b.y, x.c.y};
+    s.merge(__shfl_xor_sync(0xffffffffu, o.a, 16), __shfl_xor_sync(0xffffffffu, o.b, 16),
+            __shfl_xor_sync(0xffffffffu, o.c, 16));
+#pragma unroll
+    for (int w = 8; w > 0; w >>= 1)
+        s.merge(__shfl_xor_sync(0xffffffffu, s.a, w), __shfl_xor_sync(0xffffffffu, s.b, w),
+                __shfl_xor_sync(0xffffffffu, s.c, w));
+    return s;
+}
 __device__ __forceinline__ double warp_sum_pair(double x, double y, int lane) {
     const bool up = (lane & 16) != 0;
     double s = __dadd_rn(up ? y : x, __shfl_xor_sync(0xffffffffu, up ? x : y, 16));
@@ -1699,7 +1727,9 @@ __global__ void __launch_bounds__(32 * CC_WARPS) cprep_cold_kernel(
     const float *__restrict__ rho_max, __nv_bfloat16 *__restrict__ cs, float4 *__restrict__ cinfo,
     float2 *__restrict__ cinfoz, unsigned int *__restrict__ hz_bits) {
     dep_sync();
-    __shared__ double sums[2][CC_WARPS];  // ||c||^2 and ||c~ - c||^2 of the block's centroids
+    __shared__ float sums[2][CC_WARPS][3];  // ||c||^2 and ||c~ - c||^2 of the block's centroids,
+    __shared__ double sums64[2][CC_WARPS];  // or where these are not precise enough
+    __shared__ bool use64[CC_WARPS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float rho = *rho_max;
     float *cf = reinterpret_cast<float *>(cinfo);
@@ -1708,7 +1738,7 @@ __global__ void __launch_bounds__(32 * CC_WARPS) cprep_cold_kernel(
         if (j0 + warp < k) {  // warp-uniform
             const int j = j0 + warp;
             const float *src = C + (int64_t)j * d;
-            Sum3 c2, e2;
+            Sum3x2 c2e2;
             bool inexact = false;  // some c~ differs from c
             for (int i0 = lane; i0 - lane < dr; i0 += 32 * PREP_UNROLL) {
                 float v[PREP_UNROLL];
@@ -1722,30 +1752,40 @@ __global__ void __launch_bounds__(32 * CC_WARPS) cprep_cold_kernel(
                     cs[(int64_t)j * dp + i] = cb;
                     const float e = __fsub_rn(__bfloat162float(cb), v[u]);  // exact
                     inexact = inexact || e != 0.0f;
-                    e2.add_square(e);
-                    c2.add_square(v[u]);
+                    c2e2.add_squares(make_float2(v[u], e));
                 }
             }
             inexact = __any_sync(0xffffffffu, inexact);
-            double s = warp_sum_pair(c2.total(), e2.total(), lane);
-            const bool ok = lane < 16 ? s >= 0x1p-40 && s <= 0x1p100 : s >= 0x1p-80 || (s == 0.0 && !inexact);
-            if (!__all_sync(0xffffffffu, ok)) {
+            const Sum3 s = warp_sum_pair(c2e2, lane);
+            const bool ok = lane < 16 ? s.a >= 0x1p-40f && s.a <= 0x1p100f : s.a >= 0x1p-80f || (s.a == 0.0f && !inexact);
+            const bool wide = !__all_sync(0xffffffffu, ok);
+            if (wide) {
                 double c2d = 0.0, e2d = 0.0;
                 for (int i = lane; i < dr; i += 32) {
                     const double c = (double)src[i], t = (double)__bfloat162float(__float2bfloat16_rn(src[i])) - c;
                     c2d += c * c;
                     e2d += t * t;
                 }
-                s = warp_sum_pair(c2d, e2d, lane);
+                const double sd = warp_sum_pair(c2d, e2d, lane);
+                if ((lane & 15) == 0) sums64[lane >> 4][warp] = sd;
             }
-            if ((lane & 15) == 0) sums[lane >> 4][warp] = s;
+            if ((lane & 15) == 0) {
+                sums[lane >> 4][warp][0] = s.a;
+                sums[lane >> 4][warp][1] = s.b;
+                sums[lane >> 4][warp][2] = s.c;
+            }
+            if (lane == 0) use64[warp] = wide;
         }
         __syncthreads();
         const int j = j0 + lane;
         if (warp == 0 && lane < CC_WARPS && j < kp) {
             float c2f = INFINITY, hf = 0.0f, zf1 = 0.0f;  // records past k: never the nearest
             if (j < k) {
-                prep_bounds(sums[0][lane], sums[1][lane], (double)rho, eps_acc, eps_s, c2f, hf, zf1);
+                auto sum = [&](int i) {
+                    const float *f = sums[i][lane];
+                    return use64[lane] ? sums64[i][lane] : Sum3{f[0], f[1], f[2]}.total();
+                };
+                prep_bounds(sum(0), sum(1), (double)rho, eps_acc, eps_s, c2f, hf, zf1);
                 // maxima over the centroids (non-negative: bits order like values)
                 atomicMax(hz_bits, __float_as_uint(hf));
                 atomicMax(hz_bits + 1, __float_as_uint(zf1));
