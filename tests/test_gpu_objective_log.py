@@ -58,8 +58,10 @@ def test_objective_of_finished_iterations(skm):
     for attempt in range(12):
         got = {}
         t = threading.Thread(target=lambda: got.update(zip(("rc", "obj", "launches"), fit(50000))))
+        before = skm.skm_kernel_launches()
         t.start()
-        time.sleep(0.03 + 0.007 * attempt)
+        while t.is_alive() and skm.skm_kernel_launches() - before < first + 40 * per + 37 * attempt:
+            time.sleep(0.0002)
         skm.skm_inject_fault(LAUNCH, 1)
         t.join()
         assert got["rc"] == 3
